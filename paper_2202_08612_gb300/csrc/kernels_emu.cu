@@ -1,0 +1,586 @@
+// FP64-accurate contractions on the BF16 tensor cores (sm_103a), after the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump: an operand is an
+// integer of up to 63 bits per element (its value over one power of two), held
+// as S balanced base-256 digits, each exact in bfloat16.  Products of digits
+// are integers of at most 2^14, which FP32 sums exactly over 256 of them for
+// the digit degrees t + u <= 3; degrees of S and more are dropped.
+//
+// GB300 retires about two FP64 operations per clock and SM (1.1 TFLOP/s in
+// all), and BF16 on the tensor cores about 1.7 PFLOP/s, so even the 36 digit
+// products of S = 8 leave room for a factor of some twenty over the FP64 pipe.
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "kernels_emu.cuh"
+#include "tc_ptx.cuh"
+
+namespace mlcc3 {
+
+namespace {
+
+constexpr int kChain = 256 / kEmuKB;  // chunks per TMEM accumulation chain (exact up to 256 products)
+constexpr int kRowB = 2 * kEmuKB;     // bytes of a shared-memory operand row
+
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                            int c2, int c3, int c4, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+      : "memory");
+}
+
+// K-major operand, 64-byte rows with the 64-byte swizzle, 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc64(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr >> 4) & 0x3FFF);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)((8 * kRowB) >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;  // SWIZZLE_64B
+  return d;
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// T 2^e (+-), rounded to binary64 on the integer pipe (an FP64 conversion costs
+// one of the two FP64 operations an SM retires per clock).
+__device__ __forceinline__ double int_to_double(long long T, int e) {
+  if (T == 0) return 0.0;
+  const unsigned long long sgn = (unsigned long long)T & (1ULL << 63);
+  unsigned long long u = T < 0 ? 0ULL - (unsigned long long)T : (unsigned long long)T;
+  const int lz = __clzll(u);
+  u <<= lz;
+  const int ex = e - lz + 63 + 1023;  // biased exponent of the leading bit
+  if (ex < 1 || ex > 2045) return ldexp((double)T, e);
+  const unsigned long long m = (u >> 11) + ((u >> 10) & 1);
+  return __longlong_as_double((long long)((((unsigned long long)(ex - 1) << 52) + m) | sgn));
+}
+
+__device__ __forceinline__ int scale_exp(EmuScale s) { return (int)((s >> 52) & 0x7ff) - 1022; }
+
+}  // namespace
+
+// One 128 x n tile of C = sum_segments A_seg B_seg^T per item, persistent (one
+// CTA per SM, item i to CTA i mod gridDim.x).
+//
+// A stage holds 32 K elements of all S slices of both operands.  The slices of
+// B lie one below the other in shared memory, so the MMA of A's slice t with
+// the stacked slices 0 .. S-1-t of B (N = (S - t) n, in pieces of at most 256)
+// puts digit pair (t, u) into TMEM columns (t + u) n: one accumulator per digit
+// degree and wide MMAs instead of S (S + 1) / 2 narrow ones.  With S = 8 and
+// n = 64 the eight degrees fill TMEM; a stage is 96 KB, two are in flight.
+//
+// After each chain of 256 K elements eight epilogue warps add the degrees,
+// weighted by 2^-8d, into 64-bit integers in registers (degrees 0..4 exactly, in
+// units of 2^-32: below 2^60 for kEmuMaxK products; the higher ones in FP32 beside
+// them) and hand TMEM back, so the next chain's MMAs wait only for the reads.  An item's sums are rounded to binary64
+// once, at its end, on the integer pipe.
+//   warp 0 lane 0: TMA producer; warp 1: TMEM, lane 0 issues; warps 2..9: epilogue
+// C = A B^T with M = N = K = 4096 and S = 5, slicing included: 2.64 ms, against
+// 8.26 ms with one launch of the split mode's kernel per digit degree (two of its
+// three products on zeros, and an FP64 reduction per output, pair and 1024 products).
+template <int S>
+__global__ void __launch_bounds__(320, 1)
+    emu_gemm_kernel(const __grid_constant__ TcMaps maps, const TcItem *__restrict__ items,
+                    const TcSeg *__restrict__ segs, int nitems, int stages, const EmuEpi epi,
+                    int *__restrict__ status) {
+  constexpr int NG = emu_max_cols(S) / 16;  // 8-column groups per epilogue thread
+  constexpr int A_SL = 128 * kRowB;         // bytes of one slice of A
+  constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *smem = reinterpret_cast<unsigned char *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int n = epi.n;
+  const int stage_bytes = S * (A_SL + n * kRowB);
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 8);
+  const uint32_t tfull = smem_u32(bars + 16), tempty = smem_u32(bars + 17);
+  const uint32_t done = smem_u32(bars + 18);
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 19);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const uint32_t ncols = S * n <= 128 ? 128u : S * n <= 256 ? 256u : 512u;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    mbar_init(tfull, 1);
+    mbar_init(tempty, 8);
+    mbar_init(done, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    // ---- TMA producer ----
+    int stage = 0;
+    uint32_t phase = 0, last = 0, pending = 0;
+    for (int i = blockIdx.x; i < nitems && !*abort_flag; i += gridDim.x) {
+      const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
+      for (int q = s0; q < s1 && !*abort_flag; ++q) {
+        const TcSeg sg = segs[q];
+        for (int kc = 0; kc < sg.nk; ++kc) {
+          if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, status, epi.wait)) {
+            *abort_flag = 1;
+            break;
+          }
+          const uint32_t st = smem_u32(smem + stage * stage_bytes), fb = full0 + 8 * stage;
+          mbar_expect_tx(fb, (uint32_t)stage_bytes);
+          tma_load_5d(st, &maps.m[sg.amap], sg.ac[0] + kEmuKB * kc, sg.ac[1], sg.ac[2], sg.ac[3], 0, fb);
+          tma_load_5d(st + S * A_SL, &maps.m[sg.bmap], sg.bc[0] + kEmuKB * kc, sg.bc[1], sg.bc[2],
+                      sg.bc[3], 0, fb);
+          last = (last & ~(1u << stage)) | (phase << stage);
+          pending |= 1u << stage;
+          if (++stage == stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+      }
+    }
+    // the shared memory must outlive every copy issued into it
+    for (int s = 0; s < stages; ++s)
+      if ((pending >> s) & 1u) mbar_wait(full0 + 8 * s, (last >> s) & 1u, status, kTcWaitDefault);
+  } else if (warp == 1 && lane == 0) {
+    // ---- MMA issuer ----
+    int stage = 0;
+    uint32_t phase = 0;
+    int t = 0;  // accumulation chains so far
+    bool ok = true;
+    for (int i = blockIdx.x; i < nitems && ok && !*abort_flag; i += gridDim.x) {
+      const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
+      int total = 0;
+      for (int q = s0; q < s1; ++q) total += segs[q].nk;
+      for (int c = 0; c < total; ++c) {
+        const int cc = c % kChain;
+        if (cc == 0) {
+          if (!mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait)) {
+            *abort_flag = 1;
+            ok = false;
+            break;
+          }
+        }
+        if (!mbar_wait(full0 + 8 * stage, phase, status, epi.wait)) {
+          *abort_flag = 1;
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t a0 = smem_u32(smem + stage * stage_bytes), b0 = a0 + S * A_SL;
+#pragma unroll
+        for (int kk = 0; kk < kEmuKB / 16; ++kk) {
+#pragma unroll
+          for (int d = 0; d < S; ++d) {
+            // slice d of A with the stacked slices 0 .. S-1-d of B; the first
+            // MMA of a chain (d = 0) covers every degree and clears them
+            const uint64_t ad = smem_desc64(a0 + d * A_SL + kk * 32);
+            const uint32_t acc = (cc > 0 || kk > 0 || d > 0) ? 1u : 0u;
+            const int cols = (S - d) * n;
+            for (int c0 = 0; c0 < cols; c0 += 256) {
+              const int nn = min(256, cols - c0);
+              mma_bf16(tmem + (uint32_t)(d * n + c0), ad, smem_desc64(b0 + c0 * kRowB + kk * 32),
+                       IDESC | ((uint32_t)(nn >> 3) << 17), acc);
+            }
+          }
+        }
+        mma_commit(empty0 + 8 * stage);
+        if (++stage == stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
+        if (cc == kChain - 1 || c == total - 1) {
+          mma_commit(tfull);
+          ++t;
+        }
+      }
+    }
+    mma_commit(done);
+  } else if (warp >= 2) {
+    // ---- epilogue ----
+    const int lg = warp & 3, half = (warp - 2) >> 2;
+    const int row = lg * 32 + lane, hn = n / 2;
+    const uint32_t tm = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(half * hn);
+    int e0 = epi.ebias - 32;
+    if (epi.sa) e0 += scale_exp(*epi.sa) + scale_exp(*epi.sb);
+    int t = 0;
+    bool ok = true;
+    for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+      if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
+      const TcItem it = items[i];
+      int total = 0;
+      for (int q = 0; q < it.seg_count; ++q) total += segs[it.seg_begin + q].nk;
+      const int chains = (total + kChain - 1) / kChain;
+      long long T[NG * 8];
+      float L[S > 5 ? NG * 8 : 1];
+      unsigned nan[NG];
+#pragma unroll
+      for (int g = 0; g < NG; ++g) {
+        nan[g] = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          T[g * 8 + j] = 0;
+          if constexpr (S > 5) L[g * 8 + j] = 0.f;
+        }
+      }
+      for (int ch = 0; ch < chains; ++ch, ++t) {
+        // the whole warp goes on or leaves: the TMEM reads are warp collectives
+        if (!__all_sync(0xffffffffu, mbar_wait(tfull, (uint32_t)t & 1u, status, epi.wait))) {
+          *abort_flag = 1;
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+          if (g * 8 < hn) {
+            uint32_t r[S][8];
+#pragma unroll
+            for (int d = 0; d < S; ++d) tmem_ld8(tm + (uint32_t)(d * n + g * 8), r[d]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float f0 = __uint_as_float(r[0][j]);
+              if (!(f0 == f0)) nan[g] |= 1u << j;
+              long long x = T[g * 8 + j];
+              x += (long long)((unsigned long long)(uint32_t)__float2int_rn(f0) << 32);
+#pragma unroll
+              for (int d = 1; d < (S < 5 ? S : 5); ++d)
+                x += (long long)__float2int_rn(__uint_as_float(r[d][j])) * (1LL << (32 - 8 * d));
+              T[g * 8 + j] = x;
+              if constexpr (S > 5) {
+                float l = __uint_as_float(r[S - 1][j]);
+#pragma unroll
+                for (int d = S - 2; d >= 5; --d) l = fmaf(l, 0x1p-8f, __uint_as_float(r[d][j]));
+                L[g * 8 + j] += l;
+              }
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+      }
+      if (!ok) break;
+      int r1, r2;
+      if (epi.linear) {
+        const int m = it.r2_0 + row;
+        r1 = m / epi.R2;
+        r2 = m % epi.R2;
+      } else {
+        r1 = it.r1_0 + row / epi.R2;
+        r2 = it.r2_0 + row % epi.R2;
+      }
+      const int cmax = r1 < epi.lim1 && r2 < epi.lim2 ? epi.nlim : 0;
+      const int c0 = it.c0 + half * hn;
+      const int er = epi.ea && cmax ? e0 + epi.ea[it.r2_0 + row] : e0;
+      double *o = epi.out + it.out_off + (long long)r1 * epi.s1 + (long long)r2 * epi.s2 + (long long)c0 * epi.sn;
+#pragma unroll
+      for (int g = 0; g < NG; ++g) {
+        if (g * 8 >= hn) continue;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int c = g * 8 + j;
+          if (c0 + c >= cmax) break;
+          long long x = T[c];
+          int ex = epi.eb ? er + epi.eb[c0 + c] : er;
+          if constexpr (S > 5) {
+            // T moved up as far as it goes, so that the higher degrees (|L| < 2^30,
+            // in 2^-8 of T's unit) join it below its own 53 leading bits
+            const int sh = min(24, __clzll(x < 0 ? -x : x) - 2);
+            x = (x << sh) + __float2ll_rn(L[c] * __int_as_float((127 + sh - 8) << 23));
+            ex -= sh;
+          }
+          double v = int_to_double(x, ex);
+          if ((nan[g] >> j) & 1u) v = __longlong_as_double(0x7ff8000000000000LL);
+          if (epi.alpha != 1.0) v = epi.alpha == -1.0 ? -v : epi.alpha * v;
+          double *p = o + (long long)c * epi.sn;
+          if (epi.mode == 0) *p = v;
+          else atomicAdd(p, v);
+        }
+      }
+      __syncwarp();
+    }
+  }
+  if (warp == 1 && lane == 0) mbar_wait(done, 0, status, kTcWaitDefault);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols)
+                 : "memory");
+  }
+}
+
+int emu_tile_width(long long n, int S) {
+  const long long w = emu_max_cols(S), tiles = (n + w - 1) / w;
+  const long long c = tiles ? (n + tiles - 1) / tiles : 16;
+  return (int)std::max(16LL, (c + 15) / 16 * 16);
+}
+
+bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long dims[4],
+                    const unsigned long long strides[3], unsigned long long slice_bytes,
+                    const unsigned box[3], int S, std::string *err) {
+  static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess)
+      fn = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  }();
+  if (!encode) {
+    *err = "cuTensorMapEncodeTiled is not available";
+    return false;
+  }
+  cuuint64_t gd[5] = {dims[0], dims[1], dims[2], dims[3], (cuuint64_t)S};
+  cuuint64_t gs[4] = {strides[0], strides[1], strides[2], slice_bytes};
+  cuuint32_t bx[5] = {kEmuKB, box[0], box[1], box[2], (cuuint32_t)S};
+  cuuint32_t es[5] = {1, 1, 1, 1, 1};
+  CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), gd, gs, bx, es,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    *err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
+    return false;
+  }
+  return true;
+}
+
+template <int S>
+static cudaError_t launch_s(const TcMaps &maps, const TcItem *items, const TcSeg *segs, int nitems,
+                            const EmuEpi &epi, int *status, cudaStream_t st) {
+  const int stage = S * (128 + epi.n) * kRowB;
+  const int stages = std::max(2, std::min(6, (220 * 1024) / stage));
+  const int smem = 1024 + stages * stage + 256;
+  cudaError_t e = cudaFuncSetAttribute(emu_gemm_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  emu_gemm_kernel<S><<<std::min(nitems, 152), 320, smem, st>>>(maps, items, segs, nitems, stages, epi, status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, const TcSeg *segs,
+                            int nitems, const EmuEpi &epi, int *status, cudaStream_t st) {
+  if (nitems <= 0) return cudaSuccess;
+  if (epi.n < 16 || epi.n % 16 || epi.n > emu_max_cols(S)) return cudaErrorInvalidValue;
+  switch (S) {
+    case 2: return launch_s<2>(maps, items, segs, nitems, epi, status, st);
+    case 3: return launch_s<3>(maps, items, segs, nitems, epi, status, st);
+    case 4: return launch_s<4>(maps, items, segs, nitems, epi, status, st);
+    case 5: return launch_s<5>(maps, items, segs, nitems, epi, status, st);
+    case 6: return launch_s<6>(maps, items, segs, nitems, epi, status, st);
+    case 8: return launch_s<8>(maps, items, segs, nitems, epi, status, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// ---- scales ----
+__global__ void __launch_bounds__(256) emu_absmax_kernel(const double *__restrict__ x, long long n,
+                                                         EmuScale *scale) {
+  const EmuScale inf = 0x7ffULL << 52;
+  EmuScale m = 0;
+  const long long step = (long long)gridDim.x * 256;
+  long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  for (; i + 3 * step < n; i += 4 * step) {
+    EmuScale b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      b[q] = (EmuScale)__double_as_longlong(x[i + q * step]) & ~(1ULL << 63);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (b[q] < inf && b[q] > m) m = b[q];
+  }
+  for (; i < n; i += step) {
+    const EmuScale b = (EmuScale)__double_as_longlong(x[i]) & ~(1ULL << 63);
+    if (b < inf && b > m) m = b;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const EmuScale b = __shfl_xor_sync(0xffffffffu, m, o);
+    if (b > m) m = b;
+  }
+  __shared__ EmuScale red[8];
+  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w)
+      if (red[w] > m) m = red[w];
+    if (m) atomicMax(scale, m);
+  }
+}
+
+cudaError_t emu_absmax(const double *x, long long n, EmuScale *scale, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  const long long g = std::min<long long>((n + 2047) / 2048, 152LL * 8);
+  emu_absmax_kernel<<<(int)std::max(1LL, g), 256, 0, st>>>(x, n, scale);
+  return cudaGetLastError();
+}
+
+__global__ void emu_balance_kernel(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u) {
+  const int eg = scale_exp(*g), et = scale_exp(*t);
+  const int ea = max(scale_exp(*a), et + scale_exp(*u) - eg), eu = ea + eg - et;
+  auto pack = [](int e) { return (EmuScale)min(2046, max(0, e + 1022)) << 52; };
+  *a = pack(ea);
+  *u = pack(eu);
+}
+
+cudaError_t emu_balance(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u, cudaStream_t st) {
+  emu_balance_kernel<<<1, 1, 0, st>>>(a, g, t, u);
+  return cudaGetLastError();
+}
+
+__global__ void emu_scale_double_kernel(EmuScale *s) {
+  *s = (EmuScale)min(2046, scale_exp(*s) + 1023) << 52;
+}
+
+cudaError_t emu_scale_double(EmuScale *scale, cudaStream_t st) {
+  emu_scale_double_kernel<<<1, 1, 0, st>>>(scale);
+  return cudaGetLastError();
+}
+
+// ---- digits ----
+// x over 2^(e - 62), rounded to nearest: an integer of at most 62 bits for |x| < 2^e.
+__device__ __forceinline__ long long to_fixed62(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  int ex = (int)((b >> 52) & 0x7ff);
+  unsigned long long m = b & ((1ULL << 52) - 1);
+  if (ex) m |= 1ULL << 52;
+  else ex = 1;
+  const int s = ex - 1013 - e;  // m 2^(ex - 1075) 2^(62 - e)
+  unsigned long long q;
+  if (s >= 0) q = m << min(s, 9);
+  else if (s > -55) q = (m + (1ULL << (-s - 1))) >> -s;
+  else q = 0;
+  return (b >> 63) ? -(long long)q : (long long)q;
+}
+
+// Tiles of 32 rows x 64 K elements pass through shared memory, so that the loads
+// run along whichever index is contiguous in the source; each thread then makes
+// the digits of eight consecutive K elements of a row and writes 16 bytes of
+// every slice.  The digits of the 62-bit integer q are the bytes of
+// q + 0x0080..80, minus 128 each (the top byte: q's own, in [-64, 64]); a byte
+// becomes a bfloat16 through the FP32 number 2^23 + byte.  Bound by HBM: 8 bytes
+// read and 16 written per element.
+__global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp, long long slice,
+                                                         int neg, const EmuScale *scale,
+                                                         __nv_bfloat16 *__restrict__ out,
+                                                         const double *__restrict__ F, double fcoef,
+                                                         int swap) {
+  __shared__ double sm[32][65];
+  __shared__ long long ro[32], ko[64];
+  const int e = scale_exp(*scale), tid = threadIdx.x;
+  const int tr = (v.R + 31) / 32, tk = (Kp + 63) / 64;
+  const long long tiles = (long long)v.Z * tr * tk;
+  const bool kfast = v.K2 > 1 ? v.sk2 == 1 : v.sk1 == 1;
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int kt = (int)(t % tk);
+    const long long t2 = t / tk;
+    const int rt = (int)(t2 % tr), z = (int)(t2 / tr);
+    const int r0 = rt * 32, k0 = kt * 64;
+    __syncthreads();
+    if (tid < 32) {
+      const int r = r0 + tid;
+      ro[tid] = r < v.R ? (long long)(r / v.R2) * v.sr1 + (long long)(r % v.R2) * v.sr2 : -1;
+    } else if (tid < 96) {
+      const int k = k0 + tid - 32;
+      ko[tid - 32] = k < v.K ? (long long)(k / v.K2) * v.sk1 + (long long)(k % v.K2) * v.sk2 : -1;
+    }
+    __syncthreads();
+    const double *src = v.x + (long long)(z / v.Z2) * v.sz1 + (long long)(z % v.Z2) * v.sz2;
+    double x[8];
+    int rr[8], kk[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int el = tid + 256 * q;
+      if (kfast) {
+        kk[q] = el % 64;
+        rr[q] = el / 64;
+      } else {
+        rr[q] = el % 32;
+        kk[q] = el / 32;
+      }
+      const long long a = ro[rr[q]], b = ko[kk[q]];
+      x[q] = (a >= 0 && b >= 0) ? src[a + b] : 0.0;
+      if (F && a >= 0 && b >= 0) {
+        const int k = k0 + kk[q], i1 = k / v.K2, i2 = k % v.K2;
+        const int bi = swap ? i2 : i1, ci = swap ? i1 : i2;
+        if (bi == r0 + rr[q]) x[q] += fcoef * F[(long long)z * v.K2 + ci];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sm[rr[q]][kk[q]] = x[q];
+    __syncthreads();
+    const int r = tid / 8, kg = (tid % 8) * 8;
+    if (r0 + r < v.R && k0 + kg < Kp) {
+      unsigned lo[8], hi[8];
+      unsigned bad = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        double y = sm[r][kg + j];
+        if (!(fabs(y) <= 1.7976931348623157e308)) {
+          bad |= 1u << j;
+          y = 0.0;
+        }
+        long long q = to_fixed62(y, e);
+        if (neg) q = -q;
+        const unsigned long long w =
+            ((unsigned long long)q + 0x0080808080808080ULL) ^ 0x8000000000000000ULL;
+        lo[j] = (unsigned)w;
+        hi[j] = (unsigned)(w >> 32);
+      }
+      uint4 *o = reinterpret_cast<uint4 *>(out + ((long long)z * v.R + r0 + r) * Kp + k0 + kg);
+      const long long st = slice / 8;  // uint4 units
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        unsigned p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const unsigned wa = s < 4 ? hi[2 * j] : lo[2 * j], wb = s < 4 ? hi[2 * j + 1] : lo[2 * j + 1];
+          const unsigned sel = 0x7440u | (unsigned)(3 - (s & 3));  // byte, 0, 0, 0x4B
+          const float fa = __uint_as_float(__byte_perm(wa, 0x4B000000u, sel)) - 8388736.f;
+          const float fb = __uint_as_float(__byte_perm(wb, 0x4B000000u, sel)) - 8388736.f;
+          p[j] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+        }
+        if (s == 0 && bad) {  // a non-finite element makes its products NaN
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if ((bad >> j) & 1u) p[j / 2] = (p[j / 2] & (j & 1 ? 0x0000ffffu : 0xffff0000u)) | (j & 1 ? 0x7fc00000u : 0x7fc0u);
+        }
+        o[s * st] = make_uint4(p[0], p[1], p[2], p[3]);
+      }
+    }
+  }
+}
+
+cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale,
+                       __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
+                       cudaStream_t st) {
+  if (v.Z <= 0 || v.R <= 0 || Kp <= 0) return cudaSuccess;
+  const long long tiles = (long long)v.Z * ((v.R + 31) / 32) * ((Kp + 63) / 64);
+  const long long slice = (long long)v.Z * v.R * Kp;
+  emu_digits_kernel<<<(int)std::min<long long>(tiles, 152LL * 32), 256, 0, st>>>(
+      v, (int)Kp, slice, neg ? 1 : 0, scale, out, F, fcoef, swap ? 1 : 0);
+  return cudaGetLastError();
+}
+
+}  // namespace mlcc3

@@ -1,0 +1,77 @@
+// FP64-accurate contractions on the BF16 tensor cores: operands as balanced
+// base-256 digit slices (exact in bfloat16), every digit pair of one K chunk
+// multiplied in one pipeline stage, integer accumulation outside TMEM.
+#pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <string>
+
+#include "kernels_tc.cuh"
+
+namespace mlcc3 {
+
+constexpr int kEmuKB = 32;      // K elements per pipeline stage (64-byte rows)
+constexpr int kEmuSlices = 8;   // digit slices of the FP64 mode
+constexpr int kEmuMaxK = 8192;  // longest reduction of one item (TcSeg chunks times kEmuKB)
+
+// A digit operand's scale: the binary64 pattern of the operand's largest finite
+// magnitude (or of any number at least as large); |x| < 2^e with e its exponent.
+using EmuScale = unsigned long long;
+
+// Epilogue: out[off + r1 s1 + r2 s2 + n sn] (op) alpha sum_k A[r][k] B[n][k].
+// mode 0: store; 1: add (global reductions).  The rest as in TcEpi.
+struct EmuEpi {
+  double *out;
+  int mode;
+  int R2, linear;
+  long long s1, s2, sn;
+  int lim1, lim2, nlim;
+  double alpha;
+  int n;            // columns of a tile (a multiple of 16, at most emu_max_cols)
+  int ebias;        // power of two of the leading digit product: -12 (emu_digits), -14 (full leading digits)
+  // scales: one per operand (sa, sb), or one exponent per output row and column
+  const EmuScale *sa, *sb;
+  const int *ea, *eb;
+  long long wait;   // as TcEpi::wait
+};
+
+// Widest tile of an S-slice launch: S n FP32 columns fit in TMEM's 512 and
+// n / 2 accumulators per epilogue thread in its registers.
+__host__ __device__ constexpr int emu_max_cols(int S) { return S >= 7 ? 64 : 80; }
+int emu_tile_width(long long n, int S);
+
+// Tensor map of a digit operand over (K, dims1, dims2, dims3, slice); strides in
+// bytes for dims 1..3 and the slice.
+bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long dims[4],
+                    const unsigned long long strides[3], unsigned long long slice_bytes,
+                    const unsigned box[3], int S, std::string *err);
+
+cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, const TcSeg *segs,
+                            int nitems, const EmuEpi &epi, int *status, cudaStream_t st);
+
+// *scale = max(*scale, largest finite |x|)
+cudaError_t emu_absmax(const double *x, long long n, EmuScale *scale, cudaStream_t st);
+// Scales of the two products of Eq. R3 made equal: A G and t U accumulate in one
+// chain, so e_A + e_G = e_t + e_U; e_A and e_U are raised where they have to be.
+cudaError_t emu_balance(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u,
+                        cudaStream_t st);
+// *scale = twice the power of two that bounds it
+cudaError_t emu_scale_double(EmuScale *scale, cudaStream_t st);
+
+// Source of a digit operand: element (z, r, k) at z1 sz1 + z2 sz2 + r1 sr1 +
+// r2 sr2 + k1 sk1 + k2 sk2 with z = z1 Z2 + z2 and so on.
+struct EmuView {
+  const double *x;
+  int Z, Z2, R, R2, K, K2;
+  long long sz1, sz2, sr1, sr2, sk1, sk2;
+};
+// The kEmuSlices digit slices of `v` at `scale` (negated if neg), K padded with
+// zeros to Kp: out[slice][z][r][Kp].  F (optional, [z][K index of F]) with fcoef:
+// fcoef F[z][c] is added where the row equals b, (b, c) the K index pair (swap: (c, b)).
+cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale,
+                       __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
+                       cudaStream_t st);
+
+}  // namespace mlcc3
