@@ -57,8 +57,13 @@ extern "C" {
 #define MLCC3_ERR_TIMEOUT (-5)        /* a device wait gave up */
 #define MLCC3_ERR_STATE (-6)          /* call order: integrals not built */
 
-/* Arithmetic of the contractions.  MLCC3_FP64: every product and sum in
- * IEEE double.  MLCC3_SPLIT_BF16X3: integral-amplitude products on the
+/* Arithmetic of the contractions.  MLCC3_FP64: products and sums in IEEE
+ * double, or, for the large contractions ("fp64_tc_from"), as integers: every
+ * operand a multiple of 2^-62 of the power of two above its largest element,
+ * its digits multiplied on the tensor cores, the sums exact but for terms below
+ * 2^-64 and rounded to binary64 once.  Results are at least as accurate as sums
+ * in IEEE double (normwise); an operand with an infinity gives NaN where it
+ * enters.  MLCC3_SPLIT_BF16X3: integral-amplitude products on the
  * tensor cores from hi/lo bfloat16 splits with FP32 accumulation;
  * denominators and final reductions stay in FP64.
  * An FP16 hi/lo split is not offered: FP16's five exponent bits put the low
@@ -254,6 +259,13 @@ void mlcc3_sweep_destroy(mlcc3_sweep *sweep);
  *              over the launch's items) run on 128 x 128 CUDA-core tiles with
  *              FP32 accumulation over K ranges of at most 1024 (summed in
  *              FP64); the others on 64 x 64 tiles.  Default 10^9; 0: never.
+ *   "fp64_tc_from"  MLCC3_FP64 contexts with at least this many active virtual
+ *              orbitals (and n_o >= 2) run the O(N_V n_v^3 n_o^3) contractions and
+ *              the Cholesky-index products on the tensor cores (see MLCC3_FP64),
+ *              unless the digits of the integral blocks would take more than a
+ *              quarter of the free memory; smaller ones on the FP64 pipe.
+ *              Default 24.  A change that switches the path needs a new
+ *              mlcc3_build_integrals (MLCC3_ERR_STATE before it).
  *   "finish_fused"  1 (default): in the split-precision mode the finish of a
  *              triples build (rank-1 terms, denominators) and the contravariant
  *              transform of its blocks run as one pass over tile orbits; 0: as

@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "kernels_emu.cuh"
 #include "kernels_fp64.cuh"
 #include "kernels_tc.cuh"
 #include "mlcc3.h"
@@ -164,8 +165,17 @@ struct mlcc3_ctx {
     void *hi = nullptr, *lo = nullptr;
     CUtensorMap mhi, mlo;
     unsigned rows = 0;  // rows of the maps' box (make_split)
+    // FP64 mode: S digit slices at hi, `slice` elements apart, read through mhi
+    int S = 0;
+    long long slice = 0;
+    const mlcc3::EmuScale *scale = nullptr;
   };
   std::map<std::string, SplitOp> splits;
+  // FP64 mode: the large contractions on the tensor cores (kernels_emu.cuh), for
+  // n_v >= fp64_tc_from; the names of the operands' scales
+  bool emu = false;
+  long long fp64_tc_from = 24;
+  std::map<std::string, int> scales;
   // split layouts of triples arrays, converted once per (array, write
   // generation): slots hold the layouts converted so far of one array; every
   // path that writes a triples array marks it (wrote), which retires them

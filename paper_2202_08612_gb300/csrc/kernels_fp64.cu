@@ -10,6 +10,8 @@
 //   transpose_tl_kernel: doubles bookkeeping on the active-pair block.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kernels_fp64.cuh"
 
 namespace mlcc3 {
@@ -522,6 +524,91 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
     }
     out[it.off + ((long long)a * nv + b) * nv + c] = val;
   }
+}
+
+// Finish of a triples block whose two-index terms W are summed already (FP64 mode
+// on the tensor cores), in place: X = -(W + rank-1 terms) / (eps - omega).  A
+// warp takes a row (a, b), its lanes c.  The two-pair operand of a rank-1 term is
+// symmetric under exchange of its (occupied, virtual) pairs, so the six
+// permutations are three products counted twice.  Bound by the FP64 pipe (two
+// operations per clock and SM): 10 operations per element without rank-1 terms,
+// 17 with both.
+__global__ void __launch_bounds__(256) triples_finish64_kernel(double *__restrict__ X,
+                                                               const TripItem *__restrict__ items,
+                                                               const TripTerms terms,
+                                                               const double *__restrict__ eps, int NO,
+                                                               int nv, double omega_v,
+                                                               const double *__restrict__ omega_p,
+                                                               int *__restrict__ status) {
+  const TripItem it = items[blockIdx.y];
+  const long long i = it.i, j = it.j, k = it.k;
+  const double *ev = eps + NO;
+  const double eo = eps[it.i] + eps[it.j] + eps[it.k] + (omega_p ? *omega_p : omega_v);
+  const int rows = nv * nv, lane = threadIdx.x % 32;
+  bool singular = false;
+  for (int r = blockIdx.x * 8 + threadIdx.x / 32; r < rows; r += gridDim.x * 8) {
+    const int a = r / nv, b = r % nv;
+    const double er = ev[a] + ev[b] - eo;
+    double *x = X + it.off + (long long)r * nv;
+    // per term: two pointers along c (each times a factor of the row) and one factor times a vector along c
+    const double *p[2][3];
+    double f[2][3];
+    long long st[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      if (t >= terms.n) continue;
+      const TripTerm &m = terms.t[t];
+      const double co = 2.0 * m.coef;
+      if (m.kind == 2) {  // A[x][u] B[y][z][v][w]
+        p[t][0] = m.B + j * m.sB[0] + k * m.sB[1] + b * m.sB[2];
+        f[t][0] = co * m.A[i * m.sA[0] + a * m.sA[1]];
+        p[t][1] = m.B + i * m.sB[0] + k * m.sB[1] + a * m.sB[2];
+        f[t][1] = co * m.A[j * m.sA[0] + b * m.sA[1]];
+        p[t][2] = m.A + k * m.sA[0];
+        st[t] = m.sA[1];
+        f[t][2] = co * m.B[i * m.sB[0] + j * m.sB[1] + a * m.sB[2] + b * m.sB[3]];
+      } else {  // A[x][y][u][v] B[z][w]
+        p[t][0] = m.A + i * m.sA[0] + k * m.sA[1] + a * m.sA[2];
+        f[t][0] = co * m.B[j * m.sB[0] + b * m.sB[1]];
+        p[t][1] = m.A + j * m.sA[0] + k * m.sA[1] + b * m.sA[2];
+        f[t][1] = co * m.B[i * m.sB[0] + a * m.sB[1]];
+        p[t][2] = m.B + k * m.sB[0];
+        st[t] = m.sB[1];
+        f[t][2] = co * m.A[i * m.sA[0] + j * m.sA[1] + a * m.sA[2] + b * m.sA[3]];
+      }
+    }
+    for (int c = lane; c < nv; c += 32) {
+      double w = x[c];
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+        if (t < terms.n) {
+          w = fma(f[t][0], p[t][0][c], w);
+          w = fma(f[t][1], p[t][1][c], w);
+          w = fma(f[t][2], p[t][2][c * st[t]], w);
+        }
+      const double den = er + ev[c];
+      if (fabs(den) < 1e-3) {
+        singular = true;
+        w = 0.0;
+      } else {
+        w = -w / den;
+      }
+      x[c] = w;
+    }
+  }
+  if (singular) atomicOr(status, 1);
+}
+
+// terms: rank-1 terms (kinds 2 and 3, at most two, `sym` set, unit strides along the
+// last index of their two-pair operand).
+cudaError_t launch_finish64(double *X, const TripItem *items, int n, const TripTerms &terms,
+                            const double *eps, int NO, int nv, double omega, const double *omega_p,
+                            int *status, cudaStream_t st) {
+  if (n <= 0 || nv <= 0) return cudaSuccess;
+  if (terms.n > 2) return cudaErrorInvalidValue;
+  const int gx = std::max(1, std::min((nv * nv + 7) / 8, (16 * 152 + n - 1) / n));
+  triples_finish64_kernel<<<dim3(gx, n), 256, 0, st>>>(X, items, terms, eps, NO, nv, omega, omega_p, status);
+  return cudaGetLastError();
 }
 
 // Contravariant triples, virtual permutations with ijk fixed (Eq. contra_3):

@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "engine.cuh"
+#include "kernels_emu.cuh"
 #include "kernels_fp64.cuh"
 #include "kernels_tc.cuh"
 #include "mlcc3.h"
@@ -64,6 +65,8 @@ cudaError_t launch_finish_contra(const float *, const TripItem *, int, const Tri
                                  const double *, const float2 *, int, double, const double *,
                                  float *, float *, int *, cudaStream_t);
 __global__ void hilo_kernel(const double *, float2 *, int);
+cudaError_t launch_finish64(double *, const TripItem *, int, const TripTerms &, const double *, int,
+                            int, double, const double *, int *, cudaStream_t);
 bool encode_map(CUtensorMap *m, const void *base, const unsigned long long dims[4],
                 const unsigned long long strides[3], const unsigned box[4], std::string *err);
 cudaError_t split_bf16(const double *in, __nv_bfloat16 *hi, __nv_bfloat16 *lo, long long D0,
@@ -551,6 +554,24 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
   return out;
 }
 
+// FP64 mode: the O(N_V n_v^3 n_o^3) contractions on the tensor cores (digit
+// slices; rho and sigma at 20/200/12/60: 1868 -> 85 ms, the densities at
+// 13/101/7/37: 79 -> 18 ms, errors against 64 bits as before or smaller) from
+// fp64_tc_from active virtual orbitals on (a 4/8 system gains nothing: its calls
+// are launches, and the digits need more of them), where the operands'
+// digits (six layouts of the two integral blocks, the Cholesky factors and the
+// amplitudes at 16 bytes an element) leave most of the memory free.
+void choose_emu(mlcc3_ctx *c) {
+  S s(c);
+  c->emu = false;
+  if (c->precision != MLCC3_FP64 || s.no < 2 || s.nv < c->fp64_tc_from) return;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return;
+  const double digits = 16.0 * (8.0 * (double)s.gvsz() + 3.0 * (double)s.NJ * (double)(s.nv * s.NV) +
+                                4.0 * (double)s.blk() + 4.0 * (double)(s.no * s.nv * s.nv * s.NO));
+  c->emu = digits < 0.25 * (double)fr;
+}
+
 // Split the unique batches into chunks of at most chunk_blocks blocks (or, when
 // it is 0, as many as fit in half of the device memory left free once the
 // context's persistent arrays exist, at 156 bytes per block element: the
@@ -572,7 +593,8 @@ void make_chunks(mlcc3_ctx *c) {
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = (size_t)40 << 30;
     const double budget = 0.5 * (double)fr;
     // binary32 triples arrays in the split mode (and no separate FP32 copies)
-    const double per_elem = c->tri32 ? 108.0 : 156.0;
+    // (digit slices: eight FP64 arrays and three arrays' six layouts of 16 bytes)
+    const double per_elem = c->tri32 ? 108.0 : c->emu ? 352.0 : 156.0;
     part_max = group_max = std::max<long long>(1, (long long)(budget / (per_elem * (double)nv3)));
   }
   const std::string g = "#" + std::to_string(c->chunk_gen);
@@ -738,13 +760,16 @@ void tc_back_L(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
 void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, const std::string &okey,
                const BackSet &b, double *Zb);
 bool split_mode(const mlcc3_ctx *c);
-void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const double *F = nullptr,
-              double fcoef = 0.0);
+bool tc_mode(const mlcc3_ctx *c);
+void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const std::string &slot,
+              const double *F = nullptr, double fcoef = 0.0);
 void encode_split(mlcc3_ctx::SplitOp &op, const std::string &key, const unsigned long long dims[4],
                   const unsigned long long str[3], const unsigned bx[4]);
-mlcc3_ctx::SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G);
-mlcc3_ctx::SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk);
-void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T);
+mlcc3_ctx::SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G,
+                               const std::string &slot);
+mlcc3_ctx::SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk,
+                                const std::string &slot);
+void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T, const std::string &slot);
 void tc_integrals(mlcc3_ctx *c);
 void split_chol_kpairs(mlcc3_ctx *c);
 float *f32_copy(mlcc3_ctx *c, const std::string &key, const double *x, long long n);
@@ -801,8 +826,8 @@ void back_contract(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords,
                      {s.vb, 1, 0, 0, 0}, {s.NO, 0, 0, 0});
     });
   }
-  // split mode: the F term rides on the D-slot GEMM (split_gt folds cF/cD F_kc into it)
-  if (bset.F && !(split_mode(c) && bset.GD)) {
+  // tensor cores: the F term rides on the D-slot GEMM (split_gt folds cF/cD F_kc into it)
+  if (bset.F && !(tc_mode(c) && bset.GD)) {
     it = c->dev_items(okey + ":bF", [&] {
       std::vector<BstcItem> v;
       for (auto &o : ords)
@@ -814,7 +839,7 @@ void back_contract(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords,
     sh.M1 = s.nv; sh.M2 = s.nv; sh.K1 = s.nv;
     c->bstc(X, bset.F, Zb, sh, bset.cF, it, n, true, okey + ":bF");
   }
-  if (bset.GL && split_mode(c)) {
+  if (bset.GL && tc_mode(c)) {
     tc_back_L(c, X, ords, okey, bset, Zb);
   } else if (bset.GL) {
     it = c->dev_items(okey + ":bL", [&] {
@@ -828,7 +853,7 @@ void back_contract(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords,
     sh.M1 = s.nv; sh.M2 = s.nv; sh.K1 = s.nv; sh.N1 = s.NO;
     c->bstc(X, bset.GL, Zb, sh, bset.cL, it, n, true, okey + ":bL");
   }
-  if (bset.GD && split_mode(c)) {
+  if (bset.GD && tc_mode(c)) {
     tc_back_D(c, X, ords, okey, bset, Zb);
   } else if (bset.GD) {
     it = c->dev_items(okey + ":bD", [&] {
@@ -902,6 +927,42 @@ struct TcDev {
   int nitems;
 };
 
+// The FP64 mode's contractions on the tensor cores (digit slices, kernels_emu.cuh)
+// follow the same plans as the split mode's, with other chunks and tile widths.
+// K elements per chunk of a plan, K padded to chunks, chunks of K.
+int kblk(const mlcc3_ctx *c) { return c->emu ? kEmuKB : 64; }
+long long kpad(const mlcc3_ctx *c, long long K) { return (K + kblk(c) - 1) / kblk(c) * kblk(c); }
+int kchunks(const mlcc3_ctx *c, long long K) { return (int)(kpad(c, K) / kblk(c)); }
+// Columns of a tile over n output columns.
+int tile_w(const mlcc3_ctx *c, long long n) {
+  return c->emu ? emu_tile_width(n, kEmuSlices) : tc_tile_width(n);
+}
+// Longest accumulation chain of a plan, in chunks: tc_kcap in the split mode; the
+// digit sums are exact, their items only bounded by the integers' width.
+int kcap(const mlcc3_ctx *c) { return c->emu ? kEmuMaxK / kEmuKB : c->tc_kcap; }
+
+// Named scales of digit operands (FP64 mode on the tensor cores): device words.
+EmuScale *scale_of(mlcc3_ctx *c, const std::string &slot) {
+  constexpr int kMax = 4096;
+  EmuScale *base = static_cast<EmuScale *>(c->raw("emu:scales", sizeof(EmuScale) * kMax));
+  auto it = c->scales.find(slot);
+  if (it == c->scales.end()) {
+    if (c->scales.size() >= (size_t)kMax) throw Error{MLCC3_ERR_ARG, "too many scales"};
+    it = c->scales.emplace(slot, (int)c->scales.size()).first;
+  }
+  return base + it->second;
+}
+// scale = the largest finite magnitude of the arrays (zeroed first)
+void scale_max(mlcc3_ctx *c, const std::string &slot,
+               std::initializer_list<std::pair<const double *, long long>> xs) {
+  if (!c->emu) return;
+  EmuScale *d = scale_of(c, slot);
+  check_cuda(cudaMemsetAsync(d, 0, sizeof(EmuScale), c->stream), "scale");
+  for (auto &x : xs)
+    c->launch("emu_absmax_kernel", 0.0,
+              [&] { check_cuda(emu_absmax(x.first, x.second, d, c->stream), "emu_absmax"); });
+}
+
 void *upload_cached(mlcc3_ctx *c, const std::string &key, const void *data, size_t bytes) {
   auto it = c->items.find(key);
   if (it != c->items.end()) return it->second.first;
@@ -917,7 +978,7 @@ void *upload_cached(mlcc3_ctx *c, const std::string &key, const void *data, size
 // boundary by offsetting its K coordinates).  The tensor cores accumulate in
 // FP32 with truncation, so the error of one accumulation chain grows with its
 // length; the pieces are summed in FP64 by the atomic epilogue.
-void cap_chains(TcPlan &pl, int cap) {
+void cap_chains(TcPlan &pl, int cap, int kb) {
   if (cap <= 0) return;
   std::vector<TcItem> items;
   std::vector<TcSeg> segs;
@@ -935,8 +996,8 @@ void cap_chains(TcPlan &pl, int cap) {
         }
         const int take = std::min(cap - used, g.nk - k0);
         TcSeg h = g;
-        h.ac[0] = g.ac[0] + 64 * k0;
-        h.bc[0] = g.bc[0] + 64 * k0;
+        h.ac[0] = g.ac[0] + kb * k0;
+        h.bc[0] = g.bc[0] + kb * k0;
         h.nk = take;
         segs.push_back(h);
         items.back().seg_count += 1;
@@ -961,7 +1022,7 @@ TcDev tc_plan(mlcc3_ctx *c, const std::string &key0, const std::function<void(Tc
                  static_cast<const TcSeg *>(c->items.at(key + ":segs").first), it->second.second};
   TcPlan pl;
   build(pl);
-  cap_chains(pl, cap);
+  cap_chains(pl, cap, kblk(c));
   if ((long long)pl.items.size() > (long long)c->tc_persist_from) {
     // persistent launches hand out items round-robin: the longest chains first
     // (stable, so equal items keep their order and their operand reuse) even
@@ -985,9 +1046,36 @@ TcDev tc_plan(mlcc3_ctx *c, const std::string &key0, const std::function<void(Tc
 }
 
 // site: the contraction's tag in the per-call-site statistics ("tc_gemm_kernel:<site>").
+// FP64 mode on the tensor cores: A and B are the digit operands whose scales the
+// product takes (every pair of a launch has the same sum of exponents).
 void tc_launch(mlcc3_ctx *c, const char *site, int BN, const TcMaps &maps, const TcDev &d,
-               const TcEpi &epi, double flops) {
+               const TcEpi &epi, double flops, const mlcc3_ctx::SplitOp &A,
+               const mlcc3_ctx::SplitOp &B) {
   if (d.nitems == 0) return;
+  if (c->emu) {
+    EmuEpi x{};
+    x.out = static_cast<double *>(epi.out);
+    x.mode = epi.mode == 0 || epi.mode == 3 ? 0 : 1;
+    x.R2 = epi.R2;
+    x.linear = epi.linear;
+    x.s1 = epi.s1;
+    x.s2 = epi.s2;
+    x.sn = epi.sn;
+    x.lim1 = epi.lim1;
+    x.lim2 = epi.lim2;
+    x.nlim = epi.nlim;
+    x.alpha = (double)epi.alpha;
+    x.n = BN;
+    x.ebias = -12;
+    x.sa = A.scale;
+    x.sb = B.scale;
+    x.wait = c->tc_wait;
+    c->launch((std::string("emu_gemm_kernel:") + site).c_str(), flops, [&] {
+      check_cuda(launch_emu_gemm(kEmuSlices, maps, d.items, d.segs, d.nitems, x, c->status, c->stream),
+                 "emu_gemm");
+    });
+    return;
+  }
   const std::string name = std::string("tc_gemm_kernel:") + site;
   TcEpi e = epi;
   e.wait = c->tc_wait;
@@ -1017,14 +1105,37 @@ TcEpi make_epi(void *out, int mode, int R2, long long s1, long long s2, long lon
   return e;
 }
 
+// Digit slices of `v` as operand `key`.
+void make_digits(mlcc3_ctx *c, SplitOp &op, const std::string &key, const EmuView &v, long long Kp,
+                 bool neg, const std::string &slot, const double *F = nullptr, double fcoef = 0.0,
+                 bool swap = false) {
+  op.S = kEmuSlices;
+  op.slice = (long long)v.Z * v.R * Kp;
+  op.scale = scale_of(c, slot);
+  op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuSlices * 2);
+  op.lo = nullptr;
+  c->launch("emu_digits_kernel", 0.0, [&] {
+    check_cuda(emu_digits(v, Kp, neg, op.scale, static_cast<__nv_bfloat16 *>(op.hi), F, fcoef, swap,
+                          c->stream),
+               "emu_digits");
+  });
+}
+
 // hi/lo bfloat16 copy out[D0][D1][D2][Kp] of src (strides s0..s3, K innermost,
 // padded with zeros to a multiple of 64) and its two 4-D tensor maps.
+// In the FP64 mode the digit slices at the scale `slot`.
 SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, long long D0,
                     long long D1, long long D2, long long K, long long s0, long long s1,
-                    long long s2, long long s3, double scale, Box box, unsigned rowbox = 0) {
-  const long long Kp = (K + 63) / 64 * 64;
+                    long long s2, long long s3, double scale, Box box, const std::string &slot,
+                    unsigned rowbox = 0) {
+  const long long Kp = kpad(c, K);
   SplitOp &op = c->splits[key];
   const size_t n = (size_t)(D0 * D1 * D2 * Kp);
+  if (c->emu) {
+    make_digits(c, op, key,
+                EmuView{src, (int)(D0 * D1), (int)D1, (int)D2, (int)D2, (int)K, 1, s0, s1, 0, s2, s3, 0},
+                Kp, scale < 0.0, slot);
+  } else {
   op.hi = c->raw("split:" + key + ":hi", n * 2);
   op.lo = c->raw("split:" + key + ":lo", n * 2);
   c->launch("split_bf16_kernel", 0.0, [&] {
@@ -1032,13 +1143,14 @@ SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, lon
                           D0, D1, D2, K, Kp, s0, s1, s2, s3, scale, c->stream),
                "split_bf16");
   });
+  }
   const unsigned long long dims[4] = {(unsigned long long)Kp, (unsigned long long)D2,
                                       (unsigned long long)D1, (unsigned long long)D0};
   const unsigned long long str[3] = {(unsigned long long)(Kp * 2), (unsigned long long)(Kp * 2 * D2),
                                      (unsigned long long)(Kp * 2 * D2 * D1)};
   unsigned bx[4] = {64, 16, 8, 1};
   if (box == Box::Row) {
-    bx[1] = rowbox ? rowbox : (unsigned)tc_tile_width(c->nv);
+    bx[1] = rowbox ? rowbox : (unsigned)tile_w(c, c->nv);
     bx[2] = 1;
   }
   unsigned long long fdims[4] = {dims[0], (unsigned long long)(D0 * D1 * D2), 1ULL, 1ULL};
@@ -1050,9 +1162,7 @@ SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, lon
     md = fdims;
     ms = fstr;
   }
-  std::string err;
-  if (!encode_map(&op.mhi, op.hi, md, ms, bx, &err) || !encode_map(&op.mlo, op.lo, md, ms, bx, &err))
-    throw Error{MLCC3_ERR_CUDA, "tensor map " + key + ": " + err};
+  encode_split(op, key, md, ms, bx);
   op.rows = box == Box::Pair ? 128u : bx[1];
   return op;
 }
@@ -1060,7 +1170,7 @@ SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, lon
 // Tile width of a pair contraction with nN output columns, and the box rows of
 // its column operand (split_amp_T, split_go_T).
 int pair_bn(const mlcc3_ctx *c, long long nN) {
-  return nN > 256 ? c->tc_wide_bn : tc_tile_width(nN);
+  return !c->emu && nN > 256 ? c->tc_wide_bn : tile_w(c, nN);
 }
 
 // Operands of one two-index term of the triples expression, as split copies:
@@ -1071,18 +1181,34 @@ struct SplitTerm {
   SplitOp *P, *S, *amp;
 };
 
+// G[z][v][w][r] as pair operands key:P, rows (v, w), and key:S, rows (w, v).
+void split_pairs(mlcc3_ctx *c, const std::string &key, const double *G, long long R, long long sz,
+                 long long sv, long long sw, const std::string &slot) {
+  S s(c);
+  SplitOp &p = make_split(c, key + ":P", G, s.no, s.nv, s.nv, R, sz, sv, sw, 1, 1.0, Box::Pair, slot);
+  if (c->emu) {
+    // the same memory read through a map with the two row indices exchanged
+    SplitOp &q = c->splits[key + ":S"] = p;
+    const unsigned long long rb = (unsigned long long)kpad(c, R) * 2, nv = (unsigned long long)s.nv;
+    const unsigned long long dims[4] = {rb / 2, nv, nv, (unsigned long long)s.no};
+    const unsigned long long str[3] = {rb * nv, rb, rb * nv * nv};
+    const unsigned bx[4] = {64, 16, 8, 1};
+    encode_split(q, key + ":S", dims, str, bx);
+    return;
+  }
+  make_split(c, key + ":S", G, s.no, s.nv, s.nv, R, sz, sw, sv, 1, 1.0, Box::Pair, slot);
+}
+
 // Split copies of a D-type term: amplitude block X[x][u][y][D] and integral Gv-like [z][v][w][D].
 SplitTerm split_d(mlcc3_ctx *c, const std::string &ak, const double *amp, bool convert_a,
-                  const std::string &gk, const double *G, bool convert_g) {
+                  const std::string &gk, const double *G, bool convert_g,
+                  const std::string &aslot, const std::string &gslot) {
   S s(c);
   SplitTerm t{true, nullptr, nullptr, nullptr};
   if (convert_a)
-    make_split(c, ak + ":B", amp, s.no, s.no, s.nv, s.NV, s.bi, s.bL, s.ba, 1, 1.0, Box::Row);
+    make_split(c, ak + ":B", amp, s.no, s.no, s.nv, s.NV, s.bi, s.bL, s.ba, 1, 1.0, Box::Row, aslot);
   t.amp = &c->splits.at(ak + ":B");
-  if (convert_g) {
-    make_split(c, gk + ":P", G, s.no, s.nv, s.nv, s.NV, s.gk, s.gb, s.gc, 1, 1.0, Box::Pair);
-    make_split(c, gk + ":S", G, s.no, s.nv, s.nv, s.NV, s.gk, s.gc, s.gb, 1, 1.0, Box::Pair);
-  }
+  if (convert_g) split_pairs(c, gk, G, s.NV, s.gk, s.gb, s.gc, gslot);
   t.P = &c->splits.at(gk + ":P");
   t.S = &c->splits.at(gk + ":S");
   return t;
@@ -1090,15 +1216,13 @@ SplitTerm split_d(mlcc3_ctx *c, const std::string &ak, const double *amp, bool c
 
 // Split copies of an L-type term: amplitude Tl-like X[x][u][v][L] and integral Go-like [y][z][w][L].
 SplitTerm split_l(mlcc3_ctx *c, const std::string &ak, const double *ampl, bool convert_a,
-                  const std::string &gk, const double *Gl, bool convert_g) {
+                  const std::string &gk, const double *Gl, bool convert_g,
+                  const std::string &aslot, const std::string &gslot) {
   S s(c);
   SplitTerm t{false, nullptr, nullptr, nullptr};
-  if (convert_a) {
-    make_split(c, ak + ":P", ampl, s.no, s.nv, s.nv, s.NO, s.ti, s.ta, s.tb, 1, 1.0, Box::Pair);
-    make_split(c, ak + ":S", ampl, s.no, s.nv, s.nv, s.NO, s.ti, s.tb, s.ta, 1, 1.0, Box::Pair);
-  }
+  if (convert_a) split_pairs(c, ak, ampl, s.NO, s.ti, s.ta, s.tb, aslot);
   if (convert_g)
-    make_split(c, gk + ":N", Gl, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row);
+    make_split(c, gk + ":N", Gl, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, gslot);
   t.P = &c->splits.at(ak + ":P");
   t.S = &c->splits.at(ak + ":S");
   t.amp = &c->splits.at(gk + ":N");
@@ -1136,8 +1260,10 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
     maps.m[6 * t + 5] = st.amp->mlo;
   }
   const long long nb = (long long)bs.size();
-  float *W = static_cast<float *>(c->raw("tcW", sizeof(float) * (size_t)(c->chunk_nb * s.nv3)));
-  const long long NVk = (s.NV + 63) / 64, NOk = (s.NO + 63) / 64;
+  // FP64 mode: the sums go straight into the blocks
+  void *W = c->emu ? static_cast<void *>(out)
+                   : c->raw("tcW", sizeof(float) * (size_t)(c->chunk_nb * s.nv3));
+  const long long NVk = kchunks(c, s.NV), NOk = kchunks(c, s.NO);
   const long long nt1 = (s.nv + 7) / 8, nt2 = (s.nv + 15) / 16;
   const long long cs[3] = {s.nv * s.nv, s.nv, 1};
   std::string sig;
@@ -1146,10 +1272,15 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
   // depends only on the occupied indices at the other two positions, so the
   // batches that share them are stacked along N, up to G per tile, each with
   // its own amplitude box of BW rows and its own output block.
-  const int BW = tc_tile_width(s.nv);
-  const int G = std::max(1, std::min(c->tc_group, 256 / BW));
-  const int BN = tc_tile_width((long long)BW * G);
-  for (int o = 0; o < 3; ++o) {
+  // (FP64 mode: single batches; the eight digit degrees fill TMEM at 64 columns)
+  const int BW = tile_w(c, s.nv);
+  const int G = c->emu ? 1 : std::max(1, std::min(c->tc_group, 256 / BW));
+  const int BN = c->emu ? BW : tc_tile_width((long long)BW * G);
+  const long long ntN = c->emu ? (s.nv + BW - 1) / BW : 1;
+  for (int oo = 0; oo < 3; ++oo) {
+    // FP64 mode: position 2 first, whose columns are contiguous in the block: it
+    // stores, and the other two add along their contiguous rows
+    const int o = c->emu ? (oo + 2) % 3 : oo;
     const int p1 = o == 0 ? 1 : 0, p2 = o == 2 ? 1 : 2;
     const std::string key = "tc:" + bkey + ":" + sig + ":" + std::to_string(o) + ":g" + std::to_string(G);
     TcDev dv = tc_plan(c, key, [&](TcPlan &pl) {
@@ -1170,8 +1301,10 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
         const std::vector<long long> &us = groups[g];
         for (long long t1 = 0; t1 < nt1; ++t1)
           for (long long t2 = 0; t2 < nt2; ++t2)
-            for (size_t q0 = 0; q0 < us.size(); q0 += (size_t)G) {
+            for (size_t q0 = 0; q0 < us.size(); q0 += (size_t)G)
+            for (long long tn = 0; tn < ntN; ++tn) {
               const int nq = (int)std::min<size_t>((size_t)G, us.size() - q0);
+              const int c0 = (int)(tn * BW);
               int I[4][3];
               for (int q = 0; q < nq; ++q) {
                 const TripItem &b = bs[us[q0 + q]];
@@ -1179,7 +1312,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
                 I[q][1] = b.j;
                 I[q][2] = b.k;
               }
-              pl.tile((int)(8 * t1), (int)(16 * t2), 0, bs[us[q0]].off);
+              pl.tile((int)(8 * t1), (int)(16 * t2), c0, bs[us[q0]].off);
               pl.items.back().nq = nq;
               for (int q = 1; q < nq; ++q) pl.items.back().qoff[q - 1] = bs[us[q0 + q]].off;
               for (size_t t = 0; t < terms.size(); ++t) {
@@ -1188,12 +1321,12 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
                   int x = -1, y = -1;  // positions of the B box coordinates 2 and 3
                   if (terms[t].dtype && s0 == o) {
                     pl.seg((int)(6 * t) + (s1 < s2 ? 0 : 2), (int)(6 * t) + 4, (int)NVk,
-                           (int)(16 * t2), (int)(8 * t1), I[0][s2], 0, I[0][s1], I[0][s0]);
+                           (int)(16 * t2), (int)(8 * t1), I[0][s2], c0, I[0][s1], I[0][s0]);
                     x = s1;
                     y = s0;
                   } else if (!terms[t].dtype && s2 == o) {
                     pl.seg((int)(6 * t) + (s0 < s1 ? 0 : 2), (int)(6 * t) + 4, (int)NOk,
-                           (int)(16 * t2), (int)(8 * t1), I[0][s0], 0, I[0][s2], I[0][s1]);
+                           (int)(16 * t2), (int)(8 * t1), I[0][s0], c0, I[0][s2], I[0][s1]);
                     x = s2;
                     y = s1;
                   }
@@ -1209,11 +1342,12 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
             }
       }
     });
-    TcEpi epi = make_epi(W, o == 0 ? 0 : 1, 16, cs[p1], cs[p2], cs[o], s.nv, s.nv, s.nv, 1.0);
+    TcEpi epi = make_epi(W, oo == 0 ? 0 : 1, 16, cs[p1], cs[p2], cs[o], s.nv, s.nv, s.nv, 1.0);
     epi.qw = BW;
     double K = 0.0;
     for (auto &t : terms) K += 2.0 * (t.dtype ? (double)s.NV : (double)s.NO);
-    tc_launch(c, "build", BN, maps, dv, epi, 2.0 * (double)(s.nv * s.nv) * (double)s.nv * K * (double)nb);
+    tc_launch(c, "build", BN, maps, dv, epi, 2.0 * (double)(s.nv * s.nv) * (double)s.nv * K * (double)nb,
+              *terms[0].P, *terms[0].amp);
   }
   TripTerms tt{};
   for (auto &t : rank1) tt.t[tt.n++] = t;
@@ -1232,6 +1366,14 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
   (void)n;
   for (long long b0 = 0; b0 < nb; b0 += 65535) {
     const long long nbc = std::min<long long>(65535, nb - b0);
+    if (c->emu) {
+      c->launch("triples_finish64_kernel", 0.0, [&] {
+        check_cuda(launch_finish64(out, db + b0, (int)nbc, tt, c->eps, (int)s.NO, (int)s.nv, omega,
+                                   c->omega_dev, c->status, c->stream),
+                   "finish64");
+      });
+      continue;
+    }
     // about sixteen 256-thread blocks per SM over the launch, each a large
     // slice of one batch (the per-block operand tables are built serially)
     const long long gx = std::max<long long>(1, std::min<long long>((s.nv3 + 255) / 256, (16 * 152 + nbc - 1) / nbc));
@@ -1239,7 +1381,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
     const float2 *ehl = static_cast<const float2 *>(c->raw("ehl", sizeof(float2) * (size_t)s.nv));
     if (outt && c->tri32 && c->finish_fused) {
       c->launch(rank1.empty() ? "triples_finish_contra_kernel" : "triples_finish_contra_kernel:rank1", 0.0, [&] {
-        check_cuda(launch_finish_contra(W, db + b0, (int)nbc, tt, c->eps, ehl, (int)s.nv, omega,
+        check_cuda(launch_finish_contra(static_cast<const float *>(W), db + b0, (int)nbc, tt, c->eps, ehl, (int)s.nv, omega,
                                         c->omega_dev,
                                         keep_out ? reinterpret_cast<float *>(out) : nullptr,
                                         reinterpret_cast<float *>(outt), c->status, c->stream),
@@ -1249,7 +1391,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
     }
     const unsigned long long nvinv = ((1ULL << 40) + (unsigned long long)s.nv - 1) / (unsigned long long)s.nv;
     c->launch("triples_finish_kernel", 0.0, [&] {
-      triples_finish_kernel<<<grid, 256, 0, c->stream>>>(W, db + b0, (int)nbc, tt, c->eps, ehl,
+      triples_finish_kernel<<<grid, 256, 0, c->stream>>>(static_cast<const float *>(W), db + b0, (int)nbc, tt, c->eps, ehl,
                                                          (int)s.nv, nvinv, omega, c->omega_dev,
                                                          out, c->tri32 ? 1 : 0, c->status);
     });
@@ -1259,25 +1401,28 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
 }
 
 bool split_mode(const mlcc3_ctx *c) { return c->precision == MLCC3_SPLIT_BF16X3; }
+bool tc_mode(const mlcc3_ctx *c) { return split_mode(c) || c->emu; }
 
 // Persistent split copies of the ground-state amplitudes and integrals.
 void build_split_persistent(mlcc3_ctx *c) {
   S s(c);
-  make_split(c, "t:B", c->t2c, s.no, s.no, s.nv, s.NV, s.bi, s.bL, s.ba, 1, 1.0, Box::Row);
-  for (auto kv : {std::make_pair(std::string("Gv"), c->Gv), std::make_pair(std::string("Gb"), c->Gb)}) {
-    make_split(c, kv.first + ":P", kv.second, s.no, s.nv, s.nv, s.NV, s.gk, s.gb, s.gc, 1, 1.0, Box::Pair);
-    make_split(c, kv.first + ":S", kv.second, s.no, s.nv, s.nv, s.NV, s.gk, s.gc, s.gb, 1, 1.0, Box::Pair);
-  }
-  make_split(c, "Tl:P", c->Tl, s.no, s.nv, s.nv, s.NO, s.ti, s.ta, s.tb, 1, 1.0, Box::Pair);
-  make_split(c, "Tl:S", c->Tl, s.no, s.nv, s.nv, s.NO, s.ti, s.tb, s.ta, 1, 1.0, Box::Pair);
-  make_split(c, "Go:N", c->Go, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row);
-  make_split(c, "Gx:N", c->Gx, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row);
-  split_gt(c, "Gb", c->Gb, c->F, 0.5);  // Omega / rho: D slot g_Dbkc with 1/2 F_kc folded in
-  split_gt(c, "Gv", c->Gv);
-  split_go_T(c, "Gx:T", c->Gx);
-  split_go_T(c, "Go:T", c->Go);
-  split_amp_T(c, "t:AT", c->t2c);
-  split_tl_T(c, "Tl", c->Tl);
+  // one scale for both integrals (amplitudes) of a triples expression: their
+  // products accumulate in one chain
+  scale_max(c, "t", {{c->t2c, (long long)s.blk()}});
+  scale_max(c, "G", {{c->Gv, (long long)s.gvsz()}, {c->Go, (long long)s.gosz()}});
+  scale_max(c, "Gb", {{c->Gb, (long long)s.gvsz()}, {c->Gx, (long long)s.gosz()}});
+  make_split(c, "t:B", c->t2c, s.no, s.no, s.nv, s.NV, s.bi, s.bL, s.ba, 1, 1.0, Box::Row, "t");
+  split_pairs(c, "Gv", c->Gv, s.NV, s.gk, s.gb, s.gc, "G");
+  split_pairs(c, "Gb", c->Gb, s.NV, s.gk, s.gb, s.gc, "Gb");
+  split_pairs(c, "Tl", c->Tl, s.NO, s.ti, s.ta, s.tb, "t");
+  make_split(c, "Go:N", c->Go, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, "G");
+  make_split(c, "Gx:N", c->Gx, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, "Gb");
+  split_gt(c, "Gb", c->Gb, "Gb", c->F, 0.5);  // Omega / rho: D slot g_Dbkc with 1/2 F_kc folded in
+  split_gt(c, "Gv", c->Gv, "G");
+  split_go_T(c, "Gx:T", c->Gx, "Gb");
+  split_go_T(c, "Go:T", c->Go, "G");
+  split_amp_T(c, "t:AT", c->t2c, "t");
+  split_tl_T(c, "Tl", c->Tl, "t");
   split_chol_kpairs(c);
 }
 
@@ -1285,10 +1430,16 @@ void build_split_persistent(mlcc3_ctx *c) {
 // over (Kp, o1, -, o0) with a box of `rows` rows.
 SplitOp &make_split_k2(mlcc3_ctx *c, const std::string &key, const double *src, long long D0,
                        long long D1, long long K1, long long K2, long long s0, long long s1,
-                       long long sk1, long long sk2, unsigned rows, bool flat = false) {
-  const long long Kp = (K1 * K2 + 63) / 64 * 64;
+                       long long sk1, long long sk2, unsigned rows, const std::string &slot,
+                       bool flat = false) {
+  const long long Kp = kpad(c, K1 * K2);
   SplitOp &op = c->splits[key];
   const size_t n = (size_t)(D0 * D1 * Kp);
+  if (c->emu) {
+    make_digits(c, op, key,
+                EmuView{src, (int)D0, 1, (int)D1, (int)D1, (int)(K1 * K2), (int)K2, s0, 0, 0, s1, sk1, sk2},
+                Kp, false, slot);
+  } else {
   op.hi = c->raw("split:" + key + ":hi", n * 2);
   op.lo = c->raw("split:" + key + ":lo", n * 2);
   c->launch("split_bf16_k2_kernel", 0.0, [&] {
@@ -1296,6 +1447,7 @@ SplitOp &make_split_k2(mlcc3_ctx *c, const std::string &key, const double *src, 
                              D0, D1, K1, K2, Kp, s0, s1, sk1, sk2, 1.0, c->stream),
                "split_bf16_k2");
   });
+  }
   // rows over o1 within one o0, or (flat) over the flattened (o0, o1)
   const unsigned long long R = flat ? (unsigned long long)(D0 * D1) : (unsigned long long)D1;
   const unsigned long long dims[4] = {(unsigned long long)Kp, R, 1ULL,
@@ -1303,9 +1455,7 @@ SplitOp &make_split_k2(mlcc3_ctx *c, const std::string &key, const double *src, 
   const unsigned long long str[3] = {(unsigned long long)(Kp * 2), (unsigned long long)(Kp * 2) * R,
                                      (unsigned long long)(Kp * 2) * R};
   const unsigned bx[4] = {64, rows, 1, 1};
-  std::string err;
-  if (!encode_map(&op.mhi, op.hi, dims, str, bx, &err) || !encode_map(&op.mlo, op.lo, dims, str, bx, &err))
-    throw Error{MLCC3_ERR_CUDA, "tensor map " + key + ": " + err};
+  encode_split(op, key, dims, str, bx);
   return op;
 }
 
@@ -1322,42 +1472,58 @@ void tc_flat_gemm(mlcc3_ctx *c, const SplitOp &A, const SplitOp &B, long long M,
   maps.m[1] = A.mlo;
   maps.m[2] = B.mhi;
   maps.m[3] = B.mlo;
-  const int BN = tc_tile_width(N);
+  const int BN = tile_w(c, N);
   const long long ntM = (M + 127) / 128, ntN = (N + BN - 1) / BN;
-  const int nk = (int)((K + 63) / 64);
+  const int nk = kchunks(c, K);
   TcDev dv = tc_plan(c, "tcF:" + key, [&](TcPlan &pl) {
     for (long long tm = 0; tm < ntM; ++tm)
       for (long long tn = 0; tn < ntN; ++tn) {
         pl.tile(0, (int)(128 * tm), (int)(BN * tn), 0);
         pl.seg(0, 2, nk, (int)(128 * tm), 0, 0, (int)(BN * tn), 0, 0);
       }
-  }, c->tc_kcap);
+  }, kcap(c));
   TcEpi epi = make_epi(out, 2, R2, s1, s2, sn, M / R2, R2, N, alpha, 1);
-  tc_launch(c, "flat", BN, maps, dv, epi, 2.0 * (double)M * (double)N * (double)K);
+  tc_launch(c, "flat", BN, maps, dv, epi, 2.0 * (double)M * (double)N * (double)K, A, B);
 }
 
 // Cholesky factors as [J][(x, y)] split operands of the sigma singles tail.
 void split_chol_kpairs(mlcc3_ctx *c) {
   S s(c);
   const long long nmo = s.nmo, NO = s.NO;
-  const unsigned bj = (unsigned)tc_tile_width(s.NJ);
+  const unsigned bj = (unsigned)tile_w(c, s.NJ);
   // Lt[J][NO+b][NO+D] as K = (b, D); Lt[J][NO+c][k] and Lt[J][k][NO+c] as K = (c, k)
-  make_split_k2(c, "LvV:J", c->Lt + NO * nmo + NO, 1, s.NJ, s.nv, s.NV, 0, s.lJ, nmo, 1, bj, true);
-  make_split_k2(c, "Lvo:J", c->Lt + NO * nmo, 1, s.NJ, s.nv, s.no, 0, s.lJ, nmo, 1, bj, true);
-  make_split_k2(c, "Lov:J", c->Lt + NO, 1, s.NJ, s.nv, s.no, 0, s.lJ, 1, nmo, bj, true);
+  make_split_k2(c, "LvV:J", c->Lt + NO * nmo + NO, 1, s.NJ, s.nv, s.NV, 0, s.lJ, nmo, 1, bj, "Lt", true);
+  make_split_k2(c, "Lvo:J", c->Lt + NO * nmo, 1, s.NJ, s.nv, s.no, 0, s.lJ, nmo, 1, bj, "Lt", true);
+  make_split_k2(c, "Lov:J", c->Lt + NO, 1, s.NJ, s.nv, s.no, 0, s.lJ, 1, nmo, bj, "Lt", true);
 }
 
 // G[k][b][c][D] (Gv-like) transposed to [k][D][(b,c)] and [k][D][(c,b)].
 // The optional F[k][c] (with coefficient fcoef) is folded in as fcoef delta_{Db} F_kc:
 // the D-slot back-contraction then also carries the F_kc term of the doubles.
-void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const double *F,
-              double fcoef) {
+void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const std::string &slot,
+              const double *F, double fcoef) {
   S s(c);
-  const long long Kp = (s.nv * s.nv + 63) / 64 * 64;
+  const long long Kp = kpad(c, s.nv * s.nv);
+  std::string gslot = slot;
+  if (c->emu && F) {  // |G + fcoef F| < 2 max(|G|, |F|) for |fcoef| <= 1
+    gslot = key + ":T";
+    EmuScale *d = scale_of(c, gslot);
+    check_cuda(cudaMemsetAsync(d, 0, sizeof(EmuScale), c->stream), "scale");
+    check_cuda(emu_absmax(G, (long long)s.gvsz(), d, c->stream), "emu_absmax");
+    check_cuda(emu_absmax(F, s.no * s.nv, d, c->stream), "emu_absmax");
+    check_cuda(emu_scale_double(d, c->stream), "emu_scale_double");
+  }
   for (int swap = 0; swap < 2; ++swap) {
     const std::string k2 = key + (swap ? ":Ts" : ":T");
     SplitOp &op = c->splits[k2];
     const size_t n = (size_t)(s.no * s.NV * Kp);
+    if (c->emu) {
+      // rows D, K = (b, c) or (c, b)
+      make_digits(c, op, k2,
+                  EmuView{G, (int)s.no, 1, (int)s.NV, (int)s.NV, (int)(s.nv * s.nv), (int)s.nv, s.gk, 0, 0,
+                          1, swap ? s.gc : s.gb, swap ? s.gb : s.gc},
+                  Kp, false, gslot, F, fcoef, swap != 0);
+    } else {
     op.hi = c->raw("split:" + k2 + ":hi", n * 2);
     op.lo = c->raw("split:" + k2 + ":lo", n * 2);
     c->launch("split_transpose_kernel", 0.0, [&] {
@@ -1366,6 +1532,7 @@ void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const doubl
                                  (int)s.nv, (int)Kp, s.gk, s.gb, s.gc, swap, F, fcoef, c->stream),
                  "split_gt");
     });
+    }
     const unsigned long long dims[4] = {(unsigned long long)Kp, (unsigned long long)s.NV, 1ULL,
                                         (unsigned long long)s.no};
     const unsigned long long str[3] = {(unsigned long long)(Kp * 2),
@@ -1386,12 +1553,15 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
                const BackSet &b, double *Zb) {
   S s(c);
   if (ords.empty() || s.nv == 0) return;
-  const unsigned BN = (unsigned)tc_tile_width(s.nv);
+  const unsigned BN = (unsigned)tile_w(c, s.nv);
   // row = canonical position 0 / 1 / 2; K = the other two (ascending)
   const SplitOp &x0 = layout_XL(c, "bD:XL0", X, 0, BN);
   const SplitOp &x1 = layout_XL(c, "bD:XL1", X, 1, BN);
   const SplitOp &x2 = layout_XL(c, "bD:XL2", X, 2, BN);
-  if (b.gd_convert) split_gt(c, b.gd_key, b.GD, b.F, b.F ? b.cF / b.cD : 0.0);
+  if (b.gd_convert) {
+    if (!b.F) scale_max(c, b.gd_key, {{b.GD, (long long)s.gvsz()}});
+    split_gt(c, b.gd_key, b.GD, b.gd_key, b.F, b.F ? b.cF / b.cD : 0.0);
+  }
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   const SplitOp *ops[5] = {&c->splits.at(b.gd_key + ":T"), &c->splits.at(b.gd_key + ":Ts"), &x0, &x1,
@@ -1400,11 +1570,11 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
     maps.m[2 * i] = ops[i]->mhi;
     maps.m[2 * i + 1] = ops[i]->mlo;
   }
-  const long long ntD = (s.NV + 127) / 128;
-  const int nk = (int)((s.nv * s.nv + 63) / 64);
+  const long long ntD = (s.NV + 127) / 128, ntN = c->emu ? (s.nv + BN - 1) / BN : 1;
+  const int nk = kchunks(c, s.nv * s.nv);
   // orderings with the same r and the same canonical positions share the
   // integral operand and the layout map: up to G of them are stacked along N
-  const int G = std::max(1, std::min(c->tc_group, 256 / (int)BN));
+  const int G = c->emu ? 1 : std::max(1, std::min(c->tc_group, 256 / (int)BN));
   TcDev dv = tc_plan(c, "tcD:" + okey + ":g" + std::to_string(G), [&](TcPlan &pl) {
     std::map<std::array<int, 3>, std::vector<const Ord *>> groups;
     std::vector<std::array<int, 3>> order;
@@ -1417,13 +1587,14 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
       const std::vector<const Ord *> &os = groups[g];
       for (size_t q0 = 0; q0 < os.size(); q0 += (size_t)G) {
         const int nq = (int)std::min<size_t>((size_t)G, os.size() - q0);
-        for (long long t = 0; t < ntD; ++t) {
+        for (long long t = 0; t < ntD; ++t)
+        for (long long tn = 0; tn < ntN; ++tn) {
           const Ord &o = *os[q0];
-          pl.tile(0, (int)(128 * t), 0, o.p * s.bi + o.q * s.bL);
+          pl.tile(0, (int)(128 * t), (int)(BN * tn), o.p * s.bi + o.q * s.bL);
           pl.items.back().nq = nq;
           for (int q = 1; q < nq; ++q)
             pl.items.back().qoff[q - 1] = os[q0 + q]->p * s.bi + os[q0 + q]->q * s.bL;
-          pl.seg(g[1], 4 + 2 * g[2], nk, (int)(128 * t), 0, o.r, 0, 0, (int)(o.off / s.nv3));
+          pl.seg(g[1], 4 + 2 * g[2], nk, (int)(128 * t), 0, o.r, (int)(BN * tn), 0, (int)(o.off / s.nv3));
           TcSeg &last = pl.segs.back();
           last.nb = nq;
           for (int q = 1; q < nq; ++q) {
@@ -1433,29 +1604,32 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
         }
       }
     }
-  }, c->tc_kcap);
+  }, kcap(c));
   TcEpi epi = make_epi(Zb, 2, 128, 0, 1, s.ba, 1, s.NV, s.nv, b.cD);
   epi.qw = (int)BN;
-  tc_launch(c, "backD", tc_tile_width((long long)BN * G), maps, dv, epi,
-            2.0 * (double)s.NV * (double)s.nv * (double)(s.nv * s.nv) * (double)ords.size());
+  tc_launch(c, "backD", c->emu ? (int)BN : tc_tile_width((long long)BN * G), maps, dv, epi,
+            2.0 * (double)s.NV * (double)s.nv * (double)(s.nv * s.nv) * (double)ords.size(), *ops[0], x0);
 }
 
 // hi/lo buffers of layout L of the triples array X (chunk_nb blocks), converted
-// at most once per write of X: L = 0..2 is XL_L, L = 3..5 is R_{L-3}.
-std::pair<void *, void *> tri_layout(mlcc3_ctx *c, const double *X, int L) {
+// at most once per write of X: L = 0..2 is XL_L, L = 3..5 is R_{L-3}.  FP64 mode:
+// the digit slices, three arrays kept (96 bytes per element each).
+void tri_layout(mlcc3_ctx *c, const double *X, int L, SplitOp &op) {
   S s(c);
   const unsigned long long g = c->gen_of(X);
+  const int slots = c->emu ? 3 : 4;
   int q = -1;
-  for (int t = 0; t < 4; ++t)
+  for (int t = 0; t < slots; ++t)
     if (c->tri[t].src == X && c->tri[t].gen == g && c->tri[t].nb == c->chunk_nb) q = t;
   if (q < 0) {
     q = 0;
-    for (int t = 1; t < 4; ++t)
+    for (int t = 1; t < slots; ++t)
       if (c->tri[t].tick < c->tri[q].tick) q = t;
     c->tri[q] = mlcc3_ctx::TriSlot{};
     c->tri[q].src = X;
     c->tri[q].gen = g;
     c->tri[q].nb = c->chunk_nb;
+    scale_max(c, "tri" + std::to_string(q), {{X, c->chunk_nb * s.nv3}});
   }
   mlcc3_ctx::TriSlot &ts = c->tri[q];
   ts.tick = ++c->tri_tick;
@@ -1464,9 +1638,28 @@ std::pair<void *, void *> tri_layout(mlcc3_ctx *c, const double *X, int L) {
   const long long cs[3] = {s.nv * s.nv, s.nv, 1};
   const int k = L % 3, a = k == 0 ? 1 : 0, b = k == 2 ? 1 : 2;
   const bool xl = L < 3;
-  const long long Kp = xl ? (s.nv * s.nv + 63) / 64 * 64 : (s.nv + 63) / 64 * 64;
+  const long long Kp = kpad(c, xl ? s.nv * s.nv : s.nv);
   const size_t n = (size_t)nb * (size_t)(xl ? s.nv : s.nv * s.nv) * (size_t)Kp;
+  if (c->emu) {
+    const int nv = (int)s.nv;
+    const EmuView v = xl ? EmuView{X, (int)nb, 1, nv, nv, nv * nv, nv, s.nv3, 0, 0, cs[k], cs[a], cs[b]}
+                         : EmuView{X, (int)nb, 1, nv * nv, nv, nv, 1, s.nv3, 0, cs[a], cs[b], cs[k], 0};
+    const std::string key = "tri" + std::to_string(q) + ":" + std::to_string(L);
+    if (!(ts.mask & (1u << L))) {
+      ts.mask |= 1u << L;
+      make_digits(c, op, key, v, Kp, false, "tri" + std::to_string(q));
+    } else {
+      op.S = kEmuSlices;
+      op.slice = (long long)v.Z * v.R * Kp;
+      op.scale = scale_of(c, "tri" + std::to_string(q));
+      op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuSlices * 2);
+      op.lo = nullptr;
+    }
+    return;
+  }
   void *hi = c->raw(base + ":hi", n * 2), *lo = c->raw(base + ":lo", n * 2);
+  op.hi = hi;
+  op.lo = lo;
   if (!(ts.mask & (1u << L))) {
     ts.mask |= 1u << L;
     __nv_bfloat16 *h = static_cast<__nv_bfloat16 *>(hi), *l = static_cast<__nv_bfloat16 *>(lo);
@@ -1494,12 +1687,16 @@ std::pair<void *, void *> tri_layout(mlcc3_ctx *c, const double *X, int L) {
                               c->stream, c->is_tri32(X)), "split_bf16");
       });
   }
-  return {hi, lo};
 }
 
 void encode_split(mlcc3_ctx::SplitOp &op, const std::string &key, const unsigned long long dims[4],
                   const unsigned long long str[3], const unsigned bx[4]) {
   std::string err;
+  if (op.S > 0) {
+    if (!emu_encode_map(&op.mhi, op.hi, dims, str, (unsigned long long)op.slice * 2, bx + 1, op.S, &err))
+      throw Error{MLCC3_ERR_CUDA, "tensor map " + key + ": " + err};
+    return;
+  }
   if (!encode_map(&op.mhi, op.hi, dims, str, bx, &err) || !encode_map(&op.mlo, op.lo, dims, str, bx, &err))
     throw Error{MLCC3_ERR_CUDA, "tensor map " + key + ": " + err};
 }
@@ -1509,11 +1706,9 @@ void encode_split(mlcc3_ctx::SplitOp &op, const std::string &key, const unsigned
 // tensor maps over (K, row, -, block) with a box of `rows` rows.
 SplitOp &layout_XL(mlcc3_ctx *c, const std::string &key, const double *X, int k, unsigned rows) {
   S s(c);
-  auto hl = tri_layout(c, X, k);
   SplitOp &op = c->splits[key];
-  op.hi = hl.first;
-  op.lo = hl.second;
-  const unsigned long long Kp = (unsigned long long)((s.nv * s.nv + 63) / 64 * 64), nv = s.nv;
+  tri_layout(c, X, k, op);
+  const unsigned long long Kp = (unsigned long long)kpad(c, s.nv * s.nv), nv = s.nv;
   const unsigned long long dims[4] = {Kp, nv, 1ULL, (unsigned long long)c->chunk_nb};
   const unsigned long long str[3] = {Kp * 2, Kp * 2 * nv, Kp * 2 * nv};
   const unsigned bx[4] = {64, rows, 1, 1};
@@ -1524,11 +1719,9 @@ SplitOp &layout_XL(mlcc3_ctx *c, const std::string &key, const double *X, int k,
 // R_k: K = canonical position k, rows = the other two as (smaller, larger) pair tiles.
 SplitOp &layout_R(mlcc3_ctx *c, const std::string &key, const double *X, int k) {
   S s(c);
-  auto hl = tri_layout(c, X, 3 + k);
   SplitOp &op = c->splits[key];
-  op.hi = hl.first;
-  op.lo = hl.second;
-  const unsigned long long Kp = (unsigned long long)((s.nv + 63) / 64 * 64), nv = s.nv;
+  tri_layout(c, X, 3 + k, op);
+  const unsigned long long Kp = (unsigned long long)kpad(c, s.nv), nv = s.nv;
   const unsigned long long dims[4] = {Kp, nv, nv, (unsigned long long)c->chunk_nb};
   const unsigned long long str[3] = {Kp * 2, Kp * 2 * nv, Kp * 2 * nv * nv};
   const unsigned bx[4] = {64, 16, 8, 1};
@@ -1566,7 +1759,7 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
                                    " rows for tile width " + std::to_string(BN) +
                                    " (tc_wide_bn changed after build_integrals?)"};
   const long long nt1 = (s.nv + 7) / 8, nt2 = (s.nv + 15) / 16, ntN = (nN + BN - 1) / BN;
-  const int nk = (int)((s.nv + 63) / 64);
+  const int nk = kchunks(c, s.nv);
   for (int cls = 0; cls < 2; ++cls) {
     const std::string key = "tcP:" + okey + ":" + std::to_string(vk) + std::to_string(g) +
                             std::to_string(cls) + ":" + std::to_string(nN);
@@ -1585,12 +1778,13 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
               }
               pl.drop_empty_last();
             }
-    }, c->tc_kcap);
+    }, kcap(c));
     // rows of R are (smaller, larger) canonical positions: the view pair in
     // order (cls 0) or swapped (cls 1)
     TcEpi epi = make_epi(out, 2, 16, cls == 0 ? Sp1 : Sp2, cls == 0 ? Sp2 : Sp1, Sn, s.nv, s.nv,
                          nN, coef);
-    tc_launch(c, "pair", BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size() / 2.0);
+    tc_launch(c, "pair", BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size() / 2.0,
+              c->splits.at(xkey + ":R0"), B);
   }
 }
 
@@ -1607,7 +1801,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
   if (ords.empty() || s.nv == 0 || nN == 0) return;
   const int vk1 = vr == 0 ? 1 : 0, vk2 = vr == 2 ? 1 : 2;
   const int o1 = tpos == 0 ? 1 : 0, o2 = tpos == 2 ? 1 : 2;
-  const int BX = tc_tile_width(s.nv);
+  const int BX = tile_w(c, s.nv);
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (int k = 0; k < 3; ++k) {
@@ -1616,7 +1810,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
     maps.m[2 * k + 1] = r.mlo;
   }
   // T and Ts with 128-row boxes (rows past n read as zeros)
-  const unsigned long long Kp = (unsigned long long)((s.nv * s.nv + 63) / 64 * 64);
+  const unsigned long long Kp = (unsigned long long)kpad(c, s.nv * s.nv);
   const unsigned long long dims[4] = {Kp, (unsigned long long)nN, 1ULL, (unsigned long long)s.no};
   const unsigned long long str[3] = {Kp * 2, Kp * 2 * (unsigned long long)nN, Kp * 2 * (unsigned long long)nN};
   const unsigned bx[4] = {64, 128, 1, 1};
@@ -1628,7 +1822,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
   maps.m[8] = tsa.mhi;
   maps.m[9] = tsa.mlo;
   const long long ntM = (nN + 127) / 128, ntN = (s.nv + BX - 1) / BX;
-  const int nk = (int)((s.nv * s.nv + 63) / 64);
+  const int nk = kchunks(c, s.nv * s.nv);
   const std::string key = "tcX:" + okey + ":" + std::to_string(vr) + std::to_string(tpos) + ":" +
                           std::to_string(nN) + ":t";
   TcDev dv = tc_plan(c, key, [&](TcPlan &pl) {
@@ -1644,9 +1838,10 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
             }
             pl.drop_empty_last();
           }
-  }, c->tc_kcap);
+  }, kcap(c));
   TcEpi epi = make_epi(out, 2, 128, 0, 1, Srow, 1, nN, s.nv, coef);
-  tc_launch(c, "xt", BX, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size());
+  tc_launch(c, "xt", BX, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size(), T,
+            c->splits.at(xkey + ":XLB0"));
 }
 
 // out[c][d] (row stride ld) += alpha sum_{orderings} sum_{ab} X_{pqr}[a][b][c] Y_{pqr}[a][b][d]
@@ -1656,7 +1851,7 @@ void tc_vv(mlcc3_ctx *c, const double *X, const std::string &xkey, const double 
            long long ld, double alpha) {
   S s(c);
   if (ords.empty() || s.nv == 0) return;
-  const unsigned BN = (unsigned)tc_tile_width(s.nv);
+  const unsigned BN = (unsigned)tile_w(c, s.nv);
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (int k = 0; k < 3; ++k) {
@@ -1667,8 +1862,8 @@ void tc_vv(mlcc3_ctx *c, const double *X, const std::string &xkey, const double 
     maps.m[6 + 2 * k] = y.mhi;
     maps.m[6 + 2 * k + 1] = y.mlo;
   }
-  const long long ntM = (s.nv + 127) / 128;
-  const int nk = (int)((s.nv * s.nv + 63) / 64);
+  const long long ntM = (s.nv + 127) / 128, ntN = c->emu ? (s.nv + BN - 1) / BN : 1;
+  const int nk = kchunks(c, s.nv * s.nv);
   const size_t G = 16;  // orderings per tile (split K)
   // the mirror orderings (p,q,r) and (q,p,r) give the same segment (same block,
   // same layout: the K pair is in canonical order), so p > q runs once with
@@ -1680,46 +1875,51 @@ void tc_vv(mlcc3_ctx *c, const double *X, const std::string &xkey, const double 
     if (os.empty()) continue;
     TcDev dv = tc_plan(c, "tcV:" + okey + ":w" + std::to_string(w), [&](TcPlan &pl) {
       for (long long tm = 0; tm < ntM; ++tm)
+        for (long long tn = 0; tn < ntN; ++tn)
         for (size_t o0 = 0; o0 < os.size(); o0 += G) {
-          pl.tile(0, (int)(128 * tm), 0, 0);
+          pl.tile(0, (int)(128 * tm), (int)(BN * tn), 0);
           for (size_t i = o0; i < std::min(os.size(), o0 + G); ++i) {
             const Ord &o = os[i];
             const int u = (int)(o.off / s.nv3);
-            pl.seg(2 * o.sp[2], 6 + 2 * o.sp[2], nk, (int)(128 * tm), 0, u, 0, 0, u);
+            pl.seg(2 * o.sp[2], 6 + 2 * o.sp[2], nk, (int)(128 * tm), 0, u, (int)(BN * tn), 0, u);
           }
         }
-    }, c->tc_kcap);
+    }, kcap(c));
     TcEpi epi = make_epi(out, 2, 128, 0, ld, 1, 1, s.nv, s.nv, alpha * w);
-    tc_launch(c, "vv", (int)BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)s.nv * (double)os.size());
+    tc_launch(c, "vv", (int)BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)s.nv * (double)os.size(),
+              c->splits.at(xkey + ":XL0"), c->splits.at(ykey + ":YL0"));
   }
 }
 
 // Split copies of small operands (per call or at build):
 // amplitude block X[p][a][q][D] as [p][q][D][a] (Y1/P2 B operand)
-SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk) {
+SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk, const std::string &slot) {
   S s(c);
-  return make_split(c, key, Xblk, s.no, s.no, s.NV, s.nv, s.bi, s.bL, 1, s.ba, 1.0, Box::Row,
+  return make_split(c, key, Xblk, s.no, s.no, s.NV, s.nv, s.bi, s.bL, 1, s.ba, 1.0, Box::Row, slot,
                     (unsigned)pair_bn(c, s.NV));
 }
 // Go-like G[q][r][c][L] as [q][r][L][c] (Z_L B operand)
-SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G) {
+SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G, const std::string &slot) {
   S s(c);
-  return make_split(c, key, G, s.no, s.no, s.NO, s.nv, s.oj, s.ok, 1, s.oc, 1.0, Box::Row,
+  return make_split(c, key, G, s.no, s.no, s.NO, s.nv, s.oj, s.ok, 1, s.oc, 1.0, Box::Row, slot,
                     (unsigned)pair_bn(c, s.NO));
 }
 // Tl-like T[p][x][y][L] as [p][L][(x,y)] and [p][L][(y,x)] (tc_xt operands)
-void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T) {
+void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T, const std::string &slot) {
   S s(c);
-  const unsigned bn = (unsigned)tc_tile_width(s.NO);
-  make_split_k2(c, key + ":T", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.ta, s.tb, bn);
-  make_split_k2(c, key + ":Ts", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.tb, s.ta, bn);
+  const unsigned bn = (unsigned)tile_w(c, s.NO);
+  make_split_k2(c, key + ":T", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.ta, s.tb, bn, slot);
+  make_split_k2(c, key + ":Ts", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.tb, s.ta, bn, slot);
 }
 
 // Z[p][a][L][b] += cL sum_{qr} sum_c X_{pqr}[a][b][c] G_{qr}[c][L] on the tensor cores.
 void tc_back_L(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, const std::string &okey,
                const BackSet &b, double *Zb) {
   S s(c);
-  if (b.gl_convert) split_go_T(c, b.gl_key + ":T", b.GL);
+  if (b.gl_convert) {
+    scale_max(c, b.gl_key, {{b.GL, (long long)s.gosz()}});
+    split_go_T(c, b.gl_key + ":T", b.GL, b.gl_key);
+  }
   tc_pair(c, X, "X", c->splits.at(b.gl_key + ":T"), s.NO, ords, okey, 2, 0, s.bi, s.ba, 1, s.bL,
           b.cL, Zb);
 }
@@ -1734,7 +1934,7 @@ struct CholTerm {
 };
 void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, long long nN,
              long long Sw, long long Sk, long long Sc, double alpha, int mode, double *out,
-             const std::string &key) {
+             const std::string &key, long long Sn = 1) {
   S s(c);
   const long long M = s.no * s.nv;
   if (M == 0 || nN == 0 || nW == 0) return;
@@ -1747,12 +1947,12 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
     maps.m[4 * t + 2] = terms[t].B->mhi;
     maps.m[4 * t + 3] = terms[t].B->mlo;
   }
-  const int BN = tc_tile_width(nN);
+  const int BN = tile_w(c, nN);
   const long long ntM = (M + 127) / 128, ntN = (nN + BN - 1) / BN;
-  const int nk = (int)((s.NJ + 63) / 64);
+  const int nk = kchunks(c, s.NJ);
   // one accumulation chain per tile when it is short enough, else pieces
   // summed in FP64 into the zeroed output
-  const bool pieces = c->tc_kcap > 0 && nk * (int)terms.size() > c->tc_kcap;
+  const bool pieces = kcap(c) > 0 && nk * (int)terms.size() > kcap(c);
   if (pieces) {
     if (mode == 3) c->zero(out, (size_t)((nW - 1) * Sw + (s.no - 1) * Sk + (s.nv - 1) * Sc + nN));
     mode = 2;
@@ -1766,25 +1966,25 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
             pl.seg((int)(4 * t), (int)(4 * t + 2), nk, (int)(128 * tm), 0, 0, (int)(BN * tn),
                    (int)w, 0);
         }
-  }, pieces ? c->tc_kcap : 0);
-  TcEpi epi = make_epi(out, mode, (int)s.nv, Sk, Sc, 1, s.no, s.nv, nN, alpha, 1);
+  }, pieces ? kcap(c) : 0);
+  TcEpi epi = make_epi(out, mode, (int)s.nv, Sk, Sc, Sn, s.no, s.nv, nN, alpha, 1);
   tc_launch(c, "chol", BN, maps, dv, epi, 2.0 * (double)M * (double)nN * (double)nW * (double)s.NJ *
-                                      (double)terms.size());
+                                      (double)terms.size(), *terms[0].A, *terms[0].B);
 }
 
 // Split copies over the Cholesky index (K = J, stride lJ = n_mo^2 in Lt-like arrays).
 // rows (k,c) of X[J][r0 + c][k] (row offset r0, c stride cs, k stride ks), Flat 128-row box
 SplitOp &split_kc(mlcc3_ctx *c, const std::string &key, const double *X, long long ks, long long cs,
-                  long long Js) {
+                  long long Js, const std::string &slot) {
   S s(c);
-  return make_split(c, key, X, 1, s.no, s.nv, s.NJ, 0, ks, cs, Js, 1.0, Box::Flat, 128);
+  return make_split(c, key, X, 1, s.no, s.nv, s.NJ, 0, ks, cs, Js, 1.0, Box::Flat, slot, 128);
 }
 // rows (w, n) of X with strides (ws, ns), K = J (stride Js), Row box of BN rows
 SplitOp &split_wn(mlcc3_ctx *c, const std::string &key, const double *X, long long nW, long long nN,
-                  long long ws, long long ns, long long Js) {
+                  long long ws, long long ns, long long Js, const std::string &slot) {
   S s(c);
-  return make_split(c, key, X, 1, nW, nN, s.NJ, 0, ws, ns, Js, 1.0, Box::Row,
-                    (unsigned)tc_tile_width(nN));
+  return make_split(c, key, X, 1, nW, nN, s.NJ, 0, ws, ns, Js, 1.0, Box::Row, slot,
+                    (unsigned)tile_w(c, nN));
 }
 
 // Gv[k][b][c][D] = sum_J Lt[J][NO+c][k] Lt[J][NO+b][NO+D] and
@@ -1793,32 +1993,44 @@ void tc_integrals(mlcc3_ctx *c) {
   S s(c);
   const long long nmo = s.nmo, NO = s.NO;
   const double *Lt = c->Lt;
-  split_kc(c, "LvoT", Lt + NO * nmo, 1, nmo, s.lJ);
-  split_kc(c, "LovT", Lt + NO, nmo, 1, s.lJ);
-  split_wn(c, "LvVT", Lt + NO * nmo + NO, s.nv, s.NV, nmo, 1, s.lJ);
-  split_wn(c, "LVvT", Lt + NO * nmo + NO, s.nv, s.NV, 1, nmo, s.lJ);
-  split_wn(c, "LOoT", Lt, s.no, s.NO, 1, nmo, s.lJ);
+  scale_max(c, "Lt", {{Lt, s.NJ * s.lJ}});
+  split_kc(c, "LvoT", Lt + NO * nmo, 1, nmo, s.lJ, "Lt");
+  split_kc(c, "LovT", Lt + NO, nmo, 1, s.lJ, "Lt");
+  split_wn(c, "LvVT", Lt + NO * nmo + NO, s.nv, s.NV, nmo, 1, s.lJ, "Lt");
+  split_wn(c, "LVvT", Lt + NO * nmo + NO, s.nv, s.NV, 1, nmo, s.lJ, "Lt");
+  split_wn(c, "LOoT", Lt, s.no, s.NO, 1, nmo, s.lJ, "Lt");
   tc_chol(c, {{&c->splits.at("LvoT"), &c->splits.at("LvVT")}}, s.nv, s.NV, s.gb, s.gk, s.gc, 1.0, 3,
           c->Gv, "Gv");
   tc_chol(c, {{&c->splits.at("LovT"), &c->splits.at("LVvT")}}, s.nv, s.NV, s.gb, s.gk, s.gc, 1.0, 3,
           c->Gb, "Gb");
+  if (!c->emu) return;
+  // FP64 mode: the small blocks g_Ljck, g_jLkc, g_jbkc as well
+  const SplitOp &LoOT = split_wn(c, "LoOT", Lt, s.no, s.NO, nmo, 1, s.lJ, "Lt");
+  const SplitOp &LovB = split_wn(c, "LovB", Lt + NO, s.no, s.nv, nmo, 1, s.lJ, "Lt");
+  tc_chol(c, {{&c->splits.at("LvoT"), &c->splits.at("LOoT")}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, c->Go, "Go");
+  tc_chol(c, {{&c->splits.at("LovT"), &LoOT}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, c->Gx, "Gx");
+  tc_chol(c, {{&c->splits.at("LovT"), &LovB}}, s.no, s.nv, s.vj, s.vk, 1, 1.0, 3, c->Govov, "Govov", s.vb);
 }
 
 // Upsilon_bDck, Upsilon_Ljck, H1, H2 on the tensor cores (split mode).
 bool tc_upsilon(mlcc3_ctx *c, const double *LRvV, const double *LRvo, const double *LROo,
                 const double *PA, const double *PB, double *Uv, double *Uo, double *H1, double *H2) {
-  if (!split_mode(c)) return false;
+  if (!tc_mode(c)) return false;
   S s(c);
-  const SplitOp &rvV = split_wn(c, "LRvVT", LRvV, s.nv, s.NV, s.NV, 1, s.nv * s.NV);
-  const SplitOp &rvo = split_kc(c, "LRvoT", LRvo, 1, s.no, s.nv * s.no);
-  const SplitOp &rOo = split_wn(c, "LROoT", LROo, s.no, s.NO, 1, s.no, s.NO * s.no);
+  // one scale for the three factors: each product below pairs one with Lt
+  scale_max(c, "LR", {{LRvV, s.NJ * s.nv * s.NV}, {LRvo, s.NJ * s.nv * s.no}, {LROo, s.NJ * s.NO * s.no}});
+  const SplitOp &rvV = split_wn(c, "LRvVT", LRvV, s.nv, s.NV, s.NV, 1, s.nv * s.NV, "LR");
+  const SplitOp &rvo = split_kc(c, "LRvoT", LRvo, 1, s.no, s.nv * s.no, "LR");
+  const SplitOp &rOo = split_wn(c, "LROoT", LROo, s.no, s.NO, 1, s.no, s.NO * s.no, "LR");
   const SplitOp &vo = c->splits.at("LvoT"), &ov = c->splits.at("LovT");
   const SplitOp &vV = c->splits.at("LvVT"), &Oo = c->splits.at("LOoT");
   tc_chol(c, {{&vo, &rvV}, {&rvo, &vV}}, s.nv, s.NV, s.gb, s.gk, s.gc, 1.0, 3, Uv, "Uv");
   tc_chol(c, {{&vo, &rOo}, {&rvo, &Oo}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, Uo, "Uo");
   if (!H1) return true;  // no rho tau-term intermediates wanted
-  const SplitOp &pa = split_wn(c, "PAT", PA, s.no, s.NO, s.NO, 1, s.no * s.NO);
-  const SplitOp &pb = split_wn(c, "PBT", PB, s.nv, s.NV, s.NV, 1, s.nv * s.NV);
+  scale_max(c, "PA", {{PA, s.NJ * s.no * s.NO}});
+  scale_max(c, "PB", {{PB, s.NJ * s.nv * s.NV}});
+  const SplitOp &pa = split_wn(c, "PAT", PA, s.no, s.NO, s.NO, 1, s.no * s.NO, "PA");
+  const SplitOp &pb = split_wn(c, "PBT", PB, s.nv, s.NV, s.NV, 1, s.nv * s.NV, "PB");
   tc_chol(c, {{&ov, &pa}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, H1, "H1");
   tc_chol(c, {{&ov, &pb}}, s.nv, s.NV, s.gb, s.gk, s.gc, -1.0, 3, H2, "H2");
   return true;
@@ -1845,9 +2057,18 @@ void left_triples(mlcc3_ctx *c, const std::string &tag, const double *L1, const 
       term(1, (int)s.NO, -1.0, LcT, {s.ti, s.ta, s.tb, 1}, c->Gx, {s.oj, s.ok, s.oc, 1}),
       term(2, 0, 0.5, L1, {1, s.NO, 0, 0}, c->Govov, {s.vj, s.vk, s.vb, 1}),
       term(3, 0, 0.5, Lc, {s.bi, s.bL, s.ba, 1}, c->F, {s.nv, 1, 0, 0})};
-  if (!split_mode(c)) {
+  if (!tc_mode(c)) {
     triples(c, full, bkey, bs, omega, out);
     contra3(c, out, outt, nbt);
+    return;
+  }
+  const std::string lslot = "Lc:" + tag;
+  if (convert) scale_max(c, lslot, {{Lc, (long long)s.blk()}});
+  if (c->emu) {
+    full[2].sym = full[3].sym = 1;  // g_jbkc and Lc are symmetric under exchange of their pairs
+    SplitTerm d = split_d(c, tag + "c", Lc, convert, "Gb", c->Gb, false, lslot, "Gb");
+    SplitTerm l = split_l(c, tag + "cT", LcT, convert, "Gx", c->Gx, false, lslot, "Gb");
+    triples_split(c, {d, l}, {full[2], full[3]}, bkey, bs, omega, out, outt, nbt, keep_out);
     return;
   }
   // the rank-1 terms' operands are pair-symmetric (g_jbkc, Lc), and L1 is also
@@ -1870,8 +2091,8 @@ void left_triples(mlcc3_ctx *c, const std::string &tag, const double *L1, const 
   full[2].B32 = static_cast<const float *>(c->raw("f32:Govov", 4));
   full[3].A32 = f32_cached(c, "Lc:" + tag, Lc, (long long)s.blk(), convert);
   full[3].B32 = static_cast<const float *>(c->raw("f32:F", 4));
-  SplitTerm d = split_d(c, tag + "c", Lc, convert, "Gb", c->Gb, false);
-  SplitTerm l = split_l(c, tag + "cT", LcT, convert, "Gx", c->Gx, false);
+  SplitTerm d = split_d(c, tag + "c", Lc, convert, "Gb", c->Gb, false, lslot, "Gb");
+  SplitTerm l = split_l(c, tag + "cT", LcT, convert, "Gx", c->Gx, false, lslot, "Gb");
   triples_split(c, {d, l}, {full[2], full[3]}, bkey, bs, omega, out, outt, nbt, keep_out);
 }
 
@@ -1915,7 +2136,7 @@ void build_tau(mlcc3_ctx *c, const Chunk &ch, double **tau, double **taut) {
   if (c->tau_valid && c->tau_key == ch.key) return;
   c->tau_valid = true;
   c->tau_key = ch.key;
-  if (split_mode(c)) {
+  if (tc_mode(c)) {
     triples_split(c, tau_split_terms(c), {}, "b" + ch.key, ch.bs, 0.0, *tau, *taut, ch.nb);
   } else {
     triples(c, tau_terms(c), "b" + ch.key, ch.bs, 0.0, *tau);
@@ -2006,7 +2227,7 @@ void right_triples(mlcc3_ctx *c, const double *Rbar, const double *Rbl, const Up
                    double *out, double *outt, long long nbt, const std::string &tag = "",
                    bool convert = true, bool convert_u = true) {
   S s(c);
-  if (!split_mode(c)) {
+  if (!tc_mode(c)) {
     std::vector<TripTerm> terms = {
         term(0, (int)s.NV, 1.0, Rbar, {s.bi, s.bL, s.ba, 1}, c->Gv, {s.gk, s.gb, s.gc, 1}),
         term(1, (int)s.NO, -1.0, Rbl, {s.ti, s.ta, s.tb, 1}, c->Go, {s.oj, s.ok, s.oc, 1}),
@@ -2016,10 +2237,17 @@ void right_triples(mlcc3_ctx *c, const double *Rbar, const double *Rbl, const Up
     contra3(c, out, outt, nbt);
     return;
   }
-  SplitTerm d1 = split_d(c, "Rbar" + tag, Rbar, convert, "Gv", c->Gv, false);
-  SplitTerm l1 = split_l(c, "Rbarl" + tag, Rbl, convert, "Go", c->Go, false);
-  SplitTerm d2 = split_d(c, "t", c->t2c, false, "Uv", u.Uv, convert_u);
-  SplitTerm l2 = split_l(c, "Tl", c->Tl, false, "Uo", u.Uo, convert_u);
+  const std::string rslot = "Rbar" + tag, uslot = "U" + tag;
+  if (c->emu && convert) {
+    scale_max(c, rslot, {{Rbar, (long long)s.blk()}});
+    scale_max(c, uslot, {{u.Uv, (long long)s.gvsz()}, {u.Uo, (long long)s.gosz()}});
+    check_cuda(emu_balance(scale_of(c, rslot), scale_of(c, "G"), scale_of(c, "t"), scale_of(c, uslot),
+                           c->stream), "emu_balance");
+  }
+  SplitTerm d1 = split_d(c, "Rbar" + tag, Rbar, convert, "Gv", c->Gv, false, rslot, "G");
+  SplitTerm l1 = split_l(c, "Rbarl" + tag, Rbl, convert, "Go", c->Go, false, rslot, "G");
+  SplitTerm d2 = split_d(c, "t", c->t2c, false, "Uv", u.Uv, convert_u, "t", uslot);
+  SplitTerm l2 = split_l(c, "Tl", c->Tl, false, "Uo", u.Uo, convert_u, "t", uslot);
   triples_split(c, {d1, l1, d2, l2}, {}, bkey, bs, omega, out, outt, nbt);
 }
 
@@ -2063,13 +2291,14 @@ static void do_build_integrals(mlcc3_ctx *c, const double *chol_in, const double
   sh = Shape{};
   sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.nv; sh.N2 = s.NV; sh.K1 = s.NJ;
   // Gv[k][b][c][D] = g_bDck: A(k,c;J) = Lt[J][NO+c][k], B(J;b,D) = Lt[J][NO+b][NO+D]
-  if (split_mode(c)) {
+  if (tc_mode(c)) {
     tc_integrals(c);  // Gv, Gb on the tensor cores
   } else {
   c->bstc1(Lt + NO * nmo, Lt + NO * nmo + NO, c->Gv, sh, 1.0, mk_item(0, 0, 0, {1, nmo, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.gk, s.gc, s.gb, 1}), "Gv");
   // Gb[k][b][c][D] = g_Dbkc: A(k,c;J) = Lt[J][k][NO+c], B(J;b,D) = Lt[J][NO+D][NO+b]
   c->bstc1(Lt + NO, Lt + NO * nmo + NO, c->Gb, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, 1, nmo}, {s.gk, s.gc, s.gb, 1}), "Gb");
   }
+  if (!c->emu) {
   sh = Shape{};
   sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.no; sh.N2 = NO; sh.K1 = s.NJ;
   // Go[j][k][c][L] = g_Ljck: A(k,c;J) = Lt[J][NO+c][k], B(J;j,L) = Lt[J][L][j]
@@ -2080,8 +2309,10 @@ static void do_build_integrals(mlcc3_ctx *c, const double *chol_in, const double
   sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.no; sh.N2 = s.nv; sh.K1 = s.NJ;
   // Govov[j][b][k][c] = g_jbkc: A(k,c;J) = Lt[J][k][NO+c], B(J;j,b) = Lt[J][j][NO+b]
   c->bstc1(Lt + NO, Lt + NO, c->Govov, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.vk, 1, s.vj, s.vb}), "Govov");
+  }
   fock_ov(c, c->t1, c->F, "F");
   transpose_tl(c, c->t2c, c->Tl);
+  if (c->emu) build_split_persistent(c);
   if (split_mode(c)) {
     build_split_persistent(c);
     f32_copy(c, "Govov", c->Govov, s.no * s.nv * s.no * s.nv);
@@ -2220,9 +2451,10 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     for (double *p : {Y2, P1}) c->zero(p, s.gosz());
     c->zero(Y3, s.no * s.nv);
     const SplitOp *LcA = nullptr;
-    if (split_mode(c)) {
-      LcA = &split_amp_T(c, "Lc:AT", Lc);
-      split_tl_T(c, "LcT", LcT);
+    if (tc_mode(c)) {
+      scale_max(c, "LcA", {{Lc, (long long)s.blk()}});
+      LcA = &split_amp_T(c, "Lc:AT", Lc, "LcA");
+      split_tl_T(c, "LcT", LcT, "LcA");
     }
     const double *Lc32 = f32_operand(c, "Lc:y3", Lc, (long long)s.blk(), true);
     for (const Chunk &ch : chunks) {
@@ -2244,7 +2476,7 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
       int n = 0;
       const BstcItem *it;
       Shape sh;
-      if (split_mode(c)) {
+      if (tc_mode(c)) {
         // tensor cores: Y1/P2 (K = a, rows (b,c)), Y2/P1 (K = (a,b), rows c)
         tc_pair(c, L3t, "X", c->splits.at("t:AT"), s.NV, os, okey, 0, 2, s.gk, s.gb, s.gc, 1, 1.0, Y1);
         tc_pair(c, taut, "X", *LcA, s.NV, os, okey, 0, 2, s.gk, s.gb, s.gc, 1, 1.0, P2);
@@ -2293,9 +2525,10 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     c->zero(Z4, s.NJ * s.no * NO);
     c->zero(yv, s.NJ);
     // W[J][k][c] = sum_{b,D} Y1[k][b][c][D] Lt[J][NO+b][NO+D] - sum_{L,j} Y2[j][k][c][L] Lt[J][L][j]
-    const bool tc = split_mode(c);
+    const bool tc = tc_mode(c);
     if (tc) {
-      const SplitOp &a = make_split_k2(c, "Y1:kc", Y1, s.no, s.nv, s.nv, s.NV, s.gk, s.gc, s.gb, 1, 128, true);
+      scale_max(c, "Y1", {{Y1, (long long)s.gvsz()}});
+      const SplitOp &a = make_split_k2(c, "Y1:kc", Y1, s.no, s.nv, s.nv, s.NV, s.gk, s.gc, s.gb, 1, 128, "Y1", true);
       tc_flat_gemm(c, a, c->splits.at("LvV:J"), s.no * s.nv, s.NJ, s.nv * s.NV, W, (int)s.nv, s.nv, 1,
                    s.no * s.nv, 1.0, "sg1");
     } else {
@@ -2312,7 +2545,7 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     c->bstc1(W, Lt, sig1, sh, -1.0, mk_item(0, 0, 0, {1, 0, s.no * s.nv, s.nv, 0}, {s.lJ, 1, 0, nmo, 0}, {NO, 0, 1, 0}), "sg4");
     // Z2[J][b][D] = sum_{c,k} Y1[k][b][c][D] Lt[J][NO+c][k];  sigma[b][M] -= sum_{J,D} Z2 Lt[J][M][NO+D]
     if (tc) {
-      const SplitOp &a = make_split_k2(c, "Y1:bD", Y1, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, true);
+      const SplitOp &a = make_split_k2(c, "Y1:bD", Y1, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, "Y1", true);
       tc_flat_gemm(c, a, c->splits.at("Lvo:J"), s.nv * s.NV, s.NJ, s.nv * s.no, Z2, (int)s.NV, s.NV, 1,
                    s.nv * s.NV, 1.0, "sg5");
     } else {
@@ -2346,7 +2579,8 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     // P2 term: Q2[J][b][D] = sum_{c,k} P2[k][b][c][D] Lt[J][k][NO+c]; sigma[D][L] -= sum_{J,b} Q2 Lt[J][L][NO+b]
     c->zero(Q2, s.NJ * s.nv * s.NV);
     if (tc) {
-      const SplitOp &a = make_split_k2(c, "P2:bD", P2, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, true);
+      scale_max(c, "P2", {{P2, (long long)s.gvsz()}});
+      const SplitOp &a = make_split_k2(c, "P2:bD", P2, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, "P2", true);
       tc_flat_gemm(c, a, c->splits.at("Lov:J"), s.nv * s.NV, s.NJ, s.nv * s.no, Q2, (int)s.NV, s.NV, 1,
                    s.nv * s.NV, 1.0, "sg15");
     } else {
@@ -2651,13 +2885,13 @@ void density_left_gpu(mlcc3_ctx *c, const Chunk &ch, const double *Xt3, const do
   y3_like(c, taut, Lc, ch.own, okey, D + NO, nmo, 0.5, "y3d");
   // D_LD -= sum Xt^{abc}_{ijk} t^{ac}_{iL} t^{bD}_{jk}  (V summed over the chunks)
   double *V = dld_acc(c, acc, c->t2c, D, -1.0, "dLD");
-  if (split_mode(c))
+  if (tc_mode(c))
     tc_xt(c, Xt3, "X", c->splits.at("Tl:T"), c->splits.at("Tl:Ts"), s.NO, ch.own, okey, 1, 0,
           s.oj, s.ok, s.oc, 1.0, V);
   else
     v_like(c, Xt3, c->Tl, ch.own, okey, V);
   // D_cd += 1/2 sum Xt^{abc}_{ijk} tau^{abd}_{ijk}
-  if (split_mode(c))
+  if (tc_mode(c))
     tc_vv(c, Xt3, "X", tau, "Y", ch.own, okey, D + NO * nmo + NO, nmo, 0.5);
   else
     vv_block(c, Xt3, tau, ch.own, okey, D + NO * nmo + NO, nmo, 0.5);
@@ -2767,7 +3001,10 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     double *D = so.D0m, *sc = scall + 2 * st;
     const std::string stag = std::to_string(st);
     // split copies of the state's operands: made at the first chunk, kept per state
-    if (split_mode(c) && first) split_tl_T(c, "Rbl" + stag, Rbl);
+    if (tc_mode(c) && first) {
+      scale_max(c, "Rbl" + stag, {{Rbl, s.no * s.nv * s.nv * NO}});
+      split_tl_T(c, "Rbl" + stag, Rbl, "Rbl" + stag);
+    }
     // L3 (omega) and R3 (omega), with their contravariant forms (CVS: core batches only)
     double *L3 = c->tri_buf("L3", bw);
     double *L3t = c->tri_buf("L3t", bw);
@@ -2857,14 +3094,14 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     c->bstc1(c->t2x, W3, D + NO, sh, -1.0, mk_item(0, 0, 0, {s.bL, 1, s.bi, s.ba, 0}, {s.nv, 1, 0, 0, 0}, {nmo, 1, 0, 0}), "dLDw");
     //   D_LD -= sum lt^{abc}_{ijk} Rbar^{ac}_{iL} t^{bD}_{jk}  (V, V3 summed over the chunks)
     double *V = dld_acc(c, "D0m:" + std::to_string(st), c->t2c, D, -1.0, "dLD");
-    if (split_mode(c))
+    if (tc_mode(c))
       tc_xt(c, lt3, "X", c->splits.at("Rbl" + stag + ":T"), c->splits.at("Rbl" + stag + ":Ts"), s.NO, ch.own, okey, 1, 0,
             s.oj, s.ok, s.oc, 1.0, V);
     else
       v_like(c, lt3, Rbl, ch.own, okey, V);
     //   D_LD -= sum lt^{abc}_{ijk} Rbar^{aD}_{ik} t^{bc}_{jL}
     double *V3 = dld_acc(c, "D0m3:" + std::to_string(st), Rbar, D, -1.0, "dLD3");
-    if (split_mode(c)) {
+    if (tc_mode(c)) {
       tc_xt(c, lt3, "X", c->splits.at("Tl:T"), c->splits.at("Tl:Ts"), s.NO, ch.own, okey, 0, 1,
             s.oj, s.ok, s.oc, 1.0, V3);
     } else {
@@ -2886,7 +3123,7 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     c->bstc1(E, R1, D + NO, sh, -0.5, mk_item(0, 0, 0, {s.no, 0, 1, 0, 0}, {1, 0, 0, NO, 0}, {nmo, 0, 1, 0}), "dlD");
     // D_Ld -= 1/2 sum_c E2[c][d] R^c_L,  E2[c][d] = sum lt^{abc}_{ijk} tau^{abd}_{ijk}
     double *E2 = E + s.no * s.no;
-    if (split_mode(c))
+    if (tc_mode(c))
       tc_vv(c, lt3, "X", tau, "Y", ch.own, okey, E2, s.nv, 1.0);
     else
       vv_block(c, lt3, tau, ch.own, okey, E2, s.nv, 1.0);
@@ -2899,7 +3136,7 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     sh = Shape{}; sh.M1 = s.nv; sh.N1 = s.NV; sh.K1 = nj; sh.K2 = s.no; sh.K3 = s.nv;
     c->bstc1(U, c->t2c, D + NO * nmo + NO, sh, 1.0, mk_item(ch.p0 * s.no * s.nv * s.nv, ch.p0 * s.bi, 0, {1, 0, s.no * s.nv * s.nv, s.nv * s.nv, s.nv}, {s.bi, s.bL, s.ba, 1, 0}, {nmo, 0, 1, 0}), okey + ":dcD");
     // D_cd += 1/2 sum lt^{abc}_{ijk} R^{abd}_{ijk}
-    if (split_mode(c))
+    if (tc_mode(c))
       tc_vv(c, lt3, "X", R3, "Y", ch.own, okey, D + NO * nmo + NO, nmo, 0.5);
     else
       vv_block(c, lt3, R3, ch.own, okey, D + NO * nmo + NO, nmo, 0.5);
@@ -3038,6 +3275,7 @@ extern "C" int mlcc3_create(mlcc3_ctx **out, const mlcc3_dims *d, int precision,
       alloc(&c->dscal, 16);
       check_cuda(cudaMalloc(&c->status, sizeof(int)), "cudaMalloc status");
       check_cuda(cudaMemset(c->status, 0, sizeof(int)), "memset status");
+      choose_emu(c);
       make_batches(c);
       make_chunks(c);
     } catch (...) {
@@ -3262,6 +3500,15 @@ extern "C" int mlcc3_set_param(mlcc3_ctx *c, const char *name, long long value) 
     } else if (n == "bstc_big_from") {
       if (value < 0) throw Error{MLCC3_ERR_ARG, "bstc_big_from must be >= 0"};
       c->bstc_big_from = value;
+    } else if (n == "fp64_tc_from") {
+      if (value < 1 || value > (1LL << 30)) throw Error{MLCC3_ERR_ARG, "fp64_tc_from must be 1..2^30"};
+      c->fp64_tc_from = value;
+      if (c->precision == MLCC3_FP64) {
+        const bool was = c->emu;
+        choose_emu(c);
+        if (c->emu != was) c->built = false;  // the operands the integral build prepares differ
+        make_chunks(c);
+      }
     } else if (n == "finish_fused") {
       if (value != 0 && value != 1) throw Error{MLCC3_ERR_ARG, "finish_fused must be 0 or 1"};
       c->finish_fused = value == 1;
