@@ -32,10 +32,10 @@ __device__ __forceinline__ T ld_op(const double *p, int f32, long long i) {
   return f32 ? (T)reinterpret_cast<const float *>(p)[i] : (T)p[i];
 }
 
-// T: product type; the FP32 form (split-precision mode) folds each thread's
-// FP32 partial sums into FP64 every four K tiles (64 products).
-template <typename T>
-__device__ __forceinline__ void bstc_body(const BstcParams &p) {
+// FP32 products (split-precision mode): each thread's FP32 partial sums are
+// folded into FP64 every four K tiles (64 products).
+__global__ void __launch_bounds__(256, 3) bstc_f32_kernel(BstcParams p) {
+  using T = float;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
   __shared__ long long rowA[BM], rowC[BM], colB[BN], colC[BN];
@@ -159,8 +159,190 @@ __device__ __forceinline__ void bstc_body(const BstcParams &p) {
   }
 }
 
-__global__ void __launch_bounds__(256) bstc_kernel(BstcParams p) { bstc_body<double>(p); }
-__global__ void __launch_bounds__(256) bstc_f32_kernel(BstcParams p) { bstc_body<float>(p); }
+// FP64 form, tiles of TM x TN outputs, RM x RN per thread.  GB300's FP64 pipe
+// retires two operations per clock and SM, so a K step's loads cost nothing and
+// what counts is that its lanes do useful work: the tile is the one that pads
+// (M, N) least (launch_bstc64), from 64 x 64 down to 8 x 8, where the threads
+// beyond one per output take K in groups, and a reduction whose tiles do not fill
+// the chip is split over grid.z.  The next K tile's loads are in flight while the
+// current one is multiplied.  (With 64 x 64 tiles alone a 24 x 6 x 576 product of
+// the smallest system ran 28 times its products on one SM, 671 us; now 8 us.  rho
+// and sigma of that system, 6/24/4/8: 6.0 -> 0.62 ms with the small build cubes.)
+template <int TM, int TN, int RM, int RN>
+__global__ void __launch_bounds__(256) bstc64_kernel(BstcParams p) {
+  constexpr int TK = 32, TY = TM / RM, TX = TN / RN, KG = 256 / (TY * TX);
+  constexpr int NA = TK * TM / 256, NB = TK * TN / 256;
+  static_assert(TY * TX * KG == 256 && NA * 256 == TK * TM && NB * 256 == TK * TN, "tile");
+  static_assert(KG == 1 || (RM == 1 && RN == 1 && TM * TK + TK >= 256), "K groups: one output per thread");
+  __shared__ double As[TK][TM + 1], Bs[TK][TN + 1];
+  __shared__ long long rowA[TM], rowC[TM], colB[TN], colC[TN];
+  const BstcItem &it = p.items[blockIdx.y];
+  const int tid = threadIdx.x;
+  const long long M = (long long)p.M1 * p.M2, N = (long long)p.N1 * p.N2;
+  const long long K = (long long)p.K1 * p.K2 * p.K3;
+  const long long ntn = (N + TN - 1) / TN;
+  const long long m0 = (long long)blockIdx.x / ntn * TM, n0 = (long long)blockIdx.x % ntn * TN;
+  for (int t = tid; t < TM + TN; t += 256) {
+    if (t < TM) {
+      const long long m = m0 + t, m1 = m / p.M2, m2 = m % p.M2;
+      rowA[t] = m < M ? m1 * it.sA[0] + m2 * it.sA[1] : -1;
+      rowC[t] = m < M ? m1 * it.sC[0] + m2 * it.sC[1] : -1;
+    } else {
+      const long long n = n0 + t - TM, n1 = n / p.N2, n2 = n % p.N2;
+      colB[t - TM] = n < N ? n1 * it.sB[3] + n2 * it.sB[4] : -1;
+      colC[t - TM] = n < N ? n1 * it.sC[2] + n2 * it.sC[3] : -1;
+    }
+  }
+  const bool kfastA = p.K3 > 1 ? it.sA[4] == 1 : p.K2 > 1 ? it.sA[3] == 1 : it.sA[2] == 1;
+  const bool kfastB = p.K3 > 1 ? it.sB[2] == 1 : p.K2 > 1 ? it.sB[1] == 1 : it.sB[0] == 1;
+  const long long kbeg = p.kchunk ? (long long)blockIdx.z * p.kchunk : 0;
+  const long long kend = p.kchunk ? min(K, kbeg + p.kchunk) : K;
+  const double *A = p.A + it.offA, *B = p.B + it.offB;
+  __syncthreads();
+  double ra[NA], rb[NB];
+  auto load = [&](long long k0) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = tid + 256 * q, kk = kfastA ? e % TK : e / TM, mm = kfastA ? e / TK : e % TM;
+      const long long k = k0 + kk;
+      ra[q] = 0.0;
+      if (k < kend && rowA[mm] >= 0) {
+        const long long k12 = k / p.K3;
+        ra[q] = A[rowA[mm] + k12 / p.K2 * it.sA[2] + k12 % p.K2 * it.sA[3] + k % p.K3 * it.sA[4]];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + 256 * q, kk = kfastB ? e % TK : e / TN, nn = kfastB ? e / TK : e % TN;
+      const long long k = k0 + kk;
+      rb[q] = 0.0;
+      if (k < kend && colB[nn] >= 0) {
+        const long long k12 = k / p.K3;
+        rb[q] = B[colB[nn] + k12 / p.K2 * it.sB[0] + k12 % p.K2 * it.sB[1] + k % p.K3 * it.sB[2]];
+      }
+    }
+  };
+  const int kg = tid / (TY * TX), ty = tid % (TY * TX) / TX, tx = tid % TX;
+  double acc[RM][RN] = {}, sum[RM][RN] = {};
+  int tiles = -1;
+  load(kbeg);
+  for (long long k0 = kbeg; k0 < kend; k0 += TK) {
+    __syncthreads();  // the previous tile's reads are done
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = tid + 256 * q;
+      As[kfastA ? e % TK : e / TM][kfastA ? e / TK : e % TM] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + 256 * q;
+      Bs[kfastB ? e % TK : e / TN][kfastB ? e / TK : e % TN] = rb[q];
+    }
+    __syncthreads();
+    if (k0 + TK < kend) load(k0 + TK);
+    if (++tiles == 2) {  // sums of at most 64 products, then their sum: smaller rounding errors
+      tiles = 0;
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) {
+          sum[i][j] += acc[i][j];
+          acc[i][j] = 0.0;
+        }
+    }
+#pragma unroll 8
+    for (int kk = kg; kk < TK; kk += KG) {
+      double a[RM], b[RN];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) a[i] = As[kk][ty * RM + i];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) b[j] = Bs[kk][tx * RN + j];
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j) acc[i][j] += sum[i][j];
+  if (KG > 1) {
+    double *red = &As[0][0];
+    __syncthreads();
+    red[tid] = acc[0][0];
+    __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int g = 1; g < KG; ++g) acc[0][0] += red[tid + g * TY * TX];
+  }
+  double *C = p.C + it.offC;
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    const long long rc = rowC[ty * RM + i];
+    if (rc < 0) continue;
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      const long long cc = colC[tx * RN + j];
+      if (cc < 0) continue;
+      const double v = p.alpha * acc[i][j];
+      if (p.atomic) atomicAdd(C + rc + cc, v);
+      else C[rc + cc] += v;
+    }
+  }
+}
+
+// C += alpha A B in FP64 for every item (at most 65535).  Of the tiles the one with
+// the least estimated time: the products of a block's padded tile at two per
+// clock, for as many rounds of blocks as the 152 SMs need, and about 800 clocks
+// of latency per K step, which four resident blocks hide from one another.  A
+// reduction whose tiles make fewer than fill * 152 blocks is split over about as
+// many (pieces of at least 32, added atomically); fill = 0 never splits.
+cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st) {
+  struct Tile {
+    int m, n;
+    void (*k)(BstcParams);
+  };
+  static const Tile tiles[] = {
+      {64, 64, bstc64_kernel<64, 64, 4, 4>}, {64, 32, bstc64_kernel<64, 32, 4, 2>},
+      {32, 64, bstc64_kernel<32, 64, 2, 4>}, {32, 32, bstc64_kernel<32, 32, 2, 2>},
+      {64, 16, bstc64_kernel<64, 16, 4, 1>}, {16, 64, bstc64_kernel<16, 64, 1, 4>},
+      {32, 16, bstc64_kernel<32, 16, 2, 1>}, {16, 32, bstc64_kernel<16, 32, 1, 2>},
+      {16, 16, bstc64_kernel<16, 16, 1, 1>}, {64, 8, bstc64_kernel<64, 8, 2, 1>},
+      {8, 64, bstc64_kernel<8, 64, 1, 2>},   {32, 8, bstc64_kernel<32, 8, 1, 1>},
+      {8, 32, bstc64_kernel<8, 32, 1, 1>},   {16, 8, bstc64_kernel<16, 8, 1, 1>},
+      {8, 16, bstc64_kernel<8, 16, 1, 1>},   {8, 8, bstc64_kernel<8, 8, 1, 1>}};
+  const long long M = (long long)p.M1 * p.M2, N = (long long)p.N1 * p.N2;
+  const long long K = (long long)p.K1 * p.K2 * p.K3;
+  if (M <= 0 || N <= 0 || K <= 0 || p.nitems <= 0) return cudaSuccess;
+  const Tile *best = nullptr;
+  double cost = 0.0;
+  long long nt = 0, ks = 1;
+  for (const Tile &t : tiles) {
+    const long long ntiles = ((M + t.m - 1) / t.m) * ((N + t.n - 1) / t.n), blocks = ntiles * p.nitems;
+    long long split = 1;
+    if (fill > 0 && blocks < fill * 152LL)
+      split = std::max(1LL, std::min({(fill * 152LL + blocks - 1) / blocks, K / 32, 65535LL}));
+    const long long steps = ((K + split - 1) / split + 31) / 32;
+    const double rounds = (double)((blocks * split + 151) / 152);
+    const double c = rounds * 16.0 * t.m * t.n * (double)steps * (1.0 + 0.5 / t.m + 0.5 / t.n) +
+                     800.0 * (double)steps * std::max(1.0, 0.25 * rounds);
+    if (!best || c < cost) {
+      best = &t;
+      cost = c;
+      nt = ntiles;
+      ks = split;
+    }
+  }
+  p.kchunk = 0;
+  if (ks > 1) {
+    p.kchunk = ((K + ks - 1) / ks + 31) / 32 * 32;
+    ks = (K + p.kchunk - 1) / p.kchunk;
+    p.atomic = 1;
+  }
+  best->k<<<dim3((unsigned)nt, (unsigned)p.nitems, (unsigned)ks), 256, 0, st>>>(p);
+  return cudaGetLastError();
+}
 
 // Large contractions with a single K index (K2 = K3 = 1) in the split mode:
 // 128 x 128 tiles of C, 256 threads with 8 x 8 outputs each, K tiles of 8
@@ -388,13 +570,16 @@ __global__ void bstc_copy_kernel(BstcParams p) {
 }
 
 // ---------------------------------------------------------------------------
-// Triples block build, cube tile 8 x 8 x 8 of (a, b, c) per CTA.
+// Triples block build, cube tile TT x TT x TT of (a, b, c) per CTA.
 // ---------------------------------------------------------------------------
+// TT: 8, two elements per thread; or 4, one element per four threads, each a
+// quarter of every reduction, where the 8-wide cubes would leave SMs idle (16
+// batches of n_v = 8: 16 blocks of 47 us each at two FP64 operations a clock).
 namespace {
-constexpr int TT = 8;
 constexpr int TR = 32;
 }
 
+template <int TT>
 __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms terms,
                                                             const TripItem *__restrict__ items,
                                                             const double *__restrict__ eps, int NO,
@@ -403,11 +588,14 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
                                                             double *__restrict__ out,
                                                             int *__restrict__ status) {
   const double omega = omega_p ? *omega_p : omega_v;  // device-resident omega (graph replay)
+  constexpr int NE = TT == 8 ? 2 : 1, KG = TT == 8 ? 1 : 4;  // elements per thread, threads per element
+  static_assert(TT == 8 || TT == 4, "cube extent");
   __shared__ double Ps[TT][TR + 1];
   __shared__ double Qs[TT * TT][TR + 1];
   const TripTerm *sterm = terms.t;
   const int nterms = terms.n;
   const int tid = threadIdx.x;
+  const int kg = KG == 1 ? 0 : tid / (TT * TT * TT);
   const TripItem it = items[blockIdx.y];
   const int ntile = (nv + TT - 1) / TT;
   int tile = blockIdx.x;
@@ -418,15 +606,15 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
   tile /= ntile;
   base[0] = tile * TT;
   const int I[3] = {it.i, it.j, it.k};
-  int loc[2][3];
+  int loc[NE][3];
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    int e = tid + q * 256;
+  for (int q = 0; q < NE; ++q) {
+    int e = KG == 1 ? tid + q * 256 : tid % (TT * TT * TT);
     loc[q][0] = e / (TT * TT);
     loc[q][1] = (e / TT) % TT;
     loc[q][2] = e % TT;
   }
-  double acc[2] = {0.0, 0.0};
+  double acc[NE] = {};
   __syncthreads();
 
   for (int sg = 0; sg < 6; ++sg) {
@@ -462,7 +650,7 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
           sPr = tm.sA[3];
         }
         for (int r0 = 0; r0 < tm.R; r0 += TR) {
-          {
+          if (tid < TT * TR) {
             int row = tid / TR, rr = tid % TR;
             int g = base[ds] + row;
             double v = 0.0;
@@ -481,19 +669,19 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
           }
           __syncthreads();
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
+          for (int q = 0; q < NE; ++q) {
             const double *ps = Ps[loc[q][ds]];
             const double *qs = Qs[loc[q][dp1] * TT + loc[q][dp2]];
             double s = 0.0;
 #pragma unroll 8
-            for (int rr = 0; rr < TR; ++rr) s = fma(ps[rr], qs[rr], s);
+            for (int rr = kg * (TR / KG); rr < (kg + 1) * (TR / KG); ++rr) s = fma(ps[rr], qs[rr], s);
             acc[q] = fma(tm.coef, s, acc[q]);
           }
           __syncthreads();
         }
-      } else {
+      } else if (kg == 0) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < NE; ++q) {
           const long long u = base[s0] + loc[q][s0], v = base[s1] + loc[q][s1],
                           w = base[s2] + loc[q][s2];
           if (u >= nv || v >= nv || w >= nv) continue;
@@ -509,8 +697,17 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
       }
     }
   }
+  if (KG > 1) {
+    double *red = &Qs[0][0];
+    __syncthreads();
+    red[tid] = acc[0];
+    __syncthreads();
+    if (kg > 0) return;
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
+    for (int g = 1; g < KG; ++g) acc[0] += red[tid + g * TT * TT * TT];
+  }
+#pragma unroll
+  for (int q = 0; q < NE; ++q) {
     const int a = base[0] + loc[q][0], b = base[1] + loc[q][1], c = base[2] + loc[q][2];
     if (a >= nv || b >= nv || c >= nv) continue;
     const double den = eps[NO + a] + eps[NO + b] + eps[NO + c] - eps[it.i] - eps[it.j] -
@@ -524,6 +721,19 @@ __global__ void __launch_bounds__(256) triples_build_kernel(const TripTerms term
     }
     out[it.off + ((long long)a * nv + b) * nv + c] = val;
   }
+}
+
+// One block per cube and batch; the small cubes where 8-wide ones make fewer than
+// 152 blocks.
+cudaError_t launch_triples_build(const TripTerms &terms, const TripItem *items, int n, const double *eps,
+                                 int NO, int nv, double omega, const double *omega_p, double *out,
+                                 int *status, cudaStream_t st) {
+  const int n8 = (nv + 7) / 8, n4 = (nv + 3) / 4;
+  if ((long long)n8 * n8 * n8 * n >= 152)
+    triples_build_kernel<8><<<dim3(n8 * n8 * n8, n), 256, 0, st>>>(terms, items, eps, NO, nv, omega, omega_p, out, status);
+  else
+    triples_build_kernel<4><<<dim3(n4 * n4 * n4, n), 256, 0, st>>>(terms, items, eps, NO, nv, omega, omega_p, out, status);
+  return cudaGetLastError();
 }
 
 // Finish of a triples block whose two-index terms W are summed already (FP64 mode

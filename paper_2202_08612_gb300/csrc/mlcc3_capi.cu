@@ -28,7 +28,7 @@
 #include "mlcc3.h"
 
 namespace mlcc3 {
-__global__ void bstc_kernel(BstcParams p);
+cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st);
 __global__ void bstc_f32_kernel(BstcParams p);
 __global__ void bstc_big_kernel(BstcParams p);
 __global__ void bstc_dot_kernel(BstcParams p);
@@ -47,8 +47,8 @@ __global__ void bstc_copy_kernel(BstcParams p);
 __global__ void transpose2d_kernel(const double *, double *, int, int);
 __global__ void mirror_pairs_kernel(double *, int, int);
 __global__ void to_f32_kernel(const double *, float *, long long);
-__global__ void triples_build_kernel(const TripTerms, const TripItem *, const double *, int, int,
-                                     double, const double *, double *, int *);
+cudaError_t launch_triples_build(const TripTerms &, const TripItem *, int, const double *, int, int,
+                                 double, const double *, double *, int *, cudaStream_t);
 cudaError_t launch_contra3(const double *, double *, long long, int, cudaStream_t, bool);
 __global__ void finalize_doubles_kernel(const double *, double *, int, int, int, int, int);
 __global__ void c2_block_kernel(const double *, double *, int, int, int, int);
@@ -365,6 +365,16 @@ void mlcc3_ctx::bstc(const double *A, const double *B, double *C, const Shape &s
     check_cuda(cudaGetLastError(), "bstc launch");
     return;
   }
+  const std::string name = tag.empty() ? std::string("bstc_kernel") : "bstc_kernel:" + tag;
+  if (!f32) {
+    for (int z0 = 0; z0 < nitems; z0 += 65535) {
+      p.items = it + z0;
+      p.nitems = std::min(65535, nitems - z0);
+      launch(name.c_str(), 2.0 * M * N * (double)K * p.nitems,
+             [&] { check_cuda(launch_bstc64(p, bstc_fill, stream), "bstc64"); });
+    }
+    return;
+  }
   const long long tiles = ((N + 63) / 64) * ((M + 63) / 64);
   // split K when few output tiles face a long reduction
   long long ksplit = 1;
@@ -383,11 +393,8 @@ void mlcc3_ctx::bstc(const double *A, const double *B, double *C, const Shape &s
     p.items = it + z0;
     int nz = std::min(65535, nitems - z0);
     dim3 grid((unsigned)tiles, (unsigned)nz, (unsigned)ksplit);
-    const std::string name = tag.empty() ? std::string("bstc_kernel") : "bstc_kernel:" + tag;
-    launch(name.c_str(), 2.0 * M * N * (double)(sh.K1 * sh.K2 * sh.K3) * nz, [&] {
-      if (f32) bstc_f32_kernel<<<grid, 256, 0, stream>>>(p);
-      else bstc_kernel<<<grid, 256, 0, stream>>>(p);
-    });
+    launch(name.c_str(), 2.0 * M * N * (double)(sh.K1 * sh.K2 * sh.K3) * nz,
+           [&] { bstc_f32_kernel<<<grid, 256, 0, stream>>>(p); });
   }
   check_cuda(cudaGetLastError(), "bstc launch");
 }
@@ -691,16 +698,14 @@ void triples(mlcc3_ctx *c, const std::vector<TripTerm> &terms, const std::string
     db = static_cast<const TripItem *>(it->second.first);
   }
   n = (int)bs.size();
-  long long nt = (c->nv + 7) / 8;
-  dim3 grid((unsigned)(nt * nt * nt), (unsigned)n);
   double fl = 0.0;
   const double nv3 = (double)(c->nv * c->nv * c->nv);
   for (auto &t : terms) fl += 12.0 * nv3 * (t.kind <= 1 ? (double)t.R : 1.0);
   c->launch("triples_build_kernel", fl * n, [&] {
-    triples_build_kernel<<<grid, 256, 0, c->stream>>>(tt, db, c->eps, (int)c->NO, (int)c->nv,
-                                                      omega, c->omega_dev, out, c->status);
+    check_cuda(launch_triples_build(tt, db, n, c->eps, (int)c->NO, (int)c->nv, omega, c->omega_dev, out,
+                                    c->status, c->stream),
+               "triples_build launch");
   });
-  check_cuda(cudaGetLastError(), "triples_build launch");
 }
 
 void contra3(mlcc3_ctx *c, const double *X, double *Xt, long long nblocks) {

@@ -18,10 +18,10 @@
 
 namespace mlcc3 {
 void set_last_error(const std::string &msg);
-__global__ void bstc_kernel(BstcParams p);
+cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st);
 __global__ void bstc_gemv_kernel(BstcParams p);
-__global__ void triples_build_kernel(const TripTerms, const TripItem *, const double *, int, int,
-                                     double, const double *, double *, int *);
+cudaError_t launch_triples_build(const TripTerms &, const TripItem *, int, const double *, int, int,
+                                 double, const double *, double *, int *, cudaStream_t);
 cudaError_t launch_contra3(const double *, double *, long long, int, cudaStream_t, bool);
 __global__ void finalize_doubles_kernel(const double *, double *, int, int, int, int, int);
 }  // namespace mlcc3
@@ -176,9 +176,7 @@ extern "C" int mlcc3_triples_omega_static(mlcc3_ctx *c, double *omega1, double *
   tt.n = 2;
   tt.t[0] = TripTerm{0, (int)NV, 1.0, c->t2c, c->Gv, {bi, bL, ba, 1}, {gk, gb, gc, 1}};
   tt.t[1] = TripTerm{1, (int)NO, -1.0, c->Tl, c->Go, {ti, ta, tb, 1}, {oj, ok, oc, 1}};
-  const long long nt = (nv + 7) / 8;
-  triples_build_kernel<<<dim3((unsigned)(nt * nt * nt), (unsigned)nb), 256, 0, st>>>(
-      tt, dbatch, c->eps, (int)NO, (int)nv, 0.0, nullptr, tau, c->status);
+  launch_triples_build(tt, dbatch, (int)nb, c->eps, (int)NO, (int)nv, 0.0, nullptr, tau, c->status, st);
   // an error after the first launch drains the stream before returning, so that
   // no queued work of this call still writes the shared array afterwards
   auto drained = [&]() {
@@ -218,14 +216,13 @@ extern "C" int mlcc3_triples_omega_static(mlcc3_ctx *c, double *omega1, double *
     bp.alpha = L[k].alpha;
     bp.atomic = 1;
     const long long M = L[k].M1 * L[k].M2, N = L[k].N1;
-    const long long tiles = ((N + 63) / 64) * ((M + 63) / 64);
     for (long long z0 = 0; z0 < nord; z0 += 65535) {
       bp.items = ditems + k * nord + z0;
       bp.nitems = (int)std::min<long long>(65535, nord - z0);
       if (N == 1)  // matrix-vector form (singles and F terms): a warp per output row
         bstc_gemv_kernel<<<dim3((unsigned)((M + 7) / 8), (unsigned)bp.nitems), 256, 0, st>>>(bp);
       else
-        bstc_kernel<<<dim3((unsigned)tiles, (unsigned)bp.nitems), 256, 0, st>>>(bp);
+        launch_bstc64(bp, c->bstc_fill, st);
     }
   }
   const int g = (int)std::min<long long>((blk + 255) / 256, 152LL * 64);
