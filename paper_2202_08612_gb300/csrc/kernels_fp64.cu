@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <iterator>
 
 #include "kernels_fp64.cuh"
 
@@ -22,141 +23,283 @@ __constant__ int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 
 // Batched strided tensor contraction.
 // Tile 64 x 64 of C per CTA, K chunks of 16, 256 threads with 4 x 4 outputs.
 // ---------------------------------------------------------------------------
-namespace {
-constexpr int BM = 64, BN = 64, BK = 16;
-}
-
 // Element i of an operand that holds binary64 (f32 = 0) or binary32 values.
 template <typename T>
 __device__ __forceinline__ T ld_op(const double *p, int f32, long long i) {
   return f32 ? (T)reinterpret_cast<const float *>(p)[i] : (T)p[i];
 }
 
-// FP32 products (split-precision mode): each thread's FP32 partial sums are
-// folded into FP64 every four K tiles (64 products).
-__global__ void __launch_bounds__(256, 3) bstc_f32_kernel(BstcParams p) {
-  using T = float;
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN + 1];
-  __shared__ long long rowA[BM], rowC[BM], colB[BN], colC[BN];
-  __shared__ long long kA[BK], kB[BK];
+// binary64 -> binary32, round to nearest even, on the integer pipe where the result
+// is a normal number (a conversion there is an FP64 operation, two per clock and SM).
+__device__ __forceinline__ float narrow_f64(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if (((hi >> 20) & 0x7ff) - 897u < 253u) {
+    const unsigned long long m = (((unsigned long long)hi << 32) | lo) + 0x0fffffffu + ((lo >> 29) & 1u);
+    return __uint_as_float((((unsigned)(m >> 29) - 0xC0000000u) & 0x7fffffffu) | (hi & 0x80000000u));
+  }
+  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);  // zeros, as in the padding of a tile
+  return __double2float_rn(x);
+}
 
+// binary32 -> binary64 (exact) on the integer pipe; binary32 subnormals
+// (never produced here) become signed zeros.
+__device__ __forceinline__ double widen_f32(float f) {
+  const unsigned int b = __float_as_uint(f);
+  const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
+  const unsigned int e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
+  if (e == 0) return __longlong_as_double((long long)sign);
+  const unsigned long long ex = e == 255 ? 0x7FFull : (unsigned long long)(e + 896);
+  return __longlong_as_double((long long)(sign | (ex << 52) | ((unsigned long long)m << 29)));
+}
+
+// FP32 products (split-precision mode): every output's FP32 sum of 64 products in
+// K order is folded into an FP64 sum.  Tiles of TM x TN outputs, RM x RN per thread
+// (launch_bstc32).  Per 64 products an output costs one FP64 addition, as long as
+// its 64 FP32 products; conversions from and to binary64 would cost several times
+// that on the FP64 pipe and run on the integer pipe instead.  The next K tile's
+// loads are in flight while the current one is multiplied, its index splits made
+// one tile ahead.  blockIdx.z: the K range of kchunk elements it belongs to (as
+// bstc_f32's callers split K) and the piece of kfine (a multiple of 64) in it.
+// SHORT: at most 64 products per output, where writing C is the work: a thread's
+// columns lie TX apart (coalesced, but no vector reads of B) and the one FP32 sum
+// needs no FP64 addition of its own.
+template <int TM, int TN, int RM, int RN, bool SHORT = false>
+__global__ void __launch_bounds__(256, TM * TN <= 2048 ? 3 : TM * TN <= 4096 ? 2 : 1) bstc32_kernel(BstcParams p, int fine, long long kfine) {
+  constexpr int TK = 32, TX = TN / RN;
+  constexpr int NA = TK * TM / 256, NB = TK * TN / 256;
+  static_assert(TM / RM * TX == 256 && NA * 256 == TK * TM && NB * 256 == TK * TN, "tile");
+  __shared__ __align__(16) float As[TK][TM + 4], Bs[TK][TN + 4];
+  __shared__ long long rowA[TM], rowC[TM], colB[TN], colC[TN];
+  __shared__ long long kA[3][TK], kB[3][TK];  // -1 past the end
   const BstcItem &it = p.items[blockIdx.y];
   const int tid = threadIdx.x;
   const long long M = (long long)p.M1 * p.M2, N = (long long)p.N1 * p.N2;
   const long long K = (long long)p.K1 * p.K2 * p.K3;
-  const long long ntn = (N + BN - 1) / BN;
-  const long long m0 = ((long long)blockIdx.x / ntn) * BM, n0 = ((long long)blockIdx.x % ntn) * BN;
-
-  if (tid < BM) {
-    long long m = m0 + tid;
-    if (m < M) {
-      long long m1 = m / p.M2, m2 = m % p.M2;
-      rowA[tid] = m1 * it.sA[0] + m2 * it.sA[1];
-      rowC[tid] = m1 * it.sC[0] + m2 * it.sC[1];
+  const long long ntn = (N + TN - 1) / TN;
+  const long long m0 = (long long)blockIdx.x / ntn * TM, n0 = (long long)blockIdx.x % ntn * TN;
+  for (int t = tid; t < TM + TN; t += 256) {
+    if (t < TM) {
+      const long long m = m0 + t, m1 = m / p.M2, m2 = m % p.M2;
+      rowA[t] = m < M ? m1 * it.sA[0] + m2 * it.sA[1] : -1;
+      rowC[t] = m < M ? m1 * it.sC[0] + m2 * it.sC[1] : -1;
     } else {
-      rowA[tid] = -1;
-      rowC[tid] = -1;
-    }
-  } else if (tid < BM + BN) {
-    int t = tid - BM;
-    long long n = n0 + t;
-    if (n < N) {
-      long long n1 = n / p.N2, n2 = n % p.N2;
-      colB[t] = n1 * it.sB[3] + n2 * it.sB[4];
-      colC[t] = n1 * it.sC[2] + n2 * it.sC[3];
-    } else {
-      colB[t] = -1;
-      colC[t] = -1;
+      const long long n = n0 + t - TM, n1 = n / p.N2, n2 = n % p.N2;
+      colB[t - TM] = n < N ? n1 * it.sB[3] + n2 * it.sB[4] : -1;
+      colC[t - TM] = n < N ? n1 * it.sC[2] + n2 * it.sC[3] : -1;
     }
   }
-  const bool kfastA = (it.sA[4] == 1 && p.K3 > 1) || (p.K3 == 1 && it.sA[3] == 1 && p.K2 > 1) ||
-                      (p.K3 == 1 && p.K2 == 1 && it.sA[2] == 1);
-  const bool kfastB = (it.sB[2] == 1 && p.K3 > 1) || (p.K3 == 1 && it.sB[1] == 1 && p.K2 > 1) ||
-                      (p.K3 == 1 && p.K2 == 1 && it.sB[0] == 1);
-  const long long offA = it.offA, offB = it.offB;
-
-  const int ty = tid / 16, tx = tid % 16;
-  T acc[4][4];
-  double accd[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      acc[i][j] = T(0);
-      accd[i][j] = 0.0;
-    }
-  int tiles = 0;
-
-  const long long kbeg = p.kchunk ? (long long)blockIdx.z * p.kchunk : 0;
-  const long long kend = p.kchunk ? min(K, kbeg + p.kchunk) : K;
-  for (long long k0 = kbeg; k0 < kend; k0 += BK) {
-    if (tid < BK) {
-      long long k = k0 + tid;
-      if (k < kend) {
-        long long k3 = k % p.K3, k12 = k / p.K3;
-        long long k2 = k12 % p.K2, k1 = k12 / p.K2;
-        kA[tid] = k1 * it.sA[2] + k2 * it.sA[3] + k3 * it.sA[4];
-        kB[tid] = k1 * it.sB[0] + k2 * it.sB[1] + k3 * it.sB[2];
+  const bool kfastA = p.K3 > 1 ? it.sA[4] == 1 : p.K2 > 1 ? it.sA[3] == 1 : it.sA[2] == 1;
+  const bool kfastB = p.K3 > 1 ? it.sB[2] == 1 : p.K2 > 1 ? it.sB[1] == 1 : it.sB[0] == 1;
+  const long long z0 = p.kchunk ? (long long)(blockIdx.z / fine) * p.kchunk : 0;
+  const long long z1 = p.kchunk ? min(K, z0 + p.kchunk) : K;
+  const long long kbeg = z0 + (long long)(blockIdx.z % fine) * kfine;
+  const long long kend = min(z1, kbeg + kfine);
+  if (kbeg >= kend) return;
+  auto split_k = [&](int tile) {
+    if (tid >= TK) return;
+    const long long k = kbeg + (long long)tile * TK + tid;
+    long long a = -1, b = -1;
+    if (k < kend) {
+      long long k1, k2, k3;
+      if (K < (1LL << 31)) {
+        const unsigned u = (unsigned)k, u12 = u / (unsigned)p.K3;
+        k3 = u - u12 * (unsigned)p.K3;
+        k1 = u12 / (unsigned)p.K2;
+        k2 = u12 % (unsigned)p.K2;
       } else {
-        kA[tid] = -1;
-        kB[tid] = -1;
+        const long long k12 = k / p.K3;
+        k3 = k % p.K3;
+        k1 = k12 / p.K2;
+        k2 = k12 % p.K2;
       }
+      a = it.offA + k1 * it.sA[2] + k2 * it.sA[3] + k3 * it.sA[4];
+      b = it.offB + k1 * it.sB[0] + k2 * it.sB[1] + k3 * it.sB[2];
     }
+    kA[tile % 3][tid] = a;
+    kB[tile % 3][tid] = b;
+  };
+  // one element's bits: a binary64 pattern, or a binary32 one in the low half
+  auto fetch = [](const double *x, int f32, long long row, long long k) -> unsigned long long {
+    if (row < 0 || k < 0) return 0;
+    return f32 ? (unsigned long long)__float_as_uint(reinterpret_cast<const float *>(x)[row + k])
+               : (unsigned long long)__double_as_longlong(x[row + k]);
+  };
+  auto value = [](unsigned long long v, int f32) {
+    return f32 ? __uint_as_float((unsigned)v) : narrow_f64(__longlong_as_double((long long)v));
+  };
+  unsigned long long ra[NA], rb[NB];
+  auto load = [&](int tile) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = tid + 256 * q;
+      ra[q] = fetch(p.A, p.a32, rowA[kfastA ? e / TK : e % TM], kA[tile % 3][kfastA ? e % TK : e / TM]);
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + 256 * q;
+      rb[q] = fetch(p.B, p.b32, colB[kfastB ? e / TK : e % TN], kB[tile % 3][kfastB ? e % TK : e / TN]);
+    }
+  };
+  split_k(0);
+  split_k(1);
+  __syncthreads();
+  load(0);
+  const int ty = tid / TX, tx = tid % TX;
+  float acc[RM][RN];
+  double sum[RM][RN];
+#pragma unroll
+  for (int i = 0; i < RM; ++i)
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      acc[i][j] = 0.f;
+      sum[i][j] = 0.0;
+    }
+  const int tiles = (int)((kend - kbeg + TK - 1) / TK);
+  for (int t = 0; t < tiles; ++t) {
+    __syncthreads();  // the previous tile's reads are done
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = tid + 256 * q;
+      As[kfastA ? e % TK : e / TM][kfastA ? e / TK : e % TM] = value(ra[q], p.a32);
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + 256 * q;
+      Bs[kfastB ? e % TK : e / TN][kfastB ? e / TK : e % TN] = value(rb[q], p.b32);
+    }
+    split_k(t + 2);
     __syncthreads();
-    for (int e = tid; e < BK * BM; e += 256) {
-      int kk, mm;
-      if (kfastA) { mm = e / BK; kk = e % BK; } else { kk = e / BM; mm = e % BM; }
-      T v = T(0);
-      if (rowA[mm] >= 0 && kA[kk] >= 0) v = ld_op<T>(p.A, p.a32, offA + rowA[mm] + kA[kk]);
-      As[kk][mm] = v;
+    if (t + 1 < tiles) load(t + 1);
+#pragma unroll 8
+    for (int kk = 0; kk < TK; ++kk) {
+      float a[RM], b[RN];
+      if constexpr (RM % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < RM; i += 4) {
+          const float4 v = *reinterpret_cast<const float4 *>(&As[kk][ty * RM + i]);
+          a[i] = v.x;
+          a[i + 1] = v.y;
+          a[i + 2] = v.z;
+          a[i + 3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < RM; ++i) a[i] = As[kk][ty * RM + i];
+      }
+      if constexpr (SHORT) {
+#pragma unroll
+        for (int j = 0; j < RN; ++j) b[j] = Bs[kk][tx + TX * j];
+      } else if constexpr (RN % 4 == 0) {
+#pragma unroll
+        for (int j = 0; j < RN; j += 4) {
+          const float4 v = *reinterpret_cast<const float4 *>(&Bs[kk][tx * RN + j]);
+          b[j] = v.x;
+          b[j + 1] = v.y;
+          b[j + 2] = v.z;
+          b[j + 3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < RN; ++j) b[j] = Bs[kk][tx * RN + j];
+      }
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
-    for (int e = tid; e < BK * BN; e += 256) {
-      int kk, nn;
-      if (kfastB) { nn = e / BK; kk = e % BK; } else { kk = e / BN; nn = e % BN; }
-      T v = T(0);
-      if (colB[nn] >= 0 && kB[kk] >= 0) v = ld_op<T>(p.B, p.b32, offB + kB[kk] + colB[nn]);
-      Bs[kk][nn] = v;
-    }
-    __syncthreads();
+    if (!SHORT && ((t & 1) || t + 1 == tiles)) {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[4], b[4];
+      for (int i = 0; i < RM; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-    if (++tiles == 4) {
-      tiles = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          accd[i][j] += (double)acc[i][j];
-          acc[i][j] = T(0);
+        for (int j = 0; j < RN; ++j) {
+          sum[i][j] += widen_f32(acc[i][j]);
+          acc[i][j] = 0.f;
         }
     }
   }
   double *C = p.C + it.offC;
+  // +-1 decided on the bits: a comparison of doubles is an FP64 operation
+  const long long ab = __double_as_longlong(p.alpha);
+  const int unit = ab == 0x3ff0000000000000LL ? 1 : ab == (long long)0xbff0000000000000ULL ? -1 : 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    long long rc = rowC[ty * 4 + i];
+  for (int i = 0; i < RM; ++i) {
+    const long long rc = rowC[ty * RM + i];
     if (rc < 0) continue;
+    double old[RN];  // a row's loads before its stores, which might alias them
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      long long cc = colC[tx * 4 + j];
+    for (int j = 0; j < RN; ++j) {
+      const long long cc = colC[SHORT ? tx + TX * j : tx * RN + j];
+      old[j] = !p.atomic && cc >= 0 ? C[rc + cc] : 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      const long long cc = colC[SHORT ? tx + TX * j : tx * RN + j];
       if (cc < 0) continue;
-      double v = p.alpha * (accd[i][j] + (double)acc[i][j]);
+      const double x = SHORT ? widen_f32(acc[i][j]) : sum[i][j];
+      const double v = unit == 0 ? p.alpha * x : unit > 0 ? x : -x;
       if (p.atomic) atomicAdd(C + rc + cc, v);
-      else C[rc + cc] += v;
+      else C[rc + cc] = old[j] + v;
     }
   }
+}
+
+// C += alpha A B with FP32 products for every item (at most 65535).  p.kchunk splits
+// K as before (0: not); a launch of fewer than four blocks per SM is split further,
+// at multiples of 64 products from the start of a range, which changes no FP32 sum.
+// Of the tiles the one with the least estimated time: per K element its FP32
+// products (128 a clock), its shared-memory reads and its share of the FP64
+// additions, for as many rounds of blocks as the 152 SMs need, plus the latency
+// of a K step that four resident blocks hide from one another.
+cudaError_t launch_bstc32(BstcParams p, cudaStream_t st) {
+  struct Tile {
+    int m, n;
+    double clk;  // per K element
+    void (*k)(BstcParams, int, long long);
+  };
+  static const Tile tiles[] = {
+      {128, 64, 100.0, bstc32_kernel<128, 64, 8, 4>}, {64, 128, 100.0, bstc32_kernel<64, 128, 4, 8>},
+      {128, 32, 55.0, bstc32_kernel<128, 32, 4, 4>},  {32, 128, 55.0, bstc32_kernel<32, 128, 4, 4>},
+      {64, 64, 55.0, bstc32_kernel<64, 64, 4, 4>},    {64, 32, 32.0, bstc32_kernel<64, 32, 4, 2>},
+      {32, 64, 32.0, bstc32_kernel<32, 64, 2, 4>},    {32, 32, 24.0, bstc32_kernel<32, 32, 2, 2>},
+      {64, 16, 24.0, bstc32_kernel<64, 16, 4, 1>},    {16, 64, 24.0, bstc32_kernel<16, 64, 1, 4>},
+      {16, 16, 20.0, bstc32_kernel<16, 16, 1, 1>}};
+  static const Tile shorts[] = {
+      {32, 128, 65.0, bstc32_kernel<32, 128, 4, 4, true>}, {64, 64, 65.0, bstc32_kernel<64, 64, 4, 4, true>},
+      {128, 32, 65.0, bstc32_kernel<128, 32, 4, 4, true>}, {32, 64, 40.0, bstc32_kernel<32, 64, 2, 4, true>},
+      {64, 32, 36.0, bstc32_kernel<64, 32, 4, 2, true>},   {32, 32, 24.0, bstc32_kernel<32, 32, 2, 2, true>},
+      {16, 16, 20.0, bstc32_kernel<16, 16, 1, 1, true>}};
+  const long long M = (long long)p.M1 * p.M2, N = (long long)p.N1 * p.N2;
+  const long long K = (long long)p.K1 * p.K2 * p.K3;
+  if (M <= 0 || N <= 0 || K <= 0 || p.nitems <= 0) return cudaSuccess;
+  const long long range = p.kchunk ? p.kchunk : K, ranges = (K + range - 1) / range;
+  const Tile *best = nullptr;
+  double cost = 0.0;
+  long long nt = 0, fine = 1;
+  const bool is_short = range <= 64;
+  const Tile *from = is_short ? std::begin(shorts) : std::begin(tiles);
+  const Tile *to = is_short ? std::end(shorts) : std::end(tiles);
+  for (const Tile *tp = from; tp != to; ++tp) {
+    const Tile &t = *tp;
+    const long long ntiles = ((M + t.m - 1) / t.m) * ((N + t.n - 1) / t.n);
+    const long long blocks = ntiles * p.nitems * ranges;
+    long long f = 1;
+    if (blocks < 4 * 152)
+      f = std::max(1LL, std::min({(4 * 152 + blocks - 1) / blocks, (range + 127) / 128, 65535 / ranges}));
+    const long long steps = ((range + f - 1) / f + 31) / 32;
+    const double rounds = (double)((blocks * f + 151) / 152);
+    const double c = rounds * t.clk * 32.0 * (double)steps + 1200.0 * (double)steps * std::max(1.0, 0.25 * rounds);
+    if (!best || c < cost) {
+      best = &t;
+      cost = c;
+      nt = ntiles;
+      fine = f;
+    }
+  }
+  const long long kfine = ((range + fine - 1) / fine + 63) / 64 * 64;
+  fine = (range + kfine - 1) / kfine;
+  if (fine > 1) p.atomic = 1;
+  best->k<<<dim3((unsigned)nt, (unsigned)p.nitems, (unsigned)(ranges * fine)), 256, 0, st>>>(p, (int)fine, kfine);
+  return cudaGetLastError();
 }
 
 // FP64 form, tiles of TM x TN outputs, RM x RN per thread.  GB300's FP64 pipe
@@ -358,7 +501,7 @@ constexpr int GBM = 128, GBN = 128, GBK = 8, GPAD = 4;
 }
 
 __device__ __forceinline__ float ld_f(const double *p, int f32, long long i) {
-  return f32 ? reinterpret_cast<const float *>(p)[i] : (float)p[i];
+  return f32 ? reinterpret_cast<const float *>(p)[i] : narrow_f64(p[i]);
 }
 
 __global__ void __launch_bounds__(256, 1) bstc_big_kernel(BstcParams p) {
@@ -1116,17 +1259,6 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float bh, float bl)
   lo = t - (hi - s);
 }
 
-
-// binary32 -> binary64 (exact) on the integer pipe; binary32 subnormals
-// (never produced here) become signed zeros.
-__device__ __forceinline__ double widen_f32(float f) {
-  const unsigned int b = __float_as_uint(f);
-  const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
-  const unsigned int e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
-  if (e == 0) return __longlong_as_double((long long)sign);
-  const unsigned long long ex = e == 255 ? 0x7FFull : (unsigned long long)(e + 896);
-  return __longlong_as_double((long long)(sign | (ex << 52) | ((unsigned long long)m << 29)));
-}
 
 // q = x / d for x < 2^30 and d <= 1024 with the invariant-divisor multiplier
 // m = ceil(2^40 / d): the product overshoots x / d by less than x / 2^40 < 1 / d,

@@ -29,7 +29,7 @@
 
 namespace mlcc3 {
 cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st);
-__global__ void bstc_f32_kernel(BstcParams p);
+cudaError_t launch_bstc32(BstcParams p, cudaStream_t st);
 __global__ void bstc_big_kernel(BstcParams p);
 __global__ void bstc_dot_kernel(BstcParams p);
 __global__ void bstc_gemv_kernel(BstcParams p);
@@ -376,7 +376,8 @@ void mlcc3_ctx::bstc(const double *A, const double *B, double *C, const Shape &s
     return;
   }
   const long long tiles = ((N + 63) / 64) * ((M + 63) / 64);
-  // split K when few output tiles face a long reduction
+  // split K when few 64 x 64 output tiles face a long reduction (the ranges of the
+  // FP32 sums; launch_bstc32 splits them further at its own tile shapes)
   long long ksplit = 1;
   if (bstc_fill > 0 && tiles * nitems < 2 * 152 && K >= 1024) {
     ksplit = std::min<long long>((bstc_fill * 152LL + tiles * nitems - 1) / (tiles * nitems), K / 256);
@@ -384,19 +385,16 @@ void mlcc3_ctx::bstc(const double *A, const double *B, double *C, const Shape &s
   }
   if (ksplit > 1) {
     p.kchunk = ((K + ksplit - 1) / ksplit + 15) / 16 * 16;
-    ksplit = (K + p.kchunk - 1) / p.kchunk;
     p.atomic = 1;
   } else {
     p.kchunk = 0;
   }
   for (int z0 = 0; z0 < nitems; z0 += 65535) {
     p.items = it + z0;
-    int nz = std::min(65535, nitems - z0);
-    dim3 grid((unsigned)tiles, (unsigned)nz, (unsigned)ksplit);
-    launch(name.c_str(), 2.0 * M * N * (double)(sh.K1 * sh.K2 * sh.K3) * nz,
-           [&] { bstc_f32_kernel<<<grid, 256, 0, stream>>>(p); });
+    p.nitems = std::min(65535, nitems - z0);
+    launch(name.c_str(), 2.0 * M * N * (double)K * p.nitems,
+           [&] { check_cuda(launch_bstc32(p, stream), "bstc32"); });
   }
-  check_cuda(cudaGetLastError(), "bstc launch");
 }
 
 void mlcc3_ctx::bstc1(const double *A, const double *B, double *C, const Shape &sh, double alpha,
