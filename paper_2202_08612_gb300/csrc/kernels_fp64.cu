@@ -64,8 +64,8 @@ __device__ __forceinline__ double widen_f32(float f) {
 // columns lie TX apart (coalesced, but no vector reads of B) and the one FP32 sum
 // needs no FP64 addition of its own.
 template <int TM, int TN, int RM, int RN, bool SHORT = false>
-__global__ void __launch_bounds__(256, TM * TN <= 2048 ? 3 : TM * TN <= 4096 ? 2 : 1) bstc32_kernel(BstcParams p, int fine, long long kfine) {
-  constexpr int TK = 32, TX = TN / RN;
+__global__ void __launch_bounds__(256, TM * TN <= 1024 && RM == RN ? 3 : TM * TN <= 4096 ? 2 : 1) bstc32_kernel(BstcParams p, int fine, long long kfine) {
+  constexpr int TK = TM * TN >= 4096 ? 16 : 32, TX = TN / RN;  // (fewer loads held in registers)
   constexpr int NA = TK * TM / 256, NB = TK * TN / 256;
   static_assert(TM / RM * TX == 256 && NA * 256 == TK * TM && NB * 256 == TK * TN, "tile");
   __shared__ __align__(16) float As[TK][TM + 4], Bs[TK][TN + 4];
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(256, TM * TN <= 2048 ? 3 : TM * TN <= 4096 ? 2
 #pragma unroll
         for (int j = 0; j < RN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
-    if (!SHORT && ((t & 1) || t + 1 == tiles)) {
+    if (!SHORT && ((t + 1) % (64 / TK) == 0 || t + 1 == tiles)) {
 #pragma unroll
       for (int i = 0; i < RM; ++i)
 #pragma unroll
