@@ -2876,14 +2876,18 @@ void dld_flush(mlcc3_ctx *c) {
 
 // Triples part of the left density from (contravariant left triples Xt3,
 // covariant-combined doubles Lc, tau, contravariant tau), the chunk's share.
-// `acc`: the name of the D_LD accumulator of this density (dld_acc).
+// `acc`: the name of the D_LD accumulator of this density (dld_acc).  With E
+// [n_o][n_o] and E2 [n_v][n_v] the sums of D_kl and D_cd go there, without their
+// factors -1/2 and 1/2, and not into D.
 void density_left_gpu(mlcc3_ctx *c, const Chunk &ch, const double *Xt3, const double *Lc,
-                      const double *tau, const double *taut, double *D, const std::string &acc) {
+                      const double *tau, const double *taut, double *D, const std::string &acc,
+                      double *E = nullptr, double *E2 = nullptr) {
   S s(c);
   const long long nmo = s.nmo, NO = s.NO;
   const std::string okey = "o" + ch.key;
   // D_kl -= 1/2 sum Xt_{ijl} tau_{ijk}
-  pair_dots(c, ch, Xt3, tau, D, nmo, true, -0.5);
+  if (E) pair_dots(c, ch, Xt3, tau, E, s.no, true, 1.0);
+  else pair_dots(c, ch, Xt3, tau, D, nmo, true, -0.5);
   // D_ld += 1/2 sum Lc^{ab}_{ij} taut^{abd}_{ijl}
   y3_like(c, taut, Lc, ch.own, okey, D + NO, nmo, 0.5, "y3d");
   // D_LD -= sum Xt^{abc}_{ijk} t^{ac}_{iL} t^{bD}_{jk}  (V summed over the chunks)
@@ -2894,10 +2898,12 @@ void density_left_gpu(mlcc3_ctx *c, const Chunk &ch, const double *Xt3, const do
   else
     v_like(c, Xt3, c->Tl, ch.own, okey, V);
   // D_cd += 1/2 sum Xt^{abc}_{ijk} tau^{abd}_{ijk}
+  double *Dcd = E2 ? E2 : D + NO * nmo + NO;
+  const long long ldcd = E2 ? s.nv : nmo;
   if (tc_mode(c))
-    tc_vv(c, Xt3, "X", tau, "Y", ch.own, okey, D + NO * nmo + NO, nmo, 0.5);
+    tc_vv(c, Xt3, "X", tau, "Y", ch.own, okey, Dcd, ldcd, E2 ? 1.0 : 0.5);
   else
-    vv_block(c, Xt3, tau, ch.own, okey, D + NO * nmo + NO, nmo, 0.5);
+    vv_block(c, Xt3, tau, ch.own, okey, Dcd, ldcd, E2 ? 1.0 : 0.5);
 }
 
 }  // namespace
@@ -2982,6 +2988,9 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     check_cuda(cudaStreamSynchronize(c->stream), "one sync");
   }
   c->zero(scall, 2 * (size_t)n_st);
+  // E[l][k] = sum lt_{ijk} tau_{ijl} and E2[c][d] = sum lt^{abc}_{ijk} tau^{abd}_{ijk} of a
+  // chunk: D^{0-0}'s kl and cd blocks and, times each state's R1, two terms of its D^{0-m}
+  double *E = c->buf("dE", s.no * s.no + s.nv * s.nv), *E2 = E + s.no * s.no;
   for (const Chunk &ch : c->groups) {
     const std::string bkey = "b" + ch.key, okey = "o" + ch.key;
     const long long bw = ch.nb * s.nv3;
@@ -2994,7 +3003,15 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     const bool first = &ch == &c->groups.front();
     left_triples(c, "lam", lam1, lc, lcT, bkey, ch.bs, 0.0, lam3, lt3, ch.nb, false, first);
     // D^{0-0} (state independent)
-    density_left_gpu(c, ch, lt3, lc32, tau, taut, D00, "D00");
+    c->zero(E, s.no * s.no + s.nv * s.nv);
+    density_left_gpu(c, ch, lt3, lc32, tau, taut, D00, "D00", E, E2);
+    {
+      Shape sh;
+      sh.M1 = s.no; sh.M2 = s.no;
+      c->bstc1(E, one, D00, sh, -0.5, mk_item(0, 0, 0, {s.no, 1, 0, 0, 0}, {0, 0, 0, 0, 0}, {nmo, 1, 0, 0}), "d00kl");
+      sh = Shape{}; sh.M1 = s.nv; sh.M2 = s.nv;
+      c->bstc1(E2, one, D00 + NO * nmo + NO, sh, 0.5, mk_item(0, 0, 0, {s.nv, 1, 0, 0, 0}, {0, 0, 0, 0, 0}, {nmo, 1, 0, 0}), "d00cd");
+    }
     for (int st = 0; st < n_st; ++st) {
     const StateOps &so = sts[st];
     const double omega = omega_h[st];
@@ -3118,18 +3135,10 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
       sh = Shape{}; sh.M1 = s.nv; sh.K1 = s.nv; sh.K2 = s.nv; sh.N1 = NO;
       c->bstc(lt3, c->Tl, V3, sh, 1.0, it, n, true, okey + ":v3");
     }
-    // D_lD -= 1/2 sum_k E[l][k] R^D_k,  E[l][k] = sum lt_{ijk} tau_{ijl}
-    double *E = c->buf("dE", s.no * s.no + s.nv * s.nv);
-    c->zero(E, s.no * s.no + s.nv * s.nv);
-    pair_dots(c, ch, tau, lt3, E, s.no, false, 1.0);
+    // D_lD -= 1/2 sum_k E[l][k] R^D_k
     sh = Shape{}; sh.M1 = s.no; sh.N1 = s.NV; sh.K1 = s.no;
     c->bstc1(E, R1, D + NO, sh, -0.5, mk_item(0, 0, 0, {s.no, 0, 1, 0, 0}, {1, 0, 0, NO, 0}, {nmo, 0, 1, 0}), "dlD");
-    // D_Ld -= 1/2 sum_c E2[c][d] R^c_L,  E2[c][d] = sum lt^{abc}_{ijk} tau^{abd}_{ijk}
-    double *E2 = E + s.no * s.no;
-    if (tc_mode(c))
-      tc_vv(c, lt3, "X", tau, "Y", ch.own, okey, E2, s.nv, 1.0);
-    else
-      vv_block(c, lt3, tau, ch.own, okey, E2, s.nv, 1.0);
+    // D_Ld -= 1/2 sum_c E2[c][d] R^c_L
     sh = Shape{}; sh.M1 = NO; sh.N1 = s.nv; sh.K1 = s.nv;
     c->bstc1(R1, E2, D + NO, sh, -0.5, mk_item(0, 0, 0, {1, 0, NO, 0, 0}, {s.nv, 0, 0, 1, 0}, {nmo, 0, 1, 0}), "dLd");
     // D_ck += W3[k][c]
