@@ -170,48 +170,52 @@ __global__ void __launch_bounds__(320, 1)
     bool ok = true;
     for (int i = blockIdx.x; i < nitems && ok && !*abort_flag; i += gridDim.x) {
       const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
-      int total = 0;
-      for (int q = s0; q < s1; ++q) total += segs[q].nk;
-      for (int c = 0; c < total; ++c) {
-        const int cc = c % kChain;
-        if (cc == 0) {
-          if (!mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait)) {
+      int cc = 0;  // chunk of the accumulation chain
+      for (int q = s0; q < s1 && ok; ++q) {
+        const int nk = segs[q].nk, tail = segs[q].nb;
+        for (int kc = 0; kc < nk; ++kc) {
+          if (cc == 0) {
+            if (!mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait)) {
+              *abort_flag = 1;
+              ok = false;
+              break;
+            }
+          }
+          if (!mbar_wait(full0 + 8 * stage, phase, status, epi.wait)) {
             *abort_flag = 1;
             ok = false;
             break;
           }
-        }
-        if (!mbar_wait(full0 + 8 * stage, phase, status, epi.wait)) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t a0 = smem_u32(smem + stage * stage_bytes), b0 = a0 + S * A_SL;
+          tc_fence_after();
+          const uint32_t a0 = smem_u32(smem + stage * stage_bytes), b0 = a0 + S * A_SL;
+          const int steps = kc == nk - 1 && tail > 0 ? tail : kEmuKB / 16;
 #pragma unroll
-        for (int kk = 0; kk < kEmuKB / 16; ++kk) {
+          for (int kk = 0; kk < kEmuKB / 16; ++kk) {
+            if (kk >= steps) break;  // zeros to the end of the reduction
 #pragma unroll
-          for (int d = 0; d < S; ++d) {
-            // slice d of A with the stacked slices 0 .. S-1-d of B; the first
-            // MMA of a chain (d = 0) covers every degree and clears them
-            const uint64_t ad = smem_desc64(a0 + d * A_SL + kk * 32);
-            const uint32_t acc = (cc > 0 || kk > 0 || d > 0) ? 1u : 0u;
-            const int cols = (S - d) * n;
-            for (int c0 = 0; c0 < cols; c0 += 256) {
-              const int nn = min(256, cols - c0);
-              mma_bf16(tmem + (uint32_t)(d * n + c0), ad, smem_desc64(b0 + c0 * kRowB + kk * 32),
-                       IDESC | ((uint32_t)(nn >> 3) << 17), acc);
+            for (int d = 0; d < S; ++d) {
+              // slice d of A with the stacked slices 0 .. S-1-d of B; the first
+              // MMA of a chain (d = 0) covers every degree and clears them
+              const uint64_t ad = smem_desc64(a0 + d * A_SL + kk * 32);
+              const uint32_t acc = (cc > 0 || kk > 0 || d > 0) ? 1u : 0u;
+              const int cols = (S - d) * n;
+              for (int c0 = 0; c0 < cols; c0 += 256) {
+                const int nn = min(256, cols - c0);
+                mma_bf16(tmem + (uint32_t)(d * n + c0), ad, smem_desc64(b0 + c0 * kRowB + kk * 32),
+                         IDESC | ((uint32_t)(nn >> 3) << 17), acc);
+              }
             }
           }
-        }
-        mma_commit(empty0 + 8 * stage);
-        if (++stage == stages) {
-          stage = 0;
-          phase ^= 1u;
-        }
-        if (cc == kChain - 1 || c == total - 1) {
-          mma_commit(tfull);
-          ++t;
+          mma_commit(empty0 + 8 * stage);
+          if (++stage == stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+          if (++cc == kChain || (q == s1 - 1 && kc == nk - 1)) {
+            mma_commit(tfull);
+            ++t;
+            cc = 0;
+          }
         }
       }
     }
@@ -332,10 +336,19 @@ __global__ void __launch_bounds__(320, 1)
   }
 }
 
+// The width that wastes least: columns of all tiles, and as much as eight columns
+// per tile for reading A again.
 int emu_tile_width(long long n, int S) {
-  const long long w = emu_max_cols(S), tiles = (n + w - 1) / w;
-  const long long c = tiles ? (n + tiles - 1) / tiles : 16;
-  return (int)std::max(16LL, (c + 15) / 16 * 16);
+  int best = 16;
+  long long cost = -1;
+  for (int w = 16; w <= emu_max_cols(S); w += 16) {
+    const long long c = (n + w - 1) / w * (w + 8);
+    if (cost < 0 || c <= cost) {
+      cost = c;
+      best = w;
+    }
+  }
+  return best;
 }
 
 bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long dims[4],

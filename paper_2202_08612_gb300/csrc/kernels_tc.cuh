@@ -19,7 +19,8 @@ struct TcMaps {
 // coordinates ac (ac[0], the K coordinate, advances by 64 per chunk), and the
 // same for B with `bmap` and bc.  A grouped tile (TcItem::nq = nb > 1) stacks
 // nb B boxes of TcEpi::qw rows along N: box 0 at bc, box q at bc with
-// coordinates 2 and 3 replaced by bq[q - 1].
+// coordinates 2 and 3 replaced by bq[q - 1].  (emu_gemm_kernel: nb > 0 is the number
+// of 16-wide K steps of the last chunk that hold data.)
 struct TcSeg {
   int amap, bmap, nk, nb;
   int ac[4];

@@ -919,6 +919,10 @@ struct TcPlan {
     segs.push_back(g);
     items.back().seg_count += 1;
   }
+  // K steps of the last segment's last chunk (FP64 mode)
+  void tail(int steps) {
+    if (steps) segs.back().nb = steps;
+  }
   void drop_empty_last() {
     if (!items.empty() && items.back().seg_count == 0) items.pop_back();
   }
@@ -936,6 +940,11 @@ struct TcDev {
 int kblk(const mlcc3_ctx *c) { return c->emu ? kEmuKB : 64; }
 long long kpad(const mlcc3_ctx *c, long long K) { return (K + kblk(c) - 1) / kblk(c) * kblk(c); }
 int kchunks(const mlcc3_ctx *c, long long K) { return (int)(kpad(c, K) / kblk(c)); }
+// FP64 mode: 16-wide K steps of a reduction's last chunk that hold data (0: all),
+// in TcSeg::nb, which the split mode uses for grouped tiles.
+int ktail(const mlcc3_ctx *c, long long K) {
+  return c->emu ? (int)((K - 1) % kEmuKB / 16 + 1) % (kEmuKB / 16) : 0;
+}
 // Columns of a tile over n output columns.
 int tile_w(const mlcc3_ctx *c, long long n) {
   return c->emu ? emu_tile_width(n, kEmuSlices) : tc_tile_width(n);
@@ -1002,6 +1011,7 @@ void cap_chains(TcPlan &pl, int cap, int kb) {
         h.ac[0] = g.ac[0] + kb * k0;
         h.bc[0] = g.bc[0] + kb * k0;
         h.nk = take;
+        if (kb == kEmuKB && k0 + take < g.nk) h.nb = 0;  // a tail belongs to the last piece
         segs.push_back(h);
         items.back().seg_count += 1;
         used += take;
@@ -1025,6 +1035,14 @@ TcDev tc_plan(mlcc3_ctx *c, const std::string &key0, const std::function<void(Tc
                  static_cast<const TcSeg *>(c->items.at(key + ":segs").first), it->second.second};
   TcPlan pl;
   build(pl);
+  if (c->emu && cap > 0) {
+    // about four items per SM, of whole accumulation chains: their sums are exact,
+    // so where they are cut is free, and an item costs an epilogue
+    long long total = 0;
+    for (const TcSeg &g : pl.segs) total += g.nk;
+    constexpr int chain = 256 / kEmuKB;
+    cap = (int)std::min<long long>(cap, std::max<long long>(1, total / (152LL * 4 * chain)) * chain);
+  }
   cap_chains(pl, cap, kblk(c));
   if ((long long)pl.items.size() > (long long)c->tc_persist_from) {
     // persistent launches hand out items round-robin: the longest chains first
@@ -1170,6 +1188,24 @@ SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, lon
   return op;
 }
 
+// FP64 mode: digits of rows (r1, r2) = (r / R2, r % R2), r < R, of D0 blocks, K
+// contiguous, read in boxes of 128 rows.
+SplitOp &make_split_k2z(mlcc3_ctx *c, const std::string &key, const double *src, long long D0,
+                        long long R, long long R2, long long K, long long s0, long long s1,
+                        long long s2, const std::string &slot) {
+  const long long Kp = kpad(c, K);
+  SplitOp &op = c->splits[key];
+  make_digits(c, op, key, EmuView{src, (int)D0, 1, (int)R, (int)R2, (int)K, 1, s0, 0, s1, s2, 1, 0}, Kp,
+              false, slot);
+  const unsigned long long rb = (unsigned long long)Kp * 2;
+  const unsigned long long dims[4] = {(unsigned long long)Kp, (unsigned long long)R, 1ULL, (unsigned long long)D0};
+  const unsigned long long str[3] = {rb, rb * (unsigned long long)R, rb * (unsigned long long)R};
+  const unsigned bx[4] = {64, 128, 1, 1};
+  encode_split(op, key, dims, str, bx);
+  op.rows = 128;
+  return op;
+}
+
 // Tile width of a pair contraction with nN output columns, and the box rows of
 // its column operand (split_amp_T, split_go_T).
 int pair_bn(const mlcc3_ctx *c, long long nN) {
@@ -1184,22 +1220,18 @@ struct SplitTerm {
   SplitOp *P, *S, *amp;
 };
 
-// G[z][v][w][r] as pair operands key:P, rows (v, w), and key:S, rows (w, v).
+// G[z][v][w][r] as pair operands key:P, rows (v, w), and key:S, rows (w, v): pair
+// tiles of 8 x 16, or in the FP64 mode 128 rows of the flattened pair (29 tiles
+// instead of 32 at n_v = 60, 11 instead of 15 at 37).
 void split_pairs(mlcc3_ctx *c, const std::string &key, const double *G, long long R, long long sz,
                  long long sv, long long sw, const std::string &slot) {
   S s(c);
-  SplitOp &p = make_split(c, key + ":P", G, s.no, s.nv, s.nv, R, sz, sv, sw, 1, 1.0, Box::Pair, slot);
-  if (c->emu) {
-    // the same memory read through a map with the two row indices exchanged
-    SplitOp &q = c->splits[key + ":S"] = p;
-    const unsigned long long rb = (unsigned long long)kpad(c, R) * 2, nv = (unsigned long long)s.nv;
-    const unsigned long long dims[4] = {rb / 2, nv, nv, (unsigned long long)s.no};
-    const unsigned long long str[3] = {rb * nv, rb, rb * nv * nv};
-    const unsigned bx[4] = {64, 16, 8, 1};
-    encode_split(q, key + ":S", dims, str, bx);
-    return;
+  for (int swap = 0; swap < 2; ++swap) {
+    const long long s1 = swap ? sw : sv, s2 = swap ? sv : sw;
+    const std::string k = key + (swap ? ":S" : ":P");
+    if (c->emu) make_split_k2z(c, k, G, s.no, s.nv * s.nv, s.nv, R, sz, s1, s2, slot);
+    else make_split(c, k, G, s.no, s.nv, s.nv, R, sz, s1, s2, 1, 1.0, Box::Pair, slot);
   }
-  make_split(c, key + ":S", G, s.no, s.nv, s.nv, R, sz, sw, sv, 1, 1.0, Box::Pair, slot);
 }
 
 // Split copies of a D-type term: amplitude block X[x][u][y][D] and integral Gv-like [z][v][w][D].
@@ -1267,7 +1299,10 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
   void *W = c->emu ? static_cast<void *>(out)
                    : c->raw("tcW", sizeof(float) * (size_t)(c->chunk_nb * s.nv3));
   const long long NVk = kchunks(c, s.NV), NOk = kchunks(c, s.NO);
-  const long long nt1 = (s.nv + 7) / 8, nt2 = (s.nv + 15) / 16;
+  // row tiles: 8 x 16 pairs, or (FP64 mode) 128 of the flattened pair
+  const long long nt1 = c->emu ? 1 : (s.nv + 7) / 8;
+  const long long nt2 = c->emu ? (s.nv * s.nv + 127) / 128 : (s.nv + 15) / 16;
+  const int tr = c->emu ? 128 : 16;
   const long long cs[3] = {s.nv * s.nv, s.nv, 1};
   std::string sig;
   for (auto &t : terms) sig += t.dtype ? 'd' : 'l';
@@ -1315,7 +1350,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
                 I[q][1] = b.j;
                 I[q][2] = b.k;
               }
-              pl.tile((int)(8 * t1), (int)(16 * t2), c0, bs[us[q0]].off);
+              pl.tile((int)(8 * t1), (int)(tr * t2), c0, bs[us[q0]].off);
               pl.items.back().nq = nq;
               for (int q = 1; q < nq; ++q) pl.items.back().qoff[q - 1] = bs[us[q0 + q]].off;
               for (size_t t = 0; t < terms.size(); ++t) {
@@ -1324,16 +1359,20 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
                   int x = -1, y = -1;  // positions of the B box coordinates 2 and 3
                   if (terms[t].dtype && s0 == o) {
                     pl.seg((int)(6 * t) + (s1 < s2 ? 0 : 2), (int)(6 * t) + 4, (int)NVk,
-                           (int)(16 * t2), (int)(8 * t1), I[0][s2], c0, I[0][s1], I[0][s0]);
+                           (int)(tr * t2), (int)(8 * t1), I[0][s2], c0, I[0][s1], I[0][s0]);
                     x = s1;
                     y = s0;
                   } else if (!terms[t].dtype && s2 == o) {
                     pl.seg((int)(6 * t) + (s0 < s1 ? 0 : 2), (int)(6 * t) + 4, (int)NOk,
-                           (int)(16 * t2), (int)(8 * t1), I[0][s0], c0, I[0][s2], I[0][s1]);
+                           (int)(tr * t2), (int)(8 * t1), I[0][s0], c0, I[0][s2], I[0][s1]);
                     x = s2;
                     y = s1;
                   }
                   if (x < 0) continue;
+                  if (c->emu) {
+                    pl.tail(ktail(c, terms[t].dtype ? s.NV : s.NO));
+                    continue;
+                  }
                   TcSeg &last = pl.segs.back();
                   last.nb = nq;
                   for (int q = 1; q < nq; ++q) {
@@ -1345,7 +1384,8 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
             }
       }
     });
-    TcEpi epi = make_epi(W, oo == 0 ? 0 : 1, 16, cs[p1], cs[p2], cs[o], s.nv, s.nv, s.nv, 1.0);
+    TcEpi epi = make_epi(W, oo == 0 ? 0 : 1, c->emu ? (int)s.nv : 16, cs[p1], cs[p2], cs[o], s.nv, s.nv,
+                         s.nv, 1.0, c->emu ? 1 : 0);
     epi.qw = BW;
     double K = 0.0;
     for (auto &t : terms) K += 2.0 * (t.dtype ? (double)s.NV : (double)s.NO);
@@ -1483,6 +1523,7 @@ void tc_flat_gemm(mlcc3_ctx *c, const SplitOp &A, const SplitOp &B, long long M,
       for (long long tn = 0; tn < ntN; ++tn) {
         pl.tile(0, (int)(128 * tm), (int)(BN * tn), 0);
         pl.seg(0, 2, nk, (int)(128 * tm), 0, 0, (int)(BN * tn), 0, 0);
+        pl.tail(ktail(c, K));
       }
   }, kcap(c));
   TcEpi epi = make_epi(out, 2, R2, s1, s2, sn, M / R2, R2, N, alpha, 1);
@@ -1599,7 +1640,7 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
             pl.items.back().qoff[q - 1] = os[q0 + q]->p * s.bi + os[q0 + q]->q * s.bL;
           pl.seg(g[1], 4 + 2 * g[2], nk, (int)(128 * t), 0, o.r, (int)(BN * tn), 0, (int)(o.off / s.nv3));
           TcSeg &last = pl.segs.back();
-          last.nb = nq;
+          last.nb = c->emu ? ktail(c, s.nv * s.nv) : nq;
           for (int q = 1; q < nq; ++q) {
             last.bq[q - 1][0] = 0;
             last.bq[q - 1][1] = (int)(os[q0 + q]->off / s.nv3);
@@ -1725,9 +1766,9 @@ SplitOp &layout_R(mlcc3_ctx *c, const std::string &key, const double *X, int k) 
   SplitOp &op = c->splits[key];
   tri_layout(c, X, 3 + k, op);
   const unsigned long long Kp = (unsigned long long)kpad(c, s.nv), nv = s.nv;
-  const unsigned long long dims[4] = {Kp, nv, nv, (unsigned long long)c->chunk_nb};
-  const unsigned long long str[3] = {Kp * 2, Kp * 2 * nv, Kp * 2 * nv * nv};
-  const unsigned bx[4] = {64, 16, 8, 1};
+  const unsigned long long dims[4] = {Kp, c->emu ? nv * nv : nv, c->emu ? 1 : nv, (unsigned long long)c->chunk_nb};
+  const unsigned long long str[3] = {Kp * 2, c->emu ? Kp * 2 * nv * nv : Kp * 2 * nv, Kp * 2 * nv * nv};
+  const unsigned bx[4] = {64, c->emu ? 128u : 16u, c->emu ? 1u : 8u, 1};
   encode_split(op, key, dims, str, bx);
   return op;
 }
@@ -1761,7 +1802,9 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
     throw Error{MLCC3_ERR_ARG, "pair contraction: operand box of " + std::to_string(B.rows) +
                                    " rows for tile width " + std::to_string(BN) +
                                    " (tc_wide_bn changed after build_integrals?)"};
-  const long long nt1 = (s.nv + 7) / 8, nt2 = (s.nv + 15) / 16, ntN = (nN + BN - 1) / BN;
+  const long long nt1 = c->emu ? 1 : (s.nv + 7) / 8, ntN = (nN + BN - 1) / BN;
+  const long long nt2 = c->emu ? (s.nv * s.nv + 127) / 128 : (s.nv + 15) / 16;
+  const int tr = c->emu ? 128 : 16;  // row tiles as in triples_split
   const int nk = kchunks(c, s.nv);
   for (int cls = 0; cls < 2; ++cls) {
     const std::string key = "tcP:" + okey + ":" + std::to_string(vk) + std::to_string(g) +
@@ -1771,21 +1814,22 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
         for (long long t1 = 0; t1 < nt1; ++t1)
           for (long long t2 = 0; t2 < nt2; ++t2)
             for (long long tn = 0; tn < ntN; ++tn) {
-              pl.tile((int)(8 * t1), (int)(16 * t2), (int)(BN * tn), og * Sg);
+              pl.tile((int)(8 * t1), (int)(tr * t2), (int)(BN * tn), og * Sg);
               for (auto &o : ords) {
                 if (occ_of(o, g) != og) continue;
                 const bool ascending = o.sp[vp1] < o.sp[vp2];
                 if (ascending != (cls == 0)) continue;
-                pl.seg(2 * o.sp[vk], 6, nk, (int)(16 * t2), (int)(8 * t1), (int)(o.off / s.nv3),
+                pl.seg(2 * o.sp[vk], 6, nk, (int)(tr * t2), (int)(8 * t1), (int)(o.off / s.nv3),
                        (int)(BN * tn), occ_of(o, b2), occ_of(o, b1));
+                pl.tail(ktail(c, s.nv));
               }
               pl.drop_empty_last();
             }
     }, kcap(c));
     // rows of R are (smaller, larger) canonical positions: the view pair in
     // order (cls 0) or swapped (cls 1)
-    TcEpi epi = make_epi(out, 2, 16, cls == 0 ? Sp1 : Sp2, cls == 0 ? Sp2 : Sp1, Sn, s.nv, s.nv,
-                         nN, coef);
+    TcEpi epi = make_epi(out, 2, c->emu ? (int)s.nv : 16, cls == 0 ? Sp1 : Sp2, cls == 0 ? Sp2 : Sp1, Sn,
+                         s.nv, s.nv, nN, coef, c->emu ? 1 : 0);
     tc_launch(c, "pair", BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size() / 2.0,
               c->splits.at(xkey + ":R0"), B);
   }
@@ -1794,6 +1838,44 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
 // out[occ o1][occ o2][row][n] += coef sum_{orderings grouped by (o1, o2)}
 //      sum_{x,y at view positions (vk1 < vk2)} X_{pqr}[..] * T_{occ t}[n][(x,y)]
 // T: split [occ t][n][(x,y)] in both K orders (T, Ts), map dims (K, n, 1, occ t).
+// FP64 mode: the view rows of X on the tile's rows and n on its columns, whose
+// width follows n (N_O is mostly the smaller: 128 x 32 tiles instead of 128 x 64 at
+// N_O = 20, n_v = 60).
+void tc_xt_digits(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp &T,
+                  const SplitOp &Ts, long long nN, const std::vector<Ord> &ords, const std::string &okey,
+                  int vr, int tpos, long long S1, long long S2, long long Srow, double coef, double *out) {
+  S s(c);
+  const int vk1 = vr == 0 ? 1 : 0, vk2 = vr == 2 ? 1 : 2;
+  const int o1 = tpos == 0 ? 1 : 0, o2 = tpos == 2 ? 1 : 2;
+  TcMaps maps;
+  std::memset(&maps, 0, sizeof(maps));
+  for (int k = 0; k < 3; ++k) maps.m[2 * k] = layout_XL(c, xkey + ":XL128" + std::to_string(k), X, k, 128).mhi;
+  maps.m[6] = T.mhi;  // boxes of tile_w(N_O) rows (split_tl_T)
+  maps.m[8] = Ts.mhi;
+  const int BN = tile_w(c, nN);
+  const long long ntM = (s.nv + 127) / 128, ntN = (nN + BN - 1) / BN;
+  const std::string key = "tcX:" + okey + ":" + std::to_string(vr) + std::to_string(tpos) + ":" +
+                          std::to_string(nN) + ":x";
+  TcDev dv = tc_plan(c, key, [&](TcPlan &pl) {
+    for (long long x1 = 0; x1 < s.no; ++x1)
+      for (long long x2 = 0; x2 < s.no; ++x2)
+        for (long long tm = 0; tm < ntM; ++tm)
+          for (long long tn = 0; tn < ntN; ++tn) {
+            pl.tile(0, (int)(128 * tm), (int)(BN * tn), x1 * S1 + x2 * S2);
+            for (auto &o : ords) {
+              if (occ_of(o, o1) != x1 || occ_of(o, o2) != x2) continue;
+              pl.seg(2 * o.sp[vr], o.sp[vk1] < o.sp[vk2] ? 6 : 8, kchunks(c, s.nv * s.nv), (int)(128 * tm), 0,
+                     (int)(o.off / s.nv3), (int)(BN * tn), 0, occ_of(o, tpos));
+              pl.tail(ktail(c, s.nv * s.nv));
+            }
+            pl.drop_empty_last();
+          }
+  }, kcap(c));
+  TcEpi epi = make_epi(out, 2, 128, 0, Srow, 1, 1, s.nv, nN, coef);
+  tc_launch(c, "xt", BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size(),
+            c->splits.at(xkey + ":XL1280"), T);
+}
+
 // The tile rows are T's n (128-row tiles; n = N_O fills 100 of 128) and the
 // columns the view row of X from XL_{s_vr} (tile_width(n_v) columns, 150 of
 // 160): the other way round, the n_v rows in 128-row tiles filled 150 of 256.
@@ -1802,9 +1884,10 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
            int vr, int tpos, long long S1, long long S2, long long Srow, double coef, double *out) {
   S s(c);
   if (ords.empty() || s.nv == 0 || nN == 0) return;
+  if (c->emu) return tc_xt_digits(c, X, xkey, T, Ts, nN, ords, okey, vr, tpos, S1, S2, Srow, coef, out);
   const int vk1 = vr == 0 ? 1 : 0, vk2 = vr == 2 ? 1 : 2;
   const int o1 = tpos == 0 ? 1 : 0, o2 = tpos == 2 ? 1 : 2;
-  const int BX = tile_w(c, s.nv);
+  const int BX = tc_tile_width(s.nv);
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (int k = 0; k < 3; ++k) {
@@ -1813,7 +1896,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
     maps.m[2 * k + 1] = r.mlo;
   }
   // T and Ts with 128-row boxes (rows past n read as zeros)
-  const unsigned long long Kp = (unsigned long long)kpad(c, s.nv * s.nv);
+  const unsigned long long Kp = (unsigned long long)((s.nv * s.nv + 63) / 64 * 64);
   const unsigned long long dims[4] = {Kp, (unsigned long long)nN, 1ULL, (unsigned long long)s.no};
   const unsigned long long str[3] = {Kp * 2, Kp * 2 * (unsigned long long)nN, Kp * 2 * (unsigned long long)nN};
   const unsigned bx[4] = {64, 128, 1, 1};
@@ -1825,7 +1908,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
   maps.m[8] = tsa.mhi;
   maps.m[9] = tsa.mlo;
   const long long ntM = (nN + 127) / 128, ntN = (s.nv + BX - 1) / BX;
-  const int nk = kchunks(c, s.nv * s.nv);
+  const int nk = (int)((s.nv * s.nv + 63) / 64);
   const std::string key = "tcX:" + okey + ":" + std::to_string(vr) + std::to_string(tpos) + ":" +
                           std::to_string(nN) + ":t";
   TcDev dv = tc_plan(c, key, [&](TcPlan &pl) {
@@ -1841,7 +1924,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
             }
             pl.drop_empty_last();
           }
-  }, kcap(c));
+  }, c->tc_kcap);
   TcEpi epi = make_epi(out, 2, 128, 0, 1, Srow, 1, nN, s.nv, coef);
   tc_launch(c, "xt", BX, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size(), T,
             c->splits.at(xkey + ":XLB0"));
@@ -1885,6 +1968,7 @@ void tc_vv(mlcc3_ctx *c, const double *X, const std::string &xkey, const double 
             const Ord &o = os[i];
             const int u = (int)(o.off / s.nv3);
             pl.seg(2 * o.sp[2], 6 + 2 * o.sp[2], nk, (int)(128 * tm), 0, u, (int)(BN * tn), 0, u);
+            pl.tail(ktail(c, s.nv * s.nv));
           }
         }
     }, kcap(c));
@@ -1955,9 +2039,11 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
   const int nk = kchunks(c, s.NJ);
   // one accumulation chain per tile when it is short enough, else pieces
   // summed in FP64 into the zeroed output
-  const bool pieces = kcap(c) > 0 && nk * (int)terms.size() > kcap(c);
+  // (FP64 mode: also where whole tiles would leave SMs idle)
+  const bool pieces = (kcap(c) > 0 && nk * (int)terms.size() > kcap(c)) ||
+                      (c->emu && nW * ntM * ntN < 2 * 152 && nk * (int)terms.size() > 16);
   if (pieces) {
-    if (mode == 3) c->zero(out, (size_t)((nW - 1) * Sw + (s.no - 1) * Sk + (s.nv - 1) * Sc + nN));
+    if (mode == 3) c->zero(out, (size_t)((nW - 1) * Sw + (s.no - 1) * Sk + (s.nv - 1) * Sc + (nN - 1) * Sn + 1));
     mode = 2;
   }
   TcDev dv = tc_plan(c, "tcJ:" + key + ":" + std::to_string(terms.size()), [&](TcPlan &pl) {
@@ -1966,8 +2052,11 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
         for (long long tn = 0; tn < ntN; ++tn) {
           pl.tile(0, (int)(128 * tm), (int)(BN * tn), w * Sw);
           for (size_t t = 0; t < terms.size(); ++t)
+          {
             pl.seg((int)(4 * t), (int)(4 * t + 2), nk, (int)(128 * tm), 0, 0, (int)(BN * tn),
                    (int)w, 0);
+            pl.tail(ktail(c, s.NJ));
+          }
         }
   }, pieces ? kcap(c) : 0);
   TcEpi epi = make_epi(out, mode, (int)s.nv, Sk, Sc, Sn, s.no, s.nv, nN, alpha, 1);
