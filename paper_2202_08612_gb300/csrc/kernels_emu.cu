@@ -87,18 +87,18 @@ __device__ __forceinline__ int scale_exp(EmuScale s) { return (int)((s >> 52) & 
 // C = A B^T with M = N = K = 4096 and S = 5, slicing included: 2.64 ms, against
 // 8.26 ms with one launch of the split mode's kernel per digit degree (two of its
 // three products on zeros, and an FP64 reduction per output, pair and 1024 products).
-template <int S>
+template <int S, int N>
 __global__ void __launch_bounds__(320, 1)
     emu_gemm_kernel(const __grid_constant__ TcMaps maps, const TcItem *__restrict__ items,
                     const TcSeg *__restrict__ segs, int nitems, int stages, const EmuEpi epi,
                     int *__restrict__ status) {
-  constexpr int NG = emu_max_cols(S) / 16;  // 8-column groups per epilogue thread
+  constexpr int NG = N / 16;  // 8-column groups per epilogue thread
   constexpr int A_SL = 128 * kRowB;         // bytes of one slice of A
   constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int n = epi.n;
+  constexpr int n = N;
   const int stage_bytes = S * (A_SL + n * kRowB);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 8);
@@ -162,64 +162,70 @@ __global__ void __launch_bounds__(320, 1)
     // the shared memory must outlive every copy issued into it
     for (int s = 0; s < stages; ++s)
       if ((pending >> s) & 1u) mbar_wait(full0 + 8 * s, (last >> s) & 1u, status, kTcWaitDefault);
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer ----
+  } else if (warp == 1) {
+    // ---- MMA issuer: the warp goes through the loops together, one lane issues.  An
+    // MMA of N = 64 takes 32 clocks, so the loop around it has to be short: with the
+    // tile width a constant its descriptors are a stage's plus constants (with a
+    // runtime width the issue took about 100 clocks per MMA, and the tensor pipe ran 59%
+    // of the time) ----
+    const bool leader = elect_one();
     int stage = 0;
     uint32_t phase = 0;
     int t = 0;  // accumulation chains so far
     bool ok = true;
-    for (int i = blockIdx.x; i < nitems && ok && !*abort_flag; i += gridDim.x) {
+    for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+      if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
       int cc = 0;  // chunk of the accumulation chain
       for (int q = s0; q < s1 && ok; ++q) {
         const int nk = segs[q].nk, tail = segs[q].nb;
         for (int kc = 0; kc < nk; ++kc) {
-          if (cc == 0) {
-            if (!mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait)) {
-              *abort_flag = 1;
-              ok = false;
-              break;
-            }
-          }
-          if (!mbar_wait(full0 + 8 * stage, phase, status, epi.wait)) {
+          if (cc == 0) ok = mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait);
+          ok = __all_sync(0xffffffffu, ok && mbar_wait(full0 + 8 * stage, phase, status, epi.wait));
+          if (!ok) {
             *abort_flag = 1;
-            ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(smem + stage * stage_bytes), b0 = a0 + S * A_SL;
-          const int steps = kc == nk - 1 && tail > 0 ? tail : kEmuKB / 16;
+          const bool last = q == s1 - 1 && kc == nk - 1;
+          if (leader) {
+            const uint32_t a0 = smem_u32(smem) + stage * stage_bytes;
+            const uint64_t ad = smem_desc64(a0), bd = smem_desc64(a0 + S * A_SL);
+            const int steps = kc == nk - 1 && tail > 0 ? tail : kEmuKB / 16;
 #pragma unroll
-          for (int kk = 0; kk < kEmuKB / 16; ++kk) {
-            if (kk >= steps) break;  // zeros to the end of the reduction
+            for (int kk = 0; kk < kEmuKB / 16; ++kk) {
+              if (kk < steps) {  // zeros to the end of the reduction
 #pragma unroll
-            for (int d = 0; d < S; ++d) {
-              // slice d of A with the stacked slices 0 .. S-1-d of B; the first
-              // MMA of a chain (d = 0) covers every degree and clears them
-              const uint64_t ad = smem_desc64(a0 + d * A_SL + kk * 32);
-              const uint32_t acc = (cc > 0 || kk > 0 || d > 0) ? 1u : 0u;
-              const int cols = (S - d) * n;
-              for (int c0 = 0; c0 < cols; c0 += 256) {
-                const int nn = min(256, cols - c0);
-                mma_bf16(tmem + (uint32_t)(d * n + c0), ad, smem_desc64(b0 + c0 * kRowB + kk * 32),
-                         IDESC | ((uint32_t)(nn >> 3) << 17), acc);
+                for (int d = 0; d < S; ++d) {
+                  // slice d of A with the stacked slices 0 .. S-1-d of B; the first
+                  // MMA of a chain (d = 0) covers every degree and clears them
+                  constexpr int W = 256;
+#pragma unroll
+                  for (int c0 = 0; c0 < (S - d) * n; c0 += W) {
+                    const int nn = (S - d) * n - c0 < W ? (S - d) * n - c0 : W;
+                    mma_bf16(tmem + (uint32_t)(d * n + c0), ad + (uint64_t)((d * A_SL + kk * 32) >> 4),
+                             bd + (uint64_t)((c0 * kRowB + kk * 32) >> 4), IDESC | ((uint32_t)(nn >> 3) << 17),
+                             kk > 0 || d > 0 ? 1u : (cc > 0 ? 1u : 0u));
+                  }
+                }
               }
             }
+            mma_commit(empty0 + 8 * stage);
+            if (cc == kChain - 1 || last) mma_commit(tfull);
           }
-          mma_commit(empty0 + 8 * stage);
+          __syncwarp();
           if (++stage == stages) {
             stage = 0;
             phase ^= 1u;
           }
-          if (++cc == kChain || (q == s1 - 1 && kc == nk - 1)) {
-            mma_commit(tfull);
+          if (++cc == kChain || last) {
             ++t;
             cc = 0;
           }
         }
       }
     }
-    mma_commit(done);
+    if (leader) mma_commit(done);
   } else if (warp >= 2) {
     // ---- epilogue ----
     const int lg = warp & 3, half = (warp - 2) >> 2;
@@ -339,11 +345,13 @@ __global__ void __launch_bounds__(320, 1)
 // The width that wastes least: columns of all tiles, and as much as eight columns
 // per tile for reading A again.
 int emu_tile_width(long long n, int S) {
-  int best = 16;
-  long long cost = -1;
-  for (int w = 16; w <= emu_max_cols(S); w += 16) {
+  const int w8[] = {16, 32, 48, 64}, ws[] = {32, 80};
+  int best = 0;
+  long long cost = 0;
+  for (int i = 0; i < (S == 8 ? 4 : 2); ++i) {
+    const int w = S == 8 ? w8[i] : ws[i];
     const long long c = (n + w - 1) / w * (w + 8);
-    if (cost < 0 || c <= cost) {
+    if (!best || c <= cost) {
       cost = c;
       best = w;
     }
@@ -380,29 +388,39 @@ bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long d
   return true;
 }
 
-template <int S>
-static cudaError_t launch_s(const TcMaps &maps, const TcItem *items, const TcSeg *segs, int nitems,
+template <int S, int N>
+static cudaError_t launch_sn(const TcMaps &maps, const TcItem *items, const TcSeg *segs, int nitems,
                             const EmuEpi &epi, int *status, cudaStream_t st) {
   const int stage = S * (128 + epi.n) * kRowB;
   const int stages = std::max(2, std::min(6, (220 * 1024) / stage));
   const int smem = 1024 + stages * stage + 256;
-  cudaError_t e = cudaFuncSetAttribute(emu_gemm_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(emu_gemm_kernel<S, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  emu_gemm_kernel<S><<<std::min(nitems, 152), 320, smem, st>>>(maps, items, segs, nitems, stages, epi, status);
+  emu_gemm_kernel<S, N><<<std::min(nitems, 152), 320, smem, st>>>(maps, items, segs, nitems, stages, epi, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, const TcSeg *segs,
                             int nitems, const EmuEpi &epi, int *status, cudaStream_t st) {
   if (nitems <= 0) return cudaSuccess;
-  if (epi.n < 16 || epi.n % 16 || epi.n > emu_max_cols(S)) return cudaErrorInvalidValue;
-  switch (S) {
-    case 2: return launch_s<2>(maps, items, segs, nitems, epi, status, st);
-    case 3: return launch_s<3>(maps, items, segs, nitems, epi, status, st);
-    case 4: return launch_s<4>(maps, items, segs, nitems, epi, status, st);
-    case 5: return launch_s<5>(maps, items, segs, nitems, epi, status, st);
-    case 6: return launch_s<6>(maps, items, segs, nitems, epi, status, st);
-    case 8: return launch_s<8>(maps, items, segs, nitems, epi, status, st);
+  switch (S * 1000 + epi.n) {
+#define EMU_CASE(s, n) \
+  case s * 1000 + n: return launch_sn<s, n>(maps, items, segs, nitems, epi, status, st)
+    EMU_CASE(8, 16);
+    EMU_CASE(8, 32);
+    EMU_CASE(8, 48);
+    EMU_CASE(8, 64);
+    EMU_CASE(2, 32);
+    EMU_CASE(2, 80);
+    EMU_CASE(3, 32);
+    EMU_CASE(3, 80);
+    EMU_CASE(4, 32);
+    EMU_CASE(4, 80);
+    EMU_CASE(5, 32);
+    EMU_CASE(5, 80);
+    EMU_CASE(6, 32);
+    EMU_CASE(6, 80);
+#undef EMU_CASE
     default: return cudaErrorInvalidValue;
   }
 }
