@@ -167,6 +167,7 @@ extern "C" int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *
         sg.ac[0] = sg.bc[0] = kEmuKB * k0;
         sg.ac[1] = m0;
         sg.bc[1] = n0;
+        it.chunks = sg.nk;
         segs.push_back(sg);
         items.push_back(it);
       }

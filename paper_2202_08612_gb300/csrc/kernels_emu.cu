@@ -138,8 +138,10 @@ __global__ void __launch_bounds__(320, 1)
     uint32_t phase = 0, last = 0, pending = 0;
     for (int i = blockIdx.x; i < nitems && !*abort_flag; i += gridDim.x) {
       const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
+      TcSeg next = segs[s0];  // read one segment ahead of its loads
       for (int q = s0; q < s1 && !*abort_flag; ++q) {
-        const TcSeg sg = segs[q];
+        const TcSeg sg = next;
+        if (q + 1 < s1) next = segs[q + 1];
         for (int kc = 0; kc < sg.nk; ++kc) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, status, epi.wait)) {
             *abort_flag = 1;
@@ -177,8 +179,13 @@ __global__ void __launch_bounds__(320, 1)
       if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
       int cc = 0;  // chunk of the accumulation chain
+      int nk1 = segs[s0].nk, tail1 = segs[s0].nb;
       for (int q = s0; q < s1 && ok; ++q) {
-        const int nk = segs[q].nk, tail = segs[q].nb;
+        const int nk = nk1, tail = tail1;
+        if (q + 1 < s1) {
+          nk1 = segs[q + 1].nk;
+          tail1 = segs[q + 1].nb;
+        }
         for (int kc = 0; kc < nk; ++kc) {
           if (cc == 0) ok = mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait);
           ok = __all_sync(0xffffffffu, ok && mbar_wait(full0 + 8 * stage, phase, status, epi.wait));
@@ -238,9 +245,7 @@ __global__ void __launch_bounds__(320, 1)
     for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
       if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const TcItem it = items[i];
-      int total = 0;
-      for (int q = 0; q < it.seg_count; ++q) total += segs[it.seg_begin + q].nk;
-      const int chains = (total + kChain - 1) / kChain;
+      const int chains = (it.chunks + kChain - 1) / kChain;
       long long T[NG * 8];
       float L[S > 5 ? NG * 8 : 1];
       unsigned nan[NG];

@@ -180,6 +180,24 @@ __device__ __forceinline__ uint32_t idesc_n(uint32_t idesc, int n) {
   return (idesc & ~(0x3Fu << 17)) | ((uint32_t)(n >> 3) << 17);
 }
 
+// The MMAs of one stage: for each 16-wide K step A_hi B_hi + A_hi B_lo + A_lo B_hi.
+// The operands' descriptors are the stage's plus constants: forming each from its
+// address took as long as an MMA of 64 columns runs.
+template <int BN>
+__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t stage_addr, uint32_t idesc, bool first) {
+  constexpr int A_BYTES = 128 * 128, B_BYTES = BN * 128;
+  const uint64_t d = smem_desc(stage_addr);
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk) {
+    const uint64_t ahi = d + (uint64_t)((kk * 32) >> 4), alo = d + (uint64_t)((A_BYTES + kk * 32) >> 4);
+    const uint64_t bhi = d + (uint64_t)((2 * A_BYTES + kk * 32) >> 4);
+    const uint64_t blo = d + (uint64_t)((2 * A_BYTES + B_BYTES + kk * 32) >> 4);
+    mma_bf16(acc, ahi, bhi, idesc, kk > 0 ? 1u : (first ? 0u : 1u));
+    mma_bf16(acc, ahi, blo, idesc, 1u);
+    mma_bf16(acc, alo, bhi, idesc, 1u);
+  }
+}
+
 // Output offset of column group q of a tile.
 __device__ __forceinline__ long long group_off(const TcItem &it, int q) {
   return q == 0 ? it.out_off : it.qoff[q - 1];
@@ -211,8 +229,7 @@ __global__ void __launch_bounds__(192, 1)
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int qrows = epi.qw > 0 ? epi.qw : BN;
   const int ntile = (it.nq > 1 ? it.nq : 1) * qrows;
-  int total = 0;
-  for (int s = 0; s < it.seg_count; ++s) total += seg[s].nk;
+  const int total = it.chunks;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -274,31 +291,26 @@ __global__ void __launch_bounds__(192, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer ----
+  } else if (warp == 1) {
+    // ---- MMA issuer: the warp waits together, one lane issues ----
+    const bool leader = elect_one();
+    const uint32_t idesc = idesc_n(IDESC, ntile);
     int stage = 0;
     uint32_t phase = 0;
     for (int c = 0; c < total; ++c) {
-      if (!mbar_wait(full0 + 8 * stage, phase, status, epi.wait)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, status, epi.wait))) break;
       tc_fence_after();
-      unsigned char *st = smem + stage * STAGE;
-      const uint32_t ahi = smem_u32(st), alo = smem_u32(st + A_BYTES);
-      const uint32_t bhi = smem_u32(st + 2 * A_BYTES), blo = smem_u32(st + 2 * A_BYTES + B_BYTES);
-      const uint32_t idesc = idesc_n(IDESC, ntile);
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t off = kk * 32;
-        mma_bf16(tmem, smem_desc(ahi + off), smem_desc(bhi + off), idesc, (c > 0 || kk > 0));
-        mma_bf16(tmem, smem_desc(ahi + off), smem_desc(blo + off), idesc, 1u);
-        mma_bf16(tmem, smem_desc(alo + off), smem_desc(bhi + off), idesc, 1u);
+      if (leader) {
+        issue_mmas<BN>(tmem, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0);
+        mma_commit(empty0 + 8 * stage);
       }
-      mma_commit(empty0 + 8 * stage);
+      __syncwarp();
       if (++stage == STAGES) {
         stage = 0;
         phase ^= 1u;
       }
     }
-    mma_commit(done);  // arrives once every MMA issued above has completed
+    if (leader) mma_commit(done);  // arrives once every MMA issued above has completed
   } else if (warp >= 2) {
     // ---- epilogue ----
     // a drain wait: every MMA issued has completed before TMEM is read and freed
@@ -410,9 +422,11 @@ __global__ void __launch_bounds__(192, 1)
     bool pending[STAGES];
     for (int s = 0; s < STAGES; ++s) pending[s] = false;
     for (int i = blockIdx.x; i < nitems && !*abort_flag; i += gridDim.x) {
-      const TcItem it = items[i];
-      for (int q = 0; q < it.seg_count && !*abort_flag; ++q) {
-        const TcSeg &sg = segs[it.seg_begin + q];
+      const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
+      TcSeg next = segs[s0];  // read one segment ahead of its loads
+      for (int q = s0; q < s1 && !*abort_flag; ++q) {
+        const TcSeg sg = next;
+        if (q + 1 < s1) next = segs[q + 1];
         for (int kc = 0; kc < sg.nk; ++kc) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, status, epi.wait)) {
             *abort_flag = 1;
@@ -433,52 +447,45 @@ __global__ void __launch_bounds__(192, 1)
     // the shared memory must outlive every copy issued into it
     for (int s = 0; s < STAGES; ++s)
       if (pending[s]) mbar_wait(full0 + 8 * s, last[s], status, kTcWaitDefault);
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer ----
+  } else if (warp == 1) {
+    // ---- MMA issuer: the warp waits together, one lane issues ----
+    const bool leader = elect_one();
     int stage = 0;
     uint32_t phase = 0;
     int t = 0;
-    for (int i = blockIdx.x; i < nitems && !*abort_flag; i += gridDim.x, ++t) {
+    for (int i = blockIdx.x; i < nitems; i += gridDim.x, ++t) {
+      if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const int u = t & 1;
-      if (!mbar_wait(tempty0 + 8 * u, ((uint32_t)(t >> 1) & 1u) ^ 1u, status, epi.wait)) {
-        *abort_flag = 1;
-        break;
-      }
-      tc_fence_after();
-      const TcItem it = items[i];
-      int total = 0;
-      for (int q = 0; q < it.seg_count; ++q) total += segs[it.seg_begin + q].nk;
+      const int total = items[i].chunks;
       const uint32_t acc = tmem + (uint32_t)(u * NCOLS);
-      const uint32_t idesc = idesc_n(IDESC, (it.nq > 1 ? it.nq : 1) * qrows);
-      bool ok = true;
-      for (int c = 0; c < total; ++c) {
-        if (!mbar_wait(full0 + 8 * stage, phase, status, epi.wait)) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
+      const uint32_t idesc = idesc_n(IDESC, (items[i].nq > 1 ? items[i].nq : 1) * qrows);
+      bool ok = __all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * u, ((uint32_t)(t >> 1) & 1u) ^ 1u, status,
+                                                  epi.wait));
+      for (int c = 0; c < total && ok; ++c) {
+        ok = __all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, status, epi.wait));
+        if (!ok) break;
         tc_fence_after();
-        unsigned char *st = smem + stage * STAGE;
-        const uint32_t ahi = smem_u32(st), alo = smem_u32(st + A_BYTES);
-        const uint32_t bhi = smem_u32(st + 2 * A_BYTES), blo = smem_u32(st + 2 * A_BYTES + B_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint32_t off = kk * 32;
-          mma_bf16(acc, smem_desc(ahi + off), smem_desc(bhi + off), idesc, (c > 0 || kk > 0));
-          mma_bf16(acc, smem_desc(ahi + off), smem_desc(blo + off), idesc, 1u);
-          mma_bf16(acc, smem_desc(alo + off), smem_desc(bhi + off), idesc, 1u);
+        if (leader) {
+          issue_mmas<BN>(acc, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0);
+          mma_commit(empty0 + 8 * stage);
         }
-        mma_commit(empty0 + 8 * stage);
+        __syncwarp();
         if (++stage == STAGES) {
           stage = 0;
           phase ^= 1u;
         }
       }
-      if (!ok) break;
-      mma_commit(tfull0 + 8 * u);  // arrives when this item's MMAs have completed
+      if (!ok) {
+        *abort_flag = 1;
+        break;
+      }
+      if (leader) mma_commit(tfull0 + 8 * u);  // arrives when this item's MMAs have completed
     }
-    mma_commit(done);
-    mbar_wait(done, 0, status, kTcWaitDefault);  // every MMA issued above has completed
+    if (leader) {
+      mma_commit(done);
+      mbar_wait(done, 0, status, kTcWaitDefault);  // every MMA issued above has completed
+    }
+    __syncwarp();
   } else if (warp >= 2) {
     // ---- epilogue ----
     const int lg = warp & 3;

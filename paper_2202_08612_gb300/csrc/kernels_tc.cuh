@@ -38,6 +38,8 @@ struct TcItem {
   int r1_0, r2_0;
   int c0;             // global column of the tile's first column
   int nq;             // column groups (0 or 1: one group of BN columns)
+  int chunks;         // K chunks of all its segments
+  int pad;
   long long out_off;
   long long qoff[3];
 };

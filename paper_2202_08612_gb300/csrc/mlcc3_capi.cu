@@ -1044,6 +1044,8 @@ TcDev tc_plan(mlcc3_ctx *c, const std::string &key0, const std::function<void(Tc
     cap = (int)std::min<long long>(cap, std::max<long long>(1, total / (152LL * 4 * chain)) * chain);
   }
   cap_chains(pl, cap, kblk(c));
+  for (TcItem &i : pl.items)
+    for (int q = 0; q < i.seg_count; ++q) i.chunks += pl.segs[i.seg_begin + q].nk;
   if ((long long)pl.items.size() > (long long)c->tc_persist_from) {
     // persistent launches hand out items round-robin: the longest chains first
     // (stable, so equal items keep their order and their operand reuse) even

@@ -148,6 +148,7 @@ extern "C" int mlcc3_debug_tc_gemm(const double *A, const double *B, double *C, 
       sg.nk = (int)(Kp / 64);
       sg.ac[1] = m0;
       sg.bc[1] = n0;
+      it.chunks = sg.nk;
       segs.push_back(sg);
       items.push_back(it);
     }
