@@ -179,12 +179,12 @@ __global__ void __launch_bounds__(320, 1)
       if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const int s0 = items[i].seg_begin, s1 = s0 + items[i].seg_count;
       int cc = 0;  // chunk of the accumulation chain
-      int nk1 = segs[s0].nk, tail1 = segs[s0].nb;
+      int nk1 = segs[s0].nk, tail1 = segs[s0].tail;
       for (int q = s0; q < s1 && ok; ++q) {
         const int nk = nk1, tail = tail1;
         if (q + 1 < s1) {
           nk1 = segs[q + 1].nk;
-          tail1 = segs[q + 1].nb;
+          tail1 = segs[q + 1].tail;
         }
         for (int kc = 0; kc < nk; ++kc) {
           if (cc == 0) ok = mbar_wait(tempty, ((uint32_t)t & 1u) ^ 1u, status, epi.wait);

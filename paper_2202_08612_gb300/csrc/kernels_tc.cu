@@ -180,15 +180,17 @@ __device__ __forceinline__ uint32_t idesc_n(uint32_t idesc, int n) {
   return (idesc & ~(0x3Fu << 17)) | ((uint32_t)(n >> 3) << 17);
 }
 
-// The MMAs of one stage: for each 16-wide K step A_hi B_hi + A_hi B_lo + A_lo B_hi.
+// The MMAs of one stage: for each of the first `steps` 16-wide K steps A_hi B_hi + A_hi B_lo + A_lo B_hi.
 // The operands' descriptors are the stage's plus constants: forming each from its
 // address took as long as an MMA of 64 columns runs.
 template <int BN>
-__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t stage_addr, uint32_t idesc, bool first) {
+__device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t stage_addr, uint32_t idesc, bool first,
+                                           int steps) {
   constexpr int A_BYTES = 128 * 128, B_BYTES = BN * 128;
   const uint64_t d = smem_desc(stage_addr);
 #pragma unroll
   for (int kk = 0; kk < 4; ++kk) {
+    if (kk >= steps) break;
     const uint64_t ahi = d + (uint64_t)((kk * 32) >> 4), alo = d + (uint64_t)((A_BYTES + kk * 32) >> 4);
     const uint64_t bhi = d + (uint64_t)((2 * A_BYTES + kk * 32) >> 4);
     const uint64_t blo = d + (uint64_t)((2 * A_BYTES + B_BYTES + kk * 32) >> 4);
@@ -297,11 +299,17 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t idesc = idesc_n(IDESC, ntile);
     int stage = 0;
     uint32_t phase = 0;
+    int q = 0, left = seg[0].nk;  // segment and its chunks to go
     for (int c = 0; c < total; ++c) {
       if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, status, epi.wait))) break;
       tc_fence_after();
+      int steps = 4;
+      if (--left == 0) {
+        if (seg[q].tail > 0) steps = seg[q].tail;
+        if (c + 1 < total) left = seg[++q].nk;
+      }
       if (leader) {
-        issue_mmas<BN>(tmem, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0);
+        issue_mmas<BN>(tmem, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0, steps);
         mma_commit(empty0 + 8 * stage);
       }
       __syncwarp();
@@ -461,12 +469,30 @@ __global__ void __launch_bounds__(192, 1)
       const uint32_t idesc = idesc_n(IDESC, (items[i].nq > 1 ? items[i].nq : 1) * qrows);
       bool ok = __all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * u, ((uint32_t)(t >> 1) & 1u) ^ 1u, status,
                                                   epi.wait));
+      const TcSeg *seg = segs + items[i].seg_begin;
+      int left = seg->nk, tail = seg->tail;  // of the current segment, read one ahead
+      int nk1 = 0, tail1 = 0;
+      if (items[i].seg_count > 1) {
+        nk1 = seg[1].nk;
+        tail1 = seg[1].tail;
+      }
+      int q = 1;
       for (int c = 0; c < total && ok; ++c) {
+        int steps = 4;
+        if (--left == 0) {
+          if (tail > 0) steps = tail;
+          left = nk1;
+          tail = tail1;
+          if (++q < items[i].seg_count) {
+            nk1 = seg[q].nk;
+            tail1 = seg[q].tail;
+          }
+        }
         ok = __all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, status, epi.wait));
         if (!ok) break;
         tc_fence_after();
         if (leader) {
-          issue_mmas<BN>(acc, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0);
+          issue_mmas<BN>(acc, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0, steps);
           mma_commit(empty0 + 8 * stage);
         }
         __syncwarp();

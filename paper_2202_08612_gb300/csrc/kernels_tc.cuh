@@ -19,13 +19,14 @@ struct TcMaps {
 // coordinates ac (ac[0], the K coordinate, advances by 64 per chunk), and the
 // same for B with `bmap` and bc.  A grouped tile (TcItem::nq = nb > 1) stacks
 // nb B boxes of TcEpi::qw rows along N: box 0 at bc, box q at bc with
-// coordinates 2 and 3 replaced by bq[q - 1].  (emu_gemm_kernel: nb > 0 is the number
-// of 16-wide K steps of the last chunk that hold data.)
+// coordinates 2 and 3 replaced by bq[q - 1].  tail > 0: the 16-wide K steps of the
+// last chunk that hold data (the others are zeros to the end of the reduction).
 struct TcSeg {
   int amap, bmap, nk, nb;
   int ac[4];
   int bc[4];
   int bq[3][2];
+  int tail, pad;
 };
 
 // One 128 x N output tile: the K segments seg[seg_begin, seg_begin + seg_count)

@@ -919,10 +919,8 @@ struct TcPlan {
     segs.push_back(g);
     items.back().seg_count += 1;
   }
-  // K steps of the last segment's last chunk (FP64 mode)
-  void tail(int steps) {
-    if (steps) segs.back().nb = steps;
-  }
+  // K steps of the last segment's last chunk
+  void tail(int steps) { segs.back().tail = steps; }
   void drop_empty_last() {
     if (!items.empty() && items.back().seg_count == 0) items.pop_back();
   }
@@ -940,10 +938,10 @@ struct TcDev {
 int kblk(const mlcc3_ctx *c) { return c->emu ? kEmuKB : 64; }
 long long kpad(const mlcc3_ctx *c, long long K) { return (K + kblk(c) - 1) / kblk(c) * kblk(c); }
 int kchunks(const mlcc3_ctx *c, long long K) { return (int)(kpad(c, K) / kblk(c)); }
-// FP64 mode: 16-wide K steps of a reduction's last chunk that hold data (0: all),
-// in TcSeg::nb, which the split mode uses for grouped tiles.
+// 16-wide K steps of a reduction's last chunk that hold data (0: all).
 int ktail(const mlcc3_ctx *c, long long K) {
-  return c->emu ? (int)((K - 1) % kEmuKB / 16 + 1) % (kEmuKB / 16) : 0;
+  const int kb = kblk(c);
+  return (int)((K - 1) % kb / 16 + 1) % (kb / 16);
 }
 // Columns of a tile over n output columns.
 int tile_w(const mlcc3_ctx *c, long long n) {
@@ -1011,7 +1009,7 @@ void cap_chains(TcPlan &pl, int cap, int kb) {
         h.ac[0] = g.ac[0] + kb * k0;
         h.bc[0] = g.bc[0] + kb * k0;
         h.nk = take;
-        if (kb == kEmuKB && k0 + take < g.nk) h.nb = 0;  // a tail belongs to the last piece
+        if (k0 + take < g.nk) h.tail = 0;  // a tail belongs to the last piece
         segs.push_back(h);
         items.back().seg_count += 1;
         used += take;
@@ -1171,40 +1169,26 @@ SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, lon
                                       (unsigned long long)D1, (unsigned long long)D0};
   const unsigned long long str[3] = {(unsigned long long)(Kp * 2), (unsigned long long)(Kp * 2 * D2),
                                      (unsigned long long)(Kp * 2 * D2 * D1)};
-  unsigned bx[4] = {64, 16, 8, 1};
+  unsigned bx[4] = {64, 128, 1, 1};
   if (box == Box::Row) {
     bx[1] = rowbox ? rowbox : (unsigned)tile_w(c, c->nv);
-    bx[2] = 1;
   }
   unsigned long long fdims[4] = {dims[0], (unsigned long long)(D0 * D1 * D2), 1ULL, 1ULL};
   unsigned long long fstr[3] = {str[0], str[0] * fdims[1], str[0] * fdims[1]};
   const unsigned long long *md = dims, *ms = str;
   if (box == Box::Flat) {  // rows = the flattened (D0, D1, D2) index
     bx[1] = rowbox ? rowbox : 128;
-    bx[2] = 1;
     md = fdims;
     ms = fstr;
   }
+  const unsigned long long pdims[4] = {dims[0], (unsigned long long)(D1 * D2), 1ULL, (unsigned long long)D0};
+  const unsigned long long pstr[3] = {str[0], str[2], str[2]};
+  if (box == Box::Pair) {  // rows = the flattened (D1, D2) index
+    md = pdims;
+    ms = pstr;
+  }
   encode_split(op, key, md, ms, bx);
-  op.rows = box == Box::Pair ? 128u : bx[1];
-  return op;
-}
-
-// FP64 mode: digits of rows (r1, r2) = (r / R2, r % R2), r < R, of D0 blocks, K
-// contiguous, read in boxes of 128 rows.
-SplitOp &make_split_k2z(mlcc3_ctx *c, const std::string &key, const double *src, long long D0,
-                        long long R, long long R2, long long K, long long s0, long long s1,
-                        long long s2, const std::string &slot) {
-  const long long Kp = kpad(c, K);
-  SplitOp &op = c->splits[key];
-  make_digits(c, op, key, EmuView{src, (int)D0, 1, (int)R, (int)R2, (int)K, 1, s0, 0, s1, s2, 1, 0}, Kp,
-              false, slot);
-  const unsigned long long rb = (unsigned long long)Kp * 2;
-  const unsigned long long dims[4] = {(unsigned long long)Kp, (unsigned long long)R, 1ULL, (unsigned long long)D0};
-  const unsigned long long str[3] = {rb, rb * (unsigned long long)R, rb * (unsigned long long)R};
-  const unsigned bx[4] = {64, 128, 1, 1};
-  encode_split(op, key, dims, str, bx);
-  op.rows = 128;
+  op.rows = bx[1];
   return op;
 }
 
@@ -1222,17 +1206,16 @@ struct SplitTerm {
   SplitOp *P, *S, *amp;
 };
 
-// G[z][v][w][r] as pair operands key:P, rows (v, w), and key:S, rows (w, v): pair
-// tiles of 8 x 16, or in the FP64 mode 128 rows of the flattened pair (29 tiles
-// instead of 32 at n_v = 60, 11 instead of 15 at 37).
+// G[z][v][w][r] as pair operands key:P, rows (v, w), and key:S, rows (w, v), read in
+// tiles of 128 rows of the flattened pair (29 at n_v = 60, where 8 x 16 pair tiles
+// were 32; 26 instead of 32 at 57, 113 instead of 120 at 120).
 void split_pairs(mlcc3_ctx *c, const std::string &key, const double *G, long long R, long long sz,
                  long long sv, long long sw, const std::string &slot) {
   S s(c);
   for (int swap = 0; swap < 2; ++swap) {
     const long long s1 = swap ? sw : sv, s2 = swap ? sv : sw;
     const std::string k = key + (swap ? ":S" : ":P");
-    if (c->emu) make_split_k2z(c, k, G, s.no, s.nv * s.nv, s.nv, R, sz, s1, s2, slot);
-    else make_split(c, k, G, s.no, s.nv, s.nv, R, sz, s1, s2, 1, 1.0, Box::Pair, slot);
+    make_split(c, k, G, s.no, s.nv, s.nv, R, sz, s1, s2, 1, 1.0, Box::Pair, slot);
   }
 }
 
@@ -1301,10 +1284,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
   void *W = c->emu ? static_cast<void *>(out)
                    : c->raw("tcW", sizeof(float) * (size_t)(c->chunk_nb * s.nv3));
   const long long NVk = kchunks(c, s.NV), NOk = kchunks(c, s.NO);
-  // row tiles: 8 x 16 pairs, or (FP64 mode) 128 of the flattened pair
-  const long long nt1 = c->emu ? 1 : (s.nv + 7) / 8;
-  const long long nt2 = c->emu ? (s.nv * s.nv + 127) / 128 : (s.nv + 15) / 16;
-  const int tr = c->emu ? 128 : 16;
+  const long long ntM = (s.nv * s.nv + 127) / 128;  // tiles of 128 rows of the flattened pair
   const long long cs[3] = {s.nv * s.nv, s.nv, 1};
   std::string sig;
   for (auto &t : terms) sig += t.dtype ? 'd' : 'l';
@@ -1332,15 +1312,14 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
         if (!groups.count(g)) order.push_back(g);
         groups[g].push_back(u);
       }
-      // items of one pair tile (t1, t2) for every batch of the group follow each
+      // items of one pair tile for every batch of the group follow each
       // other: the concurrently running CTAs then share that tile's rows of the
       // group's integral-side operand (read from DRAM once per group instead of
       // once per batch), while the batches' amplitude boxes (a few MB per group)
       // stay in L2 across the tiles
       for (const auto &g : order) {
         const std::vector<long long> &us = groups[g];
-        for (long long t1 = 0; t1 < nt1; ++t1)
-          for (long long t2 = 0; t2 < nt2; ++t2)
+        for (long long tm = 0; tm < ntM; ++tm)
             for (size_t q0 = 0; q0 < us.size(); q0 += (size_t)G)
             for (long long tn = 0; tn < ntN; ++tn) {
               const int nq = (int)std::min<size_t>((size_t)G, us.size() - q0);
@@ -1352,7 +1331,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
                 I[q][1] = b.j;
                 I[q][2] = b.k;
               }
-              pl.tile((int)(8 * t1), (int)(tr * t2), c0, bs[us[q0]].off);
+              pl.tile(0, (int)(128 * tm), c0, bs[us[q0]].off);
               pl.items.back().nq = nq;
               for (int q = 1; q < nq; ++q) pl.items.back().qoff[q - 1] = bs[us[q0 + q]].off;
               for (size_t t = 0; t < terms.size(); ++t) {
@@ -1361,20 +1340,17 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
                   int x = -1, y = -1;  // positions of the B box coordinates 2 and 3
                   if (terms[t].dtype && s0 == o) {
                     pl.seg((int)(6 * t) + (s1 < s2 ? 0 : 2), (int)(6 * t) + 4, (int)NVk,
-                           (int)(tr * t2), (int)(8 * t1), I[0][s2], c0, I[0][s1], I[0][s0]);
+                           (int)(128 * tm), 0, I[0][s2], c0, I[0][s1], I[0][s0]);
                     x = s1;
                     y = s0;
                   } else if (!terms[t].dtype && s2 == o) {
                     pl.seg((int)(6 * t) + (s0 < s1 ? 0 : 2), (int)(6 * t) + 4, (int)NOk,
-                           (int)(tr * t2), (int)(8 * t1), I[0][s0], c0, I[0][s2], I[0][s1]);
+                           (int)(128 * tm), 0, I[0][s0], c0, I[0][s2], I[0][s1]);
                     x = s2;
                     y = s1;
                   }
                   if (x < 0) continue;
-                  if (c->emu) {
-                    pl.tail(ktail(c, terms[t].dtype ? s.NV : s.NO));
-                    continue;
-                  }
+                  pl.tail(ktail(c, terms[t].dtype ? s.NV : s.NO));
                   TcSeg &last = pl.segs.back();
                   last.nb = nq;
                   for (int q = 1; q < nq; ++q) {
@@ -1386,8 +1362,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
             }
       }
     });
-    TcEpi epi = make_epi(W, oo == 0 ? 0 : 1, c->emu ? (int)s.nv : 16, cs[p1], cs[p2], cs[o], s.nv, s.nv,
-                         s.nv, 1.0, c->emu ? 1 : 0);
+    TcEpi epi = make_epi(W, oo == 0 ? 0 : 1, (int)s.nv, cs[p1], cs[p2], cs[o], s.nv, s.nv, s.nv, 1.0, 1);
     epi.qw = BW;
     double K = 0.0;
     for (auto &t : terms) K += 2.0 * (t.dtype ? (double)s.NV : (double)s.NO);
@@ -1642,7 +1617,8 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
             pl.items.back().qoff[q - 1] = os[q0 + q]->p * s.bi + os[q0 + q]->q * s.bL;
           pl.seg(g[1], 4 + 2 * g[2], nk, (int)(128 * t), 0, o.r, (int)(BN * tn), 0, (int)(o.off / s.nv3));
           TcSeg &last = pl.segs.back();
-          last.nb = c->emu ? ktail(c, s.nv * s.nv) : nq;
+          last.nb = nq;
+          last.tail = ktail(c, s.nv * s.nv);
           for (int q = 1; q < nq; ++q) {
             last.bq[q - 1][0] = 0;
             last.bq[q - 1][1] = (int)(os[q0 + q]->off / s.nv3);
@@ -1762,15 +1738,15 @@ SplitOp &layout_XL(mlcc3_ctx *c, const std::string &key, const double *X, int k,
   return op;
 }
 
-// R_k: K = canonical position k, rows = the other two as (smaller, larger) pair tiles.
+// R_k: K = canonical position k, rows = the other two, flattened (smaller, larger).
 SplitOp &layout_R(mlcc3_ctx *c, const std::string &key, const double *X, int k) {
   S s(c);
   SplitOp &op = c->splits[key];
   tri_layout(c, X, 3 + k, op);
   const unsigned long long Kp = (unsigned long long)kpad(c, s.nv), nv = s.nv;
-  const unsigned long long dims[4] = {Kp, c->emu ? nv * nv : nv, c->emu ? 1 : nv, (unsigned long long)c->chunk_nb};
-  const unsigned long long str[3] = {Kp * 2, c->emu ? Kp * 2 * nv * nv : Kp * 2 * nv, Kp * 2 * nv * nv};
-  const unsigned bx[4] = {64, c->emu ? 128u : 16u, c->emu ? 1u : 8u, 1};
+  const unsigned long long dims[4] = {Kp, nv * nv, 1ULL, (unsigned long long)c->chunk_nb};
+  const unsigned long long str[3] = {Kp * 2, Kp * 2 * nv * nv, Kp * 2 * nv * nv};
+  const unsigned bx[4] = {64, 128, 1, 1};
   encode_split(op, key, dims, str, bx);
   return op;
 }
@@ -1804,24 +1780,21 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
     throw Error{MLCC3_ERR_ARG, "pair contraction: operand box of " + std::to_string(B.rows) +
                                    " rows for tile width " + std::to_string(BN) +
                                    " (tc_wide_bn changed after build_integrals?)"};
-  const long long nt1 = c->emu ? 1 : (s.nv + 7) / 8, ntN = (nN + BN - 1) / BN;
-  const long long nt2 = c->emu ? (s.nv * s.nv + 127) / 128 : (s.nv + 15) / 16;
-  const int tr = c->emu ? 128 : 16;  // row tiles as in triples_split
+  const long long ntM = (s.nv * s.nv + 127) / 128, ntN = (nN + BN - 1) / BN;
   const int nk = kchunks(c, s.nv);
   for (int cls = 0; cls < 2; ++cls) {
     const std::string key = "tcP:" + okey + ":" + std::to_string(vk) + std::to_string(g) +
                             std::to_string(cls) + ":" + std::to_string(nN);
     TcDev dv = tc_plan(c, key, [&](TcPlan &pl) {
       for (long long og = 0; og < s.no; ++og)
-        for (long long t1 = 0; t1 < nt1; ++t1)
-          for (long long t2 = 0; t2 < nt2; ++t2)
+        for (long long tm = 0; tm < ntM; ++tm)
             for (long long tn = 0; tn < ntN; ++tn) {
-              pl.tile((int)(8 * t1), (int)(tr * t2), (int)(BN * tn), og * Sg);
+              pl.tile(0, (int)(128 * tm), (int)(BN * tn), og * Sg);
               for (auto &o : ords) {
                 if (occ_of(o, g) != og) continue;
                 const bool ascending = o.sp[vp1] < o.sp[vp2];
                 if (ascending != (cls == 0)) continue;
-                pl.seg(2 * o.sp[vk], 6, nk, (int)(tr * t2), (int)(8 * t1), (int)(o.off / s.nv3),
+                pl.seg(2 * o.sp[vk], 6, nk, (int)(128 * tm), 0, (int)(o.off / s.nv3),
                        (int)(BN * tn), occ_of(o, b2), occ_of(o, b1));
                 pl.tail(ktail(c, s.nv));
               }
@@ -1830,8 +1803,8 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
     }, kcap(c));
     // rows of R are (smaller, larger) canonical positions: the view pair in
     // order (cls 0) or swapped (cls 1)
-    TcEpi epi = make_epi(out, 2, c->emu ? (int)s.nv : 16, cls == 0 ? Sp1 : Sp2, cls == 0 ? Sp2 : Sp1, Sn,
-                         s.nv, s.nv, nN, coef, c->emu ? 1 : 0);
+    TcEpi epi = make_epi(out, 2, (int)s.nv, cls == 0 ? Sp1 : Sp2, cls == 0 ? Sp2 : Sp1, Sn, s.nv, s.nv, nN,
+                         coef, 1);
     tc_launch(c, "pair", BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size() / 2.0,
               c->splits.at(xkey + ":R0"), B);
   }
@@ -1923,6 +1896,7 @@ void tc_xt(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp
               if (occ_of(o, o1) != x1 || occ_of(o, o2) != x2) continue;
               pl.seg(o.sp[vk1] < o.sp[vk2] ? 6 : 8, 2 * o.sp[vr], nk, (int)(128 * tm), 0,
                      occ_of(o, tpos), (int)(BX * tn), 0, (int)(o.off / s.nv3));
+              pl.tail(ktail(c, s.nv * s.nv));
             }
             pl.drop_empty_last();
           }
