@@ -1908,6 +1908,34 @@ __global__ void __launch_bounds__(256, 3) bstc_gemv_kernel(BstcParams p) { gemv_
 
 namespace mlcc3 {
 
+// The block's sums of its (k, l) tiles, over the H element shares, added to out
+// with one atomic each: with one per thread, 256 threads of a thousand blocks met
+// on n_o^2 addresses (1.12 -> 0.84 ms at n_o = 11, n_v = 57).  red: kPdRed bytes.
+constexpr size_t kPdRed = 256 * 8 * sizeof(double);
+__device__ __forceinline__ double to_f64(float x) { return widen_f32(x); }
+__device__ __forceinline__ double to_f64(double x) { return x; }
+__device__ __forceinline__ void pair_dots_add(unsigned char *smraw, const double (&acc)[4][4], int tile,
+                                              int h, int TT, int H, int nh, int no, double *out,
+                                              long long ldo, int kl, double f) {
+  double *red = reinterpret_cast<double *>(smraw);
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    __syncthreads();
+    if (h < H)
+#pragma unroll
+      for (int v = 0; v < 8; ++v) red[(h * TT + tile) * 8 + v] = acc[2 * half + v / 4][v % 4];
+    __syncthreads();
+    for (int q = threadIdx.x; q < TT * 8; q += 256) {
+      const int tl = q / 8, v = q % 8;
+      const int kk = 4 * (tl / nh) + 2 * half + v / 4, ll = 4 * (tl % nh) + v % 4;
+      if (kk >= no || ll >= no) continue;
+      double x = 0.0;
+      for (int g = 0; g < H; ++g) x += red[(g * TT + tl) * 8 + v];
+      atomicAdd(out + (kl ? kk * ldo + ll : ll * ldo + kk), f * x);
+    }
+  }
+}
+
 // D_kl-type pair terms: out[k][l] (kl = 1, else out[l][k]) += alpha sum_{abc}
 // X_{ijl}[abc] Y_{ijk}[abc] for the ordered pair (i, j) = (p0 + y / no, y % no),
 // y = blockIdx.y, over all k, l with stored views; blocks with j > i return (their
@@ -1923,7 +1951,11 @@ namespace mlcc3 {
 // except for ties: the binary32 form takes TA = 2, TB = 16, rows of 64 bytes),
 // and the element is
 // stored at its logical (a,b,c) position of the view's tile in shared memory
-// (padded strides, no bank conflicts along any axis; pads stay zero).  Thread
+// (padded strides, no bank conflicts along any axis; pads stay zero).  The copies'
+// index work bounded the kernel: an element's place along the physical axes depends
+// only on the thread and on which axis is a, so it is made once, and a tile's
+// offsets and limits once per view (FP32: 3.37 -> 2.99 ms at n_o = 6, n_v = 150; 0.84
+// -> 0.70 at 11, 57).  Thread
 // t keeps a 4x4 (k,l) tile (t % TT) of partial sums over the (t / TT)-th share
 // of every tile and adds it to `out` once.  T is the type of the products and
 // of the per-tile sums (FP32 in the split-precision mode, else FP64); the sums
@@ -1947,10 +1979,12 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
   extern __shared__ unsigned char smraw[];
   T *xs = reinterpret_cast<T *>(smraw);         // [no][TS]
   T *ys = xs + (size_t)no * TS;                 // [no][TS]
-  __shared__ long long s_off[32];
-  __shared__ int s_st[32][3];
-  __shared__ int s_ax[32][3];                   // logical axis of physical axis 0 (fastest), 1, 2
-  __shared__ int s_have[32];
+  // per view: shared-memory strides of the physical axes 0 (fastest), 1, 2 (.x, .y, .z)
+  // and which of them is the logical a (.w); per tile: offset of its first element
+  // and the extents inside the block along the physical axes (a byte each)
+  __shared__ int4 s_ax[32];
+  __shared__ long long s_tb[32];
+  __shared__ unsigned s_lim[32];
   const int i = p0 + (int)blockIdx.y / no, j = (int)blockIdx.y % no;
   // the ordered pair (j, i) gives the same sums as (i, j): X_{jil}[abc] =
   // X_{ijl}[bac] and Y likewise, and a <-> b only relabels the summation, so
@@ -1959,25 +1993,41 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
   const double wij = j < i ? 2.0 : 1.0;
   const int t = threadIdx.x;
   for (int q = t; q < 2 * no * TS; q += blockDim.x) xs[q] = T(0);
-  if (t < no) {
+  int st[3] = {0, 0, 0}, ax[3] = {0, 1, 2};
+  long long off0 = 0;
+  bool have = false;
+  if (t < no) {  // thread t looks after view t
     const int v = (i * no + j) * no + t;
-    s_have[t] = vhave[v];
-    s_off[t] = voff[v];
-    int st[3] = {vstr[3 * v], vstr[3 * v + 1], vstr[3 * v + 2]};
-    int ax[3] = {0, 1, 2};
+    have = vhave[v] != 0;
+    off0 = voff[v];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) st[x] = vstr[3 * v + x];
     // order the logical axes by stride (ascending): physical fastest first
+#pragma unroll
     for (int x = 0; x < 3; ++x)
-      for (int y = 0; y + 1 < 3 - x; ++y)
-        if (st[ax[y]] > st[ax[y + 1]]) {
+#pragma unroll
+      for (int y = 0; y + 1 < 3 - x; ++y) {
+        const int sy = ax[y] == 0 ? st[0] : ax[y] == 1 ? st[1] : st[2];
+        const int sz = ax[y + 1] == 0 ? st[0] : ax[y + 1] == 1 ? st[1] : st[2];
+        if (sy > sz) {
           const int tmp = ax[y];
           ax[y] = ax[y + 1];
           ax[y + 1] = tmp;
         }
-    for (int x = 0; x < 3; ++x) {
-      s_st[t][x] = st[x];
-      s_ax[t][x] = ax[x];
-    }
+      }
+    const int sp[3] = {PA, PB, 1};
+    s_ax[t] = make_int4(ax[0] == 0 ? sp[0] : ax[0] == 1 ? sp[1] : sp[2],
+                        ax[1] == 0 ? sp[0] : ax[1] == 1 ? sp[1] : sp[2],
+                        ax[2] == 0 ? sp[0] : ax[2] == 1 ? sp[1] : sp[2],
+                        ax[0] == 0 ? 0 : ax[1] == 0 ? 1 : 2);
   }
+  // this thread's element of a tile along the physical axes (f, m, s), for each place
+  // of the logical a among them (its extent differs); a second one follows along s
+  const int ef0 = t & (TA - 1), em0 = (t >> LTA) & (TB - 1);
+  const int ef1 = t & (TB - 1), em1 = (t >> LTB) & (TA - 1);
+  const int em2 = (t >> LTB) & (TB - 1);
+  const int es01 = t >> (LTA + LTB), es2 = t >> (2 * LTB);
+  const long long nv2 = (long long)nv * nv;
   __syncthreads();
   const int nh = (no + 3) / 4;
   const int TT = nh * nh;                   // 4x4 tiles of (k, l)
@@ -1994,34 +2044,40 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
   const int ntiles = ta * tb * tc;
   for (int q = blockIdx.x; q < ntiles; q += gridDim.x) {
     const int a0 = TA * (q / (tb * tc)), b0 = TB * ((q / tc) % tb), c0 = TB * (q % tc);
+    if (t < no) {
+      s_tb[t] = off0 + (long long)a0 * st[0] + (long long)b0 * st[1] + (long long)c0 * st[2];
+      const int lim[3] = {min(TA, nv - a0), min(TB, nv - b0), min(TB, nv - c0)};
+      unsigned w = 0;
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+        w |= (unsigned)(have ? (ax[x] == 0 ? lim[0] : ax[x] == 1 ? lim[1] : lim[2]) : 0) << (8 * x);
+      s_lim[t] = w;
+    }
     __syncthreads();  // the previous tile's reads are done
     for (int r = 0; r < no; ++r) {
-      const int f = s_ax[r][0], m = s_ax[r][1];
-      // TA and TB are powers of two: the split of e by shifts and masks
-      const int lf = f == 0 ? LTA : LTB, lm = m == 0 ? LTA : LTB;
-      const int mf = (1 << lf) - 1, mm = (1 << lm) - 1;
-      const bool hv = s_have[r] != 0;
-      const long long base = s_off[r];
-      const int sa = s_st[r][0], sb = s_st[r][1], sc = s_st[r][2];
+      const int4 sx = s_ax[r];
+      const unsigned lim = s_lim[r];
+      const int ef = sx.w == 0 ? ef0 : ef1;
+      const int em = sx.w == 0 ? em0 : sx.w == 1 ? em1 : em2;
+      const int es = sx.w == 2 ? es2 : es01;
+      const int ds = sx.w == 2 ? 256 >> (2 * LTB) : 256 >> (LTA + LTB);
+      const bool in = ef < (int)(lim & 255u) && em < (int)((lim >> 8) & 255u);
+      long long o = s_tb[r] + ef + (long long)em * nv + (long long)es * nv2;
+      const unsigned sp = (unsigned)((r * TS + ef * sx.x + em * sx.y + es * sx.z) * (int)sizeof(T));
+      unsigned dx = (unsigned)__cvta_generic_to_shared(xs) + sp, dy = (unsigned)__cvta_generic_to_shared(ys) + sp;
 #pragma unroll
-      for (int e = t; e < NE; e += 256) {
-        const int ef = e & mf, em = (e >> lf) & mm, es = e >> (lf + lm);
-        const int la = f == 0 ? ef : m == 0 ? em : es;
-        const int lb = f == 1 ? ef : m == 1 ? em : es;
-        const int lc = f == 2 ? ef : m == 2 ? em : es;
-        const int a = a0 + la, b = b0 + lb, c = c0 + lc;
-        const bool ok = hv && a < nv && b < nv && c < nv;
-        const long long o = ok ? base + (long long)a * sa + (long long)b * sb + (long long)c * sc : 0;
-        const int sp = r * TS + la * PA + lb * PB + lc;
+      for (int g = 0; g < NE / 256; ++g) {
         // asynchronous global -> shared copies; a missing element is zero-filled
+        const bool ok = in && es + g * ds < (int)(lim >> 16);
+        const long long oo = ok ? o + (long long)(g * ds) * nv2 : 0;
         const unsigned nbytes = ok ? (unsigned)sizeof(T) : 0u;
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(
-                         (unsigned)__cvta_generic_to_shared(xs + sp)),
-                     "l"(X + o), "n"(sizeof(T)), "r"(nbytes)
+                         dx + (unsigned)(g * ds * sx.z * (int)sizeof(T))),
+                     "l"(X + oo), "n"(sizeof(T)), "r"(nbytes)
                      : "memory");
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(
-                         (unsigned)__cvta_generic_to_shared(ys + sp)),
-                     "l"(Y + o), "n"(sizeof(T)), "r"(nbytes)
+                         dy + (unsigned)(g * ds * sx.z * (int)sizeof(T))),
+                     "l"(Y + oo), "n"(sizeof(T)), "r"(nbytes)
                      : "memory");
       }
     }
@@ -2054,25 +2110,17 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += (double)p[x][y];
+        for (int y = 0; y < 4; ++y) acc[x][y] += to_f64(p[x][y]);
     }
   }
-  if (h >= H) return;
-#pragma unroll
-  for (int dk = 0; dk < 4; ++dk)
-#pragma unroll
-    for (int dl = 0; dl < 4; ++dl) {
-      const int kk = k0 + dk, ll = l0 + dl;
-      if (kk >= no || ll >= no || acc[dk][dl] == 0.0) continue;
-      atomicAdd(out + (kl ? kk * ldo + ll : ll * ldo + kk), wij * alpha * acc[dk][dl]);
-    }
+  pair_dots_add(smraw, acc, tile, h, TT, H, nh, no, out, ldo, kl, wij * alpha);
 }
 
 // Shared-memory bytes of pair_dots_*_kernel for no views.
 size_t pair_dots_smem(int no, bool f32) {
   const int TA = f32 ? 2 : 4, TB = f32 ? 16 : 8;
   const int TE = TA * (TB * (TB + 1) + 1), TS = (TE + 31) / 32 * 32 + 1;
-  return 2 * (size_t)no * TS * (f32 ? sizeof(float) : sizeof(double));
+  return std::max(2 * (size_t)no * TS * (f32 ? sizeof(float) : sizeof(double)), kPdRed);
 }
 
 // Tiles of the (a,b,c) cube swept by pair_dots_*_kernel.
@@ -2216,21 +2264,13 @@ __global__ void __launch_bounds__(256, 2) pair_dots_phys_kernel(
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += (double)p[x][y];
+        for (int y = 0; y < 4; ++y) acc[x][y] += to_f64(p[x][y]);
     }
   }
-  if (h >= H) return;
-#pragma unroll
-  for (int dk = 0; dk < 4; ++dk)
-#pragma unroll
-    for (int dl = 0; dl < 4; ++dl) {
-      const int kk = k0 + dk, ll = l0 + dl;
-      if (kk >= no || ll >= no || acc[dk][dl] == 0.0) continue;
-      atomicAdd(out + (kl ? kk * ldo + ll : ll * ldo + kk), wij * alpha * acc[dk][dl]);
-    }
+  pair_dots_add(smraw, acc, tile, h, TT, H, nh, no, out, ldo, kl, wij * alpha);
 }
 
-size_t pair_dots_phys_smem(int no) { return 2 * (size_t)no * kPdTS * sizeof(float); }
+size_t pair_dots_phys_smem(int no) { return std::max(2 * (size_t)no * kPdTS * sizeof(float), kPdRed); }
 
 __global__ void __launch_bounds__(256) pair_dots_f64_kernel(
     const double *__restrict__ X, const double *__restrict__ Y, const long long *__restrict__ voff,
