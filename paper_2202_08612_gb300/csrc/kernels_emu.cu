@@ -87,14 +87,17 @@ __device__ __forceinline__ int scale_exp(EmuScale s) { return (int)((s >> 52) & 
 // C = A B^T with M = N = K = 4096 and S = 5, slicing included: 2.64 ms, against
 // 8.26 ms with one launch of the split mode's kernel per digit degree (two of its
 // three products on zeros, and an FP64 reduction per output, pair and 1024 products).
-template <int S, int N>
+// AMN: A's rows are the contiguous index of its map (boxes of 64 rows x 32 K of
+// every slice, two per stage).
+template <int S, int N, bool AMN>
 __global__ void __launch_bounds__(320, 1)
     emu_gemm_kernel(const __grid_constant__ TcMaps maps, const TcItem *__restrict__ items,
                     const TcSeg *__restrict__ segs, int nitems, int stages, const EmuEpi epi,
                     int *__restrict__ status) {
   constexpr int NG = N / 16;  // 8-column groups per epilogue thread
   constexpr int A_SL = 128 * kRowB;         // bytes of one slice of A
-  constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
+  constexpr uint32_t IDESC =
+      (1u << 4) | (1u << 7) | (1u << 10) | (AMN ? 1u << 15 : 0u) | ((uint32_t)(128 >> 4) << 24);
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -149,7 +152,13 @@ __global__ void __launch_bounds__(320, 1)
           }
           const uint32_t st = smem_u32(smem + stage * stage_bytes), fb = full0 + 8 * stage;
           mbar_expect_tx(fb, (uint32_t)stage_bytes);
-          tma_load_5d(st, &maps.m[sg.amap], sg.ac[0] + kEmuKB * kc, sg.ac[1], sg.ac[2], sg.ac[3], 0, fb);
+          if constexpr (AMN) {
+            for (int h = 0; h < 2; ++h)
+              tma_load_5d(st + h * (S * A_SL / 2), &maps.m[sg.amap], sg.ac[1] + 64 * h,
+                          sg.ac[0] + kEmuKB * kc, sg.ac[2], sg.ac[3], 0, fb);
+          } else {
+            tma_load_5d(st, &maps.m[sg.amap], sg.ac[0] + kEmuKB * kc, sg.ac[1], sg.ac[2], sg.ac[3], 0, fb);
+          }
           tma_load_5d(st + S * A_SL, &maps.m[sg.bmap], sg.bc[0] + kEmuKB * kc, sg.bc[1], sg.bc[2],
                       sg.bc[3], 0, fb);
           last = (last & ~(1u << stage)) | (phase << stage);
@@ -197,7 +206,8 @@ __global__ void __launch_bounds__(320, 1)
           const bool last = q == s1 - 1 && kc == nk - 1;
           if (leader) {
             const uint32_t a0 = smem_u32(smem) + stage * stage_bytes;
-            const uint64_t ad = smem_desc64(a0), bd = smem_desc64(a0 + S * A_SL);
+            const uint64_t ad = AMN ? smem_desc_mn(a0, S * A_SL / 2) : smem_desc64(a0);
+            const uint64_t bd = smem_desc64(a0 + S * A_SL);
             const int steps = kc == nk - 1 && tail > 0 ? tail : kEmuKB / 16;
 #pragma unroll
             for (int kk = 0; kk < kEmuKB / 16; ++kk) {
@@ -210,7 +220,8 @@ __global__ void __launch_bounds__(320, 1)
 #pragma unroll
                   for (int c0 = 0; c0 < (S - d) * n; c0 += W) {
                     const int nn = (S - d) * n - c0 < W ? (S - d) * n - c0 : W;
-                    mma_bf16(tmem + (uint32_t)(d * n + c0), ad + (uint64_t)((d * A_SL + kk * 32) >> 4),
+                    constexpr int a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
+                    mma_bf16(tmem + (uint32_t)(d * n + c0), ad + (uint64_t)((d * a_slice + kk * a_step) >> 4),
                              bd + (uint64_t)((c0 * kRowB + kk * 32) >> 4), IDESC | ((uint32_t)(nn >> 3) << 17),
                              kk > 0 || d > 0 ? 1u : (cc > 0 ? 1u : 0u));
                   }
@@ -366,7 +377,7 @@ int emu_tile_width(long long n, int S) {
 
 bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long dims[4],
                     const unsigned long long strides[3], unsigned long long slice_bytes,
-                    const unsigned box[3], int S, std::string *err) {
+                    const unsigned box[3], int S, std::string *err, bool mn) {
   static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -381,10 +392,10 @@ bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long d
   }
   cuuint64_t gd[5] = {dims[0], dims[1], dims[2], dims[3], (cuuint64_t)S};
   cuuint64_t gs[4] = {strides[0], strides[1], strides[2], slice_bytes};
-  cuuint32_t bx[5] = {kEmuKB, box[0], box[1], box[2], (cuuint32_t)S};
+  cuuint32_t bx[5] = {mn ? 64u : (cuuint32_t)kEmuKB, mn ? (cuuint32_t)kEmuKB : box[0], box[1], box[2], (cuuint32_t)S};
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
   CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), gd, gs, bx, es,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, mn ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     *err = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
@@ -393,28 +404,31 @@ bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long d
   return true;
 }
 
-template <int S, int N>
+template <int S, int N, bool AMN = false>
 static cudaError_t launch_sn(const TcMaps &maps, const TcItem *items, const TcSeg *segs, int nitems,
                             const EmuEpi &epi, int *status, cudaStream_t st) {
   const int stage = S * (128 + epi.n) * kRowB;
   const int stages = std::max(2, std::min(6, (220 * 1024) / stage));
   const int smem = 1024 + stages * stage + 256;
-  cudaError_t e = cudaFuncSetAttribute(emu_gemm_kernel<S, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(emu_gemm_kernel<S, N, AMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  emu_gemm_kernel<S, N><<<std::min(nitems, 152), 320, smem, st>>>(maps, items, segs, nitems, stages, epi, status);
+  emu_gemm_kernel<S, N, AMN><<<std::min(nitems, 152), 320, smem, st>>>(maps, items, segs, nitems, stages, epi, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, const TcSeg *segs,
                             int nitems, const EmuEpi &epi, int *status, cudaStream_t st) {
   if (nitems <= 0) return cudaSuccess;
-  switch (S * 1000 + epi.n) {
+  switch (S * 1000 + epi.n + (epi.amn ? 100 : 0)) {
 #define EMU_CASE(s, n) \
   case s * 1000 + n: return launch_sn<s, n>(maps, items, segs, nitems, epi, status, st)
-    EMU_CASE(8, 16);
-    EMU_CASE(8, 32);
-    EMU_CASE(8, 48);
-    EMU_CASE(8, 64);
+#define EMU_CASE2(n)  \
+  EMU_CASE(8, n);     \
+  case 8100 + n: return launch_sn<8, n, true>(maps, items, segs, nitems, epi, status, st)
+    EMU_CASE2(16);
+    EMU_CASE2(32);
+    EMU_CASE2(48);
+    EMU_CASE2(64);
     EMU_CASE(2, 32);
     EMU_CASE(2, 80);
     EMU_CASE(3, 32);
@@ -426,6 +440,7 @@ cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, cons
     EMU_CASE(6, 32);
     EMU_CASE(6, 80);
 #undef EMU_CASE
+#undef EMU_CASE2
     default: return cudaErrorInvalidValue;
   }
 }

@@ -29,6 +29,7 @@ struct EmuEpi {
   long long s1, s2, sn;
   int lim1, lim2, nlim;
   double alpha;
+  int amn;          // as TcEpi::amn (S = 8)
   int n;            // columns of a tile (a multiple of 16, at most emu_max_cols)
   int ebias;        // power of two of the leading digit product: -12 (emu_digits), -14 (full leading digits)
   // scales: one per operand (sa, sb), or one exponent per output row and column
@@ -43,10 +44,11 @@ __host__ __device__ constexpr int emu_max_cols(int S) { return S >= 7 ? 64 : 80;
 int emu_tile_width(long long n, int S);
 
 // Tensor map of a digit operand over (K, dims1, dims2, dims3, slice); strides in
-// bytes for dims 1..3 and the slice.
+// bytes for dims 1..3 and the slice.  mn: dims[0] are the rows, dims[1] is K, for
+// boxes of 64 rows x kEmuKB.
 bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long dims[4],
                     const unsigned long long strides[3], unsigned long long slice_bytes,
-                    const unsigned box[3], int S, std::string *err);
+                    const unsigned box[3], int S, std::string *err, bool mn = false);
 
 cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, const TcSeg *segs,
                             int nitems, const EmuEpi &epi, int *status, cudaStream_t st);

@@ -156,17 +156,27 @@ __host__ __device__ __forceinline__ bool epi_rows_t(const TcEpi &epi) {
 // Loads of one pipeline stage for chunk kc of segment sg: A hi/lo (128 rows),
 // then the segment's B boxes (hi into the first BN rows' region, lo into the
 // second), box q at row q * qrows.  The barrier expects exactly these bytes.
+// amn: A comes as two boxes of 64 rows x 64 K with the rows contiguous.
 template <int BN>
 __device__ __forceinline__ void issue_stage(const TcMaps &maps, const TcSeg &sg, int kc,
-                                            unsigned char *st, uint32_t fb, int qrows) {
+                                            unsigned char *st, uint32_t fb, int qrows, int amn) {
   constexpr int A_BYTES = 128 * 128;
   constexpr int B_BYTES = BN * 128;
   const int nb = sg.nb > 1 ? sg.nb : 1;
   const int qb = qrows * 128;
   mbar_expect_tx(fb, 2 * A_BYTES + 2 * nb * qb);
   const int k = sg.ac[0] + 64 * kc, kb = sg.bc[0] + 64 * kc;
-  tma_load_4d(smem_u32(st), &maps.m[sg.amap], k, sg.ac[1], sg.ac[2], sg.ac[3], fb);
-  tma_load_4d(smem_u32(st + A_BYTES), &maps.m[sg.amap + 1], k, sg.ac[1], sg.ac[2], sg.ac[3], fb);
+  if (amn) {
+    for (int h = 0; h < 2; ++h) {
+      tma_load_4d(smem_u32(st + h * (A_BYTES / 2)), &maps.m[sg.amap], sg.ac[1] + 64 * h, k, sg.ac[2],
+                  sg.ac[3], fb);
+      tma_load_4d(smem_u32(st + A_BYTES + h * (A_BYTES / 2)), &maps.m[sg.amap + 1], sg.ac[1] + 64 * h, k,
+                  sg.ac[2], sg.ac[3], fb);
+    }
+  } else {
+    tma_load_4d(smem_u32(st), &maps.m[sg.amap], k, sg.ac[1], sg.ac[2], sg.ac[3], fb);
+    tma_load_4d(smem_u32(st + A_BYTES), &maps.m[sg.amap + 1], k, sg.ac[1], sg.ac[2], sg.ac[3], fb);
+  }
   for (int q = 0; q < nb; ++q) {
     const int c2 = q ? sg.bq[q - 1][0] : sg.bc[2], c3 = q ? sg.bq[q - 1][1] : sg.bc[3];
     tma_load_4d(smem_u32(st + 2 * A_BYTES + q * qb), &maps.m[sg.bmap], kb, sg.bc[1], c2, c3, fb);
@@ -185,13 +195,16 @@ __device__ __forceinline__ uint32_t idesc_n(uint32_t idesc, int n) {
 // address took as long as an MMA of 64 columns runs.
 template <int BN>
 __device__ __forceinline__ void issue_mmas(uint32_t acc, uint32_t stage_addr, uint32_t idesc, bool first,
-                                           int steps) {
+                                           int steps, int amn) {
   constexpr int A_BYTES = 128 * 128, B_BYTES = BN * 128;
   const uint64_t d = smem_desc(stage_addr);
+  // A with contiguous rows: 16 K elements are two groups of eight, 1024 bytes each
+  const uint64_t da = amn ? smem_desc_mn(stage_addr, A_BYTES / 2) : d;
+  const uint64_t step = amn ? 2048 >> 4 : 32 >> 4;
 #pragma unroll
   for (int kk = 0; kk < 4; ++kk) {
     if (kk >= steps) break;
-    const uint64_t ahi = d + (uint64_t)((kk * 32) >> 4), alo = d + (uint64_t)((A_BYTES + kk * 32) >> 4);
+    const uint64_t ahi = da + kk * step, alo = ahi + (uint64_t)(A_BYTES >> 4);
     const uint64_t bhi = d + (uint64_t)((2 * A_BYTES + kk * 32) >> 4);
     const uint64_t blo = d + (uint64_t)((2 * A_BYTES + B_BYTES + kk * 32) >> 4);
     mma_bf16(acc, ahi, bhi, idesc, kk > 0 ? 1u : (first ? 0u : 1u));
@@ -268,7 +281,7 @@ __global__ void __launch_bounds__(192, 1)
         }
         unsigned char *st = smem + stage * STAGE;
         const uint32_t fb = full0 + 8 * stage;
-        issue_stage<BN>(maps, sg, kc, st, fb, qrows);
+        issue_stage<BN>(maps, sg, kc, st, fb, qrows, epi.amn);
         ++issued;
         if (++stage == STAGES) {
           stage = 0;
@@ -296,7 +309,7 @@ __global__ void __launch_bounds__(192, 1)
   } else if (warp == 1) {
     // ---- MMA issuer: the warp waits together, one lane issues ----
     const bool leader = elect_one();
-    const uint32_t idesc = idesc_n(IDESC, ntile);
+    const uint32_t idesc = idesc_n(IDESC, ntile) | (uint32_t)epi.amn << 15;  // 15: A's rows contiguous
     int stage = 0;
     uint32_t phase = 0;
     int q = 0, left = seg[0].nk;  // segment and its chunks to go
@@ -309,7 +322,8 @@ __global__ void __launch_bounds__(192, 1)
         if (c + 1 < total) left = seg[++q].nk;
       }
       if (leader) {
-        issue_mmas<BN>(tmem, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0, steps);
+        issue_mmas<BN>(tmem, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0, steps,
+                       epi.amn);
         mma_commit(empty0 + 8 * stage);
       }
       __syncwarp();
@@ -442,7 +456,7 @@ __global__ void __launch_bounds__(192, 1)
           }
           unsigned char *st = smem + stage * STAGE;
           const uint32_t fb = full0 + 8 * stage;
-          issue_stage<BN>(maps, sg, kc, st, fb, qrows);
+          issue_stage<BN>(maps, sg, kc, st, fb, qrows, epi.amn);
           last[stage] = phase;
           pending[stage] = true;
           if (++stage == STAGES) {
@@ -466,7 +480,8 @@ __global__ void __launch_bounds__(192, 1)
       const int u = t & 1;
       const int total = items[i].chunks;
       const uint32_t acc = tmem + (uint32_t)(u * NCOLS);
-      const uint32_t idesc = idesc_n(IDESC, (items[i].nq > 1 ? items[i].nq : 1) * qrows);
+      const uint32_t idesc =
+          idesc_n(IDESC, (items[i].nq > 1 ? items[i].nq : 1) * qrows) | (uint32_t)epi.amn << 15;
       bool ok = __all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * u, ((uint32_t)(t >> 1) & 1u) ^ 1u, status,
                                                   epi.wait));
       const TcSeg *seg = segs + items[i].seg_begin;
@@ -492,7 +507,7 @@ __global__ void __launch_bounds__(192, 1)
         if (!ok) break;
         tc_fence_after();
         if (leader) {
-          issue_mmas<BN>(acc, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0, steps);
+          issue_mmas<BN>(acc, smem_u32(smem) + (uint32_t)(stage * STAGE), idesc, c == 0, steps, epi.amn);
           mma_commit(empty0 + 8 * stage);
         }
         __syncwarp();

@@ -59,6 +59,7 @@ struct TcEpi {
   int lim1, lim2, nlim;
   float alpha;
   int qw;       // columns per group of a grouped tile (0: one group of the launch's BN)
+  int amn;      // 1: A is read with its rows contiguous (maps over (row, K, -, block))
   // clock limit of the pipeline's progress waits (0: kTcWaitDefault).  The
   // drain waits (copies and MMAs already issued) always use kTcWaitDefault.
   long long wait;

@@ -1087,6 +1087,7 @@ void tc_launch(mlcc3_ctx *c, const char *site, int BN, const TcMaps &maps, const
     x.nlim = epi.nlim;
     x.alpha = (double)epi.alpha;
     x.n = BN;
+    x.amn = epi.amn;
     x.ebias = -12;
     x.sa = A.scale;
     x.sb = B.scale;
@@ -1122,6 +1123,7 @@ TcEpi make_epi(void *out, int mode, int R2, long long s1, long long s2, long lon
   e.nlim = (int)nlim;
   e.alpha = (float)alpha;
   e.qw = 0;
+  e.amn = 0;
   e.wait = 0;
   return e;
 }
@@ -1633,10 +1635,10 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
             2.0 * (double)s.NV * (double)s.nv * (double)(s.nv * s.nv) * (double)ords.size(), *ops[0], x0);
 }
 
-// hi/lo buffers of layout L of the triples array X (chunk_nb blocks), converted
-// at most once per write of X: L = 0..2 is XL_L, L = 3..5 is R_{L-3}.  FP64 mode:
-// the digit slices, three arrays kept (96 bytes per element each).
-void tri_layout(mlcc3_ctx *c, const double *X, int L, SplitOp &op) {
+// hi/lo buffers of layout XL_k of the triples array X (chunk_nb blocks), converted
+// at most once per write of X.  FP64 mode: the digit slices, three arrays kept (48
+// bytes per element each).
+void tri_layout(mlcc3_ctx *c, const double *X, int k, SplitOp &op) {
   S s(c);
   const unsigned long long g = c->gen_of(X);
   const int slots = c->emu ? 3 : 4;
@@ -1655,59 +1657,41 @@ void tri_layout(mlcc3_ctx *c, const double *X, int L, SplitOp &op) {
   }
   mlcc3_ctx::TriSlot &ts = c->tri[q];
   ts.tick = ++c->tri_tick;
-  const std::string base = "tri" + std::to_string(q) + ":" + std::to_string(L);
+  const std::string base = "tri" + std::to_string(q) + ":" + std::to_string(k);
   const long long nb = c->chunk_nb;
   const long long cs[3] = {s.nv * s.nv, s.nv, 1};
-  const int k = L % 3, a = k == 0 ? 1 : 0, b = k == 2 ? 1 : 2;
-  const bool xl = L < 3;
-  const long long Kp = kpad(c, xl ? s.nv * s.nv : s.nv);
-  const size_t n = (size_t)nb * (size_t)(xl ? s.nv : s.nv * s.nv) * (size_t)Kp;
+  const int a = k == 0 ? 1 : 0, b = k == 2 ? 1 : 2, nv = (int)s.nv;
+  const long long Kp = kpad(c, s.nv * s.nv);
+  const bool convert = !(ts.mask & (1u << k));
+  ts.mask |= 1u << k;
   if (c->emu) {
-    const int nv = (int)s.nv;
-    const EmuView v = xl ? EmuView{X, (int)nb, 1, nv, nv, nv * nv, nv, s.nv3, 0, 0, cs[k], cs[a], cs[b]}
-                         : EmuView{X, (int)nb, 1, nv * nv, nv, nv, 1, s.nv3, 0, cs[a], cs[b], cs[k], 0};
-    const std::string key = "tri" + std::to_string(q) + ":" + std::to_string(L);
-    if (!(ts.mask & (1u << L))) {
-      ts.mask |= 1u << L;
-      make_digits(c, op, key, v, Kp, false, "tri" + std::to_string(q));
+    const EmuView v{X, (int)nb, 1, nv, nv, nv * nv, nv, s.nv3, 0, 0, cs[k], cs[a], cs[b]};
+    if (convert) {
+      make_digits(c, op, base, v, Kp, false, "tri" + std::to_string(q));
     } else {
       op.S = kEmuSlices;
       op.slice = (long long)v.Z * v.R * Kp;
       op.scale = scale_of(c, "tri" + std::to_string(q));
-      op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuSlices * 2);
+      op.hi = c->raw("digits:" + base, (size_t)op.slice * kEmuSlices * 2);
       op.lo = nullptr;
     }
     return;
   }
-  void *hi = c->raw(base + ":hi", n * 2), *lo = c->raw(base + ":lo", n * 2);
-  op.hi = hi;
-  op.lo = lo;
-  if (!(ts.mask & (1u << L))) {
-    ts.mask |= 1u << L;
-    __nv_bfloat16 *h = static_cast<__nv_bfloat16 *>(hi), *l = static_cast<__nv_bfloat16 *>(lo);
-    const int nv = (int)s.nv;
-    if (L == 2 || L == 3 || L == 4) {
-      // the layouts whose K index is not the source's contiguous one: tiled transposes
-      // XL2: [u][x2][(x0 x1)] ; R0: [u][(x1 x2)][x0] ; R1: [u x0][x2][x1]
-      const long long B = L == 4 ? nb * s.nv : nb;
-      const int R = L == 2 ? nv * nv : nv, C = L == 3 ? nv * nv : nv;
-      const long long sb = L == 4 ? s.nv * s.nv : s.nv3;
-      const long long sr = L == 2 ? s.nv : L == 3 ? s.nv * s.nv : s.nv;
-      const long long db = (long long)C * Kp;
-      c->launch("split_transpose_kernel", 0.0, [&] {
-        check_cuda(split_transpose(X, h, l, B, R, (int)Kp, C, sb, sr, db, Kp, c->stream,
-                                   c->is_tri32(X)), "split_transpose");
-      });
-    } else if (xl)
-      c->launch("split_bf16_k2_kernel", 0.0, [&] {
-        check_cuda(split_bf16_k2(X, h, l, nb, s.nv, s.nv, s.nv, Kp, s.nv3, cs[k], cs[a], cs[b], 1.0,
-                                 c->stream, c->is_tri32(X)), "split_bf16_k2");
-      });
-    else
-      c->launch("split_bf16_kernel", 0.0, [&] {
-        check_cuda(split_bf16(X, h, l, nb, s.nv, s.nv, s.nv, Kp, s.nv3, cs[a], cs[b], cs[k], 1.0,
-                              c->stream, c->is_tri32(X)), "split_bf16");
-      });
+  const size_t n = (size_t)nb * (size_t)s.nv * (size_t)Kp;
+  op.hi = c->raw(base + ":hi", n * 2);
+  op.lo = c->raw(base + ":lo", n * 2);
+  if (!convert) return;
+  __nv_bfloat16 *h = static_cast<__nv_bfloat16 *>(op.hi), *l = static_cast<__nv_bfloat16 *>(op.lo);
+  if (k == 2) {  // [u][x2][(x0 x1)]: the K index is not the source's contiguous one, tiled transpose
+    c->launch("split_transpose_kernel", 0.0, [&] {
+      check_cuda(split_transpose(X, h, l, nb, nv * nv, (int)Kp, nv, s.nv3, s.nv, s.nv * Kp, Kp, c->stream,
+                                 c->is_tri32(X)), "split_transpose");
+    });
+  } else {
+    c->launch("split_bf16_k2_kernel", 0.0, [&] {
+      check_cuda(split_bf16_k2(X, h, l, nb, s.nv, s.nv, s.nv, Kp, s.nv3, cs[k], cs[a], cs[b], 1.0,
+                               c->stream, c->is_tri32(X)), "split_bf16_k2");
+    });
   }
 }
 
@@ -1738,16 +1722,25 @@ SplitOp &layout_XL(mlcc3_ctx *c, const std::string &key, const double *X, int k,
   return op;
 }
 
-// R_k: K = canonical position k, rows = the other two, flattened (smaller, larger).
-SplitOp &layout_R(mlcc3_ctx *c, const std::string &key, const double *X, int k) {
+// The same XL_k read the other way round: rows = the flattened pair of the other two
+// positions (contiguous), K = canonical position k.  The tensor cores take such
+// an operand as it lies, so no layouts with K = k contiguous are made (they were
+// half of the conversions of a triples array).
+SplitOp &layout_XM(mlcc3_ctx *c, const std::string &key, const double *X, int k) {
   S s(c);
   SplitOp &op = c->splits[key];
-  tri_layout(c, X, 3 + k, op);
-  const unsigned long long Kp = (unsigned long long)kpad(c, s.nv), nv = s.nv;
-  const unsigned long long dims[4] = {Kp, nv * nv, 1ULL, (unsigned long long)c->chunk_nb};
-  const unsigned long long str[3] = {Kp * 2, Kp * 2 * nv * nv, Kp * 2 * nv * nv};
-  const unsigned bx[4] = {64, 128, 1, 1};
-  encode_split(op, key, dims, str, bx);
+  tri_layout(c, X, k, op);
+  const unsigned long long rb = (unsigned long long)kpad(c, s.nv * s.nv) * 2, nv = s.nv;
+  const unsigned long long dims[4] = {nv * nv, nv, 1ULL, (unsigned long long)c->chunk_nb};
+  const unsigned long long str[3] = {rb, rb * nv, rb * nv};
+  const unsigned bx[4] = {64, 64, 1, 1};
+  std::string err;
+  if (op.S > 0) {
+    if (!emu_encode_map(&op.mhi, op.hi, dims, str, (unsigned long long)op.slice * 2, bx + 1, op.S, &err, true))
+      throw Error{MLCC3_ERR_CUDA, "tensor map " + key + ": " + err};
+  } else {
+    encode_split(op, key, dims, str, bx);
+  }
   return op;
 }
 
@@ -1755,8 +1748,8 @@ int occ_of(const Ord &o, int pos) { return pos == 0 ? o.p : pos == 1 ? o.q : o.r
 
 // out[occ_g][pair][n] += coef sum_{orderings, grouped by occupied position g}
 //                        sum_{x at view position vk} X_{pqr}[..] * B_{occ b1, occ b2}[n][x]
-// Rows: the two view positions other than vk, as pair tiles read from R_{s_vk}
-// (K = canonical position s_vk).  B: a split operand [occ b1][occ b2][n][K]
+// Rows: the two view positions other than vk, flattened, K = canonical position s_vk,
+// from XL_{s_vk} read with its rows contiguous (layout_XM).  B: a split operand [occ b1][occ b2][n][K]
 // (map dims (K, n, occ b2, occ b1)) with box BN = tile_width(nN).
 // out address = out_off(occ_g) + view-pair strides (Sp1, Sp2) + n * Sn.
 void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const SplitOp &B, long long nN,
@@ -1769,7 +1762,7 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (int k = 0; k < 3; ++k) {
-    SplitOp &r = layout_R(c, xkey + ":R" + std::to_string(k), X, k);
+    SplitOp &r = layout_XM(c, xkey + ":XM" + std::to_string(k), X, k);
     maps.m[2 * k] = r.mhi;
     maps.m[2 * k + 1] = r.mlo;
   }
@@ -1801,12 +1794,13 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
               pl.drop_empty_last();
             }
     }, kcap(c));
-    // rows of R are (smaller, larger) canonical positions: the view pair in
+    // rows of XM are (smaller, larger) canonical positions: the view pair in
     // order (cls 0) or swapped (cls 1)
     TcEpi epi = make_epi(out, 2, (int)s.nv, cls == 0 ? Sp1 : Sp2, cls == 0 ? Sp2 : Sp1, Sn, s.nv, s.nv, nN,
                          coef, 1);
+    epi.amn = 1;
     tc_launch(c, "pair", BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)nN * (double)ords.size() / 2.0,
-              c->splits.at(xkey + ":R0"), B);
+              c->splits.at(xkey + ":XM0"), B);
   }
 }
 
