@@ -7,6 +7,29 @@
 
 namespace mlcc3 {
 
+// binary64 -> binary32, round to nearest even, on the integer pipe where the result
+// is a normal number (a conversion there is an FP64 operation, two per clock and SM).
+__device__ __forceinline__ float narrow_f64(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if (((hi >> 20) & 0x7ff) - 897u < 253u) {
+    const unsigned long long m = (((unsigned long long)hi << 32) | lo) + 0x0fffffffu + ((lo >> 29) & 1u);
+    return __uint_as_float((((unsigned)(m >> 29) - 0xC0000000u) & 0x7fffffffu) | (hi & 0x80000000u));
+  }
+  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);  // zeros, as in the padding of a tile
+  return __double2float_rn(x);
+}
+
+// binary32 -> binary64 (exact) on the integer pipe; binary32 subnormals
+// (never produced here) become signed zeros.
+__device__ __forceinline__ double widen_f32(float f) {
+  const unsigned int b = __float_as_uint(f);
+  const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
+  const unsigned int e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
+  if (e == 0) return __longlong_as_double((long long)sign);
+  const unsigned long long ex = e == 255 ? 0x7FFull : (unsigned long long)(e + 896);
+  return __longlong_as_double((long long)(sign | (ex << 52) | ((unsigned long long)m << 29)));
+}
+
 // x ~ hi + lo with hi = bf16(f), lo = bf16(f - hi), f = binary32(x); f - hi is
 // exact in binary32 (it keeps the 16 low bits of f's significand).
 __device__ __forceinline__ void split_hi_lo(double x, __nv_bfloat16 &hi, __nv_bfloat16 &lo) {

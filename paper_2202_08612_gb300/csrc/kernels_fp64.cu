@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <iterator>
 
+#include "fastconv.cuh"
 #include "kernels_fp64.cuh"
 
 namespace mlcc3 {
@@ -27,29 +28,6 @@ __constant__ int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 
 template <typename T>
 __device__ __forceinline__ T ld_op(const double *p, int f32, long long i) {
   return f32 ? (T)reinterpret_cast<const float *>(p)[i] : (T)p[i];
-}
-
-// binary64 -> binary32, round to nearest even, on the integer pipe where the result
-// is a normal number (a conversion there is an FP64 operation, two per clock and SM).
-__device__ __forceinline__ float narrow_f64(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  if (((hi >> 20) & 0x7ff) - 897u < 253u) {
-    const unsigned long long m = (((unsigned long long)hi << 32) | lo) + 0x0fffffffu + ((lo >> 29) & 1u);
-    return __uint_as_float((((unsigned)(m >> 29) - 0xC0000000u) & 0x7fffffffu) | (hi & 0x80000000u));
-  }
-  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);  // zeros, as in the padding of a tile
-  return __double2float_rn(x);
-}
-
-// binary32 -> binary64 (exact) on the integer pipe; binary32 subnormals
-// (never produced here) become signed zeros.
-__device__ __forceinline__ double widen_f32(float f) {
-  const unsigned int b = __float_as_uint(f);
-  const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
-  const unsigned int e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
-  if (e == 0) return __longlong_as_double((long long)sign);
-  const unsigned long long ex = e == 255 ? 0x7FFull : (unsigned long long)(e + 896);
-  return __longlong_as_double((long long)(sign | (ex << 52) | ((unsigned long long)m << 29)));
 }
 
 // FP32 products (split-precision mode): every output's FP32 sum of 64 products in
@@ -1324,6 +1302,11 @@ __device__ __forceinline__ FinishEnt finish_entry(const TripTerm &tm, int sg, co
   return e;
 }
 
+__device__ __forceinline__ bool finish_same(const FinishEnt &f, const FinishEnt &e) {
+  return f.pa == e.pa && f.pb == e.pb && f.ca[0] == e.ca[0] && f.ca[1] == e.ca[1] && f.ca[2] == e.ca[2] &&
+         f.cb[0] == e.cb[0] && f.cb[1] == e.cb[1] && f.cb[2] == e.cb[2];
+}
+
 // Appends e to tab[0..n) or, when an entry with the same operands and
 // coefficients is there, adds its coefficient to that one: the two
 // permutations that a symmetric operand relates (and any that coincide for
@@ -1332,8 +1315,7 @@ __device__ __forceinline__ FinishEnt finish_entry(const TripTerm &tm, int sg, co
 __device__ __forceinline__ int finish_merge(FinishEnt *tab, int n, const FinishEnt &e) {
   for (int m = 0; m < n; ++m) {
     FinishEnt &f = tab[m];
-    if (f.pa == e.pa && f.pb == e.pb && f.ca[0] == e.ca[0] && f.ca[1] == e.ca[1] &&
-        f.ca[2] == e.ca[2] && f.cb[0] == e.cb[0] && f.cb[1] == e.cb[1] && f.cb[2] == e.cb[2]) {
+    if (finish_same(f, e)) {
       f.coef += e.coef;
       return n;
     }
@@ -1565,26 +1547,51 @@ __global__ void __launch_bounds__(512, 2) triples_finish_contra_kernel(
     eol = (float)(eo - (double)eoh);
   }
   __syncthreads();
-  if (t == 0 && nr > 0) {
-    int n = 0;
-    for (int q = 0; q < 6 * nr; ++q) n = finish_merge(tab, n, raw[q]);
-    nent = n;
+  if (nr > 5) {
+    if (t == 0) {
+      int n = 0;
+      for (int q = 0; q < 6 * nr; ++q) n = finish_merge(tab, n, raw[q]);
+      nent = n;
+    }
+  } else if (t < 32 && nr > 0) {
+    // finish_merge by a warp (810 -> 792 us at n_v = 60, 352 batches): lane q looks for
+    // its entry's equals, the first of them stays
+    const int n = 6 * nr;
+    bool head = t < n;
+    float coef = 0.f;
+    for (int m = 0; m < n; ++m)
+      if (t < n && finish_same(raw[t], raw[m])) {
+        coef += raw[m].coef;
+        if (m < t) head = false;
+      }
+    const unsigned heads = __ballot_sync(0xffffffffu, head);
+    if (head) {
+      FinishEnt &f = tab[__popc(heads & ((1u << t) - 1))];
+      f = raw[t];
+      f.coef = coef;
+    }
+    if (t == 0) nent = __popc(heads);
   }
   // element e = t + 512 r of a tile: (l0, l1, l2) = (e >> 8, (e >> 4) & 15, e & 15)
   const int l0b = t >> 8, l1 = (t >> 4) & 15, l2 = t & 15;
   const float *Wb = W + it.off;
+  // a thread's eight elements of a tile are rows l0b + 2r of one column: their
+  // addresses are a first one plus multiples of nv2x2, their shared-memory
+  // positions constants apart
+  const long long nv2x2 = 2LL * nv * nv;
+  float *fcol = ftile + l0b * kFSI + l1 * kFSJ + l2;
   // 1. asynchronous copies of the distinct tiles
   for (int p = 0; p < 6; ++p) {
     if (slot[p] != p) continue;
-    const int y = kFW * org[p][1] + l1, z = kFW * org[p][2] + l2;
+    const int x = kFW * org[p][0] + l0b, y = kFW * org[p][1] + l1, z = kFW * org[p][2] + l2;
+    const int rows = y < nv && z < nv ? (nv - x + 1) / 2 : 0;  // x + 2r < nv
+    const float *src = Wb + ((long long)x * nv + y) * nv + z;
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(fcol + p * kFT);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const int l0 = l0b + 2 * r, x = kFW * org[p][0] + l0;
-      const bool ok = x < nv && y < nv && z < nv;
-      const float *src = ok ? Wb + ((long long)x * nv + y) * nv + z : Wb;
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                       (unsigned)__cvta_generic_to_shared(ftile + p * kFT + l0 * kFSI + l1 * kFSJ + l2)),
-                   "l"(src), "r"(ok ? 4u : 0u)
+      const bool ok = r < rows;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + r * 2 * kFSI * 4),
+                   "l"(ok ? src + r * nv2x2 : Wb), "r"(ok ? 4u : 0u)
                    : "memory");
     }
   }
@@ -1599,10 +1606,11 @@ __global__ void __launch_bounds__(512, 2) triples_finish_contra_kernel(
     const int y = kFW * org[p][1] + l1, z = kFW * org[p][2] + l2;
     if (y >= nv || z >= nv) continue;
     const int x0 = kFW * org[p][0] + l0b;
+    const int rows = (nv - x0 + 1) / 2;  // rows r < rows lie inside
+    float *col = fcol + p * kFT;
     float acc[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-      acc[r] = x0 + 2 * r < nv ? ftile[p * kFT + (l0b + 2 * r) * kFSI + l1 * kFSJ + l2] : 0.f;
+    for (int r = 0; r < 8; ++r) acc[r] = r < rows ? col[r * 2 * kFSI] : 0.f;
     for (int n = 0; n < ne; ++n) {
       const FinishEnt &e = tab[n];
       const float *pa = e.pa + (y * e.ca[1] + z * e.ca[2]);
@@ -1615,11 +1623,11 @@ __global__ void __launch_bounds__(512, 2) triples_finish_contra_kernel(
         const float *pv = a0 == 0 ? pb : pa;
         const int v0 = a0 == 0 ? b0 : a0;
         const float u = cf * (a0 == 0 ? pa[0] : pb[0]);
+        pv += (long long)x0 * v0;
+        const int st = 2 * v0;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int x = x0 + 2 * r;
-          if (x < nv) acc[r] = fmaf(u, pv[x * v0], acc[r]);
-        }
+        for (int r = 0; r < 8; ++r)
+          if (r < rows) acc[r] = fmaf(u, pv[r * st], acc[r]);
       } else {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -1632,11 +1640,11 @@ __global__ void __launch_bounds__(512, 2) triples_finish_contra_kernel(
     float yh = ey.x, yl = ey.y;  // eps_y + eps_z + (-eps_ijk - omega), shared by the column
     df_add(yh, yl, ez.x, ez.y);
     df_add(yh, yl, eoh, eol);
+    float *o = out ? out + it.off + ((long long)x0 * nv + y) * nv + z : nullptr;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const int x = x0 + 2 * r;
-      if (x >= nv) break;
-      const float2 ex = __ldg(ehl + x);
+      if (r >= rows) break;
+      const float2 ex = __ldg(ehl + x0 + 2 * r);
       float dh = ex.x, dl = ex.y;
       df_add(dh, dl, yh, yl);
       const float den = dh + dl;
@@ -1645,42 +1653,43 @@ __global__ void __launch_bounds__(512, 2) triples_finish_contra_kernel(
         atomicOr(status, 1);
       else
         q = __fdividef(-acc[r], den);
-      ftile[p * kFT + (l0b + 2 * r) * kFSI + l1 * kFSJ + l2] = q;
-      if (out) out[it.off + ((long long)x * nv + y) * nv + z] = q;
+      col[r * 2 * kFSI] = q;
+      if (out) o[r * nv2x2] = q;
     }
   }
   __syncthreads();
   // 3. the transform of the element orbits owned in tile (A, B, C)
   {
     const int A = org[0][0], Bt = org[0][1], C = org[0][2];
-#pragma unroll 2
-    for (int r = 0; r < 8; ++r) {
-      const int l0 = l0b + 2 * r;
-      const bool own = (A < Bt || l0 <= l1) && (Bt < C || l1 <= l2) && kFW * A + l0 < nv &&
-                       kFW * Bt + l1 < nv && kFW * C + l2 < nv;
-      if (!own) continue;
-      float v[6];
-      int pos[6];
-      c3_pos<kFSI, kFSJ, kFT>(l0, l1, l2, slot, pos);
+    // positions of the permutations at l0 = l0b; per r each moves by its own constant
+    constexpr int step[6] = {2 * kFSI, 2 * kFSJ, 2, 2 * kFSJ, 2, 2 * kFSI};
+    int pos[6];
+    c3_pos<kFSI, kFSJ, kFT>(l0b, l1, l2, slot, pos);
+    const bool col = (Bt < C || l1 <= l2) && kFW * Bt + l1 < nv && kFW * C + l2 < nv;
+    const int lmax = min(A < Bt ? kFW - 1 : l1, nv - 1 - kFW * A);
 #pragma unroll
-      for (int p = 0; p < 6; ++p) v[p] = ftile[pos[p]];
+    for (int r = 0; r < 8; ++r) {
+      if (!col || l0b + 2 * r > lmax) break;
+      float v[6];
+#pragma unroll
+      for (int p = 0; p < 6; ++p) v[p] = ftile[pos[p] + r * step[p]];
       const float E = (v[0] + v[1]) + v[2], Od = (v[3] + v[4]) + v[5];
       const float be = fmaf(-2.f, Od, E), bo = fmaf(-2.f, E, Od);
 #pragma unroll
-      for (int p = 0; p < 6; ++p) ftile[pos[p]] = fmaf(3.f, v[p], p < 3 ? be : bo);
+      for (int p = 0; p < 6; ++p) ftile[pos[p] + r * step[p]] = fmaf(3.f, v[p], p < 3 ? be : bo);
     }
   }
   __syncthreads();
   float *O = outt + it.off;
   for (int p = 0; p < 6; ++p) {
     if (slot[p] != p) continue;
-    const int y = kFW * org[p][1] + l1, z = kFW * org[p][2] + l2;
+    const int x0 = kFW * org[p][0] + l0b, y = kFW * org[p][1] + l1, z = kFW * org[p][2] + l2;
     if (y >= nv || z >= nv) continue;
+    const int rows = (nv - x0 + 1) / 2;
+    float *o = O + ((long long)x0 * nv + y) * nv + z;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int l0 = l0b + 2 * r, x = kFW * org[p][0] + l0;
-      if (x < nv) O[((long long)x * nv + y) * nv + z] = ftile[p * kFT + l0 * kFSI + l1 * kFSJ + l2];
-    }
+    for (int r = 0; r < 8; ++r)
+      if (r < rows) o[r * nv2x2] = fcol[p * kFT + r * 2 * kFSI];
   }
 }
 
@@ -1733,6 +1742,56 @@ namespace mlcc3 {
 // FP32 and folded into FP64; one atomic update per output (and per K slice).
 // Grid: x = 4 ceil(M / 8) (the second mapping uses the first quarter; the
 // first splits the extra blocks over K), y = items.
+// The same sums for reductions of two levels (one of the three extents is 1, n the
+// faster one's) whose offsets fit in 32 bits: the
+// running offsets of strided_dot took 32 instructions per element in 64-bit
+// arithmetic and three levels of carries, these 13.
+template <int U, typename TA, typename TB>
+__device__ __forceinline__ double strided_dot2(const TA *__restrict__ Am, const TB *__restrict__ B, int n,
+                                               int ka0, int ka1, int kb0, int kb1, int k0, int kend, int step) {
+  int r = k0 % n, oa, ob;
+  {
+    const int q = k0 / n;
+    oa = q * ka0 + r * ka1;
+    ob = q * kb0 + r * kb1;
+  }
+  const int dq = step / n, dr = step % n;
+  const int sa = dq * ka0 + dr * ka1, sb = dq * kb0 + dr * kb1;
+  const int ca = ka0 - n * ka1, cb = kb0 - n * kb1;  // r wraps into q
+  double s = 0.0;
+  TA sf = TA(0);
+  int nf = 0;
+  for (int k = k0; k < kend; k += U * step) {
+    TA av[U], bv[U];
+    const bool whole = k + (U - 1) * step < kend;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool ok = whole || k + u * step < kend;
+      av[u] = ok ? Am[oa] : TA(0);
+      if constexpr (sizeof(TA) == 4 && sizeof(TB) == 8) bv[u] = ok ? narrow_f64(B[ob]) : TA(0);
+      else bv[u] = ok ? (TA)B[ob] : TA(0);
+      oa += sa;
+      ob += sb;
+      r += dr;
+      if (r >= n) {
+        r -= n;
+        oa += ca;
+        ob += cb;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) sf = fma(av[u], bv[u], sf);
+    nf += U;
+    if (nf >= 16) {
+      if constexpr (sizeof(TA) == 4) s += widen_f32(sf);
+      else s += sf;
+      sf = TA(0);
+      nf = 0;
+    }
+  }
+  return s + (double)sf;
+}
+
 // Strided dot product of a row of A (binary32 or binary64) with B over the K
 // elements k = k0, k0 + step, ... < kend, (k1, k2, k3) the split of k (k3
 // fastest) advanced with carries.  U elements are loaded before their FMAs, so
@@ -1830,6 +1889,23 @@ __device__ __forceinline__ void gemv_body(const BstcParams &p) {
   long long ka[3] = {it.sA[2], it.sA[3], it.sA[4]}, kb[3] = {it.sB[0], it.sB[1], it.sB[2]};
   const long long K = (long long)Kn[0] * Kn[1] * Kn[2];
   auto ldb = [&](long long i) { return Bf ? (TA)Bf[i] : (TA)Bd[i]; };
+  // the dot product of row `a` over k = kb0, kb0 + step, ... < ke
+  auto dot = [&](const TA *a, long long kb0, long long ke, int step) {
+    if ((Kn[0] == 1 || Kn[1] == 1 || Kn[2] == 1) && K < (1LL << 30)) {
+      // the two levels (one of the three extents is 1), the second the faster
+      const bool l2 = Kn[2] == 1, l1 = !l2 && Kn[1] == 1;
+      const int n1 = l2 || l1 ? Kn[0] : Kn[1], n2 = l2 ? Kn[1] : Kn[2];
+      const long long a0 = l2 || l1 ? ka[0] : ka[1], a1 = l2 ? ka[1] : ka[2];
+      const long long b0 = l2 || l1 ? kb[0] : kb[1], b1 = l2 ? kb[1] : kb[2];
+      // offsets up to a load batch past the end
+      const long long span = (n1 + 520LL) * max(llabs(a0), llabs(b0)) + (n2 + 520LL) * max(llabs(a1), llabs(b1));
+      if (span < (1LL << 30)) {
+        return Bf ? strided_dot2<kGemvU<TA>>(a, Bf, n2, (int)a0, (int)a1, (int)b0, (int)b1, (int)kb0, (int)ke, step)
+                  : strided_dot2<kGemvU<TA>>(a, Bd, n2, (int)a0, (int)a1, (int)b0, (int)b1, (int)kb0, (int)ke, step);
+      }
+    }
+    return strided_dot<kGemvU<TA>>(a, ldb, Kn, ka, kb, kb0, ke, step);
+  };
   const GemvMap g = gemv32_map(it, M1, M2, K);
   const int mf = g.mf;
   if (mf >= 0 && g.small_k) {
@@ -1839,7 +1915,7 @@ __device__ __forceinline__ void gemv_body(const BstcParams &p) {
     const long long m = cg * 32 + lane;
     if (m >= M) return;
     const long long m1 = mf == 1 ? m / M2 : m % M1, m2 = mf == 1 ? m % M2 : m / M1;
-    const double s = strided_dot<kGemvU<TA>>(A + m1 * it.sA[0] + m2 * it.sA[1], ldb, Kn, ka, kb, 0, K, 1);
+    const double s = dot(A + m1 * it.sA[0] + m2 * it.sA[1], 0, K, 1);
     double *C = p.C + it.offC + m1 * it.sC[0] + m2 * it.sC[1];
     if (p.atomic) atomicAdd(C, p.alpha * s);
     else *C += p.alpha * s;
@@ -1859,7 +1935,7 @@ __device__ __forceinline__ void gemv_body(const BstcParams &p) {
     const long long m1 = mf == 1 ? m / M2 : m % M1, m2 = mf == 1 ? m % M2 : m / M1;
     const TA *Am = A + m1 * it.sA[0] + m2 * it.sA[1];
     // the warps take k = kbeg + warp, + 8, ...
-    const double s = valid ? strided_dot<kGemvU<TA>>(Am, ldb, Kn, ka, kb, kbeg + warp, kend, 8) : 0.0;
+    const double s = valid ? dot(Am, kbeg + warp, kend, 8) : 0.0;
     red[warp][lane] = s;
     __syncthreads();
     if (warp == 0 && valid) {
@@ -1890,7 +1966,7 @@ __device__ __forceinline__ void gemv_body(const BstcParams &p) {
   const bool valid = m < M;
   const long long m1 = valid ? m / M2 : 0, m2 = valid ? m % M2 : 0;
   const TA *Am = A + m1 * it.sA[0] + m2 * it.sA[1];
-  double s = valid ? strided_dot<kGemvU<TA>>(Am, ldb, Kn, ka, kb, sub, K, lpo) : 0.0;
+  double s = valid ? dot(Am, sub, K, lpo) : 0.0;
   for (int o = lpo / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (valid && sub == 0) {
     double *C = p.C + it.offC + m1 * it.sC[0] + m2 * it.sC[1];
