@@ -11,15 +11,59 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
 #include "kernels_emu.cuh"
 #include "mlcc3.h"
+#include "workpool.cuh"
 
 namespace mlcc3 {
 
 void set_last_error(const std::string &msg);
+
+namespace {
+constexpr int kMaxDev = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[kMaxDev] = {};
+}  // namespace
+
+cudaError_t work_alloc(void **p, size_t bytes, cudaStream_t st) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    if (!g_pool[dev]) {
+      cudaMemPoolProps props{};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      if ((e = cudaMemPoolCreate(&g_pool[dev], &props)) != cudaSuccess) {
+        g_pool[dev] = nullptr;
+        return e;
+      }
+      uint64_t keep = kWorkKeep;
+      cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    pool = g_pool[dev];
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
+void work_free(void *p, cudaStream_t st) {
+  if (p) cudaFreeAsync(p, st);
+}
+
+void work_trim() {
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  for (cudaMemPool_t pool : g_pool)
+    if (pool) cudaMemPoolTrimTo(pool, 0);
+}
 
 // Row r of X (one block): its exponent e[r], |X[r][k]| < 2^e[r] (0 for a zero
 // row), and its s digit slices: q = X[r][k] 2^(8s - 1 - e[r]) rounded to nearest
@@ -101,8 +145,8 @@ using namespace mlcc3;
 
 // C = A B^T (FP64 device arrays; A [M][K] rows lda apart, B [N][K] rows ldb
 // apart, C [M][N] rows ldc apart) from `slices` digit slices of each operand.
-// Allocates its temporaries (digit slices, exponents, the tile list), runs on
-// `stream` and returns when the product is in C.
+// Takes its temporaries (digit slices, exponents, the tile list) from the work
+// pool, runs on `stream` and returns when the product is in C.
 extern "C" int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *B, long long ldb,
                                   double *C, long long ldc, int M, int N, int K, int slices,
                                   void *stream) {
@@ -124,22 +168,16 @@ extern "C" int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *
   const int s = slices;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int Kp = (K + kEmuKB - 1) / kEmuKB * kEmuKB;
-  std::vector<void *> mem;
+  void *mem = nullptr;
   auto cleanup = [&] {
-    cudaStreamSynchronize(st);
-    for (void *p : mem) cudaFree(p);
+    work_free(mem, st);
+    return cudaStreamSynchronize(st);
   };
   auto fail = [&](int code, const std::string &m) {
     cleanup();
     cudaGetLastError();
     set_last_error("mlcc3_fp64emu_gemm: " + m);
     return code;
-  };
-  auto alloc = [&](size_t bytes) -> void * {
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
-    mem.push_back(p);
-    return p;
   };
   // items: output tiles, their reductions cut where few tiles would leave SMs
   // idle (pieces of at least 512) or where they exceed an item's bound; the
@@ -181,8 +219,8 @@ extern "C" int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *
   const size_t oa = part(sizeof(__nv_bfloat16) * s * M * (size_t)Kp), ob = part(sizeof(__nv_bfloat16) * s * N * (size_t)Kp);
   const size_t oea = part(sizeof(int) * M), oeb = part(sizeof(int) * N);
   const size_t oi = part(sizeof(TcItem) * items.size()), os = part(sizeof(TcSeg) * segs.size()), ost = part(sizeof(int));
-  char *base = static_cast<char *>(alloc(total));
-  if (!base) return fail(MLCC3_ERR_OOM, "cudaMalloc");
+  if (work_alloc(&mem, total, st) != cudaSuccess) return fail(MLCC3_ERR_OOM, "workspace");
+  char *base = static_cast<char *>(mem);
   __nv_bfloat16 *sa = reinterpret_cast<__nv_bfloat16 *>(base + oa), *sb = reinterpret_cast<__nv_bfloat16 *>(base + ob);
   int *ea = reinterpret_cast<int *>(base + oea), *eb = reinterpret_cast<int *>(base + oeb);
   int *status = reinterpret_cast<int *>(base + ost);
@@ -221,9 +259,11 @@ extern "C" int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *
                                   (int)items.size(), epi, status, st);
   int hst = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, status, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(MLCC3_ERR_CUDA, cudaGetErrorString(e));
-  cleanup();
+  if ((e = cleanup()) != cudaSuccess) {
+    mem = nullptr;
+    return fail(MLCC3_ERR_CUDA, cudaGetErrorString(e));
+  }
   if (hst & kStatusTimeout) {
     set_last_error("mlcc3_fp64emu_gemm: a tensor-core pipeline wait timed out");
     return MLCC3_ERR_TIMEOUT;

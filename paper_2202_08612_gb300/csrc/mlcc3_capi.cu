@@ -26,6 +26,7 @@
 #include "kernels_fp64.cuh"
 #include "kernels_tc.cuh"
 #include "mlcc3.h"
+#include "workpool.cuh"
 
 namespace mlcc3 {
 cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st);
@@ -122,7 +123,13 @@ void *mlcc3_ctx::raw(const std::string &name, size_t bytes) {
     tri_regs.erase(name);
   }
   void *p = nullptr;
-  check_cuda(cudaMalloc(&p, bytes < 256 ? 256 : bytes), ("cudaMalloc " + name).c_str());
+  cudaError_t e = cudaMalloc(&p, bytes < 256 ? 256 : bytes);
+  if (e == cudaErrorMemoryAllocation) {  // once more without what the work pool keeps
+    cudaGetLastError();
+    work_trim();
+    e = cudaMalloc(&p, bytes < 256 ? 256 : bytes);
+  }
+  check_cuda(e, ("cudaMalloc " + name).c_str());
   scratch[name] = {p, bytes};
   return p;
 }
@@ -3371,6 +3378,7 @@ extern "C" void mlcc3_destroy(mlcc3_ctx *c) {
     cudaEventDestroy(pe.stop);
   }
   for (auto e : c->event_pool) cudaEventDestroy(e);
+  work_trim();
   delete c;
 }
 
