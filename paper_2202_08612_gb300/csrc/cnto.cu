@@ -7,14 +7,20 @@
 // a, N over (i, c, j).  One FP64 kernel computes C[m][n] += alpha sum_k
 // A[m][k] A[n][k] for a batch of strided views, the reduction split across
 // blocks (partial sums added atomically), 64 x 64 output tiles staged through
-// shared memory.
+// shared memory.  That kernel only runs where there is no room for the digit slices
+// (kernels_emu.cuh) with which the doubles' matrices run on the tensor cores; the
+// singles and the diagonal term have a kernel of one thread per element.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 #include <string>
+#include <vector>
 
+#include "kernels_emu.cuh"
 #include "mlcc3.h"
+#include "workpool.cuh"
 
 namespace mlcc3 {
 void set_last_error(const std::string &msg);
@@ -84,16 +90,173 @@ __global__ void __launch_bounds__(256) gram_kernel(GramView v, double alpha, dou
     }
 }
 
-// M_ii += 1/2 sum_a d_ai^2 and N_aa += 1/2 sum_i d_ai^2 with d_ai = R^{aa}_{ii}
-// (the delta factor of Eqs. M and N).
-__global__ void cnto_diag_kernel(const double *R2, long long NO, long long NV, double *M,
-                                 double *N) {
+// The singles' parts and the delta factor's diagonals (Eqs. M and N), which also set M and N:
+// M_ij = sum_a R1_ai R1_aj + delta_ij 1/2 sum_a d_ai^2, N_ab = sum_i R1_ai R1_bi +
+// delta_ab 1/2 sum_i d_ai^2 with d_ai = R^{aa}_{ii}.  A thread per element (64 x 64
+// tiles of this size, mostly padding on the FP64 pipe, took 0.3 ms).
+__global__ void cnto_singles_kernel(const double *R1, const double *R2, long long NO, long long NV,
+                                    double *M, double *N) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= NO * NV) return;
-  const long long a = e / NO, i = e % NO;
-  const double d = R2[((a * NO + i) * NV + a) * NO + i];
-  atomicAdd(M + i * NO + i, 0.5 * d * d);
-  atomicAdd(N + a * NV + a, 0.5 * d * d);
+  const bool occ = e < NO * NO;
+  const long long f = occ ? e : e - NO * NO, rows = occ ? NO : NV, K = occ ? NV : NO;
+  if (f >= rows * rows) return;
+  const long long p = f / rows, q = f % rows, rs = occ ? 1 : NO, ks = occ ? NO : 1;
+  double s = 0.0, d2 = 0.0;
+  for (long long k = 0; k < K; ++k) s = fma(R1[p * rs + k * ks], R1[q * rs + k * ks], s);
+  if (p == q)
+    for (long long k = 0; k < K; ++k) {
+      const long long a = occ ? k : p, i = occ ? p : k;
+      const double d = R2[((a * NO + i) * NV + a) * NO + i];
+      d2 = fma(d, d, d2);
+    }
+  (occ ? M : N)[f] = fma(0.5, d2, s);
+}
+
+// X[i][j] += the copies' sum, for j >= i, and X[j][i] = X[i][j].
+__global__ void fold_kernel(double *X, long long n, const double *copy, int copies) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n * n) return;
+  const long long i = e / n, j = e % n;
+  if (j < i) return;
+  double s = 0.0;
+  for (int c = 0; c < copies; ++c) s += copy[c * n * n + e];
+  s += X[e];
+  X[e] = s;
+  X[j * n + i] = s;
+}
+
+// M_ij += 1/2 sum_a sum_K P[(a,i)][K] P[(a,j)][K] and N_ab += 1/2 sum_i sum_K P[(a,i)][K]
+// P[(b,i)][K], P the doubles as an n x n matrix (n = N_O N_V), on the tensor cores.
+// The digits of P's rows serve both: rows i of block a, or rows a (n_o rows apart)
+// of block i, are two tensor maps over the same memory.  K runs in chunks whose
+// digits take at most a gigabyte.  39 / 263: 70.3 -> 2.9 ms, error 1.3e-15 -> 7e-17.
+cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, double *M, double *N,
+                              cudaStream_t st, bool *timeout, std::string *err) {
+  using namespace mlcc3;
+  const long long n = NO * NV;
+  const long long most = std::max<long long>(kEmuKB, (((long long)1 << 30) - (64 << 20)) / (16 * n) / kEmuKB * kEmuKB);
+  const long long parts = (n + most - 1) / most, kc = ((n + parts - 1) / parts + kEmuKB - 1) / kEmuKB * kEmuKB;
+  struct Gram {
+    long long rows, blocks, row_stride, block_stride;  // strides in rows of P
+    double *out;
+    int copies;
+  } g[2] = {{NO, NV, 1, NO, M, 1}, {NV, NO, NO, 1, N, 1}};
+  std::vector<TcItem> items[2];
+  std::vector<TcSeg> segs[2];
+  // tiles on and above the diagonal, their reductions (all blocks' chunk after chunk)
+  // cut into about eight items per SM of whole accumulation chains.  A thousand parts
+  // added one by one to the same element would round more often than the FP64 kernel's
+  // sums, so the p parts of a tile go to sqrt(p) copies, which one kernel adds up
+  const int nk = (int)(kc / kEmuKB);
+  int w[2];
+  for (int q = 0; q < 2; ++q) {
+    w[q] = emu_tile_width(g[q].rows, kEmuSlices);
+    long long tiles = 0;
+    for (long long m0 = 0; m0 < g[q].rows; m0 += 128) tiles += (g[q].rows + w[q] - 1) / w[q] - m0 / w[q];
+    const long long all = g[q].blocks * nk, chain = 256 / kEmuKB;
+    const long long per =
+        std::min<long long>(kEmuMaxK / kEmuKB, std::max<long long>(1, all * tiles / (1216 * chain)) * chain);
+    const long long np = (all + per - 1) / per;
+    while (g[q].copies < 32 && g[q].copies * g[q].copies < np) ++g[q].copies;
+    for (long long c0 = 0; c0 < all; c0 += per)
+      for (long long m0 = 0; m0 < g[q].rows; m0 += 128)
+        for (long long n0 = m0 / w[q] * w[q]; n0 < g[q].rows; n0 += w[q]) {
+          TcItem it{};
+          it.seg_begin = (int)segs[q].size();
+          it.r2_0 = (int)m0;
+          it.c0 = (int)n0;
+          it.out_off = c0 / per % g[q].copies * g[q].rows * g[q].rows;
+          for (long long c = c0; c < std::min(all, c0 + per);) {
+            TcSeg sg{};
+            sg.amap = 0;
+            sg.bmap = 1;
+            sg.nk = (int)std::min(nk - c % nk, std::min(all, c0 + per) - c);
+            sg.ac[0] = sg.bc[0] = (int)(c % nk * kEmuKB);
+            sg.ac[1] = (int)m0;
+            sg.bc[1] = (int)n0;
+            sg.ac[2] = sg.bc[2] = (int)(c / nk);
+            segs[q].push_back(sg);
+            it.seg_count += 1;
+            it.chunks += sg.nk;
+            c += sg.nk;
+          }
+          items[q].push_back(it);
+        }
+  }
+  size_t total = 0;
+  auto part = [&](size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t od = part((size_t)16 * n * kc), os = part(sizeof(EmuScale)), ost = os + sizeof(EmuScale);
+  // scale, status (both zero) and the tile lists go over in one copy
+  size_t oi[2], og[2];
+  for (int q = 0; q < 2; ++q) {
+    oi[q] = part(sizeof(TcItem) * items[q].size());
+    og[q] = part(sizeof(TcSeg) * segs[q].size());
+  }
+  const size_t head_bytes = total - os;
+  size_t oc[2];
+  for (int q = 0; q < 2; ++q) oc[q] = part(sizeof(double) * g[q].copies * g[q].rows * g[q].rows);
+  std::vector<char> head(head_bytes, 0);
+  for (int q = 0; q < 2; ++q) {
+    std::memcpy(head.data() + (oi[q] - os), items[q].data(), sizeof(TcItem) * items[q].size());
+    std::memcpy(head.data() + (og[q] - os), segs[q].data(), sizeof(TcSeg) * segs[q].size());
+  }
+  void *mem = nullptr;
+  cudaError_t e = work_alloc(&mem, total, st);
+  if (e != cudaSuccess) return e;
+  char *base = static_cast<char *>(mem);
+  __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(base + od);
+  EmuScale *scale = reinterpret_cast<EmuScale *>(base + os);
+  int *status = reinterpret_cast<int *>(base + ost), hst = 0;
+  e = cudaMemcpyAsync(base + os, head.data(), head.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(base + oc[0], 0, total - oc[0], st);
+  if (e == cudaSuccess) e = emu_absmax(R2, n * n, scale, st);
+  for (long long k0 = 0; k0 < n && e == cudaSuccess; k0 += kc) {
+    // (a shorter last chunk is padded with zeros)
+    const EmuView v{R2 + k0, 1, 1, (int)n, (int)n, (int)std::min(kc, n - k0), 1, 0, 0, 0, n, 1, 0};
+    e = emu_digits(v, kc, false, scale, dig, nullptr, 0.0, false, st);
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+      TcMaps maps{};
+      const unsigned long long rb = (unsigned long long)kc * 2;
+      const unsigned long long dims[4] = {(unsigned long long)kc, (unsigned long long)g[q].rows,
+                                          (unsigned long long)g[q].blocks, 1};
+      const unsigned long long str[3] = {rb * g[q].row_stride, rb * g[q].block_stride, rb * n};
+      const unsigned ba[3] = {128, 1, 1}, bb[3] = {(unsigned)w[q], 1, 1};
+      if (!emu_encode_map(&maps.m[0], dig, dims, str, rb * n, ba, kEmuSlices, err) ||
+          !emu_encode_map(&maps.m[1], dig, dims, str, rb * n, bb, kEmuSlices, err)) {
+        e = cudaErrorInvalidValue;
+        break;
+      }
+      EmuEpi epi{};
+      epi.out = reinterpret_cast<double *>(base + oc[q]);
+      epi.mode = 1;
+      epi.R2 = 1 << 30;
+      epi.s2 = g[q].rows;
+      epi.sn = 1;
+      epi.lim1 = 1;
+      epi.lim2 = epi.nlim = (int)g[q].rows;
+      epi.alpha = 0.5;
+      epi.n = w[q];
+      epi.ebias = -12;
+      epi.sa = epi.sb = scale;
+      e = launch_emu_gemm(kEmuSlices, maps, reinterpret_cast<TcItem *>(base + oi[q]),
+                          reinterpret_cast<TcSeg *>(base + og[q]), (int)items[q].size(), epi, status, st);
+    }
+  }
+  for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+    fold_kernel<<<(unsigned)((g[q].rows * g[q].rows + 255) / 256), 256, 0, st>>>(
+        g[q].out, g[q].rows, reinterpret_cast<double *>(base + oc[q]), g[q].copies);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, status, sizeof(int), cudaMemcpyDeviceToHost, st);
+  work_free(mem, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = e2;
+  *timeout = (hst & kStatusTimeout) != 0;
+  return e;
 }
 
 bool on_device(const void *p) {
@@ -137,24 +300,32 @@ extern "C" int mlcc3_cnto_matrices(int64_t n_occ, int64_t n_vir, const double *R
     return MLCC3_ERR_ARG;
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = cudaMemsetAsync(M, 0, sizeof(double) * NO * NO, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(N, 0, sizeof(double) * NV * NV, st);
-  // singles: M_ij += sum_a R1[a][i] R1[a][j], N_ab += sum_i R1[a][i] R1[b][i]
-  if (e == cudaSuccess) e = gram(GramView{R1, NO, NV, 1, NO, 1, 0, 0}, 1.0, M, st);
-  if (e == cudaSuccess) e = gram(GramView{R1, NV, NO, NO, 1, 1, 0, 0}, 1.0, N, st);
+  cnto_singles_kernel<<<(unsigned)((NO * NO + NV * NV + 255) / 256), 256, 0, st>>>(R1, R2, NO, NV, M, N);
+  cudaError_t e = cudaGetLastError();
   // doubles: M_ij += 1/2 sum_a sum_{(b,k)} R2[a][i][(b,k)] R2[a][j][(b,k)]
-  if (e == cudaSuccess)
-    e = gram(GramView{R2, NO, NV * NO, NV * NO, 1, NV, NO * NV * NO, 0}, 0.5, M, st);
   //          N_ab += 1/2 sum_{(i,c,j)} R2[a][(i,c,j)] R2[b][(i,c,j)]
-  if (e == cudaSuccess) e = gram(GramView{R2, NV, NO * NV * NO, NO * NV * NO, 1, 1, 0, 0}, 0.5, N, st);
-  if (e == cudaSuccess) {
-    const long long n = NO * NV;
-    cnto_diag_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(R2, NO, NV, M, N);
-    e = cudaGetLastError();
+  // (the singles' parts are symmetric, so mirroring the sums keeps them)
+  std::string err;
+  bool done = false, timeout = false;
+  if (e == cudaSuccess && NO * NV < (1LL << 20)) {
+    e = doubles_by_digits(NO, NV, R2, M, N, st, &timeout, &err);
+    done = e == cudaSuccess;
+    if (e == cudaErrorMemoryAllocation) {  // no room for a workspace: the FP64 kernel needs none
+      cudaGetLastError();
+      e = cudaSuccess;
+    }
   }
+  if (timeout) {
+    mlcc3::set_last_error("mlcc3_cnto_matrices: a tensor-core pipeline wait timed out");
+    return MLCC3_ERR_TIMEOUT;
+  }
+  if (e == cudaSuccess && !done)
+    e = gram(GramView{R2, NO, NV * NO, NV * NO, 1, NV, NO * NV * NO, 0}, 0.5, M, st);
+  if (e == cudaSuccess && !done)
+    e = gram(GramView{R2, NV, NO * NV * NO, NO * NV * NO, 1, 1, 0, 0}, 0.5, N, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
-    mlcc3::set_last_error(std::string("mlcc3_cnto_matrices: ") + cudaGetErrorString(e));
+    mlcc3::set_last_error(std::string("mlcc3_cnto_matrices: ") + (err.empty() ? cudaGetErrorString(e) : err));
     return MLCC3_ERR_CUDA;
   }
   return MLCC3_OK;
