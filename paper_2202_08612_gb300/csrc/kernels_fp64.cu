@@ -1990,23 +1990,25 @@ namespace mlcc3 {
 constexpr size_t kPdRed = 256 * 8 * sizeof(double);
 __device__ __forceinline__ double to_f64(float x) { return widen_f32(x); }
 __device__ __forceinline__ double to_f64(double x) { return x; }
-__device__ __forceinline__ void pair_dots_add(unsigned char *smraw, const double (&acc)[4][4], int tile,
+template <int D>
+__device__ __forceinline__ void pair_dots_add(unsigned char *smraw, const double (&acc)[D][D], int tile,
                                               int h, int TT, int H, int nh, int no, double *out,
                                               long long ldo, int kl, double f) {
   double *red = reinterpret_cast<double *>(smraw);
 #pragma unroll
-  for (int half = 0; half < 2; ++half) {
+  for (int v0 = 0; v0 < D * D; v0 += 8) {
+    const int nv = D * D - v0 < 8 ? D * D - v0 : 8;
     __syncthreads();
     if (h < H)
 #pragma unroll
-      for (int v = 0; v < 8; ++v) red[(h * TT + tile) * 8 + v] = acc[2 * half + v / 4][v % 4];
+      for (int v = 0; v < nv; ++v) red[(h * TT + tile) * nv + v] = acc[(v0 + v) / D][(v0 + v) % D];
     __syncthreads();
-    for (int q = threadIdx.x; q < TT * 8; q += 256) {
-      const int tl = q / 8, v = q % 8;
-      const int kk = 4 * (tl / nh) + 2 * half + v / 4, ll = 4 * (tl % nh) + v % 4;
+    for (int q = threadIdx.x; q < TT * nv; q += 256) {
+      const int tl = q / nv, v = v0 + q % nv;
+      const int kk = D * (tl / nh) + v / D, ll = D * (tl % nh) + v % D;
       if (kk >= no || ll >= no) continue;
       double x = 0.0;
-      for (int g = 0; g < H; ++g) x += red[(g * TT + tl) * 8 + v];
+      for (int g = 0; g < H; ++g) x += red[(g * TT + tl) * nv + q % nv];
       atomicAdd(out + (kl ? kk * ldo + ll : ll * ldo + kk), f * x);
     }
   }
@@ -2032,11 +2034,13 @@ __device__ __forceinline__ void pair_dots_add(unsigned char *smraw, const double
 // only on the thread and on which axis is a, so it is made once, and a tile's
 // offsets and limits once per view (FP32: 3.37 -> 2.99 ms at n_o = 6, n_v = 150; 0.84
 // -> 0.70 at 11, 57).  Thread
-// t keeps a 4x4 (k,l) tile (t % TT) of partial sums over the (t / TT)-th share
-// of every tile and adds it to `out` once.  T is the type of the products and
+// t keeps a D x D (k,l) tile (t % TT) of partial sums over the (t / TT)-th share
+// of every tile and adds it to `out` once.  D = 3 where the same number of tiles holds
+// n_o: fewer outputs past n_o, whose FP64 sums took a third of the FP64 pipe, and three
+// blocks per SM instead of two (2.85 -> 1.93 ms at n_o = 6, n_v = 150).  T is the type of the products and
 // of the per-tile sums (FP32 in the split-precision mode, else FP64); the sums
 // over tiles are FP64.  Requires no <= 32.
-template <typename T, int TA, int TB>
+template <typename T, int TA, int TB, int D>
 __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
                                                const T *__restrict__ Y,
                                                const long long *__restrict__ voff,
@@ -2106,27 +2110,27 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
   const long long nv2 = (long long)nv * nv;
   __syncthreads();
   const int nh = (no + 3) / 4;
-  const int TT = nh * nh;                   // 4x4 tiles of (k, l)
+  const int TT = nh * nh;                   // D x D tiles of (k, l)
   const int H = 256 / TT;                   // element shares per tile
   const int tile = t % TT, h = t / TT;
-  const int k0 = 4 * (tile / nh), l0 = 4 * (tile % nh);
+  const int k0 = D * (tile / nh), l0 = D * (tile % nh);
   // positions of this thread's share: in FP64 even ones (the other threads waited for the
   // last share: 0.87 -> 0.36 ms at n_o = 7, n_v = 37); in FP32 TE / H each, the rest in the
   // last one (the partial sums are part of the results)
   const int e0 = sizeof(T) == 8 ? h * TE / H : h * (TE / H);
   const int e1 = sizeof(T) == 8 ? (h + 1) * TE / H : (h + 1 == H) ? TE : (h + 1) * (TE / H);
   // that last share is up to five times the others (42 positions against 8 at n_o <= 8):
-  // a thread per output sums it, in the same order, instead of one per 4 x 4 outputs
+  // a thread per output sums it, in the same order, instead of one per D x D outputs
   const bool spread = sizeof(T) == 4 && TT <= 16 && TE - (H - 1) * (TE / H) > 2 * (TE / H);
   const int hmax = spread ? H - 1 : H;
-  const bool tail = spread && t < TT * 16;
-  const int tk = 4 * (t / 16 / nh) + t % 16 / 4, tl = 4 * (t / 16 % nh) + t % 4;
+  const bool tail = spread && t < TT * D * D;
+  const int tk = D * (t / (D * D) / nh) + t % (D * D) / D, tl = D * (t / (D * D) % nh) + t % D;
   double tacc = 0.0;
-  double acc[4][4];
+  double acc[D][D];
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < D; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
+    for (int y = 0; y < D; ++y) acc[x][y] = 0.0;
   const int ta = (nv + TA - 1) / TA, tb = (nv + TB - 1) / TB, tc = (nv + TB - 1) / TB;
   const int ntiles = ta * tb * tc;
   for (int q = blockIdx.x; q < ntiles; q += gridDim.x) {
@@ -2178,33 +2182,33 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
       tacc += to_f64(q);
     }
     if (h < hmax) {
-      const T *xr[4], *yr[4];
+      const T *xr[D], *yr[D];
 #pragma unroll
-      for (int d = 0; d < 4; ++d) {
+      for (int d = 0; d < D; ++d) {
         xr[d] = xs + min(l0 + d, no - 1) * TS;
         yr[d] = ys + min(k0 + d, no - 1) * TS;
       }
-      T p[4][4];
+      T p[D][D];
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < D; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) p[x][y] = T(0);
+        for (int y = 0; y < D; ++y) p[x][y] = T(0);
       for (int e = e0; e < e1; ++e) {
-        T u[4], w[4];
+        T u[D], w[D];
 #pragma unroll
-        for (int d = 0; d < 4; ++d) {
+        for (int d = 0; d < D; ++d) {
           u[d] = xr[d][e];
           w[d] = yr[d][e];
         }
 #pragma unroll
-        for (int x = 0; x < 4; ++x)
+        for (int x = 0; x < D; ++x)
 #pragma unroll
-          for (int y = 0; y < 4; ++y) p[x][y] += w[x] * u[y];
+          for (int y = 0; y < D; ++y) p[x][y] += w[x] * u[y];
       }
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < D; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += to_f64(p[x][y]);
+        for (int y = 0; y < D; ++y) acc[x][y] += to_f64(p[x][y]);
     }
   }
   if (tail && tk < no && tl < no)
@@ -2226,11 +2230,12 @@ long long pair_dots_tiles(int nv, bool f32) {
 }
 
 // FP32 operands (FP32 copies of the triples arrays, split-precision mode).
-__global__ void __launch_bounds__(256, 2) pair_dots_f32_kernel(
+template <int D>
+__global__ void __launch_bounds__(256, D == 3 ? 3 : 2) pair_dots_f32_kernel(
     const float *__restrict__ X, const float *__restrict__ Y, const long long *__restrict__ voff,
     const int *__restrict__ vstr, const char *__restrict__ vhave, int no, int nv, int p0,
     double *__restrict__ out, long long ldo, int kl, double alpha) {
-  pair_dots_body<float, 2, 16>(X, Y, voff, vstr, vhave, no, nv, p0, out, ldo, kl, alpha);
+  pair_dots_body<float, 2, 16, D>(X, Y, voff, vstr, vhave, no, nv, p0, out, ldo, kl, alpha);
 }
 
 // Physical-order form of pair_dots_f32_kernel for n_v a multiple of 4 (every
@@ -2238,11 +2243,12 @@ __global__ void __launch_bounds__(256, 2) pair_dots_f32_kernel(
 // copied in its own storage order, sixteen bytes (four elements along the
 // stride-1 axis) per cp.async, and the products read each view through its
 // logical strides in shared memory (64, 8 or 1 per logical axis).  Thread t
-// keeps a 4x4 (k,l) tile of partial sums over a share of the tile's 64 (a,b)
+// keeps a D x D (k,l) tile of partial sums over a share of the tile's 64 (a,b)
 // rows.  Same sums as pair_dots_f32_kernel.
 constexpr int kPdTS = 512 + 4;  // floats per view tile in shared memory (16-byte multiple)
 
-__global__ void __launch_bounds__(256, 2) pair_dots_phys_kernel(
+template <int D>
+__global__ void __launch_bounds__(256, D == 3 ? 3 : 2) pair_dots_phys_kernel(
     const float *__restrict__ X, const float *__restrict__ Y, const long long *__restrict__ voff,
     const int *__restrict__ vstr, const char *__restrict__ vhave, int no, int nv, int p0,
     double *__restrict__ out, long long ldo, int kl, double alpha) {
@@ -2289,18 +2295,18 @@ __global__ void __launch_bounds__(256, 2) pair_dots_phys_kernel(
   const int TT = nh * nh;
   const int H = 256 / TT;
   const int tile = t % TT, h = t / TT;
-  const int k0 = 4 * (tile / nh), l0 = 4 * (tile % nh);
+  const int k0 = D * (tile / nh), l0 = D * (tile % nh);
   const int row0 = h * 64 / H, row1 = (h + 1) * 64 / H;  // (a,b) rows of this share
-  int xr[4], yr[4];
-  for (int d = 0; d < 4; ++d) {
+  int xr[D], yr[D];
+  for (int d = 0; d < D; ++d) {
     xr[d] = min(l0 + d, no - 1);
     yr[d] = min(k0 + d, no - 1);
   }
-  double acc[4][4];
+  double acc[D][D];
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < D; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
+    for (int y = 0; y < D; ++y) acc[x][y] = 0.0;
   const int tb = (nv + 7) / 8;
   const int ntiles = tb * tb * tb;
   const long long nv2 = (long long)nv * nv;
@@ -2328,16 +2334,16 @@ __global__ void __launch_bounds__(256, 2) pair_dots_phys_kernel(
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (h < H) {
-      float p[4][4];
+      float p[D][D];
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < D; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) p[x][y] = 0.f;
+        for (int y = 0; y < D; ++y) p[x][y] = 0.f;
       for (int row = row0; row < row1; ++row) {
         const int a = row >> 3, b = row & 7;
-        int ux[4], uy[4], cx[4], cy[4];
+        int ux[D], uy[D], cx[D], cy[D];
 #pragma unroll
-        for (int d = 0; d < 4; ++d) {
+        for (int d = 0; d < D; ++d) {
           ux[d] = xr[d] * kPdTS + a * s_sm[xr[d]][0] + b * s_sm[xr[d]][1];
           uy[d] = yr[d] * kPdTS + a * s_sm[yr[d]][0] + b * s_sm[yr[d]][1];
           cx[d] = s_sm[xr[d]][2];
@@ -2345,22 +2351,22 @@ __global__ void __launch_bounds__(256, 2) pair_dots_phys_kernel(
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          float u[4], w[4];
+          float u[D], w[D];
 #pragma unroll
-          for (int d = 0; d < 4; ++d) {
+          for (int d = 0; d < D; ++d) {
             u[d] = xs[ux[d] + c * cx[d]];
             w[d] = ys[uy[d] + c * cy[d]];
           }
 #pragma unroll
-          for (int x = 0; x < 4; ++x)
+          for (int x = 0; x < D; ++x)
 #pragma unroll
-            for (int y = 0; y < 4; ++y) p[x][y] += w[x] * u[y];
+            for (int y = 0; y < D; ++y) p[x][y] += w[x] * u[y];
         }
       }
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < D; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] += to_f64(p[x][y]);
+        for (int y = 0; y < D; ++y) acc[x][y] += to_f64(p[x][y]);
     }
   }
   pair_dots_add(smraw, acc, tile, h, TT, H, nh, no, out, ldo, kl, wij * alpha);
@@ -2368,12 +2374,18 @@ __global__ void __launch_bounds__(256, 2) pair_dots_phys_kernel(
 
 size_t pair_dots_phys_smem(int no) { return std::max(2 * (size_t)no * kPdTS * sizeof(float), kPdRed); }
 
+template <int D>
 __global__ void __launch_bounds__(256) pair_dots_f64_kernel(
     const double *__restrict__ X, const double *__restrict__ Y, const long long *__restrict__ voff,
     const int *__restrict__ vstr, const char *__restrict__ vhave, int no, int nv, int p0,
     double *__restrict__ out, long long ldo, int kl, double alpha) {
-  pair_dots_body<double, 4, 8>(X, Y, voff, vstr, vhave, no, nv, p0, out, ldo, kl, alpha);
+  pair_dots_body<double, 4, 8, D>(X, Y, voff, vstr, vhave, no, nv, p0, out, ldo, kl, alpha);
 }
+
+// The kernels for (k, l) tiles of 3 x 3 or 4 x 4 outputs.
+PairDots32 pair_dots_f32(int d) { return d == 3 ? pair_dots_f32_kernel<3> : pair_dots_f32_kernel<4>; }
+PairDots32 pair_dots_phys(int d) { return d == 3 ? pair_dots_phys_kernel<3> : pair_dots_phys_kernel<4>; }
+PairDots64 pair_dots_f64(int d) { return d == 3 ? pair_dots_f64_kernel<3> : pair_dots_f64_kernel<4>; }
 
 }  // namespace mlcc3
 

@@ -103,4 +103,11 @@ struct TripTerms {
   int n;
 };
 
+// X, Y, view offsets, strides and presence, n_o, n_v, first i, out, its rows, orientation, alpha
+template <typename T>
+using PairDots = void (*)(const T *, const T *, const long long *, const int *, const char *, int, int, int,
+                          double *, long long, int, double);
+using PairDots32 = PairDots<float>;
+using PairDots64 = PairDots<double>;
+
 }  // namespace mlcc3
