@@ -260,7 +260,7 @@ void mlcc3_sweep_destroy(mlcc3_sweep *sweep);
  *              FP32 accumulation over K ranges of at most 1024 (summed in
  *              FP64); the others on 64 x 64 tiles.  Default 10^9; 0: never.
  *   "fp64_tc_from"  MLCC3_FP64 contexts with at least this many active virtual
- *              orbitals (and n_o >= 2) run the O(N_V n_v^3 n_o^3) contractions and
+ *              orbitals, or n_o n_v at least three times it, and n_o >= 2 run the O(N_V n_v^3 n_o^3) contractions and
  *              the Cholesky-index products on the tensor cores (see MLCC3_FP64),
  *              unless the digits of the integral blocks would take more than a
  *              quarter of the free memory; smaller ones on the FP64 pipe.

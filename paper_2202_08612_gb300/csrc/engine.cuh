@@ -171,8 +171,8 @@ struct mlcc3_ctx {
     const mlcc3::EmuScale *scale = nullptr;
   };
   std::map<std::string, SplitOp> splits;
-  // FP64 mode: the large contractions on the tensor cores (kernels_emu.cuh), for
-  // n_v >= fp64_tc_from; the names of the operands' scales
+  // FP64 mode: the large contractions on the tensor cores (kernels_emu.cuh), from
+  // fp64_tc_from on (choose_emu); the names of the operands' scales
   bool emu = false;
   long long fp64_tc_from = 24;
   std::map<std::string, int> scales;

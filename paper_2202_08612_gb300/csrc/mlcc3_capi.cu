@@ -566,14 +566,17 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
 // FP64 mode: the O(N_V n_v^3 n_o^3) contractions on the tensor cores (digit
 // slices; rho and sigma at 20/200/12/60: 1868 -> 85 ms, the densities at
 // 13/101/7/37: 79 -> 18 ms, errors against 64 bits as before or smaller) from
-// fp64_tc_from active virtual orbitals on (a 4/8 system gains nothing: its calls
-// are launches, and the digits need more of them), where the operands'
+// fp64_tc_from (24) active virtual orbitals or n_o n_v = 3 fp64_tc_from on (rho and sigma,
+// FP64 pipe against digits: 4/12 0.85 against 1.15 ms, 4/16 1.34 and 1.32, 6/12 1.79 and
+// 1.20, 8/16 4.66 and 1.67, 3/24 1.87 and 1.63; below, a call is launches, and the digits
+// need more of them), where the operands'
 // digits (six layouts of the two integral blocks, the Cholesky factors and the
 // amplitudes at 16 bytes an element) leave most of the memory free.
 void choose_emu(mlcc3_ctx *c) {
   S s(c);
   c->emu = false;
-  if (c->precision != MLCC3_FP64 || s.no < 2 || s.nv < c->fp64_tc_from) return;
+  if (c->precision != MLCC3_FP64 || s.no < 2) return;
+  if (s.nv < c->fp64_tc_from && s.no * s.nv < 3 * c->fp64_tc_from) return;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return;
   const double digits = 16.0 * (8.0 * (double)s.gvsz() + 3.0 * (double)s.NJ * (double)(s.nv * s.NV) +

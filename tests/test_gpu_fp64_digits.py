@@ -79,3 +79,13 @@ def test_a_vector_that_is_not_finite_gives_nan():
     r1, r2 = c.empty_dev(c.st.R1.shape), c.empty_dev(c.st.R2.shape)
     g.jacobian_right(c.st.omega, c.to_dev(c.st.R1), c.to_dev(R2), r1, r2)
     assert np.isnan(c.host(r2)).any()
+
+
+@pytest.mark.parametrize("dims", [(9, 24, 8, 9, 30), (25, 20, 24, 3, 24), (5, 40, 2, 24, 40), (7, 24, 5, 14, 30)])
+def test_default_rule_around_its_line(dims):
+    """n_o n_v = 72 or n_v = 24 take the digits, 5/14 the FP64 pipe: the same results."""
+    _cuda()
+    c = Case(*dims, nstates=1)
+    got, simt = run_all(c, c.context()), run_all(c, c.context(params={"fp64_tc_from": 2000}))
+    for k in got:
+        assert rel_err(got[k], simt[k]) < 1e-12, (k, rel_err(got[k], simt[k]))
