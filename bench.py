@@ -1344,7 +1344,7 @@ def run_fp64emu(args):
                       "value": res[5]["tflops"], "unit": "TFLOP/s", "n_gpus": 1,
                       "steps": args.steps, "warmup": args.warmup, "higher_is_better": True,
                       "config": {"workload": f"C = A B^T, M = N = K = {n}, FP64 normal entries",
-                                 "note": "each call allocates and frees its temporaries"},
+                                 "note": "workspace from the library's stream-ordered pool"},
                       "slices": {str(k): v for k, v in res.items()},
                       "dgemm": {"ms": ms_d, "tflops": fl / ms_d / 1e9}}))
 

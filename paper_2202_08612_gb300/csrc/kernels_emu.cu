@@ -81,10 +81,10 @@ __device__ __forceinline__ int scale_exp(EmuScale s) { return (int)((s >> 52) & 
 // After each chain of 256 K elements eight epilogue warps add the degrees,
 // weighted by 2^-8d, into 64-bit integers in registers (degrees 0..4 exactly, in
 // units of 2^-32: below 2^60 for kEmuMaxK products; the higher ones in FP32 beside
-// them) and hand TMEM back, so the next chain's MMAs wait only for the reads.  An item's sums are rounded to binary64
-// once, at its end, on the integer pipe.
+// them) and hand TMEM back, so the next chain's MMAs wait only for the reads.  An
+// item's sums are rounded to binary64 once, at its end, on the integer pipe.
 //   warp 0 lane 0: TMA producer; warp 1: TMEM, lane 0 issues; warps 2..9: epilogue
-// C = A B^T with M = N = K = 4096 and S = 5, slicing included: 2.64 ms, against
+// C = A B^T with M = N = K = 4096 and S = 5, slicing included: 1.77 ms, against
 // 8.26 ms with one launch of the split mode's kernel per digit degree (two of its
 // three products on zeros, and an FP64 reduction per output, pair and 1024 products).
 // AMN: A's rows are the contiguous index of its map (boxes of 64 rows x 32 K of

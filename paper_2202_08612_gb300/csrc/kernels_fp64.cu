@@ -1,7 +1,8 @@
 // FP64 kernels of the MLCC3 triples path (sm_103a).
 //
-// * bstc_kernel: batched strided tensor contraction, C += alpha A B with
-//   per-item strides (any permuted view of a triples block is a stride set).
+// * bstc64_kernel, bstc32_kernel (FP32 products), bstc_gemv, bstc_dot: batched
+//   strided tensor contraction, C += alpha A B with per-item strides (any permuted
+//   view of a triples block is a stride set).
 // * triples_build_kernel: one n_v^3 block per unique batch i >= j >= k,
 //   X^{abc}_{ijk} = -(eps^{abc}_{ijk} - omega)^{-1} P^{abc}_{ijk} V^{abc}_{ijk}
 //   (Eq. tau3, Eq. R3, SI L3), the six pair permutations summed in registers.
@@ -22,7 +23,6 @@ __constant__ int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 
 
 // ---------------------------------------------------------------------------
 // Batched strided tensor contraction.
-// Tile 64 x 64 of C per CTA, K chunks of 16, 256 threads with 4 x 4 outputs.
 // ---------------------------------------------------------------------------
 // Element i of an operand that holds binary64 (f32 = 0) or binary32 values.
 template <typename T>

@@ -1,7 +1,7 @@
 // C ABI and host orchestration of the MLCC3 triples path.
 //
 // Every contraction of the paper's equations is expressed as a batched
-// strided contraction (bstc_kernel) over the unique batches i >= j >= k:
+// strided contraction (launch_bstc64, launch_bstc32) over the unique batches i >= j >= k:
 // the block X_{ijk} of a batch is computed once (triples_build_kernel) and
 // each distinct ordering (p,q,r) of (i,j,k) reads it through a permuted
 // stride set (pair symmetry X^{abc}_{ijk} = X^{sigma(abc)}_{sigma(ijk)},
@@ -564,13 +564,13 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
 }
 
 // FP64 mode: the O(N_V n_v^3 n_o^3) contractions on the tensor cores (digit
-// slices; rho and sigma at 20/200/12/60: 1868 -> 85 ms, the densities at
-// 13/101/7/37: 79 -> 18 ms, errors against 64 bits as before or smaller) from
+// slices; rho and sigma at 20/200/12/60: 1868 -> 61 ms, the densities at
+// 13/101/7/37: 79 -> 5.4 ms, errors against 64 bits as before or smaller) from
 // fp64_tc_from (24) active virtual orbitals or n_o n_v = 3 fp64_tc_from on (rho and sigma,
 // FP64 pipe against digits: 4/12 0.85 against 1.15 ms, 4/16 1.34 and 1.32, 6/12 1.79 and
 // 1.20, 8/16 4.66 and 1.67, 3/24 1.87 and 1.63; below, a call is launches, and the digits
 // need more of them), where the operands'
-// digits (six layouts of the two integral blocks, the Cholesky factors and the
+// digits (the layouts of the two integral blocks, the Cholesky factors and the
 // amplitudes at 16 bytes an element) leave most of the memory free.
 void choose_emu(mlcc3_ctx *c) {
   S s(c);
@@ -605,7 +605,7 @@ void make_chunks(mlcc3_ctx *c) {
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = (size_t)40 << 30;
     const double budget = 0.5 * (double)fr;
     // binary32 triples arrays in the split mode (and no separate FP32 copies)
-    // (digit slices: eight FP64 arrays and three arrays' six layouts of 16 bytes)
+    // (digit slices: eight FP64 arrays and up to 18 layouts of 16 bytes)
     const double per_elem = c->tri32 ? 108.0 : c->emu ? 352.0 : 156.0;
     part_max = group_max = std::max<long long>(1, (long long)(budget / (per_elem * (double)nv3)));
   }
