@@ -176,7 +176,8 @@ extern "C" int mlcc3_triples_omega_static(mlcc3_ctx *c, double *omega1, double *
   tt.n = 2;
   tt.t[0] = TripTerm{0, (int)NV, 1.0, c->t2c, c->Gv, {bi, bL, ba, 1}, {gk, gb, gc, 1}};
   tt.t[1] = TripTerm{1, (int)NO, -1.0, c->Tl, c->Go, {ti, ta, tb, 1}, {oj, ok, oc, 1}};
-  launch_triples_build(tt, dbatch, (int)nb, c->eps, (int)NO, (int)nv, 0.0, nullptr, tau, c->status, st);
+  const cudaError_t built =
+      launch_triples_build(tt, dbatch, (int)nb, c->eps, (int)NO, (int)nv, 0.0, nullptr, tau, c->status, st);
   // an error after the first launch drains the stream before returning, so that
   // no queued work of this call still writes the shared array afterwards
   auto drained = [&]() {
@@ -184,7 +185,7 @@ extern "C" int mlcc3_triples_omega_static(mlcc3_ctx *c, double *omega1, double *
     cudaGetLastError();
     return MLCC3_ERR_CUDA;
   };
-  if (!chk(cudaGetLastError(), "triples_build launch") ||
+  if (!chk(built, "triples_build launch") ||
       !chk(launch_contra3(tau, taut, nb, (int)nv, st, false), "contra3"))
     return drained();
   // scratch keeps the previous call's contents: clear the accumulators
@@ -219,10 +220,13 @@ extern "C" int mlcc3_triples_omega_static(mlcc3_ctx *c, double *omega1, double *
     for (long long z0 = 0; z0 < nord; z0 += 65535) {
       bp.items = ditems + k * nord + z0;
       bp.nitems = (int)std::min<long long>(65535, nord - z0);
-      if (N == 1)  // matrix-vector form (singles and F terms): a warp per output row
+      // (each launch is checked here: launch_bstc64 returns its error and clears it)
+      if (N == 1) {  // matrix-vector form (singles and F terms): a warp per output row
         bstc_gemv_kernel<<<dim3((unsigned)((M + 7) / 8), (unsigned)bp.nitems), 256, 0, st>>>(bp);
-      else
-        launch_bstc64(bp, c->bstc_fill, st);
+        if (!chk(cudaGetLastError(), "bstc_gemv launch")) return drained();
+      } else if (!chk(launch_bstc64(bp, c->bstc_fill, st), "bstc64 launch")) {
+        return drained();
+      }
     }
   }
   const int g = (int)std::min<long long>((blk + 255) / 256, 152LL * 64);
