@@ -59,11 +59,15 @@ extern "C" {
 
 /* Arithmetic of the contractions.  MLCC3_FP64: products and sums in IEEE
  * double, or, for the large contractions ("fp64_tc_from"), as integers: every
- * operand a multiple of 2^-62 of the power of two above its largest element,
- * its digits multiplied on the tensor cores, the sums exact but for terms below
- * 2^-64 and rounded to binary64 once.  Results are at least as accurate as sums
- * in IEEE double (normwise); an operand with an infinity gives NaN where it
- * enters.  MLCC3_SPLIT_BF16X3: integral-amplitude products on the
+ * operand a multiple of 2^-63 of the power of two |A| above its largest element,
+ * its base-256 digits multiplied on the tensor cores, the sums of up to 192 digit
+ * products in FP32 (exact but for sums of nearly only largest digits of one sign,
+ * and there to 2^-52 |A| |B|) and beyond that in integers, rounded to binary64
+ * once.  An output sum_k a_k b_k errs by less than 2^-47 sum_k |a_k| |b_k|, the
+ * bound of IEEE double sums over 64 products: that is checked for every output,
+ * and where the operands span too wide a range for it, or are not finite, the
+ * call runs again in IEEE double on the FP64 pipe, where the context then stays
+ * until the next mlcc3_build_integrals.  MLCC3_SPLIT_BF16X3: integral-amplitude products on the
  * tensor cores from hi/lo bfloat16 splits with FP32 accumulation;
  * denominators and final reductions stay in FP64.
  * An FP16 hi/lo split is not offered: FP16's five exponent bits put the low
@@ -198,8 +202,9 @@ int mlcc3_oscillator_strength(mlcc3_ctx *ctx, double omega, const double *D0m,
  *                        get a share of half the free device memory.
  *   mlcc3_sweep_set_system  n_vec trial vectors of system `sys`: R1, R2, rho1,
  *                        rho2 are DEVICE arrays with the shapes of
- *                        mlcc3_jacobian_right; the graph reads and writes these
- *                        addresses, so they must stay valid.
+ *                        mlcc3_jacobian_right that do not overlap (a run may
+ *                        read R1 and R2 more than once); the graph reads and
+ *                        writes these addresses, so they must stay valid.
  *   mlcc3_sweep_run      omega[sum of n_vec] (host, system-major).  The first
  *                        run (and the first after mlcc3_sweep_set_system,
  *                        mlcc3_build_integrals or a change of "chunk_blocks" on
@@ -261,7 +266,9 @@ void mlcc3_sweep_destroy(mlcc3_sweep *sweep);
  *              FP64); the others on 64 x 64 tiles.  Default 10^9; 0: never.
  *   "fp64_tc_from"  MLCC3_FP64 contexts with at least this many active virtual
  *              orbitals, or n_o n_v at least three times it, and n_o >= 2 run the O(N_V n_v^3 n_o^3) contractions and
- *              the Cholesky-index products on the tensor cores (see MLCC3_FP64),
+ *              the Cholesky-index products on the tensor cores (see MLCC3_FP64; a call
+ *              whose digits find no room in the device memory also runs on the FP64
+ *              pipe),
  *              unless the digits of the integral blocks would take more than a
  *              quarter of the free memory; smaller ones on the FP64 pipe.
  *              Default 24.  A change that switches the path needs a new
@@ -314,7 +321,9 @@ int mlcc3_set_param(mlcc3_ctx *ctx, const char *name, long long value);
  * R1 [N_V][N_O]; R2 [N_V][N_O][N_V][N_O] = R^{AB}_{IJ} in full storage (a CCSD
  * excitation vector, symmetric under (A,I) <-> (B,J)); M [N_O][N_O] and
  * N [N_V][N_V] are overwritten.  Device pointers only (MLCC3_ERR_ARG
- * otherwise); FP64; runs on `cuda_stream` and returns when it has finished.
+ * otherwise); FP64 (see MLCC3_FP64: on the tensor cores, or on the FP64 pipe where
+ * an element of M or N is too small beside the largest amplitude); runs on
+ * `cuda_stream` and returns when it has finished.
  * No context is needed. */
 int mlcc3_cnto_matrices(int64_t n_occ, int64_t n_vir, const double *R1, const double *R2,
                         double *M, double *N, void *cuda_stream);

@@ -7,8 +7,9 @@
 // a, N over (i, c, j).  One FP64 kernel computes C[m][n] += alpha sum_k
 // A[m][k] A[n][k] for a batch of strided views, the reduction split across
 // blocks (partial sums added atomically), 64 x 64 output tiles staged through
-// shared memory.  That kernel only runs where there is no room for the digit slices
-// (kernels_emu.cuh) with which the doubles' matrices run on the tensor cores; the
+// shared memory.  It runs where the digit slices (kernels_emu.cuh) with which the doubles'
+// matrices run on the tensor cores find no room, or where an element of M or N is too
+// small beside the largest amplitude for them (kStatusSpread); the
 // singles and the diagonal term have a kernel of one thread per element.
 #include <cuda_runtime.h>
 
@@ -129,12 +130,13 @@ __global__ void fold_kernel(double *X, long long n, const double *copy, int copi
 // P[(b,i)][K], P the doubles as an n x n matrix (n = N_O N_V), on the tensor cores.
 // The digits of P's rows serve both: rows i of block a, or rows a (n_o rows apart)
 // of block i, are two tensor maps over the same memory.  K runs in chunks whose
-// digits take at most a gigabyte.  39 / 263: 70.3 -> 2.9 ms, error 1.3e-15 -> 7e-17.
+// digits take at most a gigabyte.  *status: the launches' status bits (with
+// kStatusSpread M and N are left as they were).  39 / 263: 70.3 -> 3.5 ms, error 1.3e-15 -> 7e-17.
 cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, double *M, double *N,
-                              cudaStream_t st, bool *timeout, std::string *err) {
+                              cudaStream_t st, int *hstatus, std::string *err) {
   using namespace mlcc3;
   const long long n = NO * NV;
-  const long long most = std::max<long long>(kEmuKB, (((long long)1 << 30) - (64 << 20)) / (16 * n) / kEmuKB * kEmuKB);
+  const long long most = std::max<long long>(kEmuKB, (((long long)1 << 30) - (64 << 20)) / (2 * kEmuStored * n) / kEmuKB * kEmuKB);
   const long long parts = (n + most - 1) / most, kc = ((n + parts - 1) / parts + kEmuKB - 1) / kEmuKB * kEmuKB;
   struct Gram {
     long long rows, blocks, row_stride, block_stride;  // strides in rows of P
@@ -153,7 +155,7 @@ cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, doub
     w[q] = emu_tile_width(g[q].rows, kEmuSlices);
     long long tiles = 0;
     for (long long m0 = 0; m0 < g[q].rows; m0 += 128) tiles += (g[q].rows + w[q] - 1) / w[q] - m0 / w[q];
-    const long long all = g[q].blocks * nk, chain = 256 / kEmuKB;
+    const long long all = g[q].blocks * nk, chain = kEmuChain;
     const long long per =
         std::min<long long>(kEmuMaxK / kEmuKB, std::max<long long>(1, all * tiles / (1216 * chain)) * chain);
     const long long np = (all + per - 1) / per;
@@ -189,7 +191,7 @@ cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, doub
     total += (bytes + 255) / 256 * 256;
     return at;
   };
-  const size_t od = part((size_t)16 * n * kc), os = part(sizeof(EmuScale)), ost = os + sizeof(EmuScale);
+  const size_t od = part((size_t)2 * kEmuStored * n * kc), os = part(sizeof(EmuScale)), ost = os + sizeof(EmuScale);
   // scale, status (both zero) and the tile lists go over in one copy
   size_t oi[2], og[2];
   for (int q = 0; q < 2; ++q) {
@@ -225,8 +227,8 @@ cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, doub
                                           (unsigned long long)g[q].blocks, 1};
       const unsigned long long str[3] = {rb * g[q].row_stride, rb * g[q].block_stride, rb * n};
       const unsigned ba[3] = {128, 1, 1}, bb[3] = {(unsigned)w[q], 1, 1};
-      if (!emu_encode_map(&maps.m[0], dig, dims, str, rb * n, ba, kEmuSlices, err) ||
-          !emu_encode_map(&maps.m[1], dig, dims, str, rb * n, bb, kEmuSlices, err)) {
+      if (!emu_encode_map(&maps.m[0], dig, dims, str, rb * n, ba, kEmuStored, err) ||
+          !emu_encode_map(&maps.m[1], dig, dims, str, rb * n, bb, kEmuStored, err)) {
         e = cudaErrorInvalidValue;
         break;
       }
@@ -240,22 +242,24 @@ cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, doub
       epi.lim2 = epi.nlim = (int)g[q].rows;
       epi.alpha = 0.5;
       epi.n = w[q];
-      epi.ebias = -12;
+      epi.ebias = -14;
       epi.sa = epi.sb = scale;
       e = launch_emu_gemm(kEmuSlices, maps, reinterpret_cast<TcItem *>(base + oi[q]),
                           reinterpret_cast<TcSeg *>(base + og[q]), (int)items[q].size(), epi, status, st);
     }
   }
-  for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+  // the sums are added where all of them hold (the host waits here anyway)
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, status, sizeof(int), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  for (int q = 0; q < 2 && e == cudaSuccess && hst == 0; ++q) {
     fold_kernel<<<(unsigned)((g[q].rows * g[q].rows + 255) / 256), 256, 0, st>>>(
         g[q].out, g[q].rows, reinterpret_cast<double *>(base + oc[q]), g[q].copies);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, status, sizeof(int), cudaMemcpyDeviceToHost, st);
   work_free(mem, st);
   const cudaError_t e2 = cudaStreamSynchronize(st);
   if (e == cudaSuccess) e = e2;
-  *timeout = (hst & kStatusTimeout) != 0;
+  *hstatus = hst;
   return e;
 }
 
@@ -306,16 +310,17 @@ extern "C" int mlcc3_cnto_matrices(int64_t n_occ, int64_t n_vir, const double *R
   //          N_ab += 1/2 sum_{(i,c,j)} R2[a][(i,c,j)] R2[b][(i,c,j)]
   // (the singles' parts are symmetric, so mirroring the sums keeps them)
   std::string err;
-  bool done = false, timeout = false;
+  bool done = false;
+  int status = 0;
   if (e == cudaSuccess && NO * NV < (1LL << 20)) {
-    e = doubles_by_digits(NO, NV, R2, M, N, st, &timeout, &err);
-    done = e == cudaSuccess;
+    e = doubles_by_digits(NO, NV, R2, M, N, st, &status, &err);
+    done = e == cudaSuccess && status == 0;
     if (e == cudaErrorMemoryAllocation) {  // no room for a workspace: the FP64 kernel needs none
       cudaGetLastError();
       e = cudaSuccess;
     }
   }
-  if (timeout) {
+  if (status & mlcc3::kStatusTimeout) {
     mlcc3::set_last_error("mlcc3_cnto_matrices: a tensor-core pipeline wait timed out");
     return MLCC3_ERR_TIMEOUT;
   }

@@ -26,6 +26,10 @@ struct Error {
 
 void check_cuda(cudaError_t e, const char *what);
 
+// An Error code inside the library: a digit product met operands of too wide a range
+// (kStatusSpread); the call runs again on the FP64 pipe.
+constexpr int kErrSpread = -1000;
+
 // Shapes of a batched strided contraction: m = (M1,M2), n = (N1,N2), k = (K1,K2,K3).
 struct Shape {
   long long M1 = 1, M2 = 1, N1 = 1, N2 = 1, K1 = 1, K2 = 1, K3 = 1;
@@ -172,8 +176,13 @@ struct mlcc3_ctx {
   };
   std::map<std::string, SplitOp> splits;
   // FP64 mode: the large contractions on the tensor cores (kernels_emu.cuh), from
-  // fp64_tc_from on (choose_emu); the names of the operands' scales
-  bool emu = false;
+  // fp64_tc_from on (emu_rule, by choose_emu); the names of the operands' scales.  A call
+  // whose operands the digits cannot hold to FP64 accuracy, or whose digits find no room,
+  // runs again on the FP64 pipe, where the context stays (emu = false) until the next
+  // integral build
+  bool emu = false, emu_rule = false;
+  void leave_digits();
+  int path_gen = 0;  // counts leave_digits: a sweep's graph of before is stale
   long long fp64_tc_from = 24;
   std::map<std::string, int> scales;
   // split layouts of triples arrays, converted once per (array, write
@@ -194,8 +203,11 @@ struct mlcc3_ctx {
     auto it = gens.find(p);
     return it == gens.end() ? 0ULL : it->second;
   }
-  // output copies back to host pointers at the end of a call
+  // output copies to host pointers, and to device outputs that overlap an input of a call
+  // that may have to run again (on the FP64 pipe), at the end of a call; its device inputs
   std::vector<std::array<void *, 3>> pending_out;
+  std::vector<std::pair<const char *, size_t>> ins;
+  bool may_rerun = false;
 
   // launch accounting: every kernel launch is counted; with profiling on,
   // CUDA events bracket each launch on the context's stream.

@@ -3,7 +3,8 @@
 // integer of up to 63 bits per element (its value over one power of two), held
 // as S balanced base-256 digits, each exact in bfloat16.  Products of digits
 // are integers of at most 2^14, which FP32 sums exactly over 256 of them for
-// the digit degrees t + u <= 3; degrees of S and more are dropped.
+// the digit degrees t + u <= 3.  Kept are the degrees up to S - 1, and with S = 8 (the
+// FP64 mode) up to 8, which leaves out terms below 2^-69 of full scale per product.
 //
 // GB300 retires about two FP64 operations per clock and SM (1.1 TFLOP/s in
 // all), and BF16 on the tensor cores about 1.7 PFLOP/s, so even the 36 digit
@@ -20,7 +21,8 @@ namespace mlcc3 {
 
 namespace {
 
-constexpr int kChain = 256 / kEmuKB;  // chunks per TMEM accumulation chain (exact up to 256 products)
+// chunks per TMEM accumulation chain
+template <int S> constexpr int kChainOf = S == kEmuSlices ? kEmuChain : 256 / kEmuKB;
 constexpr int kRowB = 2 * kEmuKB;     // bytes of a shared-memory operand row
 
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
@@ -64,7 +66,39 @@ __device__ __forceinline__ double int_to_double(long long T, int e) {
   return __longlong_as_double((long long)((((unsigned long long)(ex - 1) << 52) + m) | sgn));
 }
 
-__device__ __forceinline__ int scale_exp(EmuScale s) { return (int)((s >> 52) & 0x7ff) - 1022; }
+// (T + M 2^-32) 2^e, rounded to binary64 once (to nearest, ties to even).
+__device__ __forceinline__ double sum_to_double(long long T, long long M, int e) {
+  unsigned long long h = (unsigned long long)(T + (M >> 32)), l = (unsigned long long)M << 32;
+  const unsigned long long sgn = h & (1ULL << 63);
+  if (sgn) {
+    h = ~h + (l == 0 ? 1 : 0);
+    l = 0ULL - l;
+  }
+  if (h == 0) {
+    if (l == 0) return 0.0;
+    h = l;
+    l = 0;
+    e -= 64;
+  }
+  const int lz = __clzll((long long)h);
+  if (lz) {
+    h = (h << lz) | (l >> (64 - lz));
+    l <<= lz;
+  }
+  const int ex = e - lz + 63 + 1023;
+  if (ex < 1 || ex > 2045) {
+    const double v = ldexp((double)h, e - lz);
+    return sgn ? -v : v;
+  }
+  unsigned long long m = h >> 11;
+  const unsigned rest = (unsigned)h & 2047u;
+  if (rest > 1024u || (rest == 1024u && (l != 0 || (m & 1)))) ++m;
+  return __longlong_as_double((long long)((((unsigned long long)(ex - 1) << 52) + m) | sgn));
+}
+
+__device__ __forceinline__ int scale_exp(EmuScale s) {
+  return (int)(((s + (1ULL << 46)) >> 52) & 0x7ff) - 1022;
+}
 
 }  // namespace
 
@@ -73,15 +107,20 @@ __device__ __forceinline__ int scale_exp(EmuScale s) { return (int)((s >> 52) & 
 //
 // A stage holds 32 K elements of all S slices of both operands.  The slices of
 // B lie one below the other in shared memory, so the MMA of A's slice t with
-// the stacked slices 0 .. S-1-t of B (N = (S - t) n, in pieces of at most 256)
+// the stacked slices of B (N = their number times n, in pieces of at most 256)
 // puts digit pair (t, u) into TMEM columns (t + u) n: one accumulator per digit
-// degree and wide MMAs instead of S (S + 1) / 2 narrow ones.  With S = 8 and
-// n = 64 the eight degrees fill TMEM; a stage is 96 KB, two are in flight.
+// degree and wide MMAs instead of narrow ones per pair.
 //
-// After each chain of 256 K elements eight epilogue warps add the degrees,
-// weighted by 2^-8d, into 64-bit integers in registers (degrees 0..4 exactly, in
-// units of 2^-32: below 2^60 for kEmuMaxK products; the higher ones in FP32 beside
-// them) and hand TMEM back, so the next chain's MMAs wait only for the reads.  An
+// S = 8, the FP64 mode: degrees 0..8 and, in a tenth group of columns, the product of the
+// operands' magnitudes (a ninth slice), which an item accumulates from its first chunk to
+// its last and which says whether the digits hold its outputs to FP64 accuracy
+// (kStatusSpread).  If they do not, the caller runs the call on the FP64 pipe.  With n = 48, 480 of TMEM's 512
+// columns; a stage is 101 KB, two are in flight.
+//
+// After each chain of K elements eight epilogue warps add the degrees, weighted by 2^-8d,
+// into 64-bit integers in registers (degrees 0..4 in units of 2^-32, below 2^60 for
+// kEmuMaxK products; degrees 5..8 in units of 2^-64, below 2^54; S = 6: degree 5 in FP32)
+// and hand TMEM back, so the next chain's MMAs wait only for the reads.  An
 // item's sums are rounded to binary64 once, at its end, on the integer pipe.
 //   warp 0 lane 0: TMA producer; warp 1: TMEM, lane 0 issues; warps 2..9: epilogue
 // C = A B^T with M = N = K = 4096 and S = 5, slicing included: 1.77 ms, against
@@ -94,6 +133,11 @@ __global__ void __launch_bounds__(320, 1)
     emu_gemm_kernel(const __grid_constant__ TcMaps maps, const TcItem *__restrict__ items,
                     const TcSeg *__restrict__ segs, int nitems, int stages, const EmuEpi epi,
                     int *__restrict__ status) {
+  constexpr bool FULL = S == kEmuSlices;       // the FP64 mode
+  constexpr int SL = FULL ? kEmuStored : S;    // slices of a stage
+  constexpr int DG = FULL ? S + 1 : S;         // digit degrees
+  constexpr int GR = FULL ? DG + 1 : S;        // groups of n columns in TMEM
+  constexpr int kChain = kChainOf<S>;
   constexpr int NG = N / 16;  // 8-column groups per epilogue thread
   constexpr int A_SL = 128 * kRowB;         // bytes of one slice of A
   constexpr uint32_t IDESC =
@@ -102,7 +146,7 @@ __global__ void __launch_bounds__(320, 1)
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr int n = N;
-  const int stage_bytes = S * (A_SL + n * kRowB);
+  constexpr int stage_bytes = SL * (A_SL + n * kRowB);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 8);
   const uint32_t tfull = smem_u32(bars + 16), tempty = smem_u32(bars + 17);
@@ -110,7 +154,8 @@ __global__ void __launch_bounds__(320, 1)
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 19);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const uint32_t ncols = S * n <= 128 ? 128u : S * n <= 256 ? 256u : 512u;
+  constexpr uint32_t ncols = GR * n <= 128 ? 128u : GR * n <= 256 ? 256u : 512u;
+  static_assert(GR * n <= 512, "TMEM columns");
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
@@ -154,12 +199,12 @@ __global__ void __launch_bounds__(320, 1)
           mbar_expect_tx(fb, (uint32_t)stage_bytes);
           if constexpr (AMN) {
             for (int h = 0; h < 2; ++h)
-              tma_load_5d(st + h * (S * A_SL / 2), &maps.m[sg.amap], sg.ac[1] + 64 * h,
+              tma_load_5d(st + h * (SL * A_SL / 2), &maps.m[sg.amap], sg.ac[1] + 64 * h,
                           sg.ac[0] + kEmuKB * kc, sg.ac[2], sg.ac[3], 0, fb);
           } else {
             tma_load_5d(st, &maps.m[sg.amap], sg.ac[0] + kEmuKB * kc, sg.ac[1], sg.ac[2], sg.ac[3], 0, fb);
           }
-          tma_load_5d(st + S * A_SL, &maps.m[sg.bmap], sg.bc[0] + kEmuKB * kc, sg.bc[1], sg.bc[2],
+          tma_load_5d(st + SL * A_SL, &maps.m[sg.bmap], sg.bc[0] + kEmuKB * kc, sg.bc[1], sg.bc[2],
                       sg.bc[3], 0, fb);
           last = (last & ~(1u << stage)) | (phase << stage);
           pending |= 1u << stage;
@@ -206,26 +251,38 @@ __global__ void __launch_bounds__(320, 1)
           const bool last = q == s1 - 1 && kc == nk - 1;
           if (leader) {
             const uint32_t a0 = smem_u32(smem) + stage * stage_bytes;
-            const uint64_t ad = AMN ? smem_desc_mn(a0, S * A_SL / 2) : smem_desc64(a0);
-            const uint64_t bd = smem_desc64(a0 + S * A_SL);
+            const uint64_t ad = AMN ? smem_desc_mn(a0, SL * A_SL / 2) : smem_desc64(a0);
+            const uint64_t bd = smem_desc64(a0 + SL * A_SL);
             const int steps = kc == nk - 1 && tail > 0 ? tail : kEmuKB / 16;
 #pragma unroll
             for (int kk = 0; kk < kEmuKB / 16; ++kk) {
               if (kk < steps) {  // zeros to the end of the reduction
+                const uint32_t add = kk > 0 || cc > 0 ? 1u : 0u;  // 0: first of the chain
+                // A's slice t with B's slices [u0, u1) into the degrees t + u0 .. t + u1 - 1
+                auto mmas = [&](int t, int u0, int u1, int group, uint32_t acc) {
+                  constexpr int W = 256, a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
+#pragma unroll
+                  for (int c0 = u0 * n; c0 < u1 * n; c0 += W) {
+                    const int nn = u1 * n - c0 < W ? u1 * n - c0 : W;
+                    mma_bf16(tmem + (uint32_t)((group - u0) * n + c0),
+                             ad + (uint64_t)((t * a_slice + kk * a_step) >> 4),
+                             bd + (uint64_t)((c0 * kRowB + kk * 32) >> 4), IDESC | ((uint32_t)(nn >> 3) << 17), acc);
+                  }
+                };
 #pragma unroll
                 for (int d = 0; d < S; ++d) {
-                  // slice d of A with the stacked slices 0 .. S-1-d of B; the first
-                  // MMA of a chain (d = 0) covers every degree and clears them
-                  constexpr int W = 256;
-#pragma unroll
-                  for (int c0 = 0; c0 < (S - d) * n; c0 += W) {
-                    const int nn = (S - d) * n - c0 < W ? (S - d) * n - c0 : W;
-                    constexpr int a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
-                    mma_bf16(tmem + (uint32_t)(d * n + c0), ad + (uint64_t)((d * a_slice + kk * a_step) >> 4),
-                             bd + (uint64_t)((c0 * kRowB + kk * 32) >> 4), IDESC | ((uint32_t)(nn >> 3) << 17),
-                             kk > 0 || d > 0 ? 1u : (cc > 0 ? 1u : 0u));
+                  // the first MMA of a chain (d = 0) covers every degree up to S - 1 and
+                  // clears them; degree S (FULL) first comes up in the last slice of d = 1
+                  const int u1 = DG - d < S ? DG - d : S;
+                  if (FULL && d == 1 && add == 0) {
+                    mmas(1, 0, S - 1, 1, 1u);
+                    mmas(1, S - 1, S, S, 0u);
+                  } else {
+                    mmas(d, 0, u1, d, d > 0 ? 1u : add);
                   }
                 }
+                if constexpr (FULL)  // magnitudes, over the whole item
+                  mmas(S, S, S + 1, DG, q > s0 || kc > 0 || kk > 0 ? 1u : 0u);
               }
             }
             mma_commit(empty0 + 8 * stage);
@@ -257,16 +314,30 @@ __global__ void __launch_bounds__(320, 1)
       if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const TcItem it = items[i];
       const int chains = (it.chunks + kChain - 1) / kChain;
+      int r1, r2;
+      if (epi.linear) {
+        const int m = it.r2_0 + row;
+        r1 = m / epi.R2;
+        r2 = m % epi.R2;
+      } else {
+        r1 = it.r1_0 + row / epi.R2;
+        r2 = it.r2_0 + row % epi.R2;
+      }
+      const int cmax = r1 < epi.lim1 && r2 < epi.lim2 ? epi.nlim : 0;
+      const int c0 = it.c0 + half * hn;
       long long T[NG * 8];
-      float L[S > 5 ? NG * 8 : 1];
+      long long U[FULL ? NG * 8 : 1];  // degrees 5..8
+      float L[S == 6 ? NG * 8 : 1];    // degree 5
       unsigned nan[NG];
+      bool weak = false;
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
         nan[g] = 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           T[g * 8 + j] = 0;
-          if constexpr (S > 5) L[g * 8 + j] = 0.f;
+          if constexpr (FULL) U[g * 8 + j] = 0;
+          if constexpr (S == 6) L[g * 8 + j] = 0.f;
         }
       }
       for (int ch = 0; ch < chains; ++ch, ++t) {
@@ -280,25 +351,44 @@ __global__ void __launch_bounds__(320, 1)
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
           if (g * 8 < hn) {
-            uint32_t r[S][8];
+            constexpr int D1 = FULL ? 5 : S;  // degrees read at a time (registers)
+            uint32_t r[D1][8];
 #pragma unroll
-            for (int d = 0; d < S; ++d) tmem_ld8(tm + (uint32_t)(d * n + g * 8), r[d]);
+            for (int d = 0; d < D1; ++d) tmem_ld8(tm + (uint32_t)(d * n + g * 8), r[d]);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const float f0 = __uint_as_float(r[0][j]);
-              if (!(f0 == f0)) nan[g] |= 1u << j;
+              if (!FULL && !(f0 == f0)) nan[g] |= 1u << j;
               long long x = T[g * 8 + j];
               x += (long long)((unsigned long long)(uint32_t)__float2int_rn(f0) << 32);
 #pragma unroll
               for (int d = 1; d < (S < 5 ? S : 5); ++d)
                 x += (long long)__float2int_rn(__uint_as_float(r[d][j])) * (1LL << (32 - 8 * d));
               T[g * 8 + j] = x;
-              if constexpr (S > 5) {
-                float l = __uint_as_float(r[S - 1][j]);
+              if constexpr (S == 6) L[g * 8 + j] += __uint_as_float(r[5][j]);
+            }
+            if constexpr (FULL) {
 #pragma unroll
-                for (int d = S - 2; d >= 5; --d) l = fmaf(l, 0x1p-8f, __uint_as_float(r[d][j]));
-                L[g * 8 + j] += l;
+              for (int d = 0; d < 4; ++d) tmem_ld8(tm + (uint32_t)((5 + d) * n + g * 8), r[d]);
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                long long x = U[g * 8 + j];
+#pragma unroll
+                for (int d = 0; d < 4; ++d)
+                  x += (long long)__float2int_rn(__uint_as_float(r[d][j])) * (1LL << (24 - 8 * d));
+                U[g * 8 + j] = x;
+              }
+              if (ch == chains - 1) {
+                const float least = (float)it.chunks * (kEmuKB * kEmuLeast);
+                tmem_ld8(tm + (uint32_t)(DG * n + g * 8), r[4]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const float m = __uint_as_float(r[4][j]);
+                  weak = weak || (c0 + g * 8 + j < cmax && !(m >= least) && m != 0.f);
+                }
               }
             }
           }
@@ -308,17 +398,7 @@ __global__ void __launch_bounds__(320, 1)
         if (lane == 0) mbar_arrive(tempty);
       }
       if (!ok) break;
-      int r1, r2;
-      if (epi.linear) {
-        const int m = it.r2_0 + row;
-        r1 = m / epi.R2;
-        r2 = m % epi.R2;
-      } else {
-        r1 = it.r1_0 + row / epi.R2;
-        r2 = it.r2_0 + row % epi.R2;
-      }
-      const int cmax = r1 < epi.lim1 && r2 < epi.lim2 ? epi.nlim : 0;
-      const int c0 = it.c0 + half * hn;
+      if (FULL && __any_sync(0xffffffffu, weak) && lane == 0) atomicOr(status, kStatusSpread);
       const int er = epi.ea && cmax ? e0 + epi.ea[it.r2_0 + row] : e0;
       double *o = epi.out + it.out_off + (long long)r1 * epi.s1 + (long long)r2 * epi.s2 + (long long)c0 * epi.sn;
 #pragma unroll
@@ -330,15 +410,20 @@ __global__ void __launch_bounds__(320, 1)
           if (c0 + c >= cmax) break;
           long long x = T[c];
           int ex = epi.eb ? er + epi.eb[c0 + c] : er;
-          if constexpr (S > 5) {
-            // T moved up as far as it goes, so that the higher degrees (|L| < 2^30,
-            // in 2^-8 of T's unit) join it below its own 53 leading bits
-            const int sh = min(24, __clzll(x < 0 ? -x : x) - 2);
-            x = (x << sh) + __float2ll_rn(L[c] * __int_as_float((127 + sh - 8) << 23));
-            ex -= sh;
+          double v;
+          if constexpr (FULL) {
+            v = sum_to_double(x, U[c], ex);
+          } else {
+            if constexpr (S == 6) {
+              // T moved up as far as it goes, so that the degree above (|L| < 2^30,
+              // in 2^-8 of T's unit) joins it below its own 53 leading bits
+              const int sh = min(24, __clzll(x < 0 ? -x : x) - 2);
+              x = (x << sh) + __float2ll_rn(L[c] * __int_as_float((127 + sh - 8) << 23));
+              ex -= sh;
+            }
+            v = int_to_double(x, ex);
+            if ((nan[g] >> j) & 1u) v = __longlong_as_double(0x7ff8000000000000LL);
           }
-          double v = int_to_double(x, ex);
-          if ((nan[g] >> j) & 1u) v = __longlong_as_double(0x7ff8000000000000LL);
           if (epi.alpha != 1.0) v = epi.alpha == -1.0 ? -v : epi.alpha * v;
           double *p = o + (long long)c * epi.sn;
           if (epi.mode == 0) *p = v;
@@ -361,10 +446,10 @@ __global__ void __launch_bounds__(320, 1)
 // The width that wastes least: columns of all tiles, and as much as eight columns
 // per tile for reading A again.
 int emu_tile_width(long long n, int S) {
-  const int w8[] = {16, 32, 48, 64}, ws[] = {32, 80};
+  const int w8[] = {16, 32, 48}, ws[] = {32, 80};
   int best = 0;
   long long cost = 0;
-  for (int i = 0; i < (S == 8 ? 4 : 2); ++i) {
+  for (int i = 0; i < (S == 8 ? 3 : 2); ++i) {
     const int w = S == 8 ? w8[i] : ws[i];
     const long long c = (n + w - 1) / w * (w + 8);
     if (!best || c <= cost) {
@@ -407,7 +492,7 @@ bool emu_encode_map(CUtensorMap *m, const void *base, const unsigned long long d
 template <int S, int N, bool AMN = false>
 static cudaError_t launch_sn(const TcMaps &maps, const TcItem *items, const TcSeg *segs, int nitems,
                             const EmuEpi &epi, int *status, cudaStream_t st) {
-  const int stage = S * (128 + epi.n) * kRowB;
+  const int stage = (S == kEmuSlices ? kEmuStored : S) * (128 + epi.n) * kRowB;
   const int stages = std::max(2, std::min(6, (220 * 1024) / stage));
   const int smem = 1024 + stages * stage + 256;
   cudaError_t e = cudaFuncSetAttribute(emu_gemm_kernel<S, N, AMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -428,7 +513,6 @@ cudaError_t launch_emu_gemm(int S, const TcMaps &maps, const TcItem *items, cons
     EMU_CASE2(16);
     EMU_CASE2(32);
     EMU_CASE2(48);
-    EMU_CASE2(64);
     EMU_CASE(2, 32);
     EMU_CASE(2, 80);
     EMU_CASE(3, 32);
@@ -487,39 +571,44 @@ cudaError_t emu_absmax(const double *x, long long n, EmuScale *scale, cudaStream
   return cudaGetLastError();
 }
 
-__global__ void emu_balance_kernel(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u) {
+__global__ void emu_balance_kernel(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u,
+                                   int *status) {
   const int eg = scale_exp(*g), et = scale_exp(*t);
-  const int ea = max(scale_exp(*a), et + scale_exp(*u) - eg), eu = ea + eg - et;
+  const bool tu = *t != 0 && *u != 0;
+  const int ea = tu ? max(scale_exp(*a), et + scale_exp(*u) - eg) : scale_exp(*a), eu = ea + eg - et;
+  if (tu && (ea > 1024 || eu > 1024 || ea < -1022 || eu < -1022)) atomicOr(status, kStatusSpread);
   auto pack = [](int e) { return (EmuScale)min(2046, max(0, e + 1022)) << 52; };
   *a = pack(ea);
   *u = pack(eu);
 }
 
-cudaError_t emu_balance(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u, cudaStream_t st) {
-  emu_balance_kernel<<<1, 1, 0, st>>>(a, g, t, u);
+cudaError_t emu_balance(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u, int *status,
+                        cudaStream_t st) {
+  emu_balance_kernel<<<1, 1, 0, st>>>(a, g, t, u, status);
   return cudaGetLastError();
 }
 
-__global__ void emu_scale_double_kernel(EmuScale *s) {
+__global__ void emu_scale_double_kernel(EmuScale *s, int *status) {
+  if (scale_exp(*s) > 1023) atomicOr(status, kStatusSpread);
   *s = (EmuScale)min(2046, scale_exp(*s) + 1023) << 52;
 }
 
-cudaError_t emu_scale_double(EmuScale *scale, cudaStream_t st) {
-  emu_scale_double_kernel<<<1, 1, 0, st>>>(scale);
+cudaError_t emu_scale_double(EmuScale *scale, int *status, cudaStream_t st) {
+  emu_scale_double_kernel<<<1, 1, 0, st>>>(scale, status);
   return cudaGetLastError();
 }
 
 // ---- digits ----
-// x over 2^(e - 62), rounded to nearest: an integer of at most 62 bits for |x| < 2^e.
-__device__ __forceinline__ long long to_fixed62(double x, int e) {
+// x over 2^(e - 63), rounded to nearest: an integer below 2^63 - 2^56 for a scale's e.
+__device__ __forceinline__ long long to_fixed63(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   int ex = (int)((b >> 52) & 0x7ff);
   unsigned long long m = b & ((1ULL << 52) - 1);
   if (ex) m |= 1ULL << 52;
   else ex = 1;
-  const int s = ex - 1013 - e;  // m 2^(ex - 1075) 2^(62 - e)
+  const int s = ex - 1012 - e;  // m 2^(ex - 1075) 2^(63 - e)
   unsigned long long q;
-  if (s >= 0) q = m << min(s, 9);
+  if (s >= 0) q = m << min(s, 10);
   else if (s > -55) q = (m + (1ULL << (-s - 1))) >> -s;
   else q = 0;
   return (b >> 63) ? -(long long)q : (long long)q;
@@ -528,10 +617,10 @@ __device__ __forceinline__ long long to_fixed62(double x, int e) {
 // Tiles of 32 rows x 64 K elements pass through shared memory, so that the loads
 // run along whichever index is contiguous in the source; each thread then makes
 // the digits of eight consecutive K elements of a row and writes 16 bytes of
-// every slice.  The digits of the 62-bit integer q are the bytes of
-// q + 0x0080..80, minus 128 each (the top byte: q's own, in [-64, 64]); a byte
+// every slice.  The digits of the integer q are the bytes of
+// q + 0x0080..80, minus 128 each (the top byte: q's own, in [-127, 127]); a byte
 // becomes a bfloat16 through the FP32 number 2^23 + byte.  Bound by HBM: 8 bytes
-// read and 16 written per element.
+// read and 18 written per element.
 __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp, long long slice,
                                                          int neg, const EmuScale *scale,
                                                          __nv_bfloat16 *__restrict__ out,
@@ -583,16 +672,22 @@ __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp
     __syncthreads();
     const int r = tid / 8, kg = (tid % 8) * 8;
     if (r0 + r < v.R && k0 + kg < Kp) {
-      unsigned lo[8], hi[8];
-      unsigned bad = 0;
+      unsigned lo[8], hi[8], mag[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         double y = sm[r][kg + j];
-        if (!(fabs(y) <= 1.7976931348623157e308)) {
-          bad |= 1u << j;
+        // |y| 2^-e in binary32 (20 bits of it), less c, in bfloat16
+        const unsigned h = (unsigned)__double2hiint(y) & 0x7fffffffu;
+        const int k = (int)(h >> 20) - 1023 - e;
+        const float m = k < -100 ? 0.f : __uint_as_float(((unsigned)(127 + k) << 23) | ((h & 0xfffffu) << 3));
+        mag[j] = __float_as_uint(m - kEmuRound) >> 16;
+        if (m == kEmuRound) mag[j] = (127u - 40u) << 7;
+        if ((h | (unsigned)__double2loint(y)) == 0) mag[j] = 0u;
+        if (h >= 0x7ff00000u) {
           y = 0.0;
+          mag[j] = 0x7fc0u;
         }
-        long long q = to_fixed62(y, e);
+        long long q = to_fixed63(y, e);
         if (neg) q = -q;
         const unsigned long long w =
             ((unsigned long long)q + 0x0080808080808080ULL) ^ 0x8000000000000000ULL;
@@ -612,13 +707,10 @@ __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp
           const float fb = __uint_as_float(__byte_perm(wb, 0x4B000000u, sel)) - 8388736.f;
           p[j] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
         }
-        if (s == 0 && bad) {  // a non-finite element makes its products NaN
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if ((bad >> j) & 1u) p[j / 2] = (p[j / 2] & (j & 1 ? 0x0000ffffu : 0xffff0000u)) | (j & 1 ? 0x7fc00000u : 0x7fc0u);
-        }
         o[s * st] = make_uint4(p[0], p[1], p[2], p[3]);
       }
+      o[8 * st] = make_uint4(mag[0] | mag[1] << 16, mag[2] | mag[3] << 16, mag[4] | mag[5] << 16,
+                             mag[6] | mag[7] << 16);
     }
   }
 }

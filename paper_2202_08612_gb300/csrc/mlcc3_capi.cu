@@ -157,6 +157,30 @@ void mlcc3_ctx::release() {
   tau_key.clear();
 }
 
+// From the tensor cores to the FP64 pipe: the digits' memory is given back, and nothing
+// that a failed call left behind is used again.
+void mlcc3_ctx::leave_digits() {
+  check_cuda(cudaStreamSynchronize(stream), "sync before the FP64 pipe");
+  cudaGetLastError();
+  emu = false;
+  path_gen += 1;
+  for (auto it = scratch.begin(); it != scratch.end();) {
+    if (it->first.compare(0, 7, "digits:") != 0) {
+      ++it;
+      continue;
+    }
+    cudaFree(it->second.first);
+    it = scratch.erase(it);
+  }
+  splits.clear();
+  for (TriSlot &t : tri) t = TriSlot{};
+  tau_valid = false;
+  tau_key.clear();
+  dld_pending.clear();
+  pending_out.clear();
+  omega_dev = nullptr;
+}
+
 double *mlcc3_ctx::buf(const std::string &name, size_t n) {
   return static_cast<double *>(raw(name, n * sizeof(double)));
 }
@@ -237,7 +261,10 @@ static bool is_device_ptr(const void *p) {
 
 const double *mlcc3_ctx::in(const double *p, size_t n, const std::string &name) {
   if (p == nullptr) throw Error{MLCC3_ERR_ARG, "null input array: " + name};
-  if (is_device_ptr(p)) return p;
+  if (is_device_ptr(p)) {
+    if (may_rerun) ins.push_back({reinterpret_cast<const char *>(p), n * sizeof(double)});
+    return p;
+  }
   double *d = buf("in:" + name, n);
   check_cuda(cudaMemcpyAsync(d, p, n * sizeof(double), cudaMemcpyHostToDevice, stream),
              "stage input");
@@ -246,20 +273,27 @@ const double *mlcc3_ctx::in(const double *p, size_t n, const std::string &name) 
 
 double *mlcc3_ctx::out(double *p, size_t n, const std::string &name) {
   if (p == nullptr) throw Error{MLCC3_ERR_ARG, "null output array: " + name};
-  if (is_device_ptr(p)) return p;
+  if (is_device_ptr(p)) {
+    const char *q = reinterpret_cast<const char *>(p);
+    bool over = false;
+    for (auto &i : ins) over = over || (q < i.first + i.second && i.first < q + n * sizeof(double));
+    if (!over) return p;
+  }
   double *d = buf("out:" + name, n);
   pending_out.push_back({(void *)p, (void *)d, (void *)(n * sizeof(double))});
   return d;
 }
 
 void mlcc3_ctx::finish() {
-  for (auto &o : pending_out)
-    check_cuda(cudaMemcpyAsync(o[0], o[1], (size_t)o[2], cudaMemcpyDeviceToHost, stream),
-               "copy output");
-  pending_out.clear();
   int st = 0;
   check_cuda(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, stream),
              "read status");
+  // a call that has to run again leaves the outputs, which may be its inputs, alone
+  if (may_rerun && !pending_out.empty()) check_cuda(cudaStreamSynchronize(stream), "synchronize");
+  if (!(st & kStatusSpread))
+    for (auto &o : pending_out)
+      check_cuda(cudaMemcpyAsync(o[0], o[1], (size_t)o[2], cudaMemcpyDefault, stream), "copy output");
+  pending_out.clear();
   check_cuda(cudaStreamSynchronize(stream), "synchronize");
   check_cuda(cudaGetLastError(), "kernel launch");
   collect_events();
@@ -269,6 +303,10 @@ void mlcc3_ctx::finish() {
     tau_valid = false;
     tau_key.clear();
     throw Error{MLCC3_ERR_TIMEOUT, "a tensor-core pipeline wait timed out"};
+  }
+  if (st & kStatusSpread) {
+    check_cuda(cudaMemsetAsync(status, 0, sizeof(int), stream), "reset status");
+    throw Error{kErrSpread, "operands of too wide a range for digit products"};
   }
   if (st & 1) {
     check_cuda(cudaMemsetAsync(status, 0, sizeof(int), stream), "reset status");
@@ -564,8 +602,8 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
 }
 
 // FP64 mode: the O(N_V n_v^3 n_o^3) contractions on the tensor cores (digit
-// slices; rho and sigma at 20/200/12/60: 1868 -> 61 ms, the densities at
-// 13/101/7/37: 79 -> 5.4 ms, errors against 64 bits as before or smaller) from
+// slices; rho and sigma at 20/200/12/60: 1868 -> 82 ms, the densities at
+// 13/101/7/37: 79 -> 6.0 ms, errors against 64 bits as before or smaller) from
 // fp64_tc_from (24) active virtual orbitals or n_o n_v = 3 fp64_tc_from on (rho and sigma,
 // FP64 pipe against digits: 4/12 0.85 against 1.15 ms, 4/16 1.34 and 1.32, 6/12 1.79 and
 // 1.20, 8/16 4.66 and 1.67, 3/24 1.87 and 1.63; below, a call is launches, and the digits
@@ -574,14 +612,14 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
 // amplitudes at 16 bytes an element) leave most of the memory free.
 void choose_emu(mlcc3_ctx *c) {
   S s(c);
-  c->emu = false;
+  c->emu_rule = false;
   if (c->precision != MLCC3_FP64 || s.no < 2) return;
   if (s.nv < c->fp64_tc_from && s.no * s.nv < 3 * c->fp64_tc_from) return;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return;
   const double digits = 16.0 * (8.0 * (double)s.gvsz() + 3.0 * (double)s.NJ * (double)(s.nv * s.NV) +
                                 4.0 * (double)s.blk() + 4.0 * (double)(s.no * s.nv * s.nv * s.NO));
-  c->emu = digits < 0.25 * (double)fr;
+  c->emu_rule = digits < 0.25 * (double)fr;
 }
 
 // Split the unique batches into chunks of at most chunk_blocks blocks (or, when
@@ -1045,7 +1083,7 @@ TcDev tc_plan(mlcc3_ctx *c, const std::string &key0, const std::function<void(Tc
     // so where they are cut is free, and an item costs an epilogue
     long long total = 0;
     for (const TcSeg &g : pl.segs) total += g.nk;
-    constexpr int chain = 256 / kEmuKB;
+    constexpr int chain = kEmuChain;
     cap = (int)std::min<long long>(cap, std::max<long long>(1, total / (152LL * 4 * chain)) * chain);
   }
   cap_chains(pl, cap, kblk(c));
@@ -1095,7 +1133,7 @@ void tc_launch(mlcc3_ctx *c, const char *site, int BN, const TcMaps &maps, const
     x.alpha = (double)epi.alpha;
     x.n = BN;
     x.amn = epi.amn;
-    x.ebias = -12;
+    x.ebias = -14;
     x.sa = A.scale;
     x.sb = B.scale;
     x.wait = c->tc_wait;
@@ -1139,10 +1177,10 @@ TcEpi make_epi(void *out, int mode, int R2, long long s1, long long s2, long lon
 void make_digits(mlcc3_ctx *c, SplitOp &op, const std::string &key, const EmuView &v, long long Kp,
                  bool neg, const std::string &slot, const double *F = nullptr, double fcoef = 0.0,
                  bool swap = false) {
-  op.S = kEmuSlices;
+  op.S = kEmuStored;
   op.slice = (long long)v.Z * v.R * Kp;
   op.scale = scale_of(c, slot);
-  op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuSlices * 2);
+  op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuStored * 2);
   op.lo = nullptr;
   c->launch("emu_digits_kernel", 0.0, [&] {
     check_cuda(emu_digits(v, Kp, neg, op.scale, static_cast<__nv_bfloat16 *>(op.hi), F, fcoef, swap,
@@ -1541,7 +1579,7 @@ void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const std::
     check_cuda(cudaMemsetAsync(d, 0, sizeof(EmuScale), c->stream), "scale");
     check_cuda(emu_absmax(G, (long long)s.gvsz(), d, c->stream), "emu_absmax");
     check_cuda(emu_absmax(F, s.no * s.nv, d, c->stream), "emu_absmax");
-    check_cuda(emu_scale_double(d, c->stream), "emu_scale_double");
+    check_cuda(emu_scale_double(d, c->status, c->stream), "emu_scale_double");
   }
   for (int swap = 0; swap < 2; ++swap) {
     const std::string k2 = key + (swap ? ":Ts" : ":T");
@@ -1643,7 +1681,7 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
 }
 
 // hi/lo buffers of layout XL_k of the triples array X (chunk_nb blocks), converted
-// at most once per write of X.  FP64 mode: the digit slices, three arrays kept (48
+// at most once per write of X.  FP64 mode: the digit slices, three arrays kept (54
 // bytes per element each).
 void tri_layout(mlcc3_ctx *c, const double *X, int k, SplitOp &op) {
   S s(c);
@@ -1676,10 +1714,10 @@ void tri_layout(mlcc3_ctx *c, const double *X, int k, SplitOp &op) {
     if (convert) {
       make_digits(c, op, base, v, Kp, false, "tri" + std::to_string(q));
     } else {
-      op.S = kEmuSlices;
+      op.S = kEmuStored;
       op.slice = (long long)v.Z * v.R * Kp;
       op.scale = scale_of(c, "tri" + std::to_string(q));
-      op.hi = c->raw("digits:" + base, (size_t)op.slice * kEmuSlices * 2);
+      op.hi = c->raw("digits:" + base, (size_t)op.slice * kEmuStored * 2);
       op.lo = nullptr;
     }
     return;
@@ -2311,7 +2349,7 @@ void right_triples(mlcc3_ctx *c, const double *Rbar, const double *Rbl, const Up
     scale_max(c, rslot, {{Rbar, (long long)s.blk()}});
     scale_max(c, uslot, {{u.Uv, (long long)s.gvsz()}, {u.Uo, (long long)s.gosz()}});
     check_cuda(emu_balance(scale_of(c, rslot), scale_of(c, "G"), scale_of(c, "t"), scale_of(c, uslot),
-                           c->stream), "emu_balance");
+                           c->status, c->stream), "emu_balance");
   }
   SplitTerm d1 = split_d(c, "Rbar" + tag, Rbar, convert, "Gv", c->Gv, false, rslot, "G");
   SplitTerm l1 = split_l(c, "Rbarl" + tag, Rbl, convert, "Go", c->Go, false, rslot, "G");
@@ -3310,6 +3348,33 @@ static int guarded(F &&f) {
   }
 }
 
+// A call on a context, f() and the wait for its results: on the tensor cores' digits where
+// the context uses them and the operands allow it, else on the FP64 pipe.
+template <class F>
+static void run_call(mlcc3_ctx *c, F &&f) {
+  if (c->emu) {
+    struct MayRerun {
+      mlcc3_ctx *c;
+      explicit MayRerun(mlcc3_ctx *x) : c(x) { c->may_rerun = true; }
+      ~MayRerun() {
+        c->may_rerun = false;
+        c->ins.clear();
+      }
+    };
+    try {
+      MayRerun guard(c);
+      f();
+      c->finish();
+      return;
+    } catch (const Error &e) {
+      if (e.code != kErrSpread && e.code != MLCC3_ERR_OOM) throw;
+    }
+    c->leave_digits();
+  }
+  f();
+  c->finish();
+}
+
 extern "C" const char *mlcc3_last_error(void) { return g_last_error.c_str(); }
 
 extern "C" int mlcc3_create(mlcc3_ctx **out, const mlcc3_dims *d, int precision,
@@ -3360,6 +3425,7 @@ extern "C" int mlcc3_create(mlcc3_ctx **out, const mlcc3_dims *d, int precision,
       check_cuda(cudaMalloc(&c->status, sizeof(int)), "cudaMalloc status");
       check_cuda(cudaMemset(c->status, 0, sizeof(int)), "memset status");
       choose_emu(c);
+      c->emu = c->emu_rule;
       make_batches(c);
       make_chunks(c);
     } catch (...) {
@@ -3400,8 +3466,8 @@ extern "C" int mlcc3_build_integrals(mlcc3_ctx *c, const double *chol, const dou
   return guarded([&] {
     if (!c) throw Error{MLCC3_ERR_ARG, "null context"};
     try {
-      do_build_integrals(c, chol, t1, eps, t2c, t2x);
-      c->finish();
+      c->emu = c->emu_rule;
+      run_call(c, [&] { do_build_integrals(c, chol, t1, eps, t2c, t2x); });
     } catch (...) {
       c->built = false;  // the integral blocks may be incomplete
       throw;
@@ -3412,8 +3478,7 @@ extern "C" int mlcc3_build_integrals(mlcc3_ctx *c, const double *chol, const dou
 extern "C" int mlcc3_triples_omega(mlcc3_ctx *c, double *omega1, double *omega2) {
   return guarded([&] {
     require_built(c);
-    do_triples_omega(c, omega1, omega2);
-    c->finish();
+    run_call(c, [&] { do_triples_omega(c, omega1, omega2); });
   });
 }
 
@@ -3424,8 +3489,7 @@ extern "C" int mlcc3_jacobian_right(mlcc3_ctx *c, int n_vec, const double *omega
     require_built(c);
     if (n_vec < 0 || (n_vec > 0 && !omega)) throw Error{MLCC3_ERR_ARG, "bad n_vec/omega"};
     if (n_vec == 0) return;
-    do_jacobian_right(c, n_vec, omega, R1, R2, rho1, rho2);
-    c->finish();
+    run_call(c, [&] { do_jacobian_right(c, n_vec, omega, R1, R2, rho1, rho2); });
   });
 }
 
@@ -3436,8 +3500,7 @@ extern "C" int mlcc3_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega,
     require_built(c);
     if (n_vec < 0 || (n_vec > 0 && !omega)) throw Error{MLCC3_ERR_ARG, "bad n_vec/omega"};
     if (n_vec == 0) return;
-    do_jacobian_left(c, n_vec, omega, L1, L2, sigma1, sigma2);
-    c->finish();
+    run_call(c, [&] { do_jacobian_left(c, n_vec, omega, L1, L2, sigma1, sigma2); });
   });
 }
 
@@ -3447,8 +3510,7 @@ extern "C" int mlcc3_transition_density(mlcc3_ctx *c, double omega, const double
                                         double *D00_T, double *Dm0_T, double *D0m_T) {
   return guarded([&] {
     require_built(c);
-    do_transition_density(c, 1, &omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T, D0m_T);
-    c->finish();
+    run_call(c, [&] { do_transition_density(c, 1, &omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T, D0m_T); });
   });
 }
 
@@ -3460,9 +3522,8 @@ extern "C" int mlcc3_transition_densities(mlcc3_ctx *c, int n_states, const doub
   return guarded([&] {
     require_built(c);
     if (n_states < 1 || !omega) throw Error{MLCC3_ERR_ARG, "bad n_states/omega"};
-    do_transition_density(c, n_states, omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T,
-                          D0m_T);
-    c->finish();
+    run_call(c, [&] { do_transition_density(c, n_states, omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T,
+                          D0m_T); });
   });
 }
 
@@ -3470,8 +3531,7 @@ extern "C" int mlcc3_ground_density(mlcc3_ctx *c, const double *lam1, const doub
                                     double *D00) {
   return guarded([&] {
     require_built(c);
-    do_ground_density(c, lam1, lam2, D00);
-    c->finish();
+    run_call(c, [&] { do_ground_density(c, lam1, lam2, D00); });
   });
 }
 
@@ -3485,8 +3545,7 @@ extern "C" int mlcc3_multiplier_transformation(mlcc3_ctx *c, const double *lam1,
     const bool cvs = c->cvs;
     c->cvs = false;
     try {
-      do_jacobian_left(c, 1, &zero, lam1, lam2, eta1, eta2);
-      c->finish();
+      run_call(c, [&] { do_jacobian_left(c, 1, &zero, lam1, lam2, eta1, eta2); });
     } catch (...) {
       c->cvs = cvs;
       throw;
@@ -3503,8 +3562,7 @@ extern "C" int mlcc3_rayleigh_quotient(mlcc3_ctx *c, double omega, const double 
     if (!R1 || !R2 || !L1 || !L2 || !omega_rq) throw Error{MLCC3_ERR_ARG, "null argument"};
     if (!(std::fabs(omega) < 1e300) || !(std::fabs(sd_part) < 1e300))
       throw Error{MLCC3_ERR_ARG, "omega or sd_part is not finite"};
-    do_rayleigh(c, omega, R1, R2, L1, L2, sd_part, omega_rq);
-    c->finish();
+    run_call(c, [&] { do_rayleigh(c, omega, R1, R2, L1, L2, sd_part, omega_rq); });
   });
 }
 
@@ -3589,9 +3647,12 @@ extern "C" int mlcc3_set_param(mlcc3_ctx *c, const char *name, long long value) 
       if (value < 1 || value > (1LL << 30)) throw Error{MLCC3_ERR_ARG, "fp64_tc_from must be 1..2^30"};
       c->fp64_tc_from = value;
       if (c->precision == MLCC3_FP64) {
-        const bool was = c->emu;
+        const bool was = c->emu_rule;
         choose_emu(c);
-        if (c->emu != was) c->built = false;  // the operands the integral build prepares differ
+        if (c->emu_rule != was) {
+          c->emu = c->emu_rule;
+          c->built = false;  // the operands the integral build prepares differ
+        }
         make_chunks(c);
       }
     } else if (n == "finish_fused") {
@@ -3692,7 +3753,7 @@ struct mlcc3_sweep {
     double *rho1 = nullptr, *rho2 = nullptr;
     long long w0 = 0;  // first frequency of this system in the omega array
     unsigned long long build_gen = 0;
-    int chunk_gen = 0;
+    int chunk_gen = 0, path_gen = 0;
     int fill = 4;
     std::vector<double> fill_ms;  // tuning times per candidate
     // tensor-core choices of the split mode and their tuning times
@@ -3793,7 +3854,8 @@ void sweep_check_status(mlcc3_sweep *sw) {
   if (bits) {
     for (auto &y : sw->sys) check_cuda(cudaMemsetAsync(y.c->status, 0, sizeof(int), sw->s0), "reset");
     check_cuda(cudaStreamSynchronize(sw->s0), "sweep sync");
-    if (bits & 2) throw Error{MLCC3_ERR_TIMEOUT, "tensor-core pipeline wait timed out"};
+    if (bits & kStatusTimeout) throw Error{MLCC3_ERR_TIMEOUT, "tensor-core pipeline wait timed out"};
+    if (bits & kStatusSpread) throw Error{kErrSpread, "operands of too wide a range for digit products"};
     throw Error{MLCC3_ERR_SINGULAR_DENOM, "|eps^{abc}_{ijk} - omega| < 1e-3 in a triples block"};
   }
 }
@@ -3801,7 +3863,7 @@ void sweep_check_status(mlcc3_sweep *sw) {
 bool sweep_stale(const mlcc3_sweep *sw) {
   if (!sw->exec) return true;
   for (auto &y : sw->sys)
-    if (y.build_gen != y.c->build_gen || y.chunk_gen != y.c->chunk_gen) return true;
+    if (y.build_gen != y.c->build_gen || y.chunk_gen != y.c->chunk_gen || y.path_gen != y.c->path_gen) return true;
   return false;
 }
 
@@ -3903,6 +3965,7 @@ void sweep_prepare(mlcc3_sweep *sw) {
   for (auto &y : sw->sys) {
     y.build_gen = y.c->build_gen;
     y.chunk_gen = y.c->chunk_gen;
+    y.path_gen = y.c->path_gen;
   }
 }
 
@@ -4039,9 +4102,27 @@ extern "C" int mlcc3_sweep_run(mlcc3_sweep *sw, const double *omega) {
       check_cuda(cudaStreamSynchronize(y.c->stream), "context sync");
       y.c->collect_events();
     }
-    if (sweep_stale(sw)) sweep_prepare(sw);
-    check_cuda(cudaGraphLaunch(sw->exec, sw->s0), "graph launch");
-    sweep_check_status(sw);
+    for (;;) {
+      try {
+        if (sweep_stale(sw)) sweep_prepare(sw);
+        check_cuda(cudaGraphLaunch(sw->exec, sw->s0), "graph launch");
+        sweep_check_status(sw);
+        return;
+      } catch (const Error &e) {
+        if (e.code != kErrSpread && e.code != MLCC3_ERR_OOM) throw;
+        // once more with the systems concerned on the FP64 pipe (each leaves once)
+        cudaStreamSynchronize(sw->s0);
+        for (auto &y : sw->sys) cudaStreamSynchronize(y.st);
+        bool left = false;
+        for (size_t q = 0; q < sw->sys.size(); ++q) {
+          mlcc3_ctx *c = sw->sys[q].c;
+          if (!c->emu || (e.code == kErrSpread && !(sw->status_pin[q] & kStatusSpread))) continue;
+          c->leave_digits();
+          left = true;
+        }
+        if (!left) throw;
+      }
+    }
   });
 }
 
