@@ -393,23 +393,62 @@ __global__ void __launch_bounds__(256) bstc64_kernel(BstcParams p) {
     __syncthreads();
     red[tid] = acc[0][0];
     __syncthreads();
-    if (kg > 0) return;
 #pragma unroll
-    for (int g = 1; g < KG; ++g) acc[0][0] += red[tid + g * TY * TX];
+    for (int g = 1; g < KG; ++g)
+      if (kg == 0) acc[0][0] += red[tid + g * TY * TX];
   }
   double *C = p.C + it.offC;
+  auto add = [&](long long rc, long long cc, double x) {
+    if (rc < 0 || cc < 0) return;
+    const double v = p.alpha * x;
+    if (p.atomic) atomicAdd(C + rc + cc, v);
+    else C[rc + cc] += v;
+  };
+  if (!p.part) {
+    if (kg > 0) return;
 #pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const long long rc = rowC[ty * RM + i];
-    if (rc < 0) continue;
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < RN; ++j) {
-      const long long cc = colC[tx * RN + j];
-      if (cc < 0) continue;
-      const double v = p.alpha * acc[i][j];
-      if (p.atomic) atomicAdd(C + rc + cc, v);
-      else C[rc + cc] += v;
+      for (int j = 0; j < RN; ++j) add(rowC[ty * RM + i], colC[tx * RN + j], acc[i][j]);
+    return;
+  }
+  // A piece of a split reduction: the last one to finish its tile adds the pieces up, in
+  // their order, and C gets one sum.  (One atomic addition per piece rounded at the size of
+  // C every time: the singles of sigma, some ten products into one array, came out with
+  // twice the error of unsplit sums.)
+  const long long tile = (long long)blockIdx.y * gridDim.x + blockIdx.x;
+  constexpr int TE = TM * TN;
+  double *part = p.part + tile * gridDim.z * TE;
+  if (kg == 0) {
+    double *mine = part + (long long)blockIdx.z * TE;
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+      for (int j = 0; j < RN; ++j) mine[(ty * RM + i) * TN + tx * RN + j] = acc[i][j];
+  }
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(p.count + tile, 1u) == gridDim.z - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid == 0) p.count[tile] = 0;  // as the next launch finds it
+  constexpr int G = TE >= 256 ? 1 : 256 / TE;  // threads per output, each every G-th piece
+  for (int o = tid % TE; o < TE; o += 256) {
+    double x = 0.0;
+#pragma unroll 8
+    for (int z = tid / TE; z < (int)gridDim.z; z += G) x += __ldcg(part + (long long)z * TE + o);
+    if (G > 1) {
+      double *red = &As[0][0];
+      __syncthreads();
+      red[tid] = x;
+      __syncthreads();
+      if (tid >= TE) return;
+#pragma unroll
+      for (int g = 1; g < G; ++g) x += red[tid + g * TE];
     }
+    add(rowC[o / TN], colC[o % TN], x);
   }
 }
 
@@ -418,8 +457,8 @@ __global__ void __launch_bounds__(256) bstc64_kernel(BstcParams p) {
 // clock, for as many rounds of blocks as the 152 SMs need, and about 800 clocks
 // of latency per K step, which four resident blocks hide from one another.  A
 // reduction whose tiles make fewer than fill * 152 blocks is split over about as
-// many (pieces of at least 32, added atomically); fill = 0 never splits.
-cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st) {
+// many (pieces of at least 32); fill = 0, or no workspace, never splits.
+cudaError_t launch_bstc64(BstcParams p, int fill, const BstcWork &w, cudaStream_t st) {
   struct Tile {
     int m, n;
     void (*k)(BstcParams);
@@ -442,8 +481,9 @@ cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st) {
   for (const Tile &t : tiles) {
     const long long ntiles = ((M + t.m - 1) / t.m) * ((N + t.n - 1) / t.n), blocks = ntiles * p.nitems;
     long long split = 1;
-    if (fill > 0 && blocks < fill * 152LL)
-      split = std::max(1LL, std::min({(fill * 152LL + blocks - 1) / blocks, K / 32, 65535LL}));
+    if (fill > 0 && w.part && blocks < std::min(fill * 152LL, kBstcCounts))
+      split = std::max(1LL, std::min({(fill * 152LL + blocks - 1) / blocks, K / 32, 65535LL,
+                                      kBstcParts / (blocks * t.m * t.n)}));
     const long long steps = ((K + split - 1) / split + 31) / 32;
     const double rounds = (double)((blocks * split + 151) / 152);
     const double c = rounds * 16.0 * t.m * t.n * (double)steps * (1.0 + 0.5 / t.m + 0.5 / t.n) +
@@ -456,10 +496,14 @@ cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st) {
     }
   }
   p.kchunk = 0;
+  p.part = nullptr;
   if (ks > 1) {
     p.kchunk = ((K + ks - 1) / ks + 31) / 32 * 32;
     ks = (K + p.kchunk - 1) / p.kchunk;
-    p.atomic = 1;
+    if (ks > 1) {
+      p.part = w.part;
+      p.count = w.count;
+    }
   }
   best->k<<<dim3((unsigned)nt, (unsigned)p.nitems, (unsigned)ks), 256, 0, st>>>(p);
   return cudaGetLastError();

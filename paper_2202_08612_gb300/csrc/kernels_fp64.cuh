@@ -60,7 +60,20 @@ struct BstcParams {
   long long kchunk;  // split-K: grid.z slices of this many K elements (0 = whole K); the
                      // binary32 matrix-vector kernel: the number of K slices (0: from the grid)
   int a32, b32;      // 1: A (B) holds binary32 elements (element offsets and strides as given)
+  // FP64 form with a split reduction (launch_bstc64): the pieces' sums, tile after tile,
+  // and a count of the pieces done for each tile, zero between launches
+  double *part;
+  unsigned *count;
 };
+
+// Workspace of launch_bstc64: kBstcParts doubles and kBstcCounts zeroed counters, used by
+// one launch at a time; null: no reduction is split.
+struct BstcWork {
+  double *part;
+  unsigned *count;
+};
+constexpr long long kBstcParts = 4LL << 20;
+constexpr long long kBstcCounts = 64 * 152;
 
 // One additive term of the pre-permutation triples expression V^{abc}_{ijk}
 // (Eq. tau3, Eq. R3, SI L3), evaluated for an ordered occupied triple

@@ -29,7 +29,7 @@
 #include "workpool.cuh"
 
 namespace mlcc3 {
-cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st);
+cudaError_t launch_bstc64(BstcParams p, int fill, const BstcWork &w, cudaStream_t st);
 cudaError_t launch_bstc32(BstcParams p, cudaStream_t st);
 __global__ void bstc_big_kernel(BstcParams p);
 __global__ void bstc_dot_kernel(BstcParams p);
@@ -409,11 +409,19 @@ void mlcc3_ctx::bstc(const double *A, const double *B, double *C, const Shape &s
   }
   const std::string name = tag.empty() ? std::string("bstc_kernel") : "bstc_kernel:" + tag;
   if (!f32) {
+    // (the counters are zeroed once; every launch leaves them so)
+    const bool first = bstc_fill > 0 && !scratch.count("bstc:count");
+    BstcWork w{};
+    if (bstc_fill > 0) {
+      w.part = buf("bstc:part", (size_t)kBstcParts);
+      w.count = static_cast<unsigned *>(raw("bstc:count", sizeof(unsigned) * (size_t)kBstcCounts));
+      if (first) check_cuda(cudaMemsetAsync(w.count, 0, sizeof(unsigned) * (size_t)kBstcCounts, stream), "bstc count");
+    }
     for (int z0 = 0; z0 < nitems; z0 += 65535) {
       p.items = it + z0;
       p.nitems = std::min(65535, nitems - z0);
       launch(name.c_str(), 2.0 * M * N * (double)K * p.nitems,
-             [&] { check_cuda(launch_bstc64(p, bstc_fill, stream), "bstc64"); });
+             [&] { check_cuda(launch_bstc64(p, bstc_fill, w, stream), "bstc64"); });
     }
     return;
   }

@@ -18,7 +18,7 @@
 
 namespace mlcc3 {
 void set_last_error(const std::string &msg);
-cudaError_t launch_bstc64(BstcParams p, int fill, cudaStream_t st);
+cudaError_t launch_bstc64(BstcParams p, int fill, const BstcWork &w, cudaStream_t st);
 __global__ void bstc_gemv_kernel(BstcParams p);
 cudaError_t launch_triples_build(const TripTerms &, const TripItem *, int, const double *, int, int,
                                  double, const double *, double *, int *, cudaStream_t);
@@ -224,7 +224,7 @@ extern "C" int mlcc3_triples_omega_static(mlcc3_ctx *c, double *omega1, double *
       if (N == 1) {  // matrix-vector form (singles and F terms): a warp per output row
         bstc_gemv_kernel<<<dim3((unsigned)((M + 7) / 8), (unsigned)bp.nitems), 256, 0, st>>>(bp);
         if (!chk(cudaGetLastError(), "bstc_gemv launch")) return drained();
-      } else if (!chk(launch_bstc64(bp, c->bstc_fill, st), "bstc64 launch")) {
+      } else if (!chk(launch_bstc64(bp, 0, BstcWork{}, st), "bstc64 launch")) {
         return drained();
       }
     }
