@@ -303,9 +303,13 @@ void mlcc3_sweep_destroy(mlcc3_sweep *sweep);
  *              returns MLCC3_ERR_TIMEOUT and drops the context's cached tau, and
  *              the context stays usable.  A small value (a few clocks) makes the
  *              waits run out: failure-path testing only.  Range 0..2^40.
- *   "bstc_fill"  split-K target of the FP64 strided contractions: a launch
- *              with few output tiles and a long reduction splits K until about
- *              bstc_fill x 152 CTAs run; 0 never splits.  Default 4.  Range 0..64.
+ *   "bstc_fill"  split-K target of the strided contractions on the CUDA cores: a
+ *              launch of few output tiles splits its reduction (pieces of at
+ *              least 32 products, in the split-precision mode 128) until about
+ *              bstc_fill x 152 blocks run; 0 never splits.  FP64 pieces are added
+ *              up in a fixed order before they meet the output; split-precision
+ *              ones are added atomically, so their last bits may differ between
+ *              calls.  Default 4.  Range 0..64.
  *   "chunk_blocks"  most unique batches whose triples blocks (n_v^3 each) the
  *              context holds on the device at once; larger systems are swept
  *              in chunks (the densities by ranges of occupied indices, which

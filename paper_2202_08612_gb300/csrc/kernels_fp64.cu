@@ -222,13 +222,14 @@ __global__ void __launch_bounds__(256, TM * TN <= 1024 && RM == RN ? 3 : TM * TN
 }
 
 // C += alpha A B with FP32 products for every item (at most 65535).  p.kchunk splits
-// K as before (0: not); a launch of fewer than four blocks per SM is split further,
-// at multiples of 64 products from the start of a range, which changes no FP32 sum.
+// K as before (0: not); a launch of fewer than fill blocks per SM is split further,
+// at multiples of 64 products from the start of a range, which changes no FP32 sum
+// (fill = 0: never).
 // Of the tiles the one with the least estimated time: per K element its FP32
 // products (128 a clock), its shared-memory reads and its share of the FP64
 // additions, for as many rounds of blocks as the 152 SMs need, plus the latency
 // of a K step that four resident blocks hide from one another.
-cudaError_t launch_bstc32(BstcParams p, cudaStream_t st) {
+cudaError_t launch_bstc32(BstcParams p, int fill, cudaStream_t st) {
   struct Tile {
     int m, n;
     double clk;  // per K element
@@ -261,8 +262,8 @@ cudaError_t launch_bstc32(BstcParams p, cudaStream_t st) {
     const long long ntiles = ((M + t.m - 1) / t.m) * ((N + t.n - 1) / t.n);
     const long long blocks = ntiles * p.nitems * ranges;
     long long f = 1;
-    if (blocks < 4 * 152)
-      f = std::max(1LL, std::min({(4 * 152 + blocks - 1) / blocks, (range + 127) / 128, 65535 / ranges}));
+    if (blocks < fill * 152LL)
+      f = std::max(1LL, std::min({(fill * 152LL + blocks - 1) / blocks, (range + 127) / 128, 65535 / ranges}));
     const long long steps = ((range + f - 1) / f + 31) / 32;
     const double rounds = (double)((blocks * f + 151) / 152);
     const double c = rounds * t.clk * 32.0 * (double)steps + 1200.0 * (double)steps * std::max(1.0, 0.25 * rounds);

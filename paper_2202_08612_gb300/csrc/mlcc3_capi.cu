@@ -30,7 +30,7 @@
 
 namespace mlcc3 {
 cudaError_t launch_bstc64(BstcParams p, int fill, const BstcWork &w, cudaStream_t st);
-cudaError_t launch_bstc32(BstcParams p, cudaStream_t st);
+cudaError_t launch_bstc32(BstcParams p, int fill, cudaStream_t st);
 __global__ void bstc_big_kernel(BstcParams p);
 __global__ void bstc_dot_kernel(BstcParams p);
 __global__ void bstc_gemv_kernel(BstcParams p);
@@ -443,7 +443,7 @@ void mlcc3_ctx::bstc(const double *A, const double *B, double *C, const Shape &s
     p.items = it + z0;
     p.nitems = std::min(65535, nitems - z0);
     launch(name.c_str(), 2.0 * M * N * (double)K * p.nitems,
-           [&] { check_cuda(launch_bstc32(p, stream), "bstc32"); });
+           [&] { check_cuda(launch_bstc32(p, bstc_fill, stream), "bstc32"); });
   }
 }
 

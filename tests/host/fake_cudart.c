@@ -17,9 +17,9 @@ static struct { char *p; size_t n; } block[NBLOCK];
 static struct { const void *f; char name[160]; } kernel[NKERNEL];
 static int nkernel, last_error;
 static size_t total = (size_t)284 << 30, used;
-static char log_[1 << 22], fail_name[80], mark_name[80];
+static char log_[1 << 22], fail_name[80], mark_name[80], watch_name[80];
 static size_t nlog;
-static long long fail_at = -1, mark_left, mark_arg, mark_bits;
+static long long fail_at = -1, mark_left, mark_arg, mark_bits, watch_z;
 
 /* ---- the test's side ---- */
 void fake_total(long long n) { total = (size_t)n; }
@@ -31,6 +31,9 @@ void fake_mark(const char *name, long long n, long long arg, long long bits) {
   snprintf(mark_name, sizeof mark_name, "%s", name);
   mark_left = n, mark_arg = arg, mark_bits = bits;
 }
+/* the largest gridDim.z of the launches whose kernel's name contains `name`, from now */
+void fake_watch(const char *name) { snprintf(watch_name, sizeof watch_name, "%s", name), watch_z = 0; }
+long long fake_watched(void) { return watch_z; }
 const char *fake_log(void) { return log_; }
 void fake_clear(void) { nlog = 0, log_[0] = 0; }
 int fake_is_live(const void *p) {
@@ -94,25 +97,28 @@ void __cudaRegisterFunction(void **h, const char *f, char *d, const char *name, 
                             void *e, int *w) {
   if (nkernel < NKERNEL) kernel[nkernel].f = f, snprintf(kernel[nkernel++].name, 160, "%s", name);
 }
+struct dim { uint32_t x, y, z; };
+static struct dim config_grid;
 static size_t config_smem;
 static void *config_stream;
 unsigned __cudaPushCallConfiguration(uint64_t gxy, uint32_t gz, uint64_t bxy, uint32_t bz, size_t smem, void *st) {
+  config_grid = (struct dim){(uint32_t)gxy, (uint32_t)(gxy >> 32), gz};
   config_smem = smem, config_stream = st;
   return 0;
 }
 int __cudaPopCallConfiguration(void *g, void *b, size_t *smem, void **st) {
   const uint32_t one[3] = {1, 1, 1};
-  memcpy(g, one, sizeof one), memcpy(b, one, sizeof one);
+  memcpy(g, &config_grid, sizeof config_grid), memcpy(b, one, sizeof one);
   *smem = config_smem, *st = config_stream;
   return OK;
 }
 int __cudaGetKernel(const void **k, const void *f) { *k = f; return OK; }
-struct dim { uint32_t x, y, z; };
 int __cudaLaunchKernel(const void *k, struct dim g, struct dim b, void **args, size_t smem, void *st) {
   const char *name = "?";
   for (int i = 0; i < nkernel; ++i)
     if (kernel[i].f == k) name = kernel[i].name;
   if (nlog + strlen(name) + 2 < sizeof log_) nlog += (size_t)sprintf(log_ + nlog, "%s\n", name);
+  if (watch_name[0] && strstr(name, watch_name) && g.z > watch_z) watch_z = g.z;
   if (fail_at >= 0 && strstr(name, fail_name) && fail_at-- == 0) return set(LAUNCH_OUT_OF_RESOURCES);
   if (mark_left > 0 && strstr(name, mark_name)) --mark_left, **(int **)args[mark_arg] |= (int)mark_bits;
   return OK;
