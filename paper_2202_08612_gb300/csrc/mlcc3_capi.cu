@@ -1716,11 +1716,11 @@ void tri_layout(mlcc3_ctx *c, const double *X, int k, SplitOp &op) {
   const int a = k == 0 ? 1 : 0, b = k == 2 ? 1 : 2, nv = (int)s.nv;
   const long long Kp = kpad(c, s.nv * s.nv);
   const bool convert = !(ts.mask & (1u << k));
-  ts.mask |= 1u << k;
   if (c->emu) {
     const EmuView v{X, (int)nb, 1, nv, nv, nv * nv, nv, s.nv3, 0, 0, cs[k], cs[a], cs[b]};
     if (convert) {
       make_digits(c, op, base, v, Kp, false, "tri" + std::to_string(q));
+      ts.mask |= 1u << k;
     } else {
       op.S = kEmuStored;
       op.slice = (long long)v.Z * v.R * Kp;
@@ -1746,6 +1746,7 @@ void tri_layout(mlcc3_ctx *c, const double *X, int k, SplitOp &op) {
                                c->stream, c->is_tri32(X)), "split_bf16_k2");
     });
   }
+  ts.mask |= 1u << k;  // (only now: the allocations above may have failed)
 }
 
 void encode_split(mlcc3_ctx::SplitOp &op, const std::string &key, const unsigned long long dims[4],

@@ -19,13 +19,15 @@ static int nkernel, last_error;
 static size_t total = (size_t)284 << 30, used;
 static char log_[1 << 22], fail_name[80], mark_name[80], watch_name[80];
 static size_t nlog;
-static long long fail_at = -1, mark_left, mark_arg, mark_bits, watch_z;
+static long long fail_at = -1, malloc_at = -1, mark_left, mark_arg, mark_bits, watch_z;
 
 /* ---- the test's side ---- */
 void fake_total(long long n) { total = (size_t)n; }
 long long fake_used(void) { return (long long)used; }
 /* the n-th launch from now (0: the next) whose kernel's name contains `name` fails */
 void fake_fail(const char *name, long long n) { snprintf(fail_name, sizeof fail_name, "%s", name); fail_at = n; }
+/* device allocations from the n-th on (0: the next) find no memory; negative: none fails */
+void fake_fail_malloc(long long n) { malloc_at = n; }
 /* the next n launches of such kernels set `bits` in the int that their argument `arg` points to */
 void fake_mark(const char *name, long long n, long long arg, long long bits) {
   snprintf(mark_name, sizeof mark_name, "%s", name);
@@ -46,7 +48,8 @@ int fake_is_live(const void *p) {
 static int set(int e) { if (e) last_error = e; return e; }
 int cudaMalloc(void **p, size_t n) {
   *p = NULL;
-  if (used + n > total) return set(OOM);
+  if (used + n > total || malloc_at == 0) return set(OOM);
+  if (malloc_at > 0) --malloc_at;
   for (int i = 0; i < NBLOCK; ++i)
     if (!block[i].p) {
       void *q = mmap(NULL, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);

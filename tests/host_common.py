@@ -24,7 +24,7 @@ F.fake_log.restype = ctypes.c_char_p
 for f in (F.fake_used, F.fake_watched):
     f.restype = ctypes.c_longlong
 for f, a in ((F.fake_total, [ctypes.c_longlong]), (F.fake_fail, [ctypes.c_char_p, ctypes.c_longlong]),
-             (F.fake_mark, [ctypes.c_char_p] + [ctypes.c_longlong] * 3), (F.fake_watch, [ctypes.c_char_p]), (F.fake_is_live, [ctypes.c_void_p])):
+             (F.fake_mark, [ctypes.c_char_p] + [ctypes.c_longlong] * 3), (F.fake_watch, [ctypes.c_char_p]), (F.fake_fail_malloc, [ctypes.c_longlong]), (F.fake_is_live, [ctypes.c_void_p])):
     f.argtypes = a
 class Dev:
     'A device array of doubles.'
