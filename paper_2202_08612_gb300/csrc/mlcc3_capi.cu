@@ -1112,8 +1112,9 @@ TcDev tc_plan(mlcc3_ctx *c, const std::string &key0, const std::function<void(Tc
     for (size_t i = 0; i < ord.size(); ++i) sorted[i] = pl.items[ord[i]];
     pl.items.swap(sorted);
   }
-  void *si = upload_cached(c, key + ":items", pl.items.data(), pl.items.size() * sizeof(TcItem));
+  // (the items last: a plan is there when they are)
   void *ss = upload_cached(c, key + ":segs", pl.segs.data(), pl.segs.size() * sizeof(TcSeg));
+  void *si = upload_cached(c, key + ":items", pl.items.data(), pl.items.size() * sizeof(TcItem));
   c->items[key + ":items"].second = (int)pl.items.size();
   return TcDev{static_cast<const TcItem *>(si), static_cast<const TcSeg *>(ss),
                (int)pl.items.size()};
@@ -2250,14 +2251,15 @@ void build_tau(mlcc3_ctx *c, const Chunk &ch, double **tau, double **taut) {
   *tau = c->tri_buf("tau", (size_t)ch.nb * s.nv3);
   *taut = c->tri_buf("taut", (size_t)ch.nb * s.nv3);
   if (c->tau_valid && c->tau_key == ch.key) return;
-  c->tau_valid = true;
-  c->tau_key = ch.key;
+  c->tau_valid = false;  // until all of it is launched
   if (tc_mode(c)) {
     triples_split(c, tau_split_terms(c), {}, "b" + ch.key, ch.bs, 0.0, *tau, *taut, ch.nb);
   } else {
     triples(c, tau_terms(c), "b" + ch.key, ch.bs, 0.0, *tau);
     contra3(c, *tau, *taut, ch.nb);
   }
+  c->tau_valid = true;
+  c->tau_key = ch.key;
 }
 
 // Upsilon blocks for one trial vector (Eqs. ups_v, ups_o) and the rho tau-term
@@ -2842,7 +2844,7 @@ void pair_dots(mlcc3_ctx *c, const Chunk &ch, const double *X, const double *Y, 
   if (n3 == 0 || s.nv == 0 || ch.p1 <= ch.p0) return;
   const std::string key = "pd" + ch.key;
   void *voff = nullptr, *vstr = nullptr, *vhave = nullptr;
-  if (c->items.find(key + ":off") == c->items.end()) {
+  if (c->items.find(key + ":have") == c->items.end()) {  // (the last of the three)
     ViewMap vm(ch.held, s.no);
     std::vector<int> str(3 * n3);
     for (long long x = 0; x < n3; ++x) {
@@ -3346,6 +3348,7 @@ static int guarded(F &&f) {
     f();
     return MLCC3_OK;
   } catch (const Error &e) {
+    cudaGetLastError();  // reported here: the next call does not meet it again
     g_last_error = e.msg;
     return e.code;
   } catch (const std::exception &e) {
