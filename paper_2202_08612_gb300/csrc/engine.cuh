@@ -127,6 +127,7 @@ struct mlcc3_ctx {
 
   // named scratch buffers, reused across calls (stream ordered)
   std::map<std::string, std::pair<void *, size_t>> scratch;
+  int addr_gen = 0;  // counts what frees some of it: a sweep's graph of before is stale
   // "release_scratch": every call ends by freeing the scratch that the integral
   // build did not create (keep_scratch / keep_splits are the build's names)
   bool release_scratch = false;
@@ -182,7 +183,6 @@ struct mlcc3_ctx {
   // integral build
   bool emu = false, emu_rule = false;
   void leave_digits();
-  int path_gen = 0;  // counts leave_digits: a sweep's graph of before is stale
   long long fp64_tc_from = 24;
   std::map<std::string, int> scales;
   // split layouts of triples arrays, converted once per (array, write

@@ -117,6 +117,7 @@ void *mlcc3_ctx::raw(const std::string &name, size_t bytes) {
     check_cuda(cudaStreamSynchronize(stream), "sync before realloc");
     cudaFree(it->second.first);
     scratch.erase(it);
+    addr_gen += 1;
     tri_regs.erase(name);
   }
   void *p = nullptr;
@@ -135,6 +136,7 @@ void *mlcc3_ctx::raw(const std::string &name, size_t bytes) {
 // create) and forget what was cached in it: split copies, triples layouts and
 // FP32 copies, tau.  The stream has been synchronised.
 void mlcc3_ctx::release() {
+  addr_gen += 1;
   for (auto it = scratch.begin(); it != scratch.end();) {
     if (keep_scratch.count(it->first)) {
       ++it;
@@ -163,7 +165,7 @@ void mlcc3_ctx::leave_digits() {
   check_cuda(cudaStreamSynchronize(stream), "sync before the FP64 pipe");
   cudaGetLastError();
   emu = false;
-  path_gen += 1;
+  addr_gen += 1;
   for (auto it = scratch.begin(); it != scratch.end();) {
     if (it->first.compare(0, 7, "digits:") != 0) {
       ++it;
@@ -3765,7 +3767,7 @@ struct mlcc3_sweep {
     double *rho1 = nullptr, *rho2 = nullptr;
     long long w0 = 0;  // first frequency of this system in the omega array
     unsigned long long build_gen = 0;
-    int chunk_gen = 0, path_gen = 0;
+    int chunk_gen = 0, addr_gen = 0;
     int fill = 4;
     std::vector<double> fill_ms;  // tuning times per candidate
     // tensor-core choices of the split mode and their tuning times
@@ -3875,7 +3877,7 @@ void sweep_check_status(mlcc3_sweep *sw) {
 bool sweep_stale(const mlcc3_sweep *sw) {
   if (!sw->exec) return true;
   for (auto &y : sw->sys)
-    if (y.build_gen != y.c->build_gen || y.chunk_gen != y.c->chunk_gen || y.path_gen != y.c->path_gen) return true;
+    if (y.build_gen != y.c->build_gen || y.chunk_gen != y.c->chunk_gen || y.addr_gen != y.c->addr_gen) return true;
   return false;
 }
 
@@ -3977,7 +3979,7 @@ void sweep_prepare(mlcc3_sweep *sw) {
   for (auto &y : sw->sys) {
     y.build_gen = y.c->build_gen;
     y.chunk_gen = y.c->chunk_gen;
-    y.path_gen = y.c->path_gen;
+    y.addr_gen = y.c->addr_gen;
   }
 }
 

@@ -93,3 +93,16 @@ def test_vectors_of_a_wide_range_run_on_the_fp64_pipe():
     sw.run(np.concatenate(omegas))  # and a replay of the new graph
     _check(cases, pipes, vecs, omegas, factors)
 
+
+
+def test_chunked_replays_after_calls_that_move_the_scratch():
+    """The densities hold more blocks at a time than the sweep's chunks: their first call moves
+    the triples arrays that the captured graph was made for."""
+    cases, ctxs, pipes, sw, vecs = _sweep({"chunk_blocks": 4})
+    omegas = [c.st.omega for c in cases]
+    for n in range(3):
+        sw.run(np.concatenate(omegas))
+        _check(cases, pipes, vecs, omegas)
+        for c, g in zip(cases, ctxs):
+            _calls_between(c, g)
+        omegas = [w + 0.01 for w in omegas]
