@@ -265,12 +265,13 @@ void mlcc3_sweep_destroy(mlcc3_sweep *sweep);
  *              FP32 accumulation over K ranges of at most 1024 (summed in
  *              FP64); the others on 64 x 64 tiles.  Default 10^9; 0: never.
  *   "fp64_tc_from"  MLCC3_FP64 contexts with at least this many active virtual
- *              orbitals, or n_o n_v at least three times it, and n_o >= 2 run the O(N_V n_v^3 n_o^3) contractions and
- *              the Cholesky-index products on the tensor cores (see MLCC3_FP64; a call
- *              whose digits find no room in the device memory also runs on the FP64
- *              pipe),
- *              unless the digits of the integral blocks would take more than a
- *              quarter of the free memory; smaller ones on the FP64 pipe.
+ *              orbitals, or n_o n_v at least three times it, and n_o >= 2 run
+ *              the O(N_V n_v^3 n_o^3) contractions and the Cholesky-index
+ *              products on the tensor cores (see MLCC3_FP64) unless the digits,
+ *              18 bytes per element of each layout, would take more than 0.4 of
+ *              the device's memory; smaller and larger ones run on the FP64
+ *              pipe, and so does a call whose digits find no room (the digits
+ *              take 1 to 4 times the memory of the triples blocks themselves).
  *              Default 24.  A change that switches the path needs a new
  *              mlcc3_build_integrals (MLCC3_ERR_STATE before it).
  *   "finish_fused"  1 (default): in the split-precision mode the finish of a

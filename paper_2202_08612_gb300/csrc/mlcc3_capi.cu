@@ -617,9 +617,35 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
 // fp64_tc_from (24) active virtual orbitals or n_o n_v = 3 fp64_tc_from on (rho and sigma,
 // FP64 pipe against digits: 4/12 0.85 against 1.15 ms, 4/16 1.34 and 1.32, 6/12 1.79 and
 // 1.20, 8/16 4.66 and 1.67, 3/24 1.87 and 1.63; below, a call is launches, and the digits
-// need more of them), where the operands'
-// digits (the layouts of the two integral blocks, the Cholesky factors and the
-// amplitudes at 16 bytes an element) leave most of the memory free.
+// need more of them), where all digits that live at once (digit_bytes) take less than 0.4
+// of the card's memory: a rule of sizes alone, so that the same system takes the same path
+// whatever else holds memory.  (Where they find no room all the same, a call runs on the
+// pipe.)
+//
+// Digit operands by kind, those of the build and those that rho, sigma or a density
+// adds: integral blocks (Gv, Gb, Upsilon, H2, Y1, P2 in their layouts) 8 + 7, Cholesky-vV
+// 3 + 2, amplitudes with N_V innermost 2 + 3, with N_O innermost 4 + 10, o-type blocks
+// 4 + 2; 2 stored bytes per slice and element, K padded to chunks.
+double digit_bytes(const mlcc3_ctx *c) {
+  const S s(c);
+  auto pad = [](long long k) { return (double)((k + kEmuKB - 1) / kEmuKB * kEmuKB); };
+  const double o = (double)s.no, v = (double)s.nv, NO = (double)s.NO, NV = (double)s.NV, NJ = (double)s.NJ;
+  const double vv = pad(s.nv * s.nv), one = std::max(pad(s.NV) / std::max(NV, 1.0), vv / std::max(v * v, 1.0));
+  return 2.0 * kEmuStored *
+         (15.0 * one * o * v * v * NV + 5.0 * v * std::max(pad(s.NJ) * NV, NJ * pad(s.NV)) +
+          5.0 * o * o * std::max(v * pad(s.NV), NV * pad(s.nv)) + 14.0 * o * std::max(v * v * pad(s.NO), NO * vv) +
+          6.0 * o * o * std::max(v * pad(s.NO), NO * pad(s.nv)) + 8.0 * o * v * pad(s.NJ));
+}
+
+// Bytes per element of a triples block that a context holds: eight arrays (tau, R3, L3,
+// lambda3 and their contravariant forms), in the split mode binary32 with the layouts of
+// four arrays (tri_layout, three each, hi and lo) and one array of sums; on digits FP64 with
+// the layouts of three arrays.  The FP64 pipe has no layouts.
+double block_bytes(const mlcc3_ctx *c) {
+  if (c->tri32) return 8 * 4.0 + 4 * 3 * 4.0 + 4.0;
+  return 8 * 8.0 + (c->emu_rule ? 3 * 3 * 2.0 * kEmuStored : 8.0);
+}
+
 void choose_emu(mlcc3_ctx *c) {
   S s(c);
   c->emu_rule = false;
@@ -627,18 +653,12 @@ void choose_emu(mlcc3_ctx *c) {
   if (s.nv < c->fp64_tc_from && s.no * s.nv < 3 * c->fp64_tc_from) return;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return;
-  const double digits = 16.0 * (8.0 * (double)s.gvsz() + 3.0 * (double)s.NJ * (double)(s.nv * s.NV) +
-                                4.0 * (double)s.blk() + 4.0 * (double)(s.no * s.nv * s.nv * s.NO));
-  c->emu_rule = digits < 0.25 * (double)fr;
+  c->emu_rule = digit_bytes(c) < 0.4 * (double)tot;
 }
 
 // Split the unique batches into chunks of at most chunk_blocks blocks (or, when
-// it is 0, as many as fit in half of the device memory left free once the
-// context's persistent arrays exist, at 156 bytes per block element: the
-// eight FP64 triples arrays the passes keep (tau, R3, L3, lambda3 and their
-// contravariant forms) plus up to 18 cached split-precision layouts of
-// triples arrays (tri_layout) and four FP32 copies (tri_f32); 108 bytes in the
-// split mode, whose triples arrays are binary32 and need no copies; scratch
+// it is 0, as many as fit, at block_bytes per element, in half of the device memory left
+// free once the context's persistent arrays and all digits exist; scratch
 // buffers persist across calls, so one size serves all).
 void make_chunks(mlcc3_ctx *c) {
   c->chunk_gen += 1;
@@ -651,11 +671,11 @@ void make_chunks(mlcc3_ctx *c) {
   if (part_max <= 0) {
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = (size_t)40 << 30;
-    const double budget = 0.5 * (double)fr;
-    // binary32 triples arrays in the split mode (and no separate FP32 copies)
-    // (digit slices: eight FP64 arrays and up to 18 layouts of 16 bytes)
-    const double per_elem = c->tri32 ? 108.0 : c->emu ? 352.0 : 156.0;
-    part_max = group_max = std::max<long long>(1, (long long)(budget / (per_elem * (double)nv3)));
+    double digits = c->emu_rule ? digit_bytes(c) : 0.0;  // less those that are there
+    for (auto &kv : c->scratch)
+      if (kv.first.compare(0, 7, "digits:") == 0) digits -= (double)kv.second.second;
+    const double budget = 0.5 * ((double)fr - std::max(0.0, digits));
+    part_max = group_max = std::max<long long>(1, (long long)(budget / (block_bytes(c) * (double)nv3)));
   }
   const std::string g = "#" + std::to_string(c->chunk_gen);
   auto partition = [&](const std::vector<TripItem> &list, const std::string &tag) {
@@ -4022,7 +4042,7 @@ extern "C" int mlcc3_sweep_create(mlcc3_sweep **out, mlcc3_ctx *const *ctxs, int
       std::vector<int> order(n_sys);
       for (int q = 0; q < n_sys; ++q) {
         const double nv = (double)ctxs[q]->nv;
-        demand[q] = 156.0 * (double)ctxs[q]->batches.size() * nv * nv * nv;
+        demand[q] = block_bytes(ctxs[q]) * (double)ctxs[q]->batches.size() * nv * nv * nv;
         order[q] = q;
       }
       std::sort(order.begin(), order.end(), [&](int a, int b) { return demand[a] < demand[b]; });
