@@ -1026,16 +1026,13 @@ int tile_w(const mlcc3_ctx *c, long long n) {
 // digit sums are exact, their items only bounded by the integers' width.
 int kcap(const mlcc3_ctx *c) { return c->emu ? kEmuMaxK / kEmuKB : c->tc_kcap; }
 
-// Named scales of digit operands (FP64 mode on the tensor cores): device words.
+// Named scales of digit operands (FP64 mode on the tensor cores): device words, in
+// buffers of kMax that stay where they are as names are added.
 EmuScale *scale_of(mlcc3_ctx *c, const std::string &slot) {
-  constexpr int kMax = 4096;
-  EmuScale *base = static_cast<EmuScale *>(c->raw("emu:scales", sizeof(EmuScale) * kMax));
-  auto it = c->scales.find(slot);
-  if (it == c->scales.end()) {
-    if (c->scales.size() >= (size_t)kMax) throw Error{MLCC3_ERR_ARG, "too many scales"};
-    it = c->scales.emplace(slot, (int)c->scales.size()).first;
-  }
-  return base + it->second;
+  constexpr int kMax = 1024;
+  const auto it = c->scales.emplace(slot, (int)c->scales.size()).first;
+  return static_cast<EmuScale *>(c->raw("emu:scales:" + std::to_string(it->second / kMax), sizeof(EmuScale) * kMax)) +
+         it->second % kMax;
 }
 // scale = the largest finite magnitude of the arrays (zeroed first)
 void scale_max(mlcc3_ctx *c, const std::string &slot,
