@@ -343,12 +343,18 @@ int mlcc3_cnto_matrices(int64_t n_occ, int64_t n_vir, const double *R1, const do
  * about 2^-(8 slices) (slices = 5: about 1e-12).  A [M][K] with rows lda
  * apart, B [N][K] rows ldb apart, C [M][N] rows ldc apart, all FP64 device
  * arrays (MLCC3_ERR_ARG otherwise, and for slices outside 2..6 or a leading
- * dimension below the row length).  Allocates its temporaries (about
- * 2 slices (M + N) K bytes), runs on `cuda_stream` and returns when C holds
+ * dimension below the row length).  Takes its temporaries (about
+ * 2 slices (M + N) K bytes) from the pool of mlcc3_release_workspace, runs on `cuda_stream` and returns when C holds
  * the product; MLCC3_ERR_OOM when an allocation fails, MLCC3_ERR_TIMEOUT when
  * a tensor-core pipeline wait ran out (C is then not valid). */
 int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *B, long long ldb, double *C,
                        long long ldc, int M, int N, int K, int slices, void *cuda_stream);
+
+/* mlcc3_cnto_matrices and mlcc3_fp64emu_gemm take their temporaries from a pool
+ * that keeps up to 1 GiB of device memory between calls (allocating and freeing
+ * it took a fifth of a 4096^3 product).  This call gives all of it that is not in
+ * use back to the device, as destroying a context does; always MLCC3_OK. */
+int mlcc3_release_workspace(void);
 
 /* Triples residual without allocating (no counterpart in the paper).
  * Some callers cannot allocate device memory at the moment they call: a

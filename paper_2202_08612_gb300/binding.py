@@ -30,7 +30,7 @@ EXPORTS = ("mlcc3_create", "mlcc3_destroy", "mlcc3_last_error", "mlcc3_build_int
            "mlcc3_sweep_create", "mlcc3_sweep_set_system", "mlcc3_sweep_run", "mlcc3_sweep_info",
            "mlcc3_sweep_destroy", "mlcc3_rayleigh_quotient", "mlcc3_ground_density",
            "mlcc3_multiplier_transformation", "mlcc3_cnto_matrices", "mlcc3_shard_batches",
-           "mlcc3_transition_densities", "mlcc3_fp64emu_gemm")
+           "mlcc3_transition_densities", "mlcc3_fp64emu_gemm", "mlcc3_release_workspace")
 
 
 class MLCC3Error(RuntimeError):
@@ -146,6 +146,11 @@ def tc_gemm(A, B, C):
     rc = lib.mlcc3_debug_tc_gemm(_ptr(A), _ptr(B), _ptr(C), M, N, K)
     if rc != 0:
         raise MLCC3Error(rc, lib.mlcc3_last_error().decode())
+
+
+def release_workspace():
+    """mlcc3_release_workspace: give back what cnto_matrices and fp64emu_gemm keep between calls."""
+    load().mlcc3_release_workspace()
 
 
 def fp64emu_gemm(A, B, C, slices=5, stream=None):

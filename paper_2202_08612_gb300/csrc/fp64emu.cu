@@ -143,6 +143,11 @@ __global__ void __launch_bounds__(128) emu_slice_rows_kernel(const double *__res
 
 using namespace mlcc3;
 
+extern "C" int mlcc3_release_workspace(void) {
+  work_trim();
+  return MLCC3_OK;
+}
+
 // C = A B^T (FP64 device arrays; A [M][K] rows lda apart, B [N][K] rows ldb
 // apart, C [M][N] rows ldc apart) from `slices` digit slices of each operand.
 // Takes its temporaries (digit slices, exponents, the tile list) from the work

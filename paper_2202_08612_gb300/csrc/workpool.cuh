@@ -2,7 +2,8 @@
 // device that keeps up to kWorkKeep bytes between calls (allocating and freeing a
 // few hundred megabytes took 0.5 of the 2.1 ms of a 4096^3 product).  The pool is
 // CUDA's, so threads and streams may share it; work_trim gives the kept memory
-// back (when a context is destroyed, and when an allocation of the library fails).
+// back (mlcc3_release_workspace, when a context is destroyed, and when an allocation of
+// the library fails).
 #pragma once
 #include <cuda_runtime.h>
 
