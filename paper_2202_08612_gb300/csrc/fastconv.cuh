@@ -19,13 +19,12 @@ __device__ __forceinline__ float narrow_f64(double x) {
   return __double2float_rn(x);
 }
 
-// binary32 -> binary64 (exact) on the integer pipe; binary32 subnormals
-// (never produced here) become signed zeros.
+// binary32 -> binary64 (exact) on the integer pipe, but for subnormals.
 __device__ __forceinline__ double widen_f32(float f) {
   const unsigned int b = __float_as_uint(f);
   const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
   const unsigned int e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
-  if (e == 0) return __longlong_as_double((long long)sign);
+  if (e == 0) return m ? (double)f : __longlong_as_double((long long)sign);
   const unsigned long long ex = e == 255 ? 0x7FFull : (unsigned long long)(e + 896);
   return __longlong_as_double((long long)(sign | (ex << 52) | ((unsigned long long)m << 29)));
 }
