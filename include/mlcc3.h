@@ -59,8 +59,9 @@ extern "C" {
 
 /* Arithmetic of the contractions.  MLCC3_FP64: products and sums in IEEE
  * double, or, for the large contractions ("fp64_tc_from"), as integers: every
- * operand a multiple of 2^-63 of the power of two |A| above its largest element,
- * its base-256 digits multiplied on the tensor cores, the sums of up to 192 digit
+ * operand a multiple of 2^-63 of the power of two |A| above the largest element
+ * of its row (of the whole operand in the triples builds and for triples
+ * arrays), its base-256 digits multiplied on the tensor cores, the sums of up to 192 digit
  * products in FP32 (exact but for sums of nearly only largest digits of one sign,
  * and there to 2^-52 |A| |B|) and beyond that in integers, rounded to binary64
  * once.  An output sum_k a_k b_k errs by less than 2^-47 sum_k |a_k| |b_k|, the

@@ -174,6 +174,7 @@ struct mlcc3_ctx {
     int S = 0;
     long long slice = 0;
     const mlcc3::EmuScale *scale = nullptr;
+    bool row_scales = false;  // one per row (make_digits)
   };
   std::map<std::string, SplitOp> splits;
   // FP64 mode: the large contractions on the tensor cores (kernels_emu.cuh), from

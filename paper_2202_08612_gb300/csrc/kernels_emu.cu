@@ -1,6 +1,7 @@
 // FP64-accurate contractions on the BF16 tensor cores (sm_103a), after the
 // error-free splitting of Ozaki, Ogita, Oishi and Rump: an operand is an
-// integer of up to 63 bits per element (its value over one power of two), held
+// integer of up to 63 bits per element (its value over a power of two that its row or
+// the whole operand shares), held
 // as S balanced base-256 digits, each exact in bfloat16.  Products of digits
 // are integers of at most 2^14, which FP32 sums exactly over 256 of them for
 // the digit degrees t + u <= 3.  Kept are the degrees up to S - 1, and with S = 8 (the
@@ -307,7 +308,8 @@ __global__ void __launch_bounds__(320, 1)
     const int row = lg * 32 + lane, hn = n / 2;
     const uint32_t tm = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(half * hn);
     int e0 = epi.ebias - 32;
-    if (epi.sa) e0 += scale_exp(*epi.sa) + scale_exp(*epi.sb);
+    if (epi.sa && !epi.ra) e0 += scale_exp(*epi.sa);
+    if (epi.sb && !epi.rb) e0 += scale_exp(*epi.sb);
     int t = 0;
     bool ok = true;
     for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
@@ -399,7 +401,9 @@ __global__ void __launch_bounds__(320, 1)
       }
       if (!ok) break;
       if (FULL && __any_sync(0xffffffffu, weak) && lane == 0) atomicOr(status, kStatusSpread);
-      const int er = epi.ea && cmax ? e0 + epi.ea[it.r2_0 + row] : e0;
+      int er = e0;
+      if (FULL && epi.ra && cmax) er += scale_exp(epi.sa[it.ea + it.r2_0 + row]);
+      if (!FULL && epi.ea && cmax) er += epi.ea[it.r2_0 + row];
       double *o = epi.out + it.out_off + (long long)r1 * epi.s1 + (long long)r2 * epi.s2 + (long long)c0 * epi.sn;
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
@@ -409,7 +413,9 @@ __global__ void __launch_bounds__(320, 1)
           const int c = g * 8 + j;
           if (c0 + c >= cmax) break;
           long long x = T[c];
-          int ex = epi.eb ? er + epi.eb[c0 + c] : er;
+          int ex = er;
+          if (FULL && epi.rb) ex += scale_exp(epi.sb[it.eb + c0 + c]);
+          if (!FULL && epi.eb) ex += epi.eb[c0 + c];
           double v;
           if constexpr (FULL) {
             v = sum_to_double(x, U[c], ex);
@@ -588,16 +594,6 @@ cudaError_t emu_balance(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuSc
   return cudaGetLastError();
 }
 
-__global__ void emu_scale_double_kernel(EmuScale *s, int *status) {
-  if (scale_exp(*s) > 1023) atomicOr(status, kStatusSpread);
-  *s = (EmuScale)min(2046, scale_exp(*s) + 1023) << 52;
-}
-
-cudaError_t emu_scale_double(EmuScale *scale, int *status, cudaStream_t st) {
-  emu_scale_double_kernel<<<1, 1, 0, st>>>(scale, status);
-  return cudaGetLastError();
-}
-
 // ---- digits ----
 // x over 2^(e - 63), rounded to nearest: an integer below 2^63 - 2^56 for a scale's e.
 __device__ __forceinline__ long long to_fixed63(double x, int e) {
@@ -621,14 +617,16 @@ __device__ __forceinline__ long long to_fixed63(double x, int e) {
 // q + 0x0080..80, minus 128 each (the top byte: q's own, in [-127, 127]); a byte
 // becomes a bfloat16 through the FP32 number 2^23 + byte.  Bound by HBM: 8 bytes
 // read and 18 written per element.
+// MAXIMA: no digits, the rows' largest magnitudes instead.
+template <bool MAXIMA>
 __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp, long long slice,
-                                                         int neg, const EmuScale *scale,
+                                                         int neg, EmuScale *scale, long long zs, int rs,
                                                          __nv_bfloat16 *__restrict__ out,
                                                          const double *__restrict__ F, double fcoef,
                                                          int swap) {
   __shared__ double sm[32][65];
   __shared__ long long ro[32], ko[64];
-  const int e = scale_exp(*scale), tid = threadIdx.x;
+  const int tid = threadIdx.x;
   const int tr = (v.R + 31) / 32, tk = (Kp + 63) / 64;
   const long long tiles = (long long)v.Z * tr * tk;
   const bool kfast = v.K2 > 1 ? v.sk2 == 1 : v.sk1 == 1;
@@ -671,7 +669,24 @@ __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp
     for (int q = 0; q < 8; ++q) sm[rr[q]][kk[q]] = x[q];
     __syncthreads();
     const int r = tid / 8, kg = (tid % 8) * 8;
+    EmuScale *const rscale = scale + z * zs + (long long)(r0 + r) * rs;
+    if constexpr (MAXIMA) {
+      EmuScale m = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const EmuScale b = (EmuScale)__double_as_longlong(sm[r][kg + j]) & ~(1ULL << 63);
+        if (b < (0x7ffULL << 52) && b > m) m = b;
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        const EmuScale b = __shfl_xor_sync(0xffffffffu, m, o);
+        if (b > m) m = b;
+      }
+      if (kg == 0 && m && r0 + r < v.R) atomicMax(rscale, m);
+      continue;
+    }
     if (r0 + r < v.R && k0 + kg < Kp) {
+      const int e = scale_exp(*rscale);
       unsigned lo[8], hi[8], mag[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -715,14 +730,23 @@ __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp
   }
 }
 
-cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale,
-                       __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
+cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale, long long zs,
+                       int rs, __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
                        cudaStream_t st) {
   if (v.Z <= 0 || v.R <= 0 || Kp <= 0) return cudaSuccess;
   const long long tiles = (long long)v.Z * ((v.R + 31) / 32) * ((Kp + 63) / 64);
   const long long slice = (long long)v.Z * v.R * Kp;
-  emu_digits_kernel<<<(int)std::min<long long>(tiles, 152LL * 32), 256, 0, st>>>(
-      v, (int)Kp, slice, neg ? 1 : 0, scale, out, F, fcoef, swap ? 1 : 0);
+  emu_digits_kernel<false><<<(int)std::min<long long>(tiles, 152LL * 32), 256, 0, st>>>(
+      v, (int)Kp, slice, neg ? 1 : 0, const_cast<EmuScale *>(scale), zs, rs, out, F, fcoef, swap ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t emu_row_maxima(const EmuView &v, EmuScale *scale, long long zs, int rs, const double *F,
+                           double fcoef, bool swap, cudaStream_t st) {
+  if (v.Z <= 0 || v.R <= 0 || v.K <= 0) return cudaSuccess;
+  const long long tiles = (long long)v.Z * ((v.R + 31) / 32) * ((v.K + 63) / 64);
+  emu_digits_kernel<true><<<(int)std::min<long long>(tiles, 152LL * 32), 256, 0, st>>>(
+      v, v.K, 0, 0, scale, zs, rs, nullptr, F, fcoef, swap ? 1 : 0);
   return cudaGetLastError();
 }
 

@@ -22,18 +22,19 @@ constexpr int kEmuChain = 6;
 constexpr int kEmuMaxK = 8192;  // longest reduction of one item (TcSeg chunks times kEmuKB)
 
 // The device status bit of a product that the digits cannot hold to FP64 accuracy.  With
-// |A|, |B| the powers of two above the operands' largest elements, rounding an operand to
+// |A|, |B| the powers of two above the largest elements that share the operands' scales (a
+// row's, or the whole operand's), rounding an operand to
 // 2^-63 of its own errs by up to 2^-64 (|A| sum |b_k| + |B| sum |a_k|) in an output, over the
 // K with a_k b_k != 0, and the digit pairs left out by up to 2^-69.4 K |A| |B|.  The kernel
 // measures, for every output, P - c (|A| sum |b_k| + |B| sum |a_k|) with P = sum |a_k| |b_k| and
-// c = 2^-12, and sets the bit unless that is zero (as every product is) or at least
-// 2^-22 K |A| |B|.  So an output errs by less than 2^-52 P + 2^-47.4 P, where FP64 sums of 64
+// c = 2^-14, and sets the bit unless that is zero (as every product is) or at least
+// 2^-22 K |A| |B|.  So an output errs by less than 2^-50 P + 2^-47.4 P, where FP64 sums of 64
 // products (2^6 roundings of 2^-53) may err by 2^-47 P; and by about as much as FP64 sums
 // where the errors have random signs (the pairs left out 2^-72 K^(1/2) |A| |B|, FP64's
 // 2^-51.5 K^(1/2) |a| |b|).  Without the bit an operand spread over 10^6 lost ten digits of
 // its small outputs.
 constexpr int kStatusSpread = 4;
-constexpr float kEmuRound = 0x1p-12f;  // c
+constexpr float kEmuRound = 0x1p-14f;  // c
 constexpr float kEmuLeast = 0x1p-22f;
 
 // A digit operand's scale: the binary64 pattern of the operand's largest finite
@@ -53,8 +54,10 @@ struct EmuEpi {
   int amn;          // as TcEpi::amn (S = 8)
   int n;            // columns of a tile (a multiple of 16, at most emu_max_cols)
   int ebias;        // power of two of the leading digit product: -14
-  // scales: one per operand (sa, sb), or one exponent per output row and column
+  // scales of the operands: one, or (ra, rb) one per row of A and of B (r2_0 + row and the
+  // column, from the item's ea and eb on); S < 8: one exponent per output row and column
   const EmuScale *sa, *sb;
+  int ra, rb;
   const int *ea, *eb;
   long long wait;   // as TcEpi::wait
 };
@@ -82,8 +85,6 @@ cudaError_t emu_absmax(const double *x, long long n, EmuScale *scale, cudaStream
 // beyond binary64's exponents set kStatusSpread.
 cudaError_t emu_balance(EmuScale *a, const EmuScale *g, const EmuScale *t, EmuScale *u,
                         int *status, cudaStream_t st);
-// *scale = twice the power of two that bounds it
-cudaError_t emu_scale_double(EmuScale *scale, int *status, cudaStream_t st);
 
 // Source of a digit operand: element (z, r, k) at z1 sz1 + z2 sz2 + r1 sr1 +
 // r2 sr2 + k1 sk1 + k2 sk2 with z = z1 Z2 + z2 and so on.
@@ -97,8 +98,13 @@ struct EmuView {
 // not finite), whose products add up to what kStatusSpread asks for and c^2 K more:
 // out[slice][z][r][Kp].  F (optional, [z][K index of F]) with fcoef:
 // fcoef F[z][c] is added where the row equals b, (b, c) the K index pair (swap: (c, b)).
-cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale,
-                       __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
+// Scale of row (z, r): scale[z zs + r rs].
+cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale, long long zs,
+                       int rs, __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
                        cudaStream_t st);
+// Those scales: the largest finite magnitude of each row's elements (of all rows that
+// share one), where it is larger than the one there.
+cudaError_t emu_row_maxima(const EmuView &v, EmuScale *scale, long long zs, int rs, const double *F,
+                           double fcoef, bool swap, cudaStream_t st);
 
 }  // namespace mlcc3

@@ -40,6 +40,7 @@ struct TcItem {
   int c0;             // global column of the tile's first column
   int nq;             // column groups (0 or 1: one group of BN columns)
   int chunks;         // K chunks of all its segments
+  int ea, eb;         // FP64 mode: first row's and column's scales (EmuEpi::ra, rb) less r2_0 and c0
   int pad;
   long long out_off;
   long long qoff[3];

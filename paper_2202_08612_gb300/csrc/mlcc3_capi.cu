@@ -839,15 +839,13 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
                const BackSet &b, double *Zb);
 bool split_mode(const mlcc3_ctx *c);
 bool tc_mode(const mlcc3_ctx *c);
-void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const std::string &slot,
-              const double *F = nullptr, double fcoef = 0.0);
+void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const double *F = nullptr,
+              double fcoef = 0.0);
 void encode_split(mlcc3_ctx::SplitOp &op, const std::string &key, const unsigned long long dims[4],
                   const unsigned long long str[3], const unsigned bx[4]);
-mlcc3_ctx::SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G,
-                               const std::string &slot);
-mlcc3_ctx::SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk,
-                                const std::string &slot);
-void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T, const std::string &slot);
+mlcc3_ctx::SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G);
+mlcc3_ctx::SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk);
+void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T);
 void tc_integrals(mlcc3_ctx *c);
 void split_chol_kpairs(mlcc3_ctx *c);
 float *f32_copy(mlcc3_ctx *c, const std::string &key, const double *x, long long n);
@@ -1164,6 +1162,8 @@ void tc_launch(mlcc3_ctx *c, const char *site, int BN, const TcMaps &maps, const
     x.ebias = -14;
     x.sa = A.scale;
     x.sb = B.scale;
+    x.ra = A.row_scales ? 1 : 0;
+    x.rb = B.row_scales ? 1 : 0;
     x.wait = c->tc_wait;
     c->launch((std::string("emu_gemm_kernel:") + site).c_str(), flops, [&] {
       check_cuda(launch_emu_gemm(kEmuSlices, maps, d.items, d.segs, d.nitems, x, c->status, c->stream),
@@ -1201,18 +1201,36 @@ TcEpi make_epi(void *out, int mode, int R2, long long s1, long long s2, long lon
   return e;
 }
 
-// Digit slices of `v` as operand `key`.
+// Digit slices of `v` as operand `key`, at the scale `slot` (scale_of), or, with a slot of
+// kRowsEach (kRowsShared) and a name, at a scale per row (z, r) (per r, shared by all z) of
+// the array of that name, which is made here unless `scales_made`.  Row scales follow
+// the row of the output alone, so every product that an accumulation chain adds up has
+// them; they serve operands whose rows are not another contraction's K.
+const char *const kRowsEach = "@", *const kRowsShared = "%";
 void make_digits(mlcc3_ctx *c, SplitOp &op, const std::string &key, const EmuView &v, long long Kp,
                  bool neg, const std::string &slot, const double *F = nullptr, double fcoef = 0.0,
-                 bool swap = false) {
+                 bool swap = false, bool scales_made = false) {
   op.S = kEmuStored;
   op.slice = (long long)v.Z * v.R * Kp;
-  op.scale = scale_of(c, slot);
+  op.row_scales = slot[0] == kRowsEach[0] || slot[0] == kRowsShared[0];
+  const long long zs = slot[0] == kRowsEach[0] ? v.R : 0, n = zs ? (long long)v.Z * v.R : v.R;
+  if (op.row_scales) {
+    EmuScale *d = static_cast<EmuScale *>(c->raw("emu:rows:" + slot.substr(1), sizeof(EmuScale) * (size_t)std::max(1LL, n)));
+    op.scale = d;
+    if (!scales_made) {
+      check_cuda(cudaMemsetAsync(d, 0, sizeof(EmuScale) * (size_t)n, c->stream), "row scales");
+      c->launch("emu_row_maxima_kernel", 0.0, [&] {
+        check_cuda(emu_row_maxima(v, d, zs, 1, F, fcoef, swap, c->stream), "emu_row_maxima");
+      });
+    }
+  } else {
+    op.scale = scale_of(c, slot);
+  }
   op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuStored * 2);
   op.lo = nullptr;
   c->launch("emu_digits_kernel", 0.0, [&] {
-    check_cuda(emu_digits(v, Kp, neg, op.scale, static_cast<__nv_bfloat16 *>(op.hi), F, fcoef, swap,
-                          c->stream),
+    check_cuda(emu_digits(v, Kp, neg, op.scale, zs, op.row_scales ? 1 : 0, static_cast<__nv_bfloat16 *>(op.hi), F,
+                          fcoef, swap, c->stream),
                "emu_digits");
   });
 }
@@ -1512,12 +1530,12 @@ void build_split_persistent(mlcc3_ctx *c) {
   split_pairs(c, "Tl", c->Tl, s.NO, s.ti, s.ta, s.tb, "t");
   make_split(c, "Go:N", c->Go, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, "G");
   make_split(c, "Gx:N", c->Gx, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, "Gb");
-  split_gt(c, "Gb", c->Gb, "Gb", c->F, 0.5);  // Omega / rho: D slot g_Dbkc with 1/2 F_kc folded in
-  split_gt(c, "Gv", c->Gv, "G");
-  split_go_T(c, "Gx:T", c->Gx, "Gb");
-  split_go_T(c, "Go:T", c->Go, "G");
-  split_amp_T(c, "t:AT", c->t2c, "t");
-  split_tl_T(c, "Tl", c->Tl, "t");
+  split_gt(c, "Gb", c->Gb, c->F, 0.5);  // Omega / rho: D slot g_Dbkc with 1/2 F_kc folded in
+  split_gt(c, "Gv", c->Gv);
+  split_go_T(c, "Gx:T", c->Gx);
+  split_go_T(c, "Go:T", c->Go);
+  split_amp_T(c, "t:AT", c->t2c);
+  split_tl_T(c, "Tl", c->Tl);
   split_chol_kpairs(c);
 }
 
@@ -1526,14 +1544,14 @@ void build_split_persistent(mlcc3_ctx *c) {
 SplitOp &make_split_k2(mlcc3_ctx *c, const std::string &key, const double *src, long long D0,
                        long long D1, long long K1, long long K2, long long s0, long long s1,
                        long long sk1, long long sk2, unsigned rows, const std::string &slot,
-                       bool flat = false) {
+                       bool flat = false, bool scales_made = false) {
   const long long Kp = kpad(c, K1 * K2);
   SplitOp &op = c->splits[key];
   const size_t n = (size_t)(D0 * D1 * Kp);
   if (c->emu) {
     make_digits(c, op, key,
                 EmuView{src, (int)D0, 1, (int)D1, (int)D1, (int)(K1 * K2), (int)K2, s0, 0, 0, s1, sk1, sk2},
-                Kp, false, slot);
+                Kp, false, slot, nullptr, 0.0, false, scales_made);
   } else {
   op.hi = c->raw("split:" + key + ":hi", n * 2);
   op.lo = c->raw("split:" + key + ":lo", n * 2);
@@ -1588,27 +1606,18 @@ void split_chol_kpairs(mlcc3_ctx *c) {
   const long long nmo = s.nmo, NO = s.NO;
   const unsigned bj = (unsigned)tile_w(c, s.NJ);
   // Lt[J][NO+b][NO+D] as K = (b, D); Lt[J][NO+c][k] and Lt[J][k][NO+c] as K = (c, k)
-  make_split_k2(c, "LvV:J", c->Lt + NO * nmo + NO, 1, s.NJ, s.nv, s.NV, 0, s.lJ, nmo, 1, bj, "Lt", true);
-  make_split_k2(c, "Lvo:J", c->Lt + NO * nmo, 1, s.NJ, s.nv, s.no, 0, s.lJ, nmo, 1, bj, "Lt", true);
-  make_split_k2(c, "Lov:J", c->Lt + NO, 1, s.NJ, s.nv, s.no, 0, s.lJ, 1, nmo, bj, "Lt", true);
+  make_split_k2(c, "LvV:J", c->Lt + NO * nmo + NO, 1, s.NJ, s.nv, s.NV, 0, s.lJ, nmo, 1, bj, "@LvV:J", true);
+  make_split_k2(c, "Lvo:J", c->Lt + NO * nmo, 1, s.NJ, s.nv, s.no, 0, s.lJ, nmo, 1, bj, "@Lvo:J", true);
+  make_split_k2(c, "Lov:J", c->Lt + NO, 1, s.NJ, s.nv, s.no, 0, s.lJ, 1, nmo, bj, "@Lov:J", true);
 }
 
 // G[k][b][c][D] (Gv-like) transposed to [k][D][(b,c)] and [k][D][(c,b)].
 // The optional F[k][c] (with coefficient fcoef) is folded in as fcoef delta_{Db} F_kc:
 // the D-slot back-contraction then also carries the F_kc term of the doubles.
-void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const std::string &slot,
-              const double *F, double fcoef) {
+void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const double *F,
+              double fcoef) {
   S s(c);
   const long long Kp = kpad(c, s.nv * s.nv);
-  std::string gslot = slot;
-  if (c->emu && F) {  // |G + fcoef F| < 2 max(|G|, |F|) for |fcoef| <= 1
-    gslot = key + ":T";
-    EmuScale *d = scale_of(c, gslot);
-    check_cuda(cudaMemsetAsync(d, 0, sizeof(EmuScale), c->stream), "scale");
-    check_cuda(emu_absmax(G, (long long)s.gvsz(), d, c->stream), "emu_absmax");
-    check_cuda(emu_absmax(F, s.no * s.nv, d, c->stream), "emu_absmax");
-    check_cuda(emu_scale_double(d, c->status, c->stream), "emu_scale_double");
-  }
   for (int swap = 0; swap < 2; ++swap) {
     const std::string k2 = key + (swap ? ":Ts" : ":T");
     SplitOp &op = c->splits[k2];
@@ -1618,7 +1627,7 @@ void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const std::
       make_digits(c, op, k2,
                   EmuView{G, (int)s.no, 1, (int)s.NV, (int)s.NV, (int)(s.nv * s.nv), (int)s.nv, s.gk, 0, 0,
                           1, swap ? s.gc : s.gb, swap ? s.gb : s.gc},
-                  Kp, false, gslot, F, fcoef, swap != 0);
+                  Kp, false, kRowsEach + key + ":T", F, fcoef, swap != 0, swap != 0);
     } else {
     op.hi = c->raw("split:" + k2 + ":hi", n * 2);
     op.lo = c->raw("split:" + k2 + ":lo", n * 2);
@@ -1655,8 +1664,7 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
   const SplitOp &x1 = layout_XL(c, "bD:XL1", X, 1, BN);
   const SplitOp &x2 = layout_XL(c, "bD:XL2", X, 2, BN);
   if (b.gd_convert) {
-    if (!b.F) scale_max(c, b.gd_key, {{b.GD, (long long)s.gvsz()}});
-    split_gt(c, b.gd_key, b.GD, b.gd_key, b.F, b.F ? b.cF / b.cD : 0.0);
+    split_gt(c, b.gd_key, b.GD, b.F, b.F ? b.cF / b.cD : 0.0);
   }
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
@@ -1687,6 +1695,7 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
         for (long long tn = 0; tn < ntN; ++tn) {
           const Ord &o = *os[q0];
           pl.tile(0, (int)(128 * t), (int)(BN * tn), o.p * s.bi + o.q * s.bL);
+          pl.items.back().ea = (int)(o.r * s.NV);  // (k, D) scales
           pl.items.back().nq = nq;
           for (int q = 1; q < nq; ++q)
             pl.items.back().qoff[q - 1] = os[q0 + q]->p * s.bi + os[q0 + q]->q * s.bL;
@@ -2024,23 +2033,23 @@ void tc_vv(mlcc3_ctx *c, const double *X, const std::string &xkey, const double 
 
 // Split copies of small operands (per call or at build):
 // amplitude block X[p][a][q][D] as [p][q][D][a] (Y1/P2 B operand)
-SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk, const std::string &slot) {
+SplitOp &split_amp_T(mlcc3_ctx *c, const std::string &key, const double *Xblk) {
   S s(c);
-  return make_split(c, key, Xblk, s.no, s.no, s.NV, s.nv, s.bi, s.bL, 1, s.ba, 1.0, Box::Row, slot,
+  return make_split(c, key, Xblk, s.no, s.no, s.NV, s.nv, s.bi, s.bL, 1, s.ba, 1.0, Box::Row, kRowsShared + key,
                     (unsigned)pair_bn(c, s.NV));
 }
 // Go-like G[q][r][c][L] as [q][r][L][c] (Z_L B operand)
-SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G, const std::string &slot) {
+SplitOp &split_go_T(mlcc3_ctx *c, const std::string &key, const double *G) {
   S s(c);
-  return make_split(c, key, G, s.no, s.no, s.NO, s.nv, s.oj, s.ok, 1, s.oc, 1.0, Box::Row, slot,
+  return make_split(c, key, G, s.no, s.no, s.NO, s.nv, s.oj, s.ok, 1, s.oc, 1.0, Box::Row, kRowsShared + key,
                     (unsigned)pair_bn(c, s.NO));
 }
 // Tl-like T[p][x][y][L] as [p][L][(x,y)] and [p][L][(y,x)] (tc_xt operands)
-void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T, const std::string &slot) {
+void split_tl_T(mlcc3_ctx *c, const std::string &key, const double *T) {
   S s(c);
   const unsigned bn = (unsigned)tile_w(c, s.NO);
-  make_split_k2(c, key + ":T", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.ta, s.tb, bn, slot);
-  make_split_k2(c, key + ":Ts", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.tb, s.ta, bn, slot);
+  make_split_k2(c, key + ":T", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.ta, s.tb, bn, kRowsShared + key);
+  make_split_k2(c, key + ":Ts", T, s.no, s.NO, s.nv, s.nv, s.ti, 1, s.tb, s.ta, bn, kRowsShared + key, false, true);
 }
 
 // Z[p][a][L][b] += cL sum_{qr} sum_c X_{pqr}[a][b][c] G_{qr}[c][L] on the tensor cores.
@@ -2048,8 +2057,7 @@ void tc_back_L(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
                const BackSet &b, double *Zb) {
   S s(c);
   if (b.gl_convert) {
-    scale_max(c, b.gl_key, {{b.GL, (long long)s.gosz()}});
-    split_go_T(c, b.gl_key + ":T", b.GL, b.gl_key);
+    split_go_T(c, b.gl_key + ":T", b.GL);
   }
   tc_pair(c, X, "X", c->splits.at(b.gl_key + ":T"), s.NO, ords, okey, 2, 0, s.bi, s.ba, 1, s.bL,
           b.cL, Zb);
@@ -2069,6 +2077,11 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
   S s(c);
   const long long M = s.no * s.nv;
   if (M == 0 || nN == 0 || nW == 0) return;
+  if (c->emu && terms.size() > 1) {  // the products have row scales of their own: one after the other
+    for (size_t t = 0; t < terms.size(); ++t)
+      tc_chol(c, {terms[t]}, nW, nN, Sw, Sk, Sc, alpha, t == 0 ? mode : 2, out, key + "+" + std::to_string(t), Sn);
+    return;
+  }
   if (terms.size() * 4 > (size_t)kTcMaps) throw Error{MLCC3_ERR_ARG, "too many Cholesky terms"};
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
@@ -2095,6 +2108,7 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
       for (long long tm = 0; tm < ntM; ++tm)
         for (long long tn = 0; tn < ntN; ++tn) {
           pl.tile(0, (int)(128 * tm), (int)(BN * tn), w * Sw);
+          pl.items.back().eb = (int)(w * nN);  // (w, n) scales
           for (size_t t = 0; t < terms.size(); ++t)
           {
             pl.seg((int)(4 * t), (int)(4 * t + 2), nk, (int)(128 * tm), 0, 0, (int)(BN * tn),
@@ -2111,15 +2125,15 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
 // Split copies over the Cholesky index (K = J, stride lJ = n_mo^2 in Lt-like arrays).
 // rows (k,c) of X[J][r0 + c][k] (row offset r0, c stride cs, k stride ks), Flat 128-row box
 SplitOp &split_kc(mlcc3_ctx *c, const std::string &key, const double *X, long long ks, long long cs,
-                  long long Js, const std::string &slot) {
+                  long long Js) {
   S s(c);
-  return make_split(c, key, X, 1, s.no, s.nv, s.NJ, 0, ks, cs, Js, 1.0, Box::Flat, slot, 128);
+  return make_split(c, key, X, 1, s.no, s.nv, s.NJ, 0, ks, cs, Js, 1.0, Box::Flat, kRowsEach + key, 128);
 }
 // rows (w, n) of X with strides (ws, ns), K = J (stride Js), Row box of BN rows
 SplitOp &split_wn(mlcc3_ctx *c, const std::string &key, const double *X, long long nW, long long nN,
-                  long long ws, long long ns, long long Js, const std::string &slot) {
+                  long long ws, long long ns, long long Js) {
   S s(c);
-  return make_split(c, key, X, 1, nW, nN, s.NJ, 0, ws, ns, Js, 1.0, Box::Row, slot,
+  return make_split(c, key, X, 1, nW, nN, s.NJ, 0, ws, ns, Js, 1.0, Box::Row, kRowsEach + key,
                     (unsigned)tile_w(c, nN));
 }
 
@@ -2129,20 +2143,19 @@ void tc_integrals(mlcc3_ctx *c) {
   S s(c);
   const long long nmo = s.nmo, NO = s.NO;
   const double *Lt = c->Lt;
-  scale_max(c, "Lt", {{Lt, s.NJ * s.lJ}});
-  split_kc(c, "LvoT", Lt + NO * nmo, 1, nmo, s.lJ, "Lt");
-  split_kc(c, "LovT", Lt + NO, nmo, 1, s.lJ, "Lt");
-  split_wn(c, "LvVT", Lt + NO * nmo + NO, s.nv, s.NV, nmo, 1, s.lJ, "Lt");
-  split_wn(c, "LVvT", Lt + NO * nmo + NO, s.nv, s.NV, 1, nmo, s.lJ, "Lt");
-  split_wn(c, "LOoT", Lt, s.no, s.NO, 1, nmo, s.lJ, "Lt");
+  split_kc(c, "LvoT", Lt + NO * nmo, 1, nmo, s.lJ);
+  split_kc(c, "LovT", Lt + NO, nmo, 1, s.lJ);
+  split_wn(c, "LvVT", Lt + NO * nmo + NO, s.nv, s.NV, nmo, 1, s.lJ);
+  split_wn(c, "LVvT", Lt + NO * nmo + NO, s.nv, s.NV, 1, nmo, s.lJ);
+  split_wn(c, "LOoT", Lt, s.no, s.NO, 1, nmo, s.lJ);
   tc_chol(c, {{&c->splits.at("LvoT"), &c->splits.at("LvVT")}}, s.nv, s.NV, s.gb, s.gk, s.gc, 1.0, 3,
           c->Gv, "Gv");
   tc_chol(c, {{&c->splits.at("LovT"), &c->splits.at("LVvT")}}, s.nv, s.NV, s.gb, s.gk, s.gc, 1.0, 3,
           c->Gb, "Gb");
   if (!c->emu) return;
   // FP64 mode: the small blocks g_Ljck, g_jLkc, g_jbkc as well
-  const SplitOp &LoOT = split_wn(c, "LoOT", Lt, s.no, s.NO, nmo, 1, s.lJ, "Lt");
-  const SplitOp &LovB = split_wn(c, "LovB", Lt + NO, s.no, s.nv, nmo, 1, s.lJ, "Lt");
+  const SplitOp &LoOT = split_wn(c, "LoOT", Lt, s.no, s.NO, nmo, 1, s.lJ);
+  const SplitOp &LovB = split_wn(c, "LovB", Lt + NO, s.no, s.nv, nmo, 1, s.lJ);
   tc_chol(c, {{&c->splits.at("LvoT"), &c->splits.at("LOoT")}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, c->Go, "Go");
   tc_chol(c, {{&c->splits.at("LovT"), &LoOT}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, c->Gx, "Gx");
   tc_chol(c, {{&c->splits.at("LovT"), &LovB}}, s.no, s.nv, s.vj, s.vk, 1, 1.0, 3, c->Govov, "Govov", s.vb);
@@ -2153,20 +2166,16 @@ bool tc_upsilon(mlcc3_ctx *c, const double *LRvV, const double *LRvo, const doub
                 const double *PA, const double *PB, double *Uv, double *Uo, double *H1, double *H2) {
   if (!tc_mode(c)) return false;
   S s(c);
-  // one scale for the three factors: each product below pairs one with Lt
-  scale_max(c, "LR", {{LRvV, s.NJ * s.nv * s.NV}, {LRvo, s.NJ * s.nv * s.no}, {LROo, s.NJ * s.NO * s.no}});
-  const SplitOp &rvV = split_wn(c, "LRvVT", LRvV, s.nv, s.NV, s.NV, 1, s.nv * s.NV, "LR");
-  const SplitOp &rvo = split_kc(c, "LRvoT", LRvo, 1, s.no, s.nv * s.no, "LR");
-  const SplitOp &rOo = split_wn(c, "LROoT", LROo, s.no, s.NO, 1, s.no, s.NO * s.no, "LR");
+  const SplitOp &rvV = split_wn(c, "LRvVT", LRvV, s.nv, s.NV, s.NV, 1, s.nv * s.NV);
+  const SplitOp &rvo = split_kc(c, "LRvoT", LRvo, 1, s.no, s.nv * s.no);
+  const SplitOp &rOo = split_wn(c, "LROoT", LROo, s.no, s.NO, 1, s.no, s.NO * s.no);
   const SplitOp &vo = c->splits.at("LvoT"), &ov = c->splits.at("LovT");
   const SplitOp &vV = c->splits.at("LvVT"), &Oo = c->splits.at("LOoT");
   tc_chol(c, {{&vo, &rvV}, {&rvo, &vV}}, s.nv, s.NV, s.gb, s.gk, s.gc, 1.0, 3, Uv, "Uv");
   tc_chol(c, {{&vo, &rOo}, {&rvo, &Oo}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, Uo, "Uo");
   if (!H1) return true;  // no rho tau-term intermediates wanted
-  scale_max(c, "PA", {{PA, s.NJ * s.no * s.NO}});
-  scale_max(c, "PB", {{PB, s.NJ * s.nv * s.NV}});
-  const SplitOp &pa = split_wn(c, "PAT", PA, s.no, s.NO, s.NO, 1, s.no * s.NO, "PA");
-  const SplitOp &pb = split_wn(c, "PBT", PB, s.nv, s.NV, s.NV, 1, s.nv * s.NV, "PB");
+  const SplitOp &pa = split_wn(c, "PAT", PA, s.no, s.NO, s.NO, 1, s.no * s.NO);
+  const SplitOp &pb = split_wn(c, "PBT", PB, s.nv, s.NV, s.NV, 1, s.nv * s.NV);
   tc_chol(c, {{&ov, &pa}}, s.no, s.NO, s.oj, s.ok, s.oc, 1.0, 3, H1, "H1");
   tc_chol(c, {{&ov, &pb}}, s.nv, s.NV, s.gb, s.gk, s.gc, -1.0, 3, H2, "H2");
   return true;
@@ -2589,9 +2598,8 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     c->zero(Y3, s.no * s.nv);
     const SplitOp *LcA = nullptr;
     if (tc_mode(c)) {
-      scale_max(c, "LcA", {{Lc, (long long)s.blk()}});
-      LcA = &split_amp_T(c, "Lc:AT", Lc, "LcA");
-      split_tl_T(c, "LcT", LcT, "LcA");
+      LcA = &split_amp_T(c, "Lc:AT", Lc);
+      split_tl_T(c, "LcT", LcT);
     }
     const double *Lc32 = f32_operand(c, "Lc:y3", Lc, (long long)s.blk(), true);
     for (const Chunk &ch : chunks) {
@@ -2664,8 +2672,7 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     // W[J][k][c] = sum_{b,D} Y1[k][b][c][D] Lt[J][NO+b][NO+D] - sum_{L,j} Y2[j][k][c][L] Lt[J][L][j]
     const bool tc = tc_mode(c);
     if (tc) {
-      scale_max(c, "Y1", {{Y1, (long long)s.gvsz()}});
-      const SplitOp &a = make_split_k2(c, "Y1:kc", Y1, s.no, s.nv, s.nv, s.NV, s.gk, s.gc, s.gb, 1, 128, "Y1", true);
+      const SplitOp &a = make_split_k2(c, "Y1:kc", Y1, s.no, s.nv, s.nv, s.NV, s.gk, s.gc, s.gb, 1, 128, "@Y1:kc", true);
       tc_flat_gemm(c, a, c->splits.at("LvV:J"), s.no * s.nv, s.NJ, s.nv * s.NV, W, (int)s.nv, s.nv, 1,
                    s.no * s.nv, 1.0, "sg1");
     } else {
@@ -2682,7 +2689,7 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     c->bstc1(W, Lt, sig1, sh, -1.0, mk_item(0, 0, 0, {1, 0, s.no * s.nv, s.nv, 0}, {s.lJ, 1, 0, nmo, 0}, {NO, 0, 1, 0}), "sg4");
     // Z2[J][b][D] = sum_{c,k} Y1[k][b][c][D] Lt[J][NO+c][k];  sigma[b][M] -= sum_{J,D} Z2 Lt[J][M][NO+D]
     if (tc) {
-      const SplitOp &a = make_split_k2(c, "Y1:bD", Y1, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, "Y1", true);
+      const SplitOp &a = make_split_k2(c, "Y1:bD", Y1, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, "@Y1:bD", true);
       tc_flat_gemm(c, a, c->splits.at("Lvo:J"), s.nv * s.NV, s.NJ, s.nv * s.no, Z2, (int)s.NV, s.NV, 1,
                    s.nv * s.NV, 1.0, "sg5");
     } else {
@@ -2716,8 +2723,7 @@ static void do_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega, const
     // P2 term: Q2[J][b][D] = sum_{c,k} P2[k][b][c][D] Lt[J][k][NO+c]; sigma[D][L] -= sum_{J,b} Q2 Lt[J][L][NO+b]
     c->zero(Q2, s.NJ * s.nv * s.NV);
     if (tc) {
-      scale_max(c, "P2", {{P2, (long long)s.gvsz()}});
-      const SplitOp &a = make_split_k2(c, "P2:bD", P2, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, "P2", true);
+      const SplitOp &a = make_split_k2(c, "P2:bD", P2, s.nv, s.NV, s.nv, s.no, s.gb, 1, s.gc, s.gk, 128, "@P2:bD", true);
       tc_flat_gemm(c, a, c->splits.at("Lov:J"), s.nv * s.NV, s.NJ, s.nv * s.no, Q2, (int)s.NV, s.NV, 1,
                    s.nv * s.NV, 1.0, "sg15");
     } else {
@@ -3162,8 +3168,7 @@ static void do_transition_density(mlcc3_ctx *c, int n_st, const double *omega_h,
     const std::string stag = std::to_string(st);
     // split copies of the state's operands: made at the first chunk, kept per state
     if (tc_mode(c) && first) {
-      scale_max(c, "Rbl" + stag, {{Rbl, s.no * s.nv * s.nv * NO}});
-      split_tl_T(c, "Rbl" + stag, Rbl, "Rbl" + stag);
+      split_tl_T(c, "Rbl" + stag, Rbl);
     }
     // L3 (omega) and R3 (omega), with their contravariant forms (CVS: core batches only)
     double *L3 = c->tri_buf("L3", bw);
