@@ -19,14 +19,39 @@ __device__ __forceinline__ float narrow_f64(double x) {
   return __double2float_rn(x);
 }
 
-// binary32 -> binary64 (exact) on the integer pipe, but for subnormals.
-__device__ __forceinline__ double widen_f32(float f) {
+// binary32 -> binary64 (exact) on the integer pipe, for numbers that are not subnormal.
+__device__ __forceinline__ double widen_normal(float f) {
   const unsigned int b = __float_as_uint(f);
   const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
   const unsigned int e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
-  if (e == 0) return m ? (double)f : __longlong_as_double((long long)sign);
+  if (e == 0) return __longlong_as_double((long long)sign);
   const unsigned long long ex = e == 255 ? 0x7FFull : (unsigned long long)(e + 896);
   return __longlong_as_double((long long)(sign | (ex << 52) | ((unsigned long long)m << 29)));
+}
+
+// The same for any number: subnormals by the hardware conversion.
+__device__ __forceinline__ double widen_f32(float f) {
+  return (__float_as_uint(f) << 1) - 1u < 0xFFFFFFu ? (double)f : widen_normal(f);
+}
+
+// sum[i] += f[i], one look for subnormals for all of them.
+template <int N>
+__device__ __forceinline__ void widen_add(double (&sum)[N], const float (&f)[N]) {
+  unsigned least = ~0u;
+#pragma unroll
+  for (int i = 0; i < N; ++i) least = min(least, (__float_as_uint(f[i]) << 1) - 1u);
+  if (least < 0xFFFFFFu) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) sum[i] += (double)f[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) sum[i] += widen_normal(f[i]);
+  }
+}
+template <int N>
+__device__ __forceinline__ void widen_add(double (&sum)[N], const double (&f)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) sum[i] += f[i];
 }
 
 // x ~ hi + lo with hi = bf16(f), lo = bf16(f - hi), f = binary32(x); f - hi is

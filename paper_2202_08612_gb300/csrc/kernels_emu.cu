@@ -316,17 +316,20 @@ __global__ void __launch_bounds__(320, 1)
       if (__shfl_sync(0xffffffffu, *abort_flag, 0)) break;
       const TcItem it = items[i];
       const int chains = (it.chunks + kChain - 1) / kChain;
-      int r1, r2;
-      if (epi.linear) {
-        const int m = it.r2_0 + row;
-        r1 = m / epi.R2;
-        r2 = m % epi.R2;
-      } else {
-        r1 = it.r1_0 + row / epi.R2;
-        r2 = it.r2_0 + row % epi.R2;
-      }
-      const int cmax = r1 < epi.lim1 && r2 < epi.lim2 ? epi.nlim : 0;
       const int c0 = it.c0 + half * hn;
+      int r1 = 0, r2 = 0, cmax = 0;
+      auto place = [&] {
+        if (epi.linear) {
+          const int m = it.r2_0 + row;
+          r1 = m / epi.R2;
+          r2 = m % epi.R2;
+        } else {
+          r1 = it.r1_0 + row / epi.R2;
+          r2 = it.r2_0 + row % epi.R2;
+        }
+        cmax = r1 < epi.lim1 && r2 < epi.lim2 ? epi.nlim : 0;
+      };
+      if (FULL) place();
       long long T[NG * 8];
       long long U[FULL ? NG * 8 : 1];  // degrees 5..8
       float L[S == 6 ? NG * 8 : 1];    // degree 5
@@ -400,6 +403,7 @@ __global__ void __launch_bounds__(320, 1)
         if (lane == 0) mbar_arrive(tempty);
       }
       if (!ok) break;
+      if (!FULL) place();  // (registers)
       if (FULL && __any_sync(0xffffffffu, weak) && lane == 0) atomicOr(status, kStatusSpread);
       int er = e0;
       if (FULL && epi.ra && cmax) er += scale_exp(epi.sa[it.ea + it.r2_0 + row]);

@@ -187,12 +187,11 @@ __global__ void __launch_bounds__(256, TM * TN <= 1024 && RM == RN ? 3 : TM * TN
     }
     if (!SHORT && ((t + 1) % (64 / TK) == 0 || t + 1 == tiles)) {
 #pragma unroll
-      for (int i = 0; i < RM; ++i)
+      for (int i = 0; i < RM; ++i) {
+        widen_add(sum[i], acc[i]);
 #pragma unroll
-        for (int j = 0; j < RN; ++j) {
-          sum[i][j] += widen_f32(acc[i][j]);
-          acc[i][j] = 0.f;
-        }
+        for (int j = 0; j < RN; ++j) acc[i][j] = 0.f;
+      }
     }
   }
   double *C = p.C + it.offC;
@@ -2257,9 +2256,7 @@ __device__ __forceinline__ void pair_dots_body(const T *__restrict__ X,
           for (int y = 0; y < D; ++y) p[x][y] += w[x] * u[y];
       }
 #pragma unroll
-      for (int x = 0; x < D; ++x)
-#pragma unroll
-        for (int y = 0; y < D; ++y) acc[x][y] += to_f64(p[x][y]);
+      for (int x = 0; x < D; ++x) widen_add(acc[x], p[x]);
     }
   }
   if (tail && tk < no && tl < no)
@@ -2415,9 +2412,7 @@ __global__ void __launch_bounds__(256, D == 3 ? 3 : 2) pair_dots_phys_kernel(
         }
       }
 #pragma unroll
-      for (int x = 0; x < D; ++x)
-#pragma unroll
-        for (int y = 0; y < D; ++y) acc[x][y] += to_f64(p[x][y]);
+      for (int x = 0; x < D; ++x) widen_add(acc[x], p[x]);
     }
   }
   pair_dots_add(smraw, acc, tile, h, TT, H, nh, no, out, ldo, kl, wij * alpha);

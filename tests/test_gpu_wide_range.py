@@ -130,3 +130,25 @@ def test_outputs_over_their_inputs(decades):
         getattr(g, call)(c.st.omega, x1, x2, z1, x2)
         assert np.linalg.norm(c.host(x2) - c.host(y2)) < TOL * np.linalg.norm(c.host(y2))
         assert np.linalg.norm(c.host(z1) - c.host(y1)) < TOL * np.linalg.norm(c.host(y1))
+
+
+def test_weak_rows_stay_on_the_tensor_cores():
+    """A vector whose elements on some inactive virtual orbitals are 10^-9 of the others makes
+    weak rows in Upsilon's factors, which have scales of their own: no FP64 build is launched,
+    and the parts of rho that come from those orbitals alone are as on the FP64 pipe."""
+    _cuda()
+    c = Case(7, 60, 3, 32, 60, nstates=1, t2_norm=0.3)
+    c.st.R1, c.st.R2 = np.array(c.st.R1), np.array(c.st.R2)
+    c.st.R1[0, 40:50] *= 1e-9
+    c.st.R2[...] = 0.0
+    outs = []
+    for start in (1, 2000):
+        g = c.context(params={"fp64_tc_from": start})
+        r1, r2 = c.empty_dev(c.st.R1.shape), c.empty_dev(c.st.R2.shape)
+        g.profile(False)
+        g.jacobian_right(c.st.omega, c.to_dev(c.st.R1), c.to_dev(c.st.R2), r1, r2)
+        names = set(g.kernel_stats())
+        assert ("triples_build_kernel" in names) == (start == 2000), names
+        outs.append((c.host(r1), c.host(r2)))
+    for x, y in zip(*outs):
+        assert np.linalg.norm(x - y) < 1e-12 * np.linalg.norm(y)
