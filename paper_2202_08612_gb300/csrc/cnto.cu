@@ -219,7 +219,7 @@ cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, doub
   for (long long k0 = 0; k0 < n && e == cudaSuccess; k0 += kc) {
     // (a shorter last chunk is padded with zeros)
     const EmuView v{R2 + k0, 1, 1, (int)n, (int)n, (int)std::min(kc, n - k0), 1, 0, 0, 0, n, 1, 0};
-    e = emu_digits(v, kc, false, scale, 0, 0, dig, nullptr, 0.0, false, st);
+    e = emu_digits(v, kc, false, scale, 0, 0, dig, st);
     for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
       TcMaps maps{};
       const unsigned long long rb = (unsigned long long)kc * 2;

@@ -625,9 +625,7 @@ __device__ __forceinline__ long long to_fixed63(double x, int e) {
 template <bool MAXIMA>
 __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp, long long slice,
                                                          int neg, EmuScale *scale, long long zs, int rs,
-                                                         __nv_bfloat16 *__restrict__ out,
-                                                         const double *__restrict__ F, double fcoef,
-                                                         int swap) {
+                                                         __nv_bfloat16 *__restrict__ out) {
   __shared__ double sm[32][65];
   __shared__ long long ro[32], ko[64];
   const int tid = threadIdx.x;
@@ -663,11 +661,6 @@ __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp
       }
       const long long a = ro[rr[q]], b = ko[kk[q]];
       x[q] = (a >= 0 && b >= 0) ? src[a + b] : 0.0;
-      if (F && a >= 0 && b >= 0) {
-        const int k = k0 + kk[q], i1 = k / v.K2, i2 = k % v.K2;
-        const int bi = swap ? i2 : i1, ci = swap ? i1 : i2;
-        if (bi == r0 + rr[q]) x[q] += fcoef * F[(long long)z * v.K2 + ci];
-      }
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) sm[rr[q]][kk[q]] = x[q];
@@ -735,22 +728,20 @@ __global__ void __launch_bounds__(256) emu_digits_kernel(const EmuView v, int Kp
 }
 
 cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale, long long zs,
-                       int rs, __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
-                       cudaStream_t st) {
+                       int rs, __nv_bfloat16 *out, cudaStream_t st) {
   if (v.Z <= 0 || v.R <= 0 || Kp <= 0) return cudaSuccess;
   const long long tiles = (long long)v.Z * ((v.R + 31) / 32) * ((Kp + 63) / 64);
   const long long slice = (long long)v.Z * v.R * Kp;
   emu_digits_kernel<false><<<(int)std::min<long long>(tiles, 152LL * 32), 256, 0, st>>>(
-      v, (int)Kp, slice, neg ? 1 : 0, const_cast<EmuScale *>(scale), zs, rs, out, F, fcoef, swap ? 1 : 0);
+      v, (int)Kp, slice, neg ? 1 : 0, const_cast<EmuScale *>(scale), zs, rs, out);
   return cudaGetLastError();
 }
 
-cudaError_t emu_row_maxima(const EmuView &v, EmuScale *scale, long long zs, int rs, const double *F,
-                           double fcoef, bool swap, cudaStream_t st) {
+cudaError_t emu_row_maxima(const EmuView &v, EmuScale *scale, long long zs, int rs, cudaStream_t st) {
   if (v.Z <= 0 || v.R <= 0 || v.K <= 0) return cudaSuccess;
   const long long tiles = (long long)v.Z * ((v.R + 31) / 32) * ((v.K + 63) / 64);
   emu_digits_kernel<true><<<(int)std::min<long long>(tiles, 152LL * 32), 256, 0, st>>>(
-      v, v.K, 0, 0, scale, zs, rs, nullptr, F, fcoef, swap ? 1 : 0);
+      v, v.K, 0, 0, scale, zs, rs, nullptr);
   return cudaGetLastError();
 }
 

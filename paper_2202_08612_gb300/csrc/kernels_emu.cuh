@@ -96,15 +96,11 @@ struct EmuView {
 // The kEmuSlices digit slices of `v` at `scale` (negated if neg), K padded with zeros to
 // Kp, and as slice kEmuSlices |x| 2^-e - c in bfloat16 (zero only for x = 0, NaN where x is
 // not finite), whose products add up to what kStatusSpread asks for and c^2 K more:
-// out[slice][z][r][Kp].  F (optional, [z][K index of F]) with fcoef:
-// fcoef F[z][c] is added where the row equals b, (b, c) the K index pair (swap: (c, b)).
-// Scale of row (z, r): scale[z zs + r rs].
+// out[slice][z][r][Kp].  Scale of row (z, r): scale[z zs + r rs].
 cudaError_t emu_digits(const EmuView &v, long long Kp, bool neg, const EmuScale *scale, long long zs,
-                       int rs, __nv_bfloat16 *out, const double *F, double fcoef, bool swap,
-                       cudaStream_t st);
+                       int rs, __nv_bfloat16 *out, cudaStream_t st);
 // Those scales: the largest finite magnitude of each row's elements (of all rows that
 // share one), where it is larger than the one there.
-cudaError_t emu_row_maxima(const EmuView &v, EmuScale *scale, long long zs, int rs, const double *F,
-                           double fcoef, bool swap, cudaStream_t st);
+cudaError_t emu_row_maxima(const EmuView &v, EmuScale *scale, long long zs, int rs, cudaStream_t st);
 
 }  // namespace mlcc3

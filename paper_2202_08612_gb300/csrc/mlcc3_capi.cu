@@ -902,8 +902,9 @@ void back_contract(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords,
                      {s.vb, 1, 0, 0, 0}, {s.NO, 0, 0, 0});
     });
   }
-  // tensor cores: the F term rides on the D-slot GEMM (split_gt folds cF/cD F_kc into it)
-  if (bset.F && !(tc_mode(c) && bset.GD)) {
+  // split mode: the F term rides on the D-slot GEMM (split_gt folds cF/cD F_kc into it).  Not
+  // on digits: an F_kc far above its row of the integrals would set the row's scale
+  if (bset.F && !(split_mode(c) && bset.GD)) {
     it = c->dev_items(okey + ":bF", [&] {
       std::vector<BstcItem> v;
       for (auto &o : ords)
@@ -1208,8 +1209,7 @@ TcEpi make_epi(void *out, int mode, int R2, long long s1, long long s2, long lon
 // them; they serve operands whose rows are not another contraction's K.
 const char *const kRowsEach = "@", *const kRowsShared = "%";
 void make_digits(mlcc3_ctx *c, SplitOp &op, const std::string &key, const EmuView &v, long long Kp,
-                 bool neg, const std::string &slot, const double *F = nullptr, double fcoef = 0.0,
-                 bool swap = false, bool scales_made = false) {
+                 bool neg, const std::string &slot, bool scales_made = false) {
   op.S = kEmuStored;
   op.slice = (long long)v.Z * v.R * Kp;
   op.row_scales = slot[0] == kRowsEach[0] || slot[0] == kRowsShared[0];
@@ -1220,7 +1220,7 @@ void make_digits(mlcc3_ctx *c, SplitOp &op, const std::string &key, const EmuVie
     if (!scales_made) {
       check_cuda(cudaMemsetAsync(d, 0, sizeof(EmuScale) * (size_t)n, c->stream), "row scales");
       c->launch("emu_row_maxima_kernel", 0.0, [&] {
-        check_cuda(emu_row_maxima(v, d, zs, 1, F, fcoef, swap, c->stream), "emu_row_maxima");
+        check_cuda(emu_row_maxima(v, d, zs, 1, c->stream), "emu_row_maxima");
       });
     }
   } else {
@@ -1229,8 +1229,8 @@ void make_digits(mlcc3_ctx *c, SplitOp &op, const std::string &key, const EmuVie
   op.hi = c->raw("digits:" + key, (size_t)op.slice * kEmuStored * 2);
   op.lo = nullptr;
   c->launch("emu_digits_kernel", 0.0, [&] {
-    check_cuda(emu_digits(v, Kp, neg, op.scale, zs, op.row_scales ? 1 : 0, static_cast<__nv_bfloat16 *>(op.hi), F,
-                          fcoef, swap, c->stream),
+    check_cuda(emu_digits(v, Kp, neg, op.scale, zs, op.row_scales ? 1 : 0, static_cast<__nv_bfloat16 *>(op.hi),
+                          c->stream),
                "emu_digits");
   });
 }
@@ -1530,7 +1530,9 @@ void build_split_persistent(mlcc3_ctx *c) {
   split_pairs(c, "Tl", c->Tl, s.NO, s.ti, s.ta, s.tb, "t");
   make_split(c, "Go:N", c->Go, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, "G");
   make_split(c, "Gx:N", c->Gx, s.no, s.no, s.nv, s.NO, s.oj, s.ok, s.oc, 1, -1.0, Box::Row, "Gb");
-  split_gt(c, "Gb", c->Gb, c->F, 0.5);  // Omega / rho: D slot g_Dbkc with 1/2 F_kc folded in
+  // Omega / rho: D slot g_Dbkc, in the split mode with 1/2 F_kc folded in
+  if (c->emu) split_gt(c, "Gb", c->Gb);
+  else split_gt(c, "Gb", c->Gb, c->F, 0.5);
   split_gt(c, "Gv", c->Gv);
   split_go_T(c, "Gx:T", c->Gx);
   split_go_T(c, "Go:T", c->Go);
@@ -1551,7 +1553,7 @@ SplitOp &make_split_k2(mlcc3_ctx *c, const std::string &key, const double *src, 
   if (c->emu) {
     make_digits(c, op, key,
                 EmuView{src, (int)D0, 1, (int)D1, (int)D1, (int)(K1 * K2), (int)K2, s0, 0, 0, s1, sk1, sk2},
-                Kp, false, slot, nullptr, 0.0, false, scales_made);
+                Kp, false, slot, scales_made);
   } else {
   op.hi = c->raw("split:" + key + ":hi", n * 2);
   op.lo = c->raw("split:" + key + ":lo", n * 2);
@@ -1612,8 +1614,8 @@ void split_chol_kpairs(mlcc3_ctx *c) {
 }
 
 // G[k][b][c][D] (Gv-like) transposed to [k][D][(b,c)] and [k][D][(c,b)].
-// The optional F[k][c] (with coefficient fcoef) is folded in as fcoef delta_{Db} F_kc:
-// the D-slot back-contraction then also carries the F_kc term of the doubles.
+// Split mode: the optional F[k][c] (with coefficient fcoef) is folded in as fcoef delta_{Db}
+// F_kc: the D-slot back-contraction then also carries the F_kc term of the doubles.
 void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const double *F,
               double fcoef) {
   S s(c);
@@ -1627,7 +1629,7 @@ void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const doubl
       make_digits(c, op, k2,
                   EmuView{G, (int)s.no, 1, (int)s.NV, (int)s.NV, (int)(s.nv * s.nv), (int)s.nv, s.gk, 0, 0,
                           1, swap ? s.gc : s.gb, swap ? s.gb : s.gc},
-                  Kp, false, kRowsEach + key + ":T", F, fcoef, swap != 0, swap != 0);
+                  Kp, false, kRowsEach + key + ":T", swap != 0);
     } else {
     op.hi = c->raw("split:" + k2 + ":hi", n * 2);
     op.lo = c->raw("split:" + k2 + ":lo", n * 2);
@@ -1664,7 +1666,8 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
   const SplitOp &x1 = layout_XL(c, "bD:XL1", X, 1, BN);
   const SplitOp &x2 = layout_XL(c, "bD:XL2", X, 2, BN);
   if (b.gd_convert) {
-    split_gt(c, b.gd_key, b.GD, b.F, b.F ? b.cF / b.cD : 0.0);
+    if (c->emu) split_gt(c, b.gd_key, b.GD);
+    else split_gt(c, b.gd_key, b.GD, b.F, b.F ? b.cF / b.cD : 0.0);
   }
   TcMaps maps;
   std::memset(&maps, 0, sizeof(maps));
