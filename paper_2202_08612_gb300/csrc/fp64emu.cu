@@ -232,10 +232,17 @@ extern "C" int mlcc3_fp64emu_gemm(const double *A, long long lda, const double *
   cudaMemsetAsync(status, 0, sizeof(int), st);
   cudaMemcpyAsync(base + oi, items.data(), sizeof(TcItem) * items.size(), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(base + os, segs.data(), sizeof(TcSeg) * segs.size(), cudaMemcpyHostToDevice, st);
+  // C is cleared before the operands are sliced (beside the copies above; between kernels
+  // it takes 6 us more), unless it may be one of them
+  auto over = [&](const double *x, long long rows, long long ld) {
+    return C < x + rows * ld && x < C + (long long)M * ldc;
+  };
+  const bool in_place = over(A, M, lda) || over(B, N, ldb);
+  auto clear = [&] { cudaMemset2DAsync(C, sizeof(double) * ldc, 0, sizeof(double) * N, M, st); };
+  if (pieces > 1 && !in_place) clear();
   emu_slice_rows_kernel<<<M, 128, 0, st>>>(A, M, K, lda, Kp, s, ea, sa);
   emu_slice_rows_kernel<<<N, 128, 0, st>>>(B, N, K, ldb, Kp, s, eb, sb);
-  // (after both operands have been read: C may be one of them)
-  if (pieces > 1) cudaMemset2DAsync(C, sizeof(double) * ldc, 0, sizeof(double) * N, M, st);
+  if (pieces > 1 && in_place) clear();
   if (cudaGetLastError() != cudaSuccess) return fail(MLCC3_ERR_CUDA, "slice kernels");
   TcMaps maps{};
   std::string err;

@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(320, 1)
                 const uint32_t add = kk > 0 || cc > 0 ? 1u : 0u;  // 0: first of the chain
                 // A's slice t with B's slices [u0, u1) into the degrees t + u0 .. t + u1 - 1
                 auto mmas = [&](int t, int u0, int u1, int group, uint32_t acc) {
-                  constexpr int W = 256, a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
+                  constexpr int W = FULL ? 256 : 256 / n * n, a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
 #pragma unroll
                   for (int c0 = u0 * n; c0 < u1 * n; c0 += W) {
                     const int nn = u1 * n - c0 < W ? u1 * n - c0 : W;
