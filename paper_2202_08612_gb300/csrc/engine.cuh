@@ -178,11 +178,14 @@ struct mlcc3_ctx {
   };
   std::map<std::string, SplitOp> splits;
   // FP64 mode: the large contractions on the tensor cores (kernels_emu.cuh), from
-  // fp64_tc_from on (emu_rule, by choose_emu); the names of the operands' scales.  A call
-  // whose operands the digits cannot hold to FP64 accuracy, or whose digits find no room,
-  // runs again on the FP64 pipe, where the context stays (emu = false) until the next
-  // integral build
+  // fp64_tc_from on (emu_rule, by choose_emu); the names of the operands' scales.  A kind
+  // of call whose operands the digits could not hold to FP64 accuracy runs on the FP64
+  // pipe until the next integral build (pipe_calls, a bit per kind: another state's or
+  // another quantity's operands are others); where the build's own operands are the
+  // reason, or digits found no room, every call does (leave_digits: emu = false)
   bool emu = false, emu_rule = false;
+  unsigned pipe_calls = 0;
+  void forget_call();
   void leave_digits();
   long long fp64_tc_from = 24;
   std::map<std::string, int> scales;

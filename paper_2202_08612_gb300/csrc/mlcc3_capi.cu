@@ -159,13 +159,23 @@ void mlcc3_ctx::release() {
   tau_key.clear();
 }
 
-// From the tensor cores to the FP64 pipe: the digits' memory is given back, and nothing
-// that a failed call left behind is used again.
-void mlcc3_ctx::leave_digits() {
+// Nothing that a failed call on digits left behind is used again.
+void mlcc3_ctx::forget_call() {
   check_cuda(cudaStreamSynchronize(stream), "sync before the FP64 pipe");
   cudaGetLastError();
-  emu = false;
   addr_gen += 1;
+  for (TriSlot &t : tri) t = TriSlot{};
+  tau_valid = false;
+  tau_key.clear();
+  dld_pending.clear();
+  pending_out.clear();
+  omega_dev = nullptr;
+}
+
+// From the tensor cores to the FP64 pipe: the digits' memory is given back.
+void mlcc3_ctx::leave_digits() {
+  forget_call();
+  emu = false;
   for (auto it = scratch.begin(); it != scratch.end();) {
     if (it->first.compare(0, 7, "digits:") != 0) {
       ++it;
@@ -175,12 +185,6 @@ void mlcc3_ctx::leave_digits() {
     it = scratch.erase(it);
   }
   splits.clear();
-  for (TriSlot &t : tri) t = TriSlot{};
-  tau_valid = false;
-  tau_key.clear();
-  dld_pending.clear();
-  pending_out.clear();
-  omega_dev = nullptr;
 }
 
 double *mlcc3_ctx::buf(const std::string &name, size_t n) {
@@ -1250,13 +1254,13 @@ SplitOp &make_split(mlcc3_ctx *c, const std::string &key, const double *src, lon
                 EmuView{src, (int)(D0 * D1), (int)D1, (int)D2, (int)D2, (int)K, 1, s0, s1, 0, s2, s3, 0},
                 Kp, scale < 0.0, slot);
   } else {
-  op.hi = c->raw("split:" + key + ":hi", n * 2);
-  op.lo = c->raw("split:" + key + ":lo", n * 2);
-  c->launch("split_bf16_kernel", 0.0, [&] {
-    check_cuda(split_bf16(src, static_cast<__nv_bfloat16 *>(op.hi), static_cast<__nv_bfloat16 *>(op.lo),
-                          D0, D1, D2, K, Kp, s0, s1, s2, s3, scale, c->stream),
-               "split_bf16");
-  });
+    op.hi = c->raw("split:" + key + ":hi", n * 2);
+    op.lo = c->raw("split:" + key + ":lo", n * 2);
+    c->launch("split_bf16_kernel", 0.0, [&] {
+      check_cuda(split_bf16(src, static_cast<__nv_bfloat16 *>(op.hi), static_cast<__nv_bfloat16 *>(op.lo),
+                            D0, D1, D2, K, Kp, s0, s1, s2, s3, scale, c->stream),
+                 "split_bf16");
+    });
   }
   const unsigned long long dims[4] = {(unsigned long long)Kp, (unsigned long long)D2,
                                       (unsigned long long)D1, (unsigned long long)D0};
@@ -1413,7 +1417,7 @@ void triples_split(mlcc3_ctx *c, const std::vector<SplitTerm> &terms,
       for (const auto &g : order) {
         const std::vector<long long> &us = groups[g];
         for (long long tm = 0; tm < ntM; ++tm)
-            for (size_t q0 = 0; q0 < us.size(); q0 += (size_t)G)
+          for (size_t q0 = 0; q0 < us.size(); q0 += (size_t)G)
             for (long long tn = 0; tn < ntN; ++tn) {
               const int nq = (int)std::min<size_t>((size_t)G, us.size() - q0);
               const int c0 = (int)(tn * BW);
@@ -1555,13 +1559,13 @@ SplitOp &make_split_k2(mlcc3_ctx *c, const std::string &key, const double *src, 
                 EmuView{src, (int)D0, 1, (int)D1, (int)D1, (int)(K1 * K2), (int)K2, s0, 0, 0, s1, sk1, sk2},
                 Kp, false, slot, scales_made);
   } else {
-  op.hi = c->raw("split:" + key + ":hi", n * 2);
-  op.lo = c->raw("split:" + key + ":lo", n * 2);
-  c->launch("split_bf16_k2_kernel", 0.0, [&] {
-    check_cuda(split_bf16_k2(src, static_cast<__nv_bfloat16 *>(op.hi), static_cast<__nv_bfloat16 *>(op.lo),
-                             D0, D1, K1, K2, Kp, s0, s1, sk1, sk2, 1.0, c->stream),
-               "split_bf16_k2");
-  });
+    op.hi = c->raw("split:" + key + ":hi", n * 2);
+    op.lo = c->raw("split:" + key + ":lo", n * 2);
+    c->launch("split_bf16_k2_kernel", 0.0, [&] {
+      check_cuda(split_bf16_k2(src, static_cast<__nv_bfloat16 *>(op.hi), static_cast<__nv_bfloat16 *>(op.lo),
+                               D0, D1, K1, K2, Kp, s0, s1, sk1, sk2, 1.0, c->stream),
+                 "split_bf16_k2");
+    });
   }
   // rows over o1 within one o0, or (flat) over the flattened (o0, o1)
   const unsigned long long R = flat ? (unsigned long long)(D0 * D1) : (unsigned long long)D1;
@@ -1631,14 +1635,14 @@ void split_gt(mlcc3_ctx *c, const std::string &key, const double *G, const doubl
                           1, swap ? s.gc : s.gb, swap ? s.gb : s.gc},
                   Kp, false, kRowsEach + key + ":T", swap != 0);
     } else {
-    op.hi = c->raw("split:" + k2 + ":hi", n * 2);
-    op.lo = c->raw("split:" + k2 + ":lo", n * 2);
-    c->launch("split_transpose_kernel", 0.0, [&] {
-      check_cuda(split_gt_launch(G, static_cast<__nv_bfloat16 *>(op.hi),
-                                 static_cast<__nv_bfloat16 *>(op.lo), (int)s.no, (int)s.NV,
-                                 (int)s.nv, (int)Kp, s.gk, s.gb, s.gc, swap, F, fcoef, c->stream),
-                 "split_gt");
-    });
+      op.hi = c->raw("split:" + k2 + ":hi", n * 2);
+      op.lo = c->raw("split:" + k2 + ":lo", n * 2);
+      c->launch("split_transpose_kernel", 0.0, [&] {
+        check_cuda(split_gt_launch(G, static_cast<__nv_bfloat16 *>(op.hi),
+                                   static_cast<__nv_bfloat16 *>(op.lo), (int)s.no, (int)s.NV,
+                                   (int)s.nv, (int)Kp, s.gk, s.gb, s.gc, swap, F, fcoef, c->stream),
+                   "split_gt");
+      });
     }
     const unsigned long long dims[4] = {(unsigned long long)Kp, (unsigned long long)s.NV, 1ULL,
                                         (unsigned long long)s.no};
@@ -1695,22 +1699,22 @@ void tc_back_D(mlcc3_ctx *c, const double *X, const std::vector<Ord> &ords, cons
       for (size_t q0 = 0; q0 < os.size(); q0 += (size_t)G) {
         const int nq = (int)std::min<size_t>((size_t)G, os.size() - q0);
         for (long long t = 0; t < ntD; ++t)
-        for (long long tn = 0; tn < ntN; ++tn) {
-          const Ord &o = *os[q0];
-          pl.tile(0, (int)(128 * t), (int)(BN * tn), o.p * s.bi + o.q * s.bL);
-          pl.items.back().ea = (int)(o.r * s.NV);  // (k, D) scales
-          pl.items.back().nq = nq;
-          for (int q = 1; q < nq; ++q)
-            pl.items.back().qoff[q - 1] = os[q0 + q]->p * s.bi + os[q0 + q]->q * s.bL;
-          pl.seg(g[1], 4 + 2 * g[2], nk, (int)(128 * t), 0, o.r, (int)(BN * tn), 0, (int)(o.off / s.nv3));
-          TcSeg &last = pl.segs.back();
-          last.nb = nq;
-          last.tail = ktail(c, s.nv * s.nv);
-          for (int q = 1; q < nq; ++q) {
-            last.bq[q - 1][0] = 0;
-            last.bq[q - 1][1] = (int)(os[q0 + q]->off / s.nv3);
+          for (long long tn = 0; tn < ntN; ++tn) {
+            const Ord &o = *os[q0];
+            pl.tile(0, (int)(128 * t), (int)(BN * tn), o.p * s.bi + o.q * s.bL);
+            pl.items.back().ea = (int)(o.r * s.NV);  // (k, D) scales
+            pl.items.back().nq = nq;
+            for (int q = 1; q < nq; ++q)
+              pl.items.back().qoff[q - 1] = os[q0 + q]->p * s.bi + os[q0 + q]->q * s.bL;
+            pl.seg(g[1], 4 + 2 * g[2], nk, (int)(128 * t), 0, o.r, (int)(BN * tn), 0, (int)(o.off / s.nv3));
+            TcSeg &last = pl.segs.back();
+            last.nb = nq;
+            last.tail = ktail(c, s.nv * s.nv);
+            for (int q = 1; q < nq; ++q) {
+              last.bq[q - 1][0] = 0;
+              last.bq[q - 1][1] = (int)(os[q0 + q]->off / s.nv3);
+            }
           }
-        }
       }
     }
   }, kcap(c));
@@ -1867,18 +1871,18 @@ void tc_pair(mlcc3_ctx *c, const double *X, const std::string &xkey, const Split
     TcDev dv = tc_plan(c, key, [&](TcPlan &pl) {
       for (long long og = 0; og < s.no; ++og)
         for (long long tm = 0; tm < ntM; ++tm)
-            for (long long tn = 0; tn < ntN; ++tn) {
-              pl.tile(0, (int)(128 * tm), (int)(BN * tn), og * Sg);
-              for (auto &o : ords) {
-                if (occ_of(o, g) != og) continue;
-                const bool ascending = o.sp[vp1] < o.sp[vp2];
-                if (ascending != (cls == 0)) continue;
-                pl.seg(2 * o.sp[vk], 6, nk, (int)(128 * tm), 0, (int)(o.off / s.nv3),
-                       (int)(BN * tn), occ_of(o, b2), occ_of(o, b1));
-                pl.tail(ktail(c, s.nv));
-              }
-              pl.drop_empty_last();
+          for (long long tn = 0; tn < ntN; ++tn) {
+            pl.tile(0, (int)(128 * tm), (int)(BN * tn), og * Sg);
+            for (auto &o : ords) {
+              if (occ_of(o, g) != og) continue;
+              const bool ascending = o.sp[vp1] < o.sp[vp2];
+              if (ascending != (cls == 0)) continue;
+              pl.seg(2 * o.sp[vk], 6, nk, (int)(128 * tm), 0, (int)(o.off / s.nv3),
+                     (int)(BN * tn), occ_of(o, b2), occ_of(o, b1));
+              pl.tail(ktail(c, s.nv));
             }
+            pl.drop_empty_last();
+          }
     }, kcap(c));
     // rows of XM are (smaller, larger) canonical positions: the view pair in
     // order (cls 0) or swapped (cls 1)
@@ -2018,15 +2022,15 @@ void tc_vv(mlcc3_ctx *c, const double *X, const std::string &xkey, const double 
     TcDev dv = tc_plan(c, "tcV:" + okey + ":w" + std::to_string(w), [&](TcPlan &pl) {
       for (long long tm = 0; tm < ntM; ++tm)
         for (long long tn = 0; tn < ntN; ++tn)
-        for (size_t o0 = 0; o0 < os.size(); o0 += G) {
-          pl.tile(0, (int)(128 * tm), (int)(BN * tn), 0);
-          for (size_t i = o0; i < std::min(os.size(), o0 + G); ++i) {
-            const Ord &o = os[i];
-            const int u = (int)(o.off / s.nv3);
-            pl.seg(2 * o.sp[2], 6 + 2 * o.sp[2], nk, (int)(128 * tm), 0, u, (int)(BN * tn), 0, u);
-            pl.tail(ktail(c, s.nv * s.nv));
+          for (size_t o0 = 0; o0 < os.size(); o0 += G) {
+            pl.tile(0, (int)(128 * tm), (int)(BN * tn), 0);
+            for (size_t i = o0; i < std::min(os.size(), o0 + G); ++i) {
+              const Ord &o = os[i];
+              const int u = (int)(o.off / s.nv3);
+              pl.seg(2 * o.sp[2], 6 + 2 * o.sp[2], nk, (int)(128 * tm), 0, u, (int)(BN * tn), 0, u);
+              pl.tail(ktail(c, s.nv * s.nv));
+            }
           }
-        }
     }, kcap(c));
     TcEpi epi = make_epi(out, 2, 128, 0, ld, 1, 1, s.nv, s.nv, alpha * w);
     tc_launch(c, "vv", (int)BN, maps, dv, epi, 2.0 * (double)s.nv3 * (double)s.nv * (double)os.size(),
@@ -2112,8 +2116,7 @@ void tc_chol(mlcc3_ctx *c, const std::vector<CholTerm> &terms, long long nW, lon
         for (long long tn = 0; tn < ntN; ++tn) {
           pl.tile(0, (int)(128 * tm), (int)(BN * tn), w * Sw);
           pl.items.back().eb = (int)(w * nN);  // (w, n) scales
-          for (size_t t = 0; t < terms.size(); ++t)
-          {
+          for (size_t t = 0; t < terms.size(); ++t) {
             pl.seg((int)(4 * t), (int)(4 * t + 2), nk, (int)(128 * tm), 0, 0, (int)(BN * tn),
                    (int)w, 0);
             pl.tail(ktail(c, s.NJ));
@@ -2443,21 +2446,21 @@ static void do_build_integrals(mlcc3_ctx *c, const double *chol_in, const double
   if (tc_mode(c)) {
     tc_integrals(c);  // Gv, Gb on the tensor cores
   } else {
-  c->bstc1(Lt + NO * nmo, Lt + NO * nmo + NO, c->Gv, sh, 1.0, mk_item(0, 0, 0, {1, nmo, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.gk, s.gc, s.gb, 1}), "Gv");
-  // Gb[k][b][c][D] = g_Dbkc: A(k,c;J) = Lt[J][k][NO+c], B(J;b,D) = Lt[J][NO+D][NO+b]
-  c->bstc1(Lt + NO, Lt + NO * nmo + NO, c->Gb, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, 1, nmo}, {s.gk, s.gc, s.gb, 1}), "Gb");
+    c->bstc1(Lt + NO * nmo, Lt + NO * nmo + NO, c->Gv, sh, 1.0, mk_item(0, 0, 0, {1, nmo, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.gk, s.gc, s.gb, 1}), "Gv");
+    // Gb[k][b][c][D] = g_Dbkc: A(k,c;J) = Lt[J][k][NO+c], B(J;b,D) = Lt[J][NO+D][NO+b]
+    c->bstc1(Lt + NO, Lt + NO * nmo + NO, c->Gb, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, 1, nmo}, {s.gk, s.gc, s.gb, 1}), "Gb");
   }
   if (!c->emu) {
-  sh = Shape{};
-  sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.no; sh.N2 = NO; sh.K1 = s.NJ;
-  // Go[j][k][c][L] = g_Ljck: A(k,c;J) = Lt[J][NO+c][k], B(J;j,L) = Lt[J][L][j]
-  c->bstc1(Lt + NO * nmo, Lt, c->Go, sh, 1.0, mk_item(0, 0, 0, {1, nmo, s.lJ, 0, 0}, {s.lJ, 0, 0, 1, nmo}, {s.ok, s.oc, s.oj, 1}), "Go");
-  // Gx[j][k][c][L] = g_jLkc: A(k,c;J) = Lt[J][k][NO+c], B(J;j,L) = Lt[J][j][L]
-  c->bstc1(Lt + NO, Lt, c->Gx, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.ok, s.oc, s.oj, 1}), "Gx");
-  sh = Shape{};
-  sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.no; sh.N2 = s.nv; sh.K1 = s.NJ;
-  // Govov[j][b][k][c] = g_jbkc: A(k,c;J) = Lt[J][k][NO+c], B(J;j,b) = Lt[J][j][NO+b]
-  c->bstc1(Lt + NO, Lt + NO, c->Govov, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.vk, 1, s.vj, s.vb}), "Govov");
+    sh = Shape{};
+    sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.no; sh.N2 = NO; sh.K1 = s.NJ;
+    // Go[j][k][c][L] = g_Ljck: A(k,c;J) = Lt[J][NO+c][k], B(J;j,L) = Lt[J][L][j]
+    c->bstc1(Lt + NO * nmo, Lt, c->Go, sh, 1.0, mk_item(0, 0, 0, {1, nmo, s.lJ, 0, 0}, {s.lJ, 0, 0, 1, nmo}, {s.ok, s.oc, s.oj, 1}), "Go");
+    // Gx[j][k][c][L] = g_jLkc: A(k,c;J) = Lt[J][k][NO+c], B(J;j,L) = Lt[J][j][L]
+    c->bstc1(Lt + NO, Lt, c->Gx, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.ok, s.oc, s.oj, 1}), "Gx");
+    sh = Shape{};
+    sh.M1 = s.no; sh.M2 = s.nv; sh.N1 = s.no; sh.N2 = s.nv; sh.K1 = s.NJ;
+    // Govov[j][b][k][c] = g_jbkc: A(k,c;J) = Lt[J][k][NO+c], B(J;j,b) = Lt[J][j][NO+b]
+    c->bstc1(Lt + NO, Lt + NO, c->Govov, sh, 1.0, mk_item(0, 0, 0, {nmo, 1, s.lJ, 0, 0}, {s.lJ, 0, 0, nmo, 1}, {s.vk, 1, s.vj, s.vb}), "Govov");
   }
   fock_ov(c, c->t1, c->F, "F");
   transpose_tl(c, c->t2c, c->Tl);
@@ -3387,11 +3390,26 @@ static int guarded(F &&f) {
   }
 }
 
+// Kinds of call (mlcc3_ctx::pipe_calls), each with and without the skip rule of a core mask.
+enum Call { kBuild, kOmega, kRight, kLeft, kMultiplier, kDensity, kGroundDensity, kRayleigh };
+static unsigned call_bit(const mlcc3_ctx *c, Call k) { return 1u << (2 * k + (cvs_on(c) ? 1 : 0)); }
+
+// The FP64 pipe for the time of a call that has left the digits.
+struct OnPipe {
+  mlcc3_ctx *c;
+  bool emu;
+  OnPipe(mlcc3_ctx *x, bool pipe) : c(x), emu(x->emu) {
+    if (pipe) c->emu = false;
+  }
+  ~OnPipe() { c->emu = emu; }
+};
+
 // A call on a context, f() and the wait for its results: on the tensor cores' digits where
 // the context uses them and the operands allow it, else on the FP64 pipe.
 template <class F>
-static void run_call(mlcc3_ctx *c, F &&f) {
-  if (c->emu) {
+static void run_call(mlcc3_ctx *c, Call kind, F &&f) {
+  const unsigned bit = call_bit(c, kind);
+  if (c->emu && !(c->pipe_calls & bit)) {
     struct MayRerun {
       mlcc3_ctx *c;
       explicit MayRerun(mlcc3_ctx *x) : c(x) { c->may_rerun = true; }
@@ -3400,6 +3418,7 @@ static void run_call(mlcc3_ctx *c, F &&f) {
         c->ins.clear();
       }
     };
+    int code = 0;
     try {
       MayRerun guard(c);
       f();
@@ -3407,9 +3426,16 @@ static void run_call(mlcc3_ctx *c, F &&f) {
       return;
     } catch (const Error &e) {
       if (e.code != kErrSpread && e.code != MLCC3_ERR_OOM) throw;
+      code = e.code;
     }
-    c->leave_digits();
+    if (kind == kBuild || code == MLCC3_ERR_OOM) {
+      c->leave_digits();
+    } else {
+      c->forget_call();
+      c->pipe_calls |= bit;
+    }
   }
+  OnPipe pipe(c, true);
   f();
   c->finish();
 }
@@ -3506,7 +3532,8 @@ extern "C" int mlcc3_build_integrals(mlcc3_ctx *c, const double *chol, const dou
     if (!c) throw Error{MLCC3_ERR_ARG, "null context"};
     try {
       c->emu = c->emu_rule;
-      run_call(c, [&] { do_build_integrals(c, chol, t1, eps, t2c, t2x); });
+      c->pipe_calls = 0;
+      run_call(c, kBuild, [&] { do_build_integrals(c, chol, t1, eps, t2c, t2x); });
     } catch (...) {
       c->built = false;  // the integral blocks may be incomplete
       throw;
@@ -3517,7 +3544,7 @@ extern "C" int mlcc3_build_integrals(mlcc3_ctx *c, const double *chol, const dou
 extern "C" int mlcc3_triples_omega(mlcc3_ctx *c, double *omega1, double *omega2) {
   return guarded([&] {
     require_built(c);
-    run_call(c, [&] { do_triples_omega(c, omega1, omega2); });
+    run_call(c, kOmega, [&] { do_triples_omega(c, omega1, omega2); });
   });
 }
 
@@ -3528,7 +3555,7 @@ extern "C" int mlcc3_jacobian_right(mlcc3_ctx *c, int n_vec, const double *omega
     require_built(c);
     if (n_vec < 0 || (n_vec > 0 && !omega)) throw Error{MLCC3_ERR_ARG, "bad n_vec/omega"};
     if (n_vec == 0) return;
-    run_call(c, [&] { do_jacobian_right(c, n_vec, omega, R1, R2, rho1, rho2); });
+    run_call(c, kRight, [&] { do_jacobian_right(c, n_vec, omega, R1, R2, rho1, rho2); });
   });
 }
 
@@ -3539,7 +3566,7 @@ extern "C" int mlcc3_jacobian_left(mlcc3_ctx *c, int n_vec, const double *omega,
     require_built(c);
     if (n_vec < 0 || (n_vec > 0 && !omega)) throw Error{MLCC3_ERR_ARG, "bad n_vec/omega"};
     if (n_vec == 0) return;
-    run_call(c, [&] { do_jacobian_left(c, n_vec, omega, L1, L2, sigma1, sigma2); });
+    run_call(c, kLeft, [&] { do_jacobian_left(c, n_vec, omega, L1, L2, sigma1, sigma2); });
   });
 }
 
@@ -3549,7 +3576,7 @@ extern "C" int mlcc3_transition_density(mlcc3_ctx *c, double omega, const double
                                         double *D00_T, double *Dm0_T, double *D0m_T) {
   return guarded([&] {
     require_built(c);
-    run_call(c, [&] { do_transition_density(c, 1, &omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T, D0m_T); });
+    run_call(c, kDensity, [&] { do_transition_density(c, 1, &omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T, D0m_T); });
   });
 }
 
@@ -3561,7 +3588,7 @@ extern "C" int mlcc3_transition_densities(mlcc3_ctx *c, int n_states, const doub
   return guarded([&] {
     require_built(c);
     if (n_states < 1 || !omega) throw Error{MLCC3_ERR_ARG, "bad n_states/omega"};
-    run_call(c, [&] { do_transition_density(c, n_states, omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T,
+    run_call(c, kDensity, [&] { do_transition_density(c, n_states, omega, lam1, lam2, R1, R2, L1, L2, D00_in, D00_T, Dm0_T,
                           D0m_T); });
   });
 }
@@ -3570,7 +3597,7 @@ extern "C" int mlcc3_ground_density(mlcc3_ctx *c, const double *lam1, const doub
                                     double *D00) {
   return guarded([&] {
     require_built(c);
-    run_call(c, [&] { do_ground_density(c, lam1, lam2, D00); });
+    run_call(c, kGroundDensity, [&] { do_ground_density(c, lam1, lam2, D00); });
   });
 }
 
@@ -3584,7 +3611,7 @@ extern "C" int mlcc3_multiplier_transformation(mlcc3_ctx *c, const double *lam1,
     const bool cvs = c->cvs;
     c->cvs = false;
     try {
-      run_call(c, [&] { do_jacobian_left(c, 1, &zero, lam1, lam2, eta1, eta2); });
+      run_call(c, kMultiplier, [&] { do_jacobian_left(c, 1, &zero, lam1, lam2, eta1, eta2); });
     } catch (...) {
       c->cvs = cvs;
       throw;
@@ -3601,7 +3628,7 @@ extern "C" int mlcc3_rayleigh_quotient(mlcc3_ctx *c, double omega, const double 
     if (!R1 || !R2 || !L1 || !L2 || !omega_rq) throw Error{MLCC3_ERR_ARG, "null argument"};
     if (!(std::fabs(omega) < 1e300) || !(std::fabs(sd_part) < 1e300))
       throw Error{MLCC3_ERR_ARG, "omega or sd_part is not finite"};
-    run_call(c, [&] { do_rayleigh(c, omega, R1, R2, L1, L2, sd_part, omega_rq); });
+    run_call(c, kRayleigh, [&] { do_rayleigh(c, omega, R1, R2, L1, L2, sd_part, omega_rq); });
   });
 }
 
@@ -3830,6 +3857,7 @@ void sweep_pass(mlcc3_sweep *sw, bool multi, int only = -1, int nvec_cap = 0) {
     const bool prof = c->prof;
     c->stream = multi ? y.st : sw->s0;
     c->prof = false;  // no per-launch events inside graphs
+    OnPipe pipe(c, (c->pipe_calls & call_bit(c, kRight)) != 0);
     try {
       if (multi) check_cuda(cudaStreamWaitEvent(y.st, sw->fork, 0), "sweep wait");
       c->tau_valid = false;
@@ -4155,8 +4183,14 @@ extern "C" int mlcc3_sweep_run(mlcc3_sweep *sw, const double *omega) {
         bool left = false;
         for (size_t q = 0; q < sw->sys.size(); ++q) {
           mlcc3_ctx *c = sw->sys[q].c;
-          if (!c->emu || (e.code == kErrSpread && !(sw->status_pin[q] & kStatusSpread))) continue;
-          c->leave_digits();
+          if (!c->emu || (c->pipe_calls & call_bit(c, kRight))) continue;
+          if (e.code == kErrSpread && !(sw->status_pin[q] & kStatusSpread)) continue;
+          if (e.code == MLCC3_ERR_OOM) {
+            c->leave_digits();
+          } else {
+            c->forget_call();
+            c->pipe_calls |= call_bit(c, kRight);
+          }
           left = true;
         }
         if (!left) throw;

@@ -1,6 +1,7 @@
 """When an FP64 context's digit products may not be used (operands of too wide a range, no
-room for the digits), the call runs again on the FP64 pipe and the context stays there until
-the next integral build; other errors stay errors."""
+room for the digits), the call runs again on the FP64 pipe, and calls of its kind (all calls,
+if the build or the room was the reason) stay there until the next integral build; other
+errors stay errors."""
 from host_common import run_host
 
 SETUP = """
@@ -23,19 +24,23 @@ def test_wide_range_runs_again_on_the_pipe(tmp_path_factory):
     F.fake_mark(b"emu_gemm", 1, 6, 4)
     assert right() == 0
     s = launches(); assert digits(s) and pipe(s)
-    for call in (left, right):  # the context stays on the pipe
-        assert call() == 0
-        s = launches(); assert not digits(s) and pipe(s)
+    assert right() == 0                    # this kind of call stays on the pipe
+    s = launches(); assert not digits(s) and pipe(s)
+    assert left() == 0                     # another one does not
+    s = launches(); assert digits(s) and not pipe(s)
+    assert right() == 0
+    s = launches(); assert not digits(s) and pipe(s)
     assert L.mlcc3_build_integrals(c, *[x.p for x in inputs]) == 0
     assert digits(launches())
-    assert left() == 0
+    assert right() == 0
     s = launches(); assert digits(s) and not pipe(s)
     # in the build itself: nothing of it stays on digits
     F.fake_mark(b"emu_gemm", 1, 6, 4)
     assert L.mlcc3_build_integrals(c, *[x.p for x in inputs]) == 0
     launches()
-    assert right() == 0
-    s = launches(); assert not digits(s) and pipe(s)
+    for call in (left, right):
+        assert call() == 0
+        s = launches(); assert not digits(s) and pipe(s)
     """)
 
 
@@ -97,4 +102,9 @@ def test_sweep_leaves_the_digits(tmp_path_factory):
     s = launches(); assert digits(s) and pipe(s)
     assert run() == 0
     assert launches() == ["graph", "launch"]
+    assert right() == 0                    # the same kind of call on the first context
+    s = launches(); assert not digits(s) and pipe(s)
+    assert left() == 0
+    s = launches(); assert digits(s) and not pipe(s)
+    assert run() == 0
     """)
