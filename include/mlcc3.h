@@ -67,8 +67,9 @@ extern "C" {
  * once.  An output sum_k a_k b_k errs by less than 2^-47 sum_k |a_k| |b_k|, the
  * bound of IEEE double sums over 64 products: that is checked for every output,
  * and where the operands span too wide a range for it, or are not finite, the
- * call runs again in IEEE double on the FP64 pipe, where the context then stays
- * until the next mlcc3_build_integrals.  MLCC3_SPLIT_BF16X3: integral-amplitude products on the
+ * call runs again in IEEE double on the FP64 pipe, where calls of its kind (those
+ * with and without the skip rule of a core mask apart) then stay until the next
+ * mlcc3_build_integrals.  MLCC3_SPLIT_BF16X3: integral-amplitude products on the
  * tensor cores from hi/lo bfloat16 splits with FP32 accumulation;
  * denominators and final reductions stay in FP64.
  * An FP16 hi/lo split is not offered: FP16's five exponent bits put the low
@@ -264,7 +265,8 @@ void mlcc3_sweep_destroy(mlcc3_sweep *sweep);
  *              and at least this many multiply-adds per launch (M N K summed
  *              over the launch's items) run on 128 x 128 CUDA-core tiles with
  *              FP32 accumulation over K ranges of at most 1024 (summed in
- *              FP64); the others on 64 x 64 tiles.  Default 10^9; 0: never.
+ *              FP64); the others on tiles chosen by their extents, 64 products
+ *              per FP32 sum.  Default 10^9; 0: never.
  *   "fp64_tc_from"  MLCC3_FP64 contexts with at least this many active virtual
  *              orbitals, or n_o n_v at least three times it, and n_o >= 2 run
  *              the O(N_V n_v^3 n_o^3) contractions and the Cholesky-index
@@ -338,8 +340,8 @@ int mlcc3_cnto_matrices(int64_t n_occ, int64_t n_vir, const double *R1, const do
  * Sec. 3 at FP64 accuracy, by error-free splitting after Ozaki, Ogita, Oishi
  * and Rump): every row of A and of B is scaled by a power of two and written
  * as `slices` balanced base-256 digits (integers in [-128, 128], exact in
- * bfloat16); the digit slices are multiplied on tcgen05 with FP32 sums that
- * are exact over K chains of up to 1024, the chains added in FP64; the digit
+ * bfloat16); the digit slices are multiplied on tcgen05 with FP32 sums over K
+ * chains of 256 (exact for t + u <= 3), the chains added as integers; the digit
  * pairs (t, u) with t + u < slices are kept, so the normwise relative error is
  * about 2^-(8 slices) (slices = 5: about 1e-12).  A [M][K] with rows lda
  * apart, B [N][K] rows ldb apart, C [M][N] rows ldc apart, all FP64 device
@@ -368,7 +370,8 @@ int mlcc3_release_workspace(void);
  * index tables) from one fixed 32 MiB device array compiled into the
  * library, which every device that loads the library holds until exit.  It
  * calls no cudaMalloc, cudaFree or other allocating routine.
- * It computes in FP64 (the FP64 kernels of the MLCC3_FP64 mode) and takes
+ * It computes in FP64 on the FP64 pipe, whatever "fp64_tc_from" says (a system
+ * whose mlcc3_triples_omega runs on the tensor cores is far slower here), and takes
  * MLCC3_FP64 contexts only: a split-precision context gets MLCC3_ERR_STATE.
  * Requirements: mlcc3_build_integrals has run on `ctx` (that call allocates,
  * so make it during set-up); omega1/omega2 are device pointers (host arrays

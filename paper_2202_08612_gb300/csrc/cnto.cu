@@ -131,7 +131,7 @@ __global__ void fold_kernel(double *X, long long n, const double *copy, int copi
 // The digits of P's rows serve both: rows i of block a, or rows a (n_o rows apart)
 // of block i, are two tensor maps over the same memory.  K runs in chunks whose
 // digits take at most a gigabyte.  *status: the launches' status bits (with
-// kStatusSpread M and N are left as they were).  39 / 263: 70.3 -> 3.5 ms, error 1.3e-15 -> 7e-17.
+// kStatusSpread M and N are left as they were).  39 / 263: 70.3 -> 3.6 ms, error 1.3e-15 -> 7e-17.
 cudaError_t doubles_by_digits(long long NO, long long NV, const double *R2, double *M, double *N,
                               cudaStream_t st, int *hstatus, std::string *err) {
   using namespace mlcc3;

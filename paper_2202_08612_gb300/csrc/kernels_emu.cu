@@ -1,14 +1,14 @@
 // FP64-accurate contractions on the BF16 tensor cores (sm_103a), after the
 // error-free splitting of Ozaki, Ogita, Oishi and Rump: an operand is an
-// integer of up to 63 bits per element (its value over a power of two that its row or
-// the whole operand shares), held
-// as S balanced base-256 digits, each exact in bfloat16.  Products of digits
-// are integers of at most 2^14, which FP32 sums exactly over 256 of them for
-// the digit degrees t + u <= 3.  Kept are the degrees up to S - 1, and with S = 8 (the
-// FP64 mode) up to 8, which leaves out terms below 2^-69 of full scale per product.
+// integer of up to 63 bits per element (its value over a power of two that its
+// row or the whole operand shares), held as S balanced base-256 digits, each
+// exact in bfloat16.  Products of digits are integers of at most 2^14, which
+// FP32 sums exactly over 256 of them for the digit degrees t + u <= 3.  Kept are
+// the degrees up to S - 1, and with S = 8 (the FP64 mode) up to 8, which leaves
+// out terms below 2^-69 of full scale per product.
 //
 // GB300 retires about two FP64 operations per clock and SM (1.1 TFLOP/s in
-// all), and BF16 on the tensor cores about 1.7 PFLOP/s, so even the 36 digit
+// all), and BF16 on the tensor cores about 1.7 PFLOP/s, so even the 43 digit
 // products of S = 8 leave room for a factor of some twenty over the FP64 pipe.
 #include <cudaTypedefs.h>
 
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(320, 1)
                 const uint32_t add = kk > 0 || cc > 0 ? 1u : 0u;  // 0: first of the chain
                 // A's slice t with B's slices [u0, u1) into the degrees t + u0 .. t + u1 - 1
                 auto mmas = [&](int t, int u0, int u1, int group, uint32_t acc) {
-                  constexpr int W = FULL ? 256 : 256 / n * n, a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
+                  constexpr int W = 256 / n * n, a_slice = AMN ? A_SL / 2 : A_SL, a_step = AMN ? 2048 : 32;
 #pragma unroll
                   for (int c0 = u0 * n; c0 < u1 * n; c0 += W) {
                     const int nn = u1 * n - c0 < W ? u1 * n - c0 : W;

@@ -37,7 +37,7 @@ __device__ __forceinline__ T ld_op(const double *p, int f32, long long i) {
 // that on the FP64 pipe and run on the integer pipe instead.  The next K tile's
 // loads are in flight while the current one is multiplied, its index splits made
 // one tile ahead.  blockIdx.z: the K range of kchunk elements it belongs to (as
-// bstc_f32's callers split K) and the piece of kfine (a multiple of 64) in it.
+// mlcc3_ctx::bstc splits K) and the piece of kfine (a multiple of 64) in it.
 // SHORT: at most 64 products per output, where writing C is the work: a thread's
 // columns lie TX apart (coalesced, but no vector reads of B) and the one FP32 sum
 // needs no FP64 addition of its own.
@@ -227,7 +227,8 @@ __global__ void __launch_bounds__(256, TM * TN <= 1024 && RM == RN ? 3 : TM * TN
 // Of the tiles the one with the least estimated time: per K element its FP32
 // products (128 a clock), its shared-memory reads and its share of the FP64
 // additions, for as many rounds of blocks as the 152 SMs need, plus the latency
-// of a K step that four resident blocks hide from one another.
+// of a K step that four resident blocks hide from one another.  (clk and the latency are
+// estimates by hand from these counts, not fits; every tile is chosen for some shape.)
 cudaError_t launch_bstc32(BstcParams p, int fill, cudaStream_t st) {
   struct Tile {
     int m, n;
@@ -1777,25 +1778,9 @@ __global__ void hilo_kernel(const double *__restrict__ x, float2 *__restrict__ y
 
 namespace mlcc3 {
 
-// Matrix-vector form of the batched strided contraction for a binary32 A (the
-// split mode's triples arrays are permuted views of n_v^3 blocks, so the
-// index that is contiguous in memory may be an output index or a reduction
-// index, depending on the item).  Each block takes one item and picks the
-// mapping whose loads run along the contiguous index:
-//  * an output index contiguous: the 32 lanes take 32 consecutive outputs
-//    along it and the 8 warps split K (sums of the warps added in shared
-//    memory);
-//  * otherwise: lpo lanes per output (about K / 16, 4 to 32; a short
-//    reduction over a whole warp was mostly shuffles and atomics), the lanes
-//    of an output along K with the contiguous K index (if any) the fastest.
-// FP32 products (B binary32 when b32, else converted), 16 per lane summed in
-// FP32 and folded into FP64; one atomic update per output (and per K slice).
-// Grid: x = 4 ceil(M / 8) (the second mapping uses the first quarter; the
-// first splits the extra blocks over K), y = items.
-// The same sums for reductions of two levels (one of the three extents is 1, n the
-// faster one's) whose offsets fit in 32 bits: the
-// running offsets of strided_dot took 32 instructions per element in 64-bit
-// arithmetic and three levels of carries, these 13.
+// strided_dot (below) for reductions of two levels (one of the three extents is 1, n the
+// faster one's) whose offsets fit in 32 bits: its running offsets took 32 instructions per
+// element in 64-bit arithmetic and three levels of carries, these 13.
 template <int U, typename TA, typename TB>
 __device__ __forceinline__ double strided_dot2(const TA *__restrict__ Am, const TB *__restrict__ B, int n,
                                                int ka0, int ka1, int kb0, int kb1, int k0, int kend, int step) {

@@ -616,12 +616,12 @@ std::vector<TripItem> shard_of(const std::vector<TripItem> &list, int count, int
 }
 
 // FP64 mode: the O(N_V n_v^3 n_o^3) contractions on the tensor cores (digit
-// slices; rho and sigma at 20/200/12/60: 1868 -> 82 ms, the densities at
-// 13/101/7/37: 79 -> 6.0 ms, errors against 64 bits as before or smaller) from
+// slices; rho and sigma at 20/200/12/60: 1868 -> 85 ms, the densities at
+// 13/101/7/37: 79 -> 6.1 ms, errors against 64 bits as before or smaller) from
 // fp64_tc_from (24) active virtual orbitals or n_o n_v = 3 fp64_tc_from on (rho and sigma,
-// FP64 pipe against digits: 4/12 0.85 against 1.15 ms, 4/16 1.34 and 1.32, 6/12 1.79 and
-// 1.20, 8/16 4.66 and 1.67, 3/24 1.87 and 1.63; below, a call is launches, and the digits
-// need more of them), where all digits that live at once (digit_bytes) take less than 0.4
+// FP64 pipe against digits at n_o/n_v: 6/12 2.11 and 1.38 ms, 8/9 3.08 and 1.44, 9/8 2.29 and
+// 1.60, 4/18 2.81 and 1.86, 3/24 2.64 and 1.98, 2/24 1.80 and 1.84; below, a call is launches,
+// and the digits need more of them), where all digits that live at once (digit_bytes) take less than 0.4
 // of the card's memory: a rule of sizes alone, so that the same system takes the same path
 // whatever else holds memory.  (Where they find no room all the same, a call runs on the
 // pipe.)
