@@ -152,3 +152,19 @@ def test_weak_rows_stay_on_the_tensor_cores():
         outs.append((c.host(r1), c.host(r2)))
     for x, y in zip(*outs):
         assert np.linalg.norm(x - y) < 1e-12 * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("decades", [0.0, 4.0])
+def test_host_arrays(decades):
+    """Inputs and outputs in host memory, of calls that run once and of ones that run again."""
+    _cuda()
+    c, factor = _fall_off(Case(7, 40, 3, 32, 60, nstates=2, t2_norm=0.3), decades)
+    ref, g = c.context(params={"fp64_tc_from": 2000}), c.context(params={"fp64_tc_from": 1}, device=False)
+    for call, X1, X2 in (("jacobian_right", c.st.R1, c.st.R2), ("jacobian_left", c.st.L1, c.st.L2)):
+        y1, y2 = c.empty_dev(X1.shape), c.empty_dev(X2.shape)
+        getattr(ref, call)(c.st.omega, c.to_dev(X1), c.to_dev(X2), y1, y2)
+        for _ in range(2):
+            z1, z2 = np.full(X1.shape, 7.0), np.full(X2.shape, 7.0)
+            getattr(g, call)(c.st.omega, np.ascontiguousarray(X1), np.ascontiguousarray(X2), z1, z2)
+            for x, y, f in ((z1, c.host(y1), factor["o1"]), (z2, c.host(y2), factor["o2"])):
+                assert np.max(np.abs(x - y) / f) < TOL * np.max(np.abs(y) / f), call
